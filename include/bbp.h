@@ -82,7 +82,8 @@ typedef struct bbp_stats {
   uint64_t head_terms;      /* head terms (modular exponentiations) */
   uint64_t head_launches;   /* head-kernel launches */
   uint64_t kernel_launches; /* all kernel launches */
-  double imad_model;        /* 32-bit integer multiply instructions the head terms need (model) */
+  double imad_model;        /* 32-bit integer multiplies the evaluation needs (model), term by term or, for
+                               a whole query summed by primes, by that form */
   double head_ms;           /* device time of the head launches (profile = 1), else 0 */
 } bbp_stats;
 
@@ -125,7 +126,11 @@ bbp_status bbp_partial_sum_async(bbp_plan p, bbp_formula f, uint32_t denominator
                                  uint64_t k_end, uint64_t n, uint32_t P, uint32_t* d_out_limbs,
                                  void* stream);
 
-/* Bits n .. n+P-1 of pi by Eq. 2.  out: caller-owned ceil(P/8) host bytes, MSB first.
+/* Bits n .. n+P-1 of pi by Eq. 2.  Whole queries by Eq. 2 with 1e8 <= n <= 2^45 and guard
+ * bits to spare are summed over the primes up to n instead of over the terms (partial
+ * fractions of the moduli); the sum is checked on the device, and where it is too close
+ * to a carry to have the term-by-term sum's bits for certain, the terms are summed.  The
+ * bits and the certified count are the term-by-term ones in every case.  out: caller-owned ceil(P/8) host bytes, MSB first.
  * valid_bits (may be NULL): how many leading bits the guard-bit error bound certifies
  * (|S - exact| < N + J + 1 units for N evaluated terms and J series).  Blocks. */
 bbp_status bbp_bits(bbp_plan p, uint64_t n, uint32_t P, uint8_t* out, uint32_t* valid_bits);
@@ -136,7 +141,8 @@ bbp_status bbp_bits_formula(bbp_plan p, bbp_formula f, uint64_t n, uint32_t P, u
 
 /* Device-pointer form: d_out (ceil(P/8) bytes), d_valid (one uint32, may be NULL)
  * and d_limbs (W/32 uint32 of the raw sum, may be NULL) are caller-owned device
- * memory; returns once queued on `stream` (NULL: the plan's stream). */
+ * memory; returns once queued on `stream` (NULL: the plan's stream).  With d_limbs the
+ * terms are summed one by one (the raw sum holds every term's rounding). */
 bbp_status bbp_bits_async(bbp_plan p, bbp_formula f, uint64_t n, uint32_t P, uint8_t* d_out,
                           uint32_t* d_valid, uint32_t* d_limbs, void* stream);
 

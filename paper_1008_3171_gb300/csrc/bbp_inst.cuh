@@ -7,6 +7,9 @@
 #error "define BBP_LMAX (accumulator limbs) before including bbp_inst.cuh"
 #endif
 
+#include <algorithm>
+
+#include "bbp_primes.cuh"
 #include "bbp_tile.cuh"
 
 #define BBP_CAT2(a, b) a##b
@@ -47,7 +50,29 @@ int queue_occupancy_t() {
   return n > 0 ? n : 1;
 }
 
+template <typename K>
+cudaError_t launch_prime_t(K kernel, const PrimeArgs& a, int sms, cudaStream_t s) {
+  int n = 0;
+  const cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, kernel, kHeadThreads, 0);
+  if (e != cudaSuccess) return e;
+  kernel<<<std::max(1, n) * sms, kHeadThreads, 0, s>>>(a);
+  return cudaGetLastError();
+}
+
 }  // namespace
+
+cudaError_t BBP_CAT(launch_prime_l, BBP_LMAX)(const PrimeArgs& a, PrimeKernel k, int sms, cudaStream_t s) {
+  switch (k) {
+    case kPrimes0: return launch_prime_t(prime_kernel<BBP_LMAX, 0>, a, sms, s);
+    case kPrimes1: return launch_prime_t(prime_kernel<BBP_LMAX, 1>, a, sms, s);
+    case kPrimes3: return launch_prime_t(prime_kernel<BBP_LMAX, 3>, a, sms, s);
+    case kSums1: return launch_prime_t(prime_sum_kernel<Arith1, BBP_LMAX>, a, sms, s);
+    case kSums2: return launch_prime_t(prime_sum_kernel<Arith2, BBP_LMAX>, a, sms, s);
+    case kPrimeWarps: return launch_prime_t(prime_power_kernel<Arith1, true, BBP_LMAX>, a, sms, s);
+    case kPowers: return launch_prime_t(prime_power_kernel<Arith2, false, BBP_LMAX>, a, sms, s);
+  }
+  return cudaErrorInvalidValue;
+}
 
 // path 0..3 (kNumPaths), streams 1 or 2 (anything else runs 1)
 cudaError_t BBP_CAT(launch_head_l, BBP_LMAX)(const HeadArgs& a, int path, int streams, int blocks, int threads,

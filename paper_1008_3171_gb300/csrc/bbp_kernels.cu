@@ -78,6 +78,7 @@ __global__ void tail_kernel(const TailArgs A) {
 // The tail ranges of several series in one launch: thread i takes the i-th term of
 // the ranges laid end to end.
 __global__ void tail_set_kernel(const TailSet S) {
+  if (S.gate && *S.gate == 0u) return;
   uint64_t i = static_cast<uint64_t>(blockIdx.x) * blockDim.x + threadIdx.x;
   uint32_t r = 0;
   while (r < S.n && i >= S.a[r].count) i -= S.a[r++].count;
@@ -91,7 +92,8 @@ __global__ void tail_set_kernel(const TailSet S) {
 
 // ---------------------------------------------------------------- fold / finalize
 
-__global__ void zero_slots_kernel(unsigned long long* slots, int L) {
+__global__ void zero_slots_kernel(unsigned long long* slots, int L, const uint32_t* gate) {
+  if (gate && *gate == 0u) return;
   for (int i = threadIdx.x; i < L; i += blockDim.x) slots[i] = 0;
 }
 
@@ -112,8 +114,8 @@ __global__ void fold_limbs_kernel(const unsigned long long* slots, int L, uint32
 }
 
 __global__ void finalize_bits_kernel(const unsigned long long* slots, int L, uint32_t P, uint64_t bound,
-                                     uint8_t* out, uint32_t* valid, uint32_t* out_limbs) {
-  if (threadIdx.x != 0 || blockIdx.x != 0) return;
+                                     uint8_t* out, uint32_t* valid, uint32_t* out_limbs, const uint32_t* gate) {
+  if (threadIdx.x != 0 || blockIdx.x != 0 || (gate && *gate == 0u)) return;
   finalize_into(slots, L, P, bound, out, valid, out_limbs);
 }
 
@@ -257,6 +259,16 @@ cudaError_t launch_head(const HeadArgs& a, int path, int streams, int lmax, int 
   }
 }
 
+cudaError_t launch_prime(const PrimeArgs& a, PrimeKernel k, int lmax, int sms, cudaStream_t s) {
+  switch (lmax) {
+#define BBP_CASE(L) \
+  case L: return launch_prime_l##L(a, k, sms, s);
+    BBP_LMAX_CASES(BBP_CASE)
+#undef BBP_CASE
+    default: return cudaErrorInvalidValue;
+  }
+}
+
 cudaError_t launch_timestamp(unsigned long long* where, cudaStream_t s) {
   timestamp_kernel<<<1, 32, 0, s>>>(where);
   return cudaGetLastError();
@@ -292,8 +304,8 @@ cudaError_t launch_tail_set(const TailSet& set, cudaStream_t s) {
   return cudaGetLastError();
 }
 
-cudaError_t launch_zero_slots(unsigned long long* slots, int L, cudaStream_t s) {
-  zero_slots_kernel<<<1, 64, 0, s>>>(slots, L);
+cudaError_t launch_zero_slots(unsigned long long* slots, int L, cudaStream_t s, const uint32_t* gate) {
+  zero_slots_kernel<<<1, 64, 0, s>>>(slots, L, gate);
   return cudaGetLastError();
 }
 
@@ -303,8 +315,9 @@ cudaError_t launch_fold_limbs(const unsigned long long* slots, int L, uint32_t* 
 }
 
 cudaError_t launch_finalize_bits(const unsigned long long* slots, int L, uint32_t P, uint64_t bound,
-                                 uint8_t* out_bytes, uint32_t* valid_bits, uint32_t* out_limbs, cudaStream_t s) {
-  finalize_bits_kernel<<<1, 32, 0, s>>>(slots, L, P, bound, out_bytes, valid_bits, out_limbs);
+                                 uint8_t* out_bytes, uint32_t* valid_bits, uint32_t* out_limbs, cudaStream_t s,
+                                 const uint32_t* gate) {
+  finalize_bits_kernel<<<1, 32, 0, s>>>(slots, L, P, bound, out_bytes, valid_bits, out_limbs, gate);
   return cudaGetLastError();
 }
 

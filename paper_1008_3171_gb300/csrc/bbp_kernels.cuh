@@ -4,6 +4,8 @@
 #include <cstdint>
 #include <cuda_runtime.h>
 
+#include "bbp_primes.h"
+
 namespace bbp {
 
 // One contiguous run of head terms (exponent e >= 0) of one series:
@@ -25,6 +27,7 @@ struct HeadArgs {
   uint32_t first_max;    // largest first-window value the moduli allow (>= 2^first - 1); a warp
                          // whose top first + 1 exponent bits stay within it takes one more bit
   unsigned long long* slots;  // L carry-save accumulators, limb i at slots[i]
+  const uint32_t* gate;  // head launches: nothing is done when *gate is 0 (NULL: always done)
 };
 
 // Tail terms (e < 0): t = floor(2^(W+e) / m), one thread per term.
@@ -48,6 +51,7 @@ constexpr int kMaxTailSet = 7;
 struct TailSet {
   TailArgs a[kMaxTailSet];
   uint32_t n;  // ranges in use
+  const uint32_t* gate;  // as in HeadArgs
 };
 
 constexpr int kMaxLimbs = 40;    // W <= 1280 bits
@@ -94,6 +98,22 @@ struct BatchDev {
   unsigned long long* done_ns;     // completion time per query (device global timer, ns)
 };
 
+// ---------------------------------------------------------------- prime form
+//
+// Arguments of the prime kernels (bbp_primes.cuh): primes base + list[i], i < *count.
+struct PrimeArgs {
+  const uint32_t* list;
+  const uint32_t* count;
+  uint32_t cap;        // length of the list buffer
+  uint32_t L;          // limbs
+  uint64_t base;
+  uint64_t e;          // exponent of 2 before a part's own constants
+  uint64_t A, B, C;    // largest moduli of the three sums
+  unsigned long long* slots;
+  uint32_t nclasses;
+  PrimeClass classes[kMaxPrimeClasses];
+};
+
 // Launch helpers (defined in bbp_kernels.cu).  They return cudaGetLastError().
 // path: 0 = one-word moduli, bitlen <= 29; 1 = two-word moduli, bitlen <= 46;
 //       2 = two-word moduli, bitlen <= 60; 3 = one-word moduli of 30 or 31 bits.
@@ -102,10 +122,12 @@ cudaError_t launch_head(const HeadArgs& a, int path, int streams, int lmax, int 
                         int threads = kHeadThreads);
 cudaError_t launch_tail(const TailArgs& a, cudaStream_t s);
 cudaError_t launch_tail_set(const TailSet& set, cudaStream_t s);
-cudaError_t launch_zero_slots(unsigned long long* slots, int L, cudaStream_t s);
+// gate: as in HeadArgs
+cudaError_t launch_zero_slots(unsigned long long* slots, int L, cudaStream_t s, const uint32_t* gate = nullptr);
 cudaError_t launch_fold_limbs(const unsigned long long* slots, int L, uint32_t* out_limbs, cudaStream_t s);
 cudaError_t launch_finalize_bits(const unsigned long long* slots, int L, uint32_t P, uint64_t bound,
-                                 uint8_t* out_bytes, uint32_t* valid_bits, uint32_t* out_limbs, cudaStream_t s);
+                                 uint8_t* out_bytes, uint32_t* valid_bits, uint32_t* out_limbs, cudaStream_t s,
+                                 const uint32_t* gate = nullptr);
 // One persistent launch over the head jobs [job_begin, job_end) of one variant;
 // *cursor (relative to job_begin) must be 0.  blocks = resident CTAs.
 cudaError_t launch_queue(const BatchDev& b, uint32_t job_begin, uint32_t job_end, unsigned int* cursor, int path,
@@ -120,13 +142,19 @@ int queue_occupancy(int path, int streams, int lmax);
 int head_lmax_for(int L, int bump = 0);
 // Resident CTAs per SM of that instantiation at `threads` per CTA.
 int head_occupancy(int path, int streams, int lmax, int threads = kHeadThreads);
+// A prime kernel over the primes of `a`, on every SM.  kPrimes0, 1, 3: prime_kernel on
+// that modulus path (primes above A / 23); kSums1, kSums2: prime_sum_kernel in one or two
+// words; kPrimeWarps: prime_power_kernel, a = 1 (p < 2^31); kPowers: a >= 2 (p < 2^23).
+enum PrimeKernel { kPrimes0, kPrimes1, kPrimes3, kSums1, kSums2, kPrimeWarps, kPowers };
+cudaError_t launch_prime(const PrimeArgs& a, PrimeKernel k, int lmax, int sms, cudaStream_t s);
 // Per accumulator class (bbp_lmax*.cu): the launchers the dispatchers above call.
 #define BBP_DECLARE_LMAX(L)                                                                                    \
   cudaError_t launch_head_l##L(const HeadArgs& a, int path, int streams, int blocks, int threads, cudaStream_t s); \
   int head_occupancy_l##L(int path, int streams, int threads);                                                 \
   cudaError_t launch_queue_l##L(const BatchDev& b, uint32_t jb, uint32_t je, unsigned int* cursor, int path,      \
                                 int streams, int blocks, cudaStream_t s);                                      \
-  int queue_occupancy_l##L(int path, int streams);
+  int queue_occupancy_l##L(int path, int streams);                                                             \
+  cudaError_t launch_prime_l##L(const PrimeArgs& a, PrimeKernel k, int sms, cudaStream_t s);
 BBP_DECLARE_LMAX(3)
 BBP_DECLARE_LMAX(4)
 BBP_DECLARE_LMAX(6)

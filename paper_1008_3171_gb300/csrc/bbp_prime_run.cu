@@ -1,0 +1,215 @@
+// Runs the prime form of a query's head sum (bbp_primes.h) on a plan: base primes, the
+// prime powers with long sums, then the primes up to n in lists of bounded length, each
+// sieved and summed.  One list buffer and one stream: a list's kernels end before the
+// next is sieved.
+//
+// Measured on a GB300, whole bbp_bits calls, term by term -> by primes: n = 1e9, P = 128:
+// 15.6 -> 4.28 ms; n = 3e8, P = 1000: 7.87 -> 2.56 ms; n = 4e10, P = 256: 1004 -> 125 ms
+// (of which 60 in prime_kernel, 30 sieving, 35 in the sums mod p).
+#include <cuda_runtime.h>
+
+#include <algorithm>
+#include <cmath>
+#include <new>
+#include <vector>
+
+#include "bbp_kernels.cuh"
+#include "bbp_planner.h"
+#include "bbp_runtime.h"
+#include "bbp_sieve.cuh"
+
+namespace bbp {
+
+namespace {
+
+constexpr uint32_t kMaxBase = (1u << 23) - 1;       // base primes up to here: 564,162 odd ones
+constexpr uint32_t kBaseCap = 565000;
+constexpr uint32_t kMaxListCap = 24u << 20;         // primes of one list (96 MB)
+constexpr uint32_t kMaxLists = 1u << 16;
+constexpr uint64_t kLongSum = 16000;                // primes below A / this take a warp each
+
+uint64_t isqrt(uint64_t v) {
+  uint64_t r = static_cast<uint64_t>(std::sqrt(static_cast<double>(v)));
+  while (r * r > v) --r;
+  while ((r + 1) * (r + 1) <= v) ++r;
+  return r;
+}
+
+}  // namespace
+
+}  // namespace bbp
+
+struct PrimeState {
+  uint32_t* list = nullptr;
+  uint32_t list_cap = 0;
+  uint32_t* primes = nullptr;  // base primes, their reciprocals and counts
+  uint64_t* inv = nullptr;
+  uint32_t* counts = nullptr;  // [0] base primes, [1] those from 67 on, [2] redo, [4 + i] list i
+};
+
+namespace bbp {
+
+namespace {
+constexpr size_t kCountHead = 4;
+
+// Primes of one list for a query at position n: all of them up to the limit.
+uint32_t list_length(uint64_t n) {
+  const double x = static_cast<double>(n);
+  return static_cast<uint32_t>(std::min<double>(kMaxListCap, 1.2 * x / std::log(x) + 4096.0));
+}
+}  // namespace
+
+void release_prime_state(bbp_plan p) {
+  PrimeState* s = p->primes;
+  if (!s) return;
+  cudaFree(s->list);
+  cudaFree(s->primes);
+  cudaFree(s->inv);
+  cudaFree(s->counts);
+  delete s;
+  p->primes = nullptr;
+}
+
+// The workspace for position n; false if it is not there and cannot be made now (a
+// stream capture is going on, or memory is short): the caller then runs term by term.
+bool prime_workspace(bbp_plan p, uint64_t n, cudaStream_t st) {
+  const uint32_t want = list_length(n);
+  if (p->primes && p->primes->list_cap >= want) return true;
+  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(st, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone) {
+    cudaGetLastError();
+    return false;
+  }
+  if (!p->primes) {
+    PrimeState* s = new (std::nothrow) PrimeState();
+    if (!s) return false;
+    p->primes = s;
+    if (cudaMalloc(&s->primes, sizeof(uint32_t) * kBaseCap) != cudaSuccess ||
+        cudaMalloc(&s->inv, sizeof(uint64_t) * kBaseCap) != cudaSuccess ||
+        cudaMalloc(&s->counts, sizeof(uint32_t) * (kCountHead + kMaxLists)) != cudaSuccess) {
+      cudaGetLastError();
+      release_prime_state(p);
+      return false;
+    }
+  }
+  PrimeState* s = p->primes;
+  cudaFree(s->list);  // waits for the work that reads it
+  s->list = nullptr;
+  s->list_cap = 0;
+  if (cudaMalloc(&s->list, sizeof(uint32_t) * want) != cudaSuccess) {
+    cudaGetLastError();
+    return false;
+  }
+  s->list_cap = want;
+  return true;
+}
+
+uint32_t* prime_redo_flag(bbp_plan p) { return p->primes->counts + 2; }
+
+// Adds the prime form of the head terms covered by prime_limits(n - 1) to `slots`, and
+// enqueues the check of the finished sum (the terms it does not cover must be in `slots`
+// already).  *launches counts the kernels.
+bbp_status launch_prime_form(bbp_plan p, uint64_t n, uint32_t W, uint32_t P, uint64_t bound,
+                             unsigned long long* slots, uint8_t* d_out, uint32_t* d_valid, cudaStream_t st,
+                             uint64_t* launches) {
+  PrimeState* S = p->primes;
+  const int lmax = head_lmax_for(static_cast<int>(W / 32));
+  if (lmax == 0) return BBP_EINVAL;
+  const PrimeLimits lim = prime_limits(n - 1);
+  const std::vector<PrimeClass> classes = prime_classes(lim);
+  if (classes.empty() || classes.size() > static_cast<size_t>(kMaxPrimeClasses)) return BBP_EINVAL;
+  PrimeArgs a{};
+  a.L = W / 32;
+  a.A = lim.A;
+  a.B = lim.B;
+  a.C = lim.C;
+  a.slots = slots;
+  a.nclasses = static_cast<uint32_t>(classes.size());
+  std::copy(classes.begin(), classes.end(), a.classes);
+  const uint64_t e = n - 1 + W;
+  cudaError_t err = cudaSuccess;
+  auto chk = [&](cudaError_t r) { if (err == cudaSuccess) err = r; };
+
+  const uint64_t root = isqrt(lim.A);
+  const uint32_t base_to = static_cast<uint32_t>(std::min<uint64_t>(kMaxBase, std::max(root, lim.A / kLongSum)));
+  const uint64_t bottom = classes.back().above;
+  // lists: primes in (base_to, A], cut where their kernel changes
+  struct Span { uint64_t lo, hi; PrimeKernel k; };
+  std::vector<Span> spans;
+  {
+    const uint64_t cuts[] = {bottom, (1ull << 29) - 1, (1ull << 31) - 1, lim.A};
+    std::vector<uint64_t> c(std::begin(cuts), std::end(cuts));
+    std::sort(c.begin(), c.end());
+    uint64_t lo = base_to;
+    for (uint64_t hi : c) {
+      hi = std::min(hi, lim.A);
+      if (hi <= lo) continue;
+      PrimeKernel k;
+      if (hi <= bottom) k = hi < (1ull << 31) ? kSums1 : kSums2;
+      else k = hi < (1ull << 29) ? kPrimes0 : hi < (1ull << 31) ? kPrimes3 : kPrimes1;
+      spans.push_back(Span{lo, hi, k});
+      lo = hi;
+    }
+  }
+  // segments: large enough that a base prime's first multiple is not most of its work
+  const uint32_t words = root < (1u << 16) ? 4096u : root < (1u << 17) ? 8192u : 16384u;
+  const uint64_t seg = 64ull * words;
+  const int sieve_blocks = sieve_occupancy(static_cast<int>(words)) * p->sm_count;
+  struct List { uint64_t base, lo, hi; uint32_t segments; PrimeKernel k; };
+  std::vector<List> lists;
+  for (const Span& s : spans) {
+    uint64_t lo = s.lo;
+    while (lo < s.hi) {
+      const uint64_t base = (lo + 1) / seg * seg;
+      // about 1 / ln x of the numbers are primes; a list that came out longer than the buffer
+      // would be seen by the check
+      const double room = 0.85 * S->list_cap * (std::log(static_cast<double>(std::max<uint64_t>(lo, 1000))) - 1.1);
+      const uint64_t nseg = std::max<uint64_t>(1, static_cast<uint64_t>(room) / seg);
+      const uint64_t hi = std::min(s.hi, base + nseg * seg - 1);
+      lists.push_back(List{base, lo, hi, static_cast<uint32_t>((hi - base) / seg + 1), s.k});
+      lo = hi;
+    }
+  }
+  if (lists.size() > kMaxLists) return BBP_ERANGE;
+
+  chk(cudaMemsetAsync(S->counts, 0, sizeof(uint32_t) * (kCountHead + lists.size()), st));
+  chk(launch_base_primes(base_to, S->primes, S->inv, S->counts, S->counts + 1, st));
+  a.list = S->primes;
+  a.count = S->counts;
+  a.cap = kBaseCap;
+  a.base = 0;
+  a.e = e;
+  chk(launch_prime(a, kPrimeWarps, lmax, p->sm_count, st));
+  chk(launch_prime(a, kPowers, lmax, p->sm_count, st));
+  *launches += 3;
+  SieveArgs v{};
+  v.words = words;
+  v.primes = S->primes + kSieveTinyPrimes;
+  v.inv = S->inv + kSieveTinyPrimes;
+  v.nprimes = S->counts + 1;
+  v.list = S->list;
+  v.cap = S->list_cap;
+  a.list = S->list;
+  a.cap = S->list_cap;
+  for (size_t i = 0; i < lists.size(); ++i) {
+    const List& l = lists[i];
+    v.base = l.base;
+    v.above = l.lo;
+    v.upto = l.hi;
+    v.segments = l.segments;
+    v.count = S->counts + kCountHead + i;
+    chk(launch_sieve(v, static_cast<int>(std::min<uint64_t>(l.segments, sieve_blocks)), st));
+    a.base = l.base;
+    a.count = v.count;
+    // one-word products with H leave a factor 2^-64, two-word ladders start with 2^64, one-word ones with 2^32
+    a.e = l.k == kSums1 || l.k == kSums2 ? e : l.k == kPrimes1 ? e - kPrimeShift : e - kPrimeShift + 32;
+    chk(launch_prime(a, l.k, lmax, p->sm_count, st));
+    *launches += 2;
+  }
+  chk(launch_prime_check(slots, static_cast<int>(W / 32), P, bound, S->counts + kCountHead,
+                         static_cast<uint32_t>(lists.size()), S->list_cap, d_out, d_valid, S->counts + 2, st));
+  *launches += 1;
+  return err == cudaSuccess ? BBP_OK : BBP_ECUDA;
+}
+
+}  // namespace bbp

@@ -1,0 +1,110 @@
+// Host side of the prime form of a query's head sum (bbp_primes.h).
+#include "bbp_primes.h"
+
+#include <algorithm>
+#include <cmath>
+#include <numeric>
+
+#include "bbp_planner.h"
+
+namespace bbp {
+
+namespace {
+
+uint64_t odd_down(uint64_t v) { return v == 0 ? 0 : (v & 1 ? v : v - 1); }
+
+uint32_t pow_mod(uint32_t e, uint32_t m) {  // 2^e mod m
+  uint64_t r = 1 % m;
+  for (uint32_t i = 0; i < e; ++i) r = r * 2 % m;
+  return static_cast<uint32_t>(r);
+}
+
+}  // namespace
+
+PrimeLimits prime_limits(uint64_t d) {
+  // A: exponents d + 3 - m (and d + 1 - m for multiples of 5) are not negative up to
+  // m = d + 1.  C: d - 1 - 5 (m - 1) / 2 is not negative up to 1 + 2 (d - 1) / 5.
+  PrimeLimits l;
+  l.A = odd_down(d + 1);
+  l.B = odd_down(l.A / 5);
+  l.C = d >= 1 ? odd_down(1 + 2 * (d - 1) / 5) : 0;
+  return l;
+}
+
+uint64_t prime_first_k(const PrimeLimits& lim, uint32_t j) {
+  const SeriesDef& s = formula_def(0).s[j];
+  const uint64_t top = s.a == 10 ? lim.A : lim.C;
+  return top < s.b ? 0 : (top - s.b) / s.a + 1;
+}
+
+std::vector<PrimeClass> prime_classes(const PrimeLimits& lim) {
+  std::vector<uint64_t> cuts;  // H changes below each of these
+  for (uint32_t c = 1; c <= kPrimeMaxC + 2; c += 2) cuts.push_back(lim.A / c);
+  const uint64_t bottom = lim.A / (kPrimeMaxC + 2);
+  for (uint32_t c = 1; lim.C / c > bottom; c += 2) cuts.push_back(lim.C / c);
+  for (uint32_t c = 1; lim.B / c > bottom; c += 2) cuts.push_back(lim.B / c);
+  std::sort(cuts.begin(), cuts.end(), std::greater<uint64_t>());
+  cuts.erase(std::unique(cuts.begin(), cuts.end()), cuts.end());
+  std::vector<PrimeClass> out;
+  for (size_t i = 1; i < cuts.size(); ++i) {
+    const uint64_t p = cuts[i] + 1;  // the class: cuts[i] < p <= cuts[i - 1]
+    const uint64_t ca = lim.A / p, cb = lim.B / p, cc = lim.C / p;
+    PrimeClass k{};
+    k.above = cuts[i];
+    uint64_t den = 1;
+    for (uint64_t c = 3; c <= ca; c += 2) den = std::lcm(den, c);
+    int64_t num = 0;
+    for (uint64_t c = 1, e = 0; c <= ca; c += 2, ++e) {
+      const int64_t f = static_cast<int64_t>(den / c);
+      auto scaled = [&](int64_t v, uint64_t bits) { return v * (int64_t{1} << bits); };
+      num += scaled(e & 1 ? -f : f, kPrimeShift + 2 - 2 * e);
+      if (c <= cb) num -= scaled(e & 1 ? -f : f, kPrimeShift - 4 - 10 * e);
+      if (c <= cc) num -= scaled(e & 2 ? -f : f, kPrimeShift - 1 - 5 * e);
+    }
+    k.num = static_cast<uint64_t>(num);
+    k.den = static_cast<uint32_t>(den);
+    uint64_t inv = den;  // Newton-Hensel lifting of den^-1 mod 2^64 (x = den: correct to 3 bits)
+    for (int it = 0; it < 5; ++it) inv *= 2 - den * inv;
+    k.den_inv = inv;
+    k.neg_inv = 0u - static_cast<uint32_t>(inv);
+    k.r2 = pow_mod(64, k.den);
+    k.r3 = pow_mod(96, k.den);
+    uint32_t lambda = 1;
+    uint32_t rest = k.den;
+    for (uint32_t f = 3; f <= kPrimeMaxC; f += 2) {
+      uint32_t q = 1;
+      while (rest % f == 0) {
+        rest /= f;
+        q *= f;
+      }
+      if (q > 1) lambda = std::lcm(lambda, q / f * (f - 1));
+    }
+    k.lambda = lambda - 1;
+    out.push_back(k);
+  }
+  return out;
+}
+
+double prime_form_imad(const PrimeLimits& lim, int limbs) {
+  const double top = static_cast<double>(lim.A), bottom = top / (kPrimeMaxC + 2), root = std::sqrt(top);
+  double total = 0;
+  for (double x = root; x < top;) {  // in steps of 1 % of x
+    const double hi = std::min(top, x * 1.01), mid = 0.5 * (x + hi);
+    const int l = bitlen(static_cast<uint64_t>(mid));
+    const bool wide = l > 31;
+    const double ladder = wide ? 13.0 * (l - 5) : 4.0 * (l - 4), digits = (wide ? 4.0 : 2.0) * limbs + 6.0;
+    const double summands = 0.8 * top / mid;  // odd c up to A / p, and up to 0.2 and 0.4 of that
+    const double per = mid > bottom ? ladder + digits + (wide ? 16.0 : 10.0) : 2.0 * ladder + digits + 12.0 * summands;
+    total += per * (hi - x) / std::log(mid);
+    x = hi;
+  }
+  return total;
+}
+
+bool prime_form_serves(int formula, uint64_t n, uint32_t P, uint32_t W, uint64_t bound) {
+  if (formula != 0 || n < kPrimeMinN || n > kPrimeMaxN) return false;
+  // the result is uncertain for 6 bound in 2^(W - P) positions: ask for less than one in 64
+  return bitlen(bound) + 9 <= static_cast<int>(W - P);
+}
+
+}  // namespace bbp

@@ -1,0 +1,78 @@
+// The prime form of a whole query's head sum (Bellard's formula, Eq. 2), host side:
+// limits, classes and launch arguments.  Pure C++, no CUDA calls.
+//
+// Every head term is 2^e / m mod 1 with m odd.  Splitting 1/m into partial fractions
+// over the prime powers q = p^a that divide m exactly,
+//
+//   1/m = sum_q ((m/q)^-1 mod q) / q   (mod 1),
+//
+// and collecting by q turns the sum over about 0.7 n terms into a sum over the prime
+// powers up to n, about n / ln n of them: one modular exponentiation 2^d mod p per
+// prime serves every term whose modulus p divides.  In terms of odd m,
+//
+//   series 10k+1, 10k+3, 10k+5, 10k+7, 10k+9 together
+//       =  8 sum_m chi(m) 2^(d-m) / m  -  2 sum_m chi(m) 2^(d-5m) / m      (A and B)
+//   series 4k+1, 4k+3 together
+//       = -  sum_m psi(m) 2^(d-1-5(m-1)/2) / m                             (C)
+//
+// with chi(m) = (-1)^((m-1)/2) and psi(m) = +1 for m = 1, 3 mod 8, -1 for 5, 7 mod 8 (the
+// second sum of A, B corrects the multiples of 5, whose sign and exponent differ).
+// For a prime p, m = c p with p not dividing c: 2^(cp) = 2^c mod p, and
+// psi(p) 2^((p-1)/2) = chi(p) mod p, so p's part is
+//
+//   chi(p) 2^d H / p,   H = 4 sum_(c <= A/p) chi(c) 4^-i / c - 1/16 sum_(c <= B/p) chi(c) 1024^-i / c
+//                           - 1/2 sum_(c <= C/p) psi(c) 32^-i / c    (mod p),  c = 2i + 1 odd,
+//
+// where A, B, C are the largest m of the three sums.  H is one rational number for all
+// primes with the same three limits.
+#pragma once
+
+#include <cstdint>
+#include <vector>
+
+namespace bbp {
+
+// Largest moduli of the three sums: every term of a modulus up to these is a head
+// term.  The (at most one) head term above `A` and all tail terms are left to the
+// term-by-term kernels.
+struct PrimeLimits {
+  uint64_t A = 0, B = 0, C = 0;
+};
+PrimeLimits prime_limits(uint64_t d);
+// First k of series j (formula 0) that the prime form does not cover.
+uint64_t prime_first_k(const PrimeLimits& lim, uint32_t j);
+
+// Primes with the same H = num / (den 2^kPrimeShift): those above `above`, up to the
+// previous class's `above`.
+constexpr int kPrimeShift = 24;   // every denominator of H up to kPrimeMaxC divides den 2^24
+constexpr uint32_t kPrimeMaxC = 21;  // classes reach down to A / (kPrimeMaxC + 2)
+constexpr int kMaxPrimeClasses = 20;
+struct PrimeClass {
+  uint64_t above;
+  uint64_t num;      // H den 2^24 < 2^54
+  uint64_t den_inv;  // den^-1 mod 2^64
+  uint32_t den;      // lcm of the odd numbers up to A / p: 1, 3, 15, ... < 2^24
+  uint32_t neg_inv;  // -den^-1 mod 2^32
+  uint32_t r2, r3;   // 2^64 mod den, 2^96 mod den
+  uint32_t lambda;   // exponent of the group of units mod den, minus 1
+  uint32_t pad;
+};
+// Classes in descending order of `above`; the last one's `above` is A / (kPrimeMaxC + 2).
+std::vector<PrimeClass> prime_classes(const PrimeLimits& lim);
+
+// Whether the prime form serves this query: position in range, and the error bound
+// small enough against the guard bits that its result is almost always certain to
+// equal the term-by-term one (see prime_check in bbp_primes.cu).
+bool prime_form_serves(int formula, uint64_t n, uint32_t P, uint32_t W, uint64_t bound);
+
+// 32-bit product halves the prime form multiplies for a query of `limbs` limbs (a model,
+// counted as in head_term_imad, with the primes' number taken as the integral of
+// 1 / ln x): per prime above A / 23 the squarings of its ladder, the product with H and
+// the quotient digits; per prime below, a ladder with a product at each bit, and 12 per
+// summand of its sums.
+double prime_form_imad(const PrimeLimits& lim, int limbs);
+
+constexpr uint64_t kPrimeMinN = 100'000'000;  // below, the terms take no longer (1.4 ms each at 1e8, P = 64)
+constexpr uint64_t kPrimeMaxN = 1ull << 45;   // sieving primes below 2^23
+
+}  // namespace bbp

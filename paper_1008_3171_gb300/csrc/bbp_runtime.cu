@@ -18,6 +18,7 @@
 #include "bbp.h"
 #include "bbp_kernels.cuh"
 #include "bbp_planner.h"
+#include "bbp_primes.h"
 #include "bbp_runtime.h"
 
 using namespace bbp;
@@ -115,7 +116,8 @@ bbp_status bbp_plan_create(bbp_plan* out, const bbp_plan_opts* opts) {
             cudaMalloc(&p->d_bytes, kMaxWorkingBits / 8) == cudaSuccess &&
             cudaMalloc(&p->d_valid, sizeof(uint32_t)) == cudaSuccess &&
             cudaMallocHost(&p->h_stage, 4096) == cudaSuccess &&
-            cudaEventCreate(&p->ev0) == cudaSuccess && cudaEventCreate(&p->ev1) == cudaSuccess;
+            cudaEventCreate(&p->ev0) == cudaSuccess && cudaEventCreate(&p->ev1) == cudaSuccess &&
+            cudaEventCreate(&p->ev2) == cudaSuccess;
   if (!ok) {
     bbp_plan_destroy(p);
     return BBP_ENOMEM;
@@ -131,6 +133,7 @@ bbp_status bbp_plan_destroy(bbp_plan p) {
   release_serve_state(p);
   if (p->stream) cudaStreamSynchronize(p->stream);
   release_batch_state(p);
+  release_prime_state(p);
   cudaFree(p->d_slots);
   cudaFree(p->d_limbs);
   cudaFree(p->d_bytes);
@@ -138,6 +141,7 @@ bbp_status bbp_plan_destroy(bbp_plan p) {
   cudaFreeHost(p->h_stage);
   if (p->ev0) cudaEventDestroy(p->ev0);
   if (p->ev1) cudaEventDestroy(p->ev1);
+  if (p->ev2) cudaEventDestroy(p->ev2);
   if (p->own_stream && p->stream) cudaStreamDestroy(p->stream);
   delete p;
   return BBP_OK;
@@ -171,13 +175,14 @@ namespace bbp {
 
 // Launches every range of `ranges` (all of one query, same W) into `slots`.
 bbp_status launch_ranges(bbp_plan p, int f, uint64_t n, uint32_t W, const std::vector<TermRange>& ranges,
-                         unsigned long long* slots, cudaStream_t st) {
+                         unsigned long long* slots, cudaStream_t st, const uint32_t* gate) {
   const FormulaDef& F = formula_def(f);
   const uint32_t L = W / 32;
   const int lmax = pick_lmax(W, p->limb_bump);
   if (lmax == 0) return BBP_EINVAL;
   float total_ms = 0;
   TailSet tails{};
+  tails.gate = gate;
   for (const TermRange& r : ranges) {
     const SeriesDef& s = F.s[r.j];
     const bool odd_start = F.alternating && (r.k_begin & 1ull);
@@ -220,6 +225,7 @@ bbp_status launch_ranges(bbp_plan p, int f, uint64_t n, uint32_t W, const std::v
     a.first = r.first;
     a.first_max = r.first_max;
     a.slots = slots;
+    a.gate = gate;
     const int streams = head_streams(p, r.path);
     const int warps_per_block = p->cta / 32;
     const int occ = head_occupancy(r.path, streams, lmax, p->cta);
@@ -276,6 +282,82 @@ bbp_status plan_query(bbp_plan p, int f, uint64_t n, uint32_t W, int j_only, uin
 
 extern "C" {
 
+}  // extern "C"
+
+namespace {
+
+// How a whole query is summed: term by term; by the prime form, whose check may ask for
+// the terms (the caller reads the flag); or by the prime form with the term kernels
+// queued behind it, which do nothing unless the check asks for them.
+enum Form { kTerms, kPrimeOnly, kPrimeOrTerms };
+
+// Queues a whole query.  *by_primes (may be NULL): whether the prime form runs.
+bbp_status enqueue_bits(bbp_plan p, int f, uint64_t n, uint32_t P, uint32_t W, uint8_t* d_out, uint32_t* d_valid,
+                        uint32_t* d_limbs, cudaStream_t s, Form form, bool* by_primes) {
+  if (by_primes) *by_primes = false;
+  const FormulaDef& F = formula_def(f);
+  std::vector<TermRange> ranges;
+  uint64_t N = 0;
+  const bbp_status st = plan_query(p, f, n, W, -1, 0, UINT64_MAX, ranges, &N);
+  if (st != BBP_OK) return st;
+  BBP_CUDA(cudaSetDevice(p->device));
+  const int L = static_cast<int>(W / 32);
+  const uint64_t bound = N + F.count + 1;  // |S - exact| < N + J + 1 units
+  // The raw sum itself depends on every term's rounding: only the terms give it.
+  const uint32_t* gate = nullptr;
+  uint64_t prime_launches = 0;
+  float prime_ms = 0;
+  p->stats = bbp_stats{};
+  if (form != kTerms && !d_limbs && prime_form_serves(f, n, P, W, bound) && prime_workspace(p, n, s)) {
+    const PrimeLimits lim = prime_limits(n - 1);
+    std::vector<TermRange> rest;  // tails, and a head term past the limits
+    for (uint32_t j = 0; j < F.count; ++j) {
+      const bbp_status rs = plan_query(p, f, n, W, static_cast<int>(j), prime_first_k(lim, j), UINT64_MAX, rest, nullptr);
+      if (rs != BBP_OK) return rs;
+    }
+    if (p->profile) BBP_CUDA(cudaEventRecord(p->ev2, s));
+    BBP_CUDA(launch_zero_slots(p->d_slots, L, s));
+    const bbp_status ls = launch_ranges(p, f, n, W, rest, p->d_slots, s);
+    if (ls != BBP_OK) return ls;
+    const bbp_status ps = launch_prime_form(p, n, W, P, bound, p->d_slots, d_out, d_valid, s, &prime_launches);
+    if (ps != BBP_OK) return ps;
+    if (p->profile) {
+      BBP_CUDA(cudaEventRecord(p->ev1, s));
+      BBP_CUDA(cudaEventSynchronize(p->ev1));
+      BBP_CUDA(cudaEventElapsedTime(&prime_ms, p->ev2, p->ev1));
+    }
+    prime_launches += p->stats.kernel_launches + 1;
+    gate = prime_redo_flag(p);
+    if (by_primes) *by_primes = true;
+  }
+  if (gate && form == kPrimeOnly) {
+    p->stats = bbp_stats{};
+    for (const TermRange& r : ranges) {
+      p->stats.terms += r.count;
+      if (!r.tail) p->stats.head_terms += r.count;
+    }
+    p->stats.imad_model = prime_form_imad(prime_limits(n - 1), L);
+    p->stats.head_launches = prime_launches;
+    p->stats.kernel_launches = prime_launches;
+    p->stats.head_ms = prime_ms;
+    return BBP_OK;
+  }
+  p->stats = bbp_stats{};
+  BBP_CUDA(launch_zero_slots(p->d_slots, L, s, gate));
+  const bbp_status ls = launch_ranges(p, f, n, W, ranges, p->d_slots, s, gate);
+  if (ls != BBP_OK) return ls;
+  BBP_CUDA(launch_finalize_bits(p->d_slots, L, P, bound, d_out, d_valid, d_limbs, s, gate));
+  p->stats.kernel_launches += 2 + prime_launches;
+  p->stats.head_launches += prime_launches;
+  p->stats.head_ms += prime_ms;
+  if (gate) p->stats.imad_model = prime_form_imad(prime_limits(n - 1), L);
+  return BBP_OK;
+}
+
+}  // namespace
+
+extern "C" {
+
 bbp_status bbp_partial_sum_async(bbp_plan p, bbp_formula f, uint32_t denominator, uint64_t k_begin,
                                  uint64_t k_end, uint64_t n, uint32_t P, uint32_t* d_out_limbs, void* stream) {
   if (!p || !valid_formula(f) || n == 0 || P == 0 || k_begin > k_end || !d_out_limbs) return BBP_EINVAL;
@@ -313,20 +395,8 @@ bbp_status bbp_bits_async(bbp_plan p, bbp_formula f, uint64_t n, uint32_t P, uin
   if (!p || !valid_formula(f) || n == 0 || P == 0 || !d_out) return BBP_EINVAL;
   uint32_t W;
   if (!working_bits(P, p->guard, &W)) return BBP_EINVAL;
-  std::vector<TermRange> ranges;
-  uint64_t N = 0;
-  const bbp_status st = plan_query(p, f, n, W, -1, 0, UINT64_MAX, ranges, &N);
-  if (st != BBP_OK) return st;
-  BBP_CUDA(cudaSetDevice(p->device));
-  cudaStream_t s = stream ? static_cast<cudaStream_t>(stream) : p->stream;
-  p->stats = bbp_stats{};
-  BBP_CUDA(launch_zero_slots(p->d_slots, static_cast<int>(W / 32), s));
-  const bbp_status ls = launch_ranges(p, f, n, W, ranges, p->d_slots, s);
-  if (ls != BBP_OK) return ls;
-  const uint64_t bound = N + formula_def(f).count + 1;  // |S - exact| < N + J + 1 units
-  BBP_CUDA(launch_finalize_bits(p->d_slots, static_cast<int>(W / 32), P, bound, d_out, d_valid, d_limbs, s));
-  p->stats.kernel_launches += 2;
-  return BBP_OK;
+  return enqueue_bits(p, f, n, P, W, d_out, d_valid, d_limbs, stream ? static_cast<cudaStream_t>(stream) : p->stream,
+                      kPrimeOrTerms, nullptr);
 }
 
 bbp_status bbp_shard_range(bbp_formula f, uint32_t denominator, uint64_t n, uint32_t W, uint32_t shard,
@@ -416,15 +486,25 @@ bbp_status bbp_finalize_async(bbp_plan p, bbp_formula f, uint64_t n, uint32_t P,
 
 bbp_status bbp_bits_formula(bbp_plan p, bbp_formula f, uint64_t n, uint32_t P, uint8_t* out, uint32_t* valid_bits) {
   if (!p || !out) return BBP_EINVAL;
-  bbp_status st = bbp_bits_async(p, f, n, P, p->d_bytes, p->d_valid, nullptr, p->stream);
-  if (st != BBP_OK) return st;
+  uint32_t W;
+  if (!valid_formula(f) || n == 0 || P == 0 || !working_bits(P, p->guard, &W)) return BBP_EINVAL;
   const uint32_t nbytes = (P + 7) / 8;
   uint8_t* h = static_cast<uint8_t*>(p->h_stage);
-  BBP_CUDA(cudaMemcpyAsync(h, p->d_bytes, nbytes, cudaMemcpyDeviceToHost, p->stream));
-  BBP_CUDA(cudaMemcpyAsync(h + 2048, p->d_valid, sizeof(uint32_t), cudaMemcpyDeviceToHost, p->stream));
-  BBP_CUDA(cudaStreamSynchronize(p->stream));
+  uint32_t valid = 0;
+  for (Form form = kPrimeOnly;; form = kTerms) {
+    bool by_primes = false;
+    const bbp_status st = enqueue_bits(p, f, n, P, W, p->d_bytes, p->d_valid, nullptr, p->stream, form, &by_primes);
+    if (st != BBP_OK) return st;
+    BBP_CUDA(cudaMemcpyAsync(h, p->d_bytes, nbytes, cudaMemcpyDeviceToHost, p->stream));
+    BBP_CUDA(cudaMemcpyAsync(h + 2048, p->d_valid, sizeof(uint32_t), cudaMemcpyDeviceToHost, p->stream));
+    if (by_primes)
+      BBP_CUDA(cudaMemcpyAsync(h + 2052, prime_redo_flag(p), sizeof(uint32_t), cudaMemcpyDeviceToHost, p->stream));
+    BBP_CUDA(cudaStreamSynchronize(p->stream));
+    uint32_t redo = 0;
+    if (by_primes) std::memcpy(&redo, h + 2052, sizeof(redo));
+    if (redo == 0) break;
+  }
   std::memcpy(out, h, nbytes);
-  uint32_t valid;
   std::memcpy(&valid, h + 2048, sizeof(valid));
   if (valid_bits) *valid_bits = valid;
   if (p->strict && valid < P) return BBP_EINVALID_BITS;

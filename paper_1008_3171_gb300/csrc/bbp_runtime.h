@@ -32,8 +32,9 @@ struct bbp_plan_s {
   uint8_t* d_bytes = nullptr;
   uint32_t* d_valid = nullptr;
   void* h_stage = nullptr;  // 4 KiB pinned staging
-  cudaEvent_t ev0 = nullptr, ev1 = nullptr;
+  cudaEvent_t ev0 = nullptr, ev1 = nullptr, ev2 = nullptr;
   bbp_stats stats{};
+  struct PrimeState* primes = nullptr;  // workspace of the prime form (bbp_prime_run.cu)
   // batched state (bbp_batch.cu) and serving engine (bbp_serve.cu)
   struct BatchState* batch = nullptr;
   struct ServeEngine* serve = nullptr;
@@ -54,7 +55,14 @@ bbp_status cuda_status(cudaError_t e);
 bbp_status plan_query(bbp_plan p, int f, uint64_t n, uint32_t W, int j_only, uint64_t k_lo, uint64_t k_hi,
                       std::vector<TermRange>& ranges, uint64_t* n_terms);
 bbp_status launch_ranges(bbp_plan p, int f, uint64_t n, uint32_t W, const std::vector<TermRange>& ranges,
-                         unsigned long long* slots, cudaStream_t st);
+                         unsigned long long* slots, cudaStream_t st, const uint32_t* gate = nullptr);
+// Prime form of a query's head sum (bbp_prime_run.cu)
+bool prime_workspace(bbp_plan p, uint64_t n, cudaStream_t st);
+uint32_t* prime_redo_flag(bbp_plan p);
+bbp_status launch_prime_form(bbp_plan p, uint64_t n, uint32_t W, uint32_t P, uint64_t bound,
+                             unsigned long long* slots, uint8_t* d_out, uint32_t* d_valid, cudaStream_t st,
+                             uint64_t* launches);
+void release_prime_state(bbp_plan p);
 void load_tune_table(bbp_plan p, const char* path);
 void release_batch_state(bbp_plan p);
 void release_serve_state(bbp_plan p);

@@ -252,6 +252,7 @@ __device__ __forceinline__ void process_tile(const HeadArgs& A, const uint64_t t
 
 template <int LMAX, int PATH, int S>
 __global__ void __launch_bounds__(kHeadThreads) head_kernel(const HeadArgs A, const uint64_t ntiles) {
+  if (A.gate && *A.gate == 0u) return;
   const uint32_t lane = threadIdx.x & 31u;
   const uint32_t wid = threadIdx.x >> 5;
   const uint64_t warp = (static_cast<uint64_t>(blockIdx.x) * blockDim.x + threadIdx.x) >> 5;

@@ -1,0 +1,98 @@
+"""Whole queries summed by primes (bbp_bits, bbp_bits_async without the raw sum) against the
+term-by-term kernels (bbp_accumulate_async + bbp_finalize_async): the same bits and the same
+certified count, tolerance 0, at positions where the prime form's limits, classes, lists and
+words change, and where its check sends the query back to the terms."""
+
+import pytest
+
+pytestmark = pytest.mark.gpu
+
+torch = pytest.importorskip("torch")
+
+
+@pytest.fixture(scope="module")
+def bbp():
+    import paper_1008_3171_gb300 as m
+
+    return m
+
+
+@pytest.fixture(scope="module")
+def plans(bbp):
+    ps = {G: bbp.Plan(device=0, guard_bits=G) for G in (32, 64)}
+    yield ps
+    for p in ps.values():
+        p.close()
+
+
+def by_terms(bbp, plan, n, P):
+    L = plan.working_bits(P) // 32
+    slots = torch.zeros(L, dtype=torch.int64, device="cuda")
+    out = torch.zeros((P + 7) // 8, dtype=torch.uint8, device="cuda")
+    valid = torch.zeros(1, dtype=torch.int32, device="cuda")
+    torch.cuda.synchronize()
+    bbp.bbp_accumulate_async(plan.handle, 0, n, P, 0, 1, slots.data_ptr())
+    bbp.bbp_finalize_async(plan.handle, 0, n, P, slots.data_ptr(), out.data_ptr(), valid.data_ptr())
+    torch.cuda.synchronize()
+    return int.from_bytes(bytes(out.cpu().numpy()), "big") >> (8 * len(out) - P), int(valid[0])
+
+
+def by_async(bbp, plan, n, P):
+    out = torch.zeros((P + 7) // 8, dtype=torch.uint8, device="cuda")
+    valid = torch.zeros(1, dtype=torch.int32, device="cuda")
+    torch.cuda.synchronize()
+    bbp.bbp_bits_async(plan.handle, 0, n, P, out.data_ptr(), valid.data_ptr())
+    torch.cuda.synchronize()
+    return int.from_bytes(bytes(out.cpu().numpy()), "big") >> (8 * len(out) - P), int(valid[0])
+
+
+# the smallest position that takes primes and its neighbours (n - 1 and n - 2 even and odd, A a
+# multiple of 5 or not), 2^27, 2^29 and 2^31 (word and path changes above and below the moduli),
+# A / 23 past 2^31 (sums in two words), several lists
+@pytest.mark.parametrize("n,P", [(10**8 - 1, 64), (10**8, 64), (10**8 + 1, 100), (10**8 + 3, 256), (10**8 + 4, 448),
+                                 (10**8 + 5, 1000), (2**27 + 1, 704), (2**29 - 1, 128), (2**29 + 3, 32),
+                                 (2**31 - 1, 64), (2**31 + 2, 256), (23 * 2**29 + 7, 128), (23 * 2**31 + 11, 256)])
+def test_equals_the_terms(bbp, plans, n, P):
+    assert plans[64].bits(n, P) == by_terms(bbp, plans[64], n, P)
+
+
+def test_check_sends_uncertain_positions_to_the_terms(bbp, plans):
+    """G = 32 and P = 60: 36 bits below the output for a bound of 2^26.1 units, so about one
+    position in 160 lies within three bounds of a carry.  Those and the others agree."""
+    plan, P = plans[32], 60
+    redone = 0
+    for n in range(10**8 + 1, 10**8 + 801):
+        got = plan.bits(n, P)
+        terms_run = plan.stats()["imad_model"] > 4e9   # 7.5e9 for the terms, about 1e9 for the primes
+        redone += terms_run
+        if terms_run or n % 64 == 0:
+            want = by_terms(bbp, plan, n, P)
+            assert got == want, n
+            assert by_async(bbp, plan, n, P) == want, n
+    assert 0 < redone < 40   # 5 expected
+
+
+def test_async_on_a_stream_and_under_capture(bbp, plans):
+    """Queued on a caller's stream, captured into a graph and replayed; a plan whose workspace is
+    not there yet is captured term by term."""
+    n, P = 10**8 + 77, 128
+    want = by_terms(bbp, plans[64], n, P)
+    for fresh in (True, False):
+        plan = bbp.Plan(device=0, guard_bits=64)
+        if not fresh:
+            plan.bits(n, P)
+        out = torch.zeros(P // 8, dtype=torch.uint8, device="cuda")
+        valid = torch.zeros(1, dtype=torch.int32, device="cuda")
+        stream = torch.cuda.Stream()
+        torch.cuda.synchronize()
+        graph = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(graph, stream=stream):
+            bbp.bbp_bits_async(plan.handle, 0, n, P, out.data_ptr(), valid.data_ptr(), 0, stream.cuda_stream)
+        for _ in range(2):
+            out.zero_()
+            valid.zero_()
+            graph.replay()
+            torch.cuda.synchronize()
+            assert (int.from_bytes(bytes(out.cpu().numpy()), "big"), int(valid[0])) == want
+        del graph
+        plan.close()
