@@ -260,6 +260,43 @@ __device__ __forceinline__ void sqr_redc64_p1(uint32_t& x0, uint32_t& x1, uint32
   x1 = r1;
 }
 
+// Half-reduced squaring: x <- (x^2 + u m) / 2^32 with one reduction step, for x^2 < 2^96
+// (x < 2^48): the result is below x^2 / 2^32 + m, which must stay below 2^64.  The first
+// half of sqr_redc64_p1.
+__device__ __forceinline__ void sqr_half64_p1(uint32_t& x0, uint32_t& x1, const Mod64& M) {
+  uint32_t y0, y1;
+  asm("{\n\t"
+      ".reg .u32 a0, a1, d1, s0, h0, b0, b1, q0, u, h, z0, z1, n0, n1, np, cy;\n\t"
+      ".reg .u64 p;\n\t"
+      "mov.u32        a0, %2;\n\t"
+      "mov.u32        a1, %3;\n\t"
+      "mov.u32        n0, %4;\n\t"
+      "mov.u32        n1, %5;\n\t"
+      "mov.u32        np, %6;\n\t"
+      "shf.l.wrap.b32 d1, 0, a1, 1;\n\t"       // 2 x1 (x1 < 2^16)
+      "mul.wide.u32   p, a0, a0;\n\t"
+      "mov.b64        {s0, h0}, p;\n\t"
+      "mul.wide.u32   p, a0, d1;\n\t"
+      "mov.b64        {b0, b1}, p;\n\t"
+      "mul.lo.u32     q0, a1, a1;\n\t"
+      "mul.lo.u32     u, s0, np;\n\t"
+      "mul.hi.u32     h, u, n0;\n\t"
+      "mul.wide.u32   p, u, n1;\n\t"
+      "mov.b64        {z0, z1}, p;\n\t"
+      "add.cc.u32     cy, s0, -1;\n\t"         // carry out = (s0 != 0)
+      "addc.cc.u32    h0, h0, b0;\n\t"
+      "addc.u32       b1, b1, q0;\n\t"
+      "add.cc.u32     h0, h0, z0;\n\t"
+      "addc.u32       b1, b1, z1;\n\t"
+      "add.cc.u32     %0, h0, h;\n\t"
+      "addc.u32       %1, b1, 0;\n\t"
+      "}"
+      : "=r"(y0), "=r"(y1)
+      : "r"(x0), "r"(x1), "r"(M.m0), "r"(M.m1), "r"(M.mp));
+  x0 = y0;
+  x1 = y1;
+}
+
 // x < 2m  ->  x mod m
 __device__ __forceinline__ void reduce_once64(uint32_t& x0, uint32_t& x1, const Mod64& M) {
   uint32_t y0, y1, borrow;

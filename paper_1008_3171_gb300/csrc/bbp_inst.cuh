@@ -52,8 +52,11 @@ int queue_occupancy_t() {
 
 template <typename K>
 cudaError_t launch_prime_t(K kernel, const PrimeArgs& a, int sms, cudaStream_t s) {
+  // the sieve's CTAs need the SM's shared memory while these run
+  cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributePreferredSharedMemoryCarveout,
+                                       cudaSharedmemCarveoutMaxShared);
   int n = 0;
-  const cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, kernel, kHeadThreads, 0);
+  if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, kernel, kHeadThreads, 0);
   if (e != cudaSuccess) return e;
   kernel<<<std::max(1, n) * sms, kHeadThreads, 0, s>>>(a);
   return cudaGetLastError();
@@ -63,9 +66,10 @@ cudaError_t launch_prime_t(K kernel, const PrimeArgs& a, int sms, cudaStream_t s
 
 cudaError_t BBP_CAT(launch_prime_l, BBP_LMAX)(const PrimeArgs& a, PrimeKernel k, int sms, cudaStream_t s) {
   switch (k) {
-    case kPrimes0: return launch_prime_t(prime_kernel<BBP_LMAX, 0>, a, sms, s);
-    case kPrimes1: return launch_prime_t(prime_kernel<BBP_LMAX, 1>, a, sms, s);
-    case kPrimes3: return launch_prime_t(prime_kernel<BBP_LMAX, 3>, a, sms, s);
+    case kPrimes0: return launch_prime_t(prime_kernel<BBP_LMAX, 0, false>, a, sms, s);
+    case kPrimes1: return launch_prime_t(prime_kernel<BBP_LMAX, 1, false>, a, sms, s);
+    case kPrimesHalf: return launch_prime_t(prime_kernel<BBP_LMAX, 1, true>, a, sms, s);
+    case kPrimes3: return launch_prime_t(prime_kernel<BBP_LMAX, 3, false>, a, sms, s);
     case kSums1: return launch_prime_t(prime_sum_kernel<Arith1, BBP_LMAX>, a, sms, s);
     case kSums2: return launch_prime_t(prime_sum_kernel<Arith2, BBP_LMAX>, a, sms, s);
     case kPrimeWarps: return launch_prime_t(prime_power_kernel<Arith1, true, BBP_LMAX>, a, sms, s);

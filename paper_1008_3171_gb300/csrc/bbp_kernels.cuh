@@ -104,6 +104,7 @@ struct BatchDev {
 struct PrimeArgs {
   const uint32_t* list;
   const uint32_t* count;
+  uint32_t* taken;     // primes handed out to warps so far (prime_power_kernel: not used)
   uint32_t cap;        // length of the list buffer
   uint32_t L;          // limbs
   uint64_t base;
@@ -143,9 +144,9 @@ int head_lmax_for(int L, int bump = 0);
 // Resident CTAs per SM of that instantiation at `threads` per CTA.
 int head_occupancy(int path, int streams, int lmax, int threads = kHeadThreads);
 // A prime kernel over the primes of `a`, on every SM.  kPrimes0, 1, 3: prime_kernel on
-// that modulus path (primes above A / 23); kSums1, kSums2: prime_sum_kernel in one or two
+// that modulus path (primes above A / 23), kPrimesHalf on path 1 up to kPrimeHalfMax; kSums1, kSums2: prime_sum_kernel in one or two
 // words; kPrimeWarps: prime_power_kernel, a = 1 (p < 2^31); kPowers: a >= 2 (p < 2^23).
-enum PrimeKernel { kPrimes0, kPrimes1, kPrimes3, kSums1, kSums2, kPrimeWarps, kPowers };
+enum PrimeKernel { kPrimes0, kPrimes1, kPrimesHalf, kPrimes3, kSums1, kSums2, kPrimeWarps, kPowers };
 cudaError_t launch_prime(const PrimeArgs& a, PrimeKernel k, int lmax, int sms, cudaStream_t s);
 // Per accumulator class (bbp_lmax*.cu): the launchers the dispatchers above call.
 #define BBP_DECLARE_LMAX(L)                                                                                    \

@@ -4,8 +4,9 @@
 // next is sieved.
 //
 // Measured on a GB300, whole bbp_bits calls, term by term -> by primes: n = 1e9, P = 128:
-// 15.6 -> 4.28 ms; n = 3e8, P = 1000: 7.87 -> 2.56 ms; n = 4e10, P = 256: 1004 -> 125 ms
-// (of which 60 in prime_kernel, 30 sieving, 35 in the sums mod p).
+// 15.6 -> 2.05 ms; n = 3e8, P = 1000: 7.89 -> 1.20 ms; n = 4e10, P = 256: 1005 -> 89.7 ms;
+// n = 1e12, P = 256: 27.1 -> 2.86 s.  At 4e10 the kernels alone take 52 ms (primes above
+// A / 23), 10 (below), 11 and 2 (prime powers) and 20 (sieve).
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -24,7 +25,7 @@ namespace {
 
 constexpr uint32_t kMaxBase = (1u << 23) - 1;       // base primes up to here: 564,162 odd ones
 constexpr uint32_t kBaseCap = 565000;
-constexpr uint32_t kMaxListCap = 24u << 20;         // primes of one list (96 MB)
+constexpr uint32_t kMaxListCap = 24u << 20;         // primes of one list (96 MB), two lists
 constexpr uint32_t kMaxLists = 1u << 16;
 constexpr uint64_t kLongSum = 16000;                // primes below A / this take a warp each
 
@@ -40,11 +41,15 @@ uint64_t isqrt(uint64_t v) {
 }  // namespace bbp
 
 struct PrimeState {
-  uint32_t* list = nullptr;
+  uint32_t* list[2] = {};
   uint32_t list_cap = 0;
-  uint32_t* primes = nullptr;  // base primes, their reciprocals and counts
-  uint64_t* inv = nullptr;
-  uint32_t* counts = nullptr;  // [0] base primes, [1] those from 67 on, [2] redo, [4 + i] list i
+  uint32_t* primes = nullptr;  // base primes
+  bbp::SievePrime* sieve_primes = nullptr;
+  // [0] base primes, [1] those from 17 on, [2] redo; then the length of each list, then the
+  // primes of each handed out so far
+  uint32_t* counts = nullptr;
+  cudaStream_t sieve = nullptr, sums = nullptr;  // beside the caller's stream
+  cudaEvent_t ready[2] = {}, used[2] = {}, base = nullptr, done = nullptr;
 };
 
 namespace bbp {
@@ -57,14 +62,42 @@ uint32_t list_length(uint64_t n) {
   const double x = static_cast<double>(n);
   return static_cast<uint32_t>(std::min<double>(kMaxListCap, 1.2 * x / std::log(x) + 4096.0));
 }
+
+bool make_state(PrimeState* s) {
+  int low = 0, high = 0;
+  bool ok = cudaDeviceGetStreamPriorityRange(&low, &high) == cudaSuccess &&
+            cudaStreamCreateWithPriority(&s->sieve, cudaStreamNonBlocking, high) == cudaSuccess &&
+            cudaStreamCreateWithPriority(&s->sums, cudaStreamNonBlocking, high) == cudaSuccess &&
+            cudaMalloc(&s->primes, sizeof(uint32_t) * kBaseCap) == cudaSuccess &&
+            cudaMalloc(&s->sieve_primes, sizeof(SievePrime) * kBaseCap) == cudaSuccess &&
+            cudaMalloc(&s->counts, sizeof(uint32_t) * (kCountHead + 2 * kMaxLists)) == cudaSuccess;
+  auto event = [&](cudaEvent_t* e) {
+    ok = ok && cudaEventCreateWithFlags(e, cudaEventDisableTiming) == cudaSuccess;
+  };
+  for (cudaEvent_t& e : s->ready) event(&e);
+  for (cudaEvent_t& e : s->used) event(&e);
+  event(&s->base);
+  event(&s->done);
+  return ok;
+}
 }  // namespace
 
 void release_prime_state(bbp_plan p) {
   PrimeState* s = p->primes;
   if (!s) return;
-  cudaFree(s->list);
+  if (s->sieve) cudaStreamSynchronize(s->sieve);
+  if (s->sums) cudaStreamSynchronize(s->sums);
+  for (cudaEvent_t e : s->ready)
+    if (e) cudaEventDestroy(e);
+  for (cudaEvent_t e : s->used)
+    if (e) cudaEventDestroy(e);
+  if (s->base) cudaEventDestroy(s->base);
+  if (s->done) cudaEventDestroy(s->done);
+  if (s->sieve) cudaStreamDestroy(s->sieve);
+  if (s->sums) cudaStreamDestroy(s->sums);
+  for (uint32_t* l : s->list) cudaFree(l);
   cudaFree(s->primes);
-  cudaFree(s->inv);
+  cudaFree(s->sieve_primes);
   cudaFree(s->counts);
   delete s;
   p->primes = nullptr;
@@ -81,24 +114,23 @@ bool prime_workspace(bbp_plan p, uint64_t n, cudaStream_t st) {
     return false;
   }
   if (!p->primes) {
-    PrimeState* s = new (std::nothrow) PrimeState();
-    if (!s) return false;
-    p->primes = s;
-    if (cudaMalloc(&s->primes, sizeof(uint32_t) * kBaseCap) != cudaSuccess ||
-        cudaMalloc(&s->inv, sizeof(uint64_t) * kBaseCap) != cudaSuccess ||
-        cudaMalloc(&s->counts, sizeof(uint32_t) * (kCountHead + kMaxLists)) != cudaSuccess) {
+    p->primes = new (std::nothrow) PrimeState();
+    if (!p->primes) return false;
+    if (!make_state(p->primes)) {
       cudaGetLastError();
       release_prime_state(p);
       return false;
     }
   }
   PrimeState* s = p->primes;
-  cudaFree(s->list);  // waits for the work that reads it
-  s->list = nullptr;
   s->list_cap = 0;
-  if (cudaMalloc(&s->list, sizeof(uint32_t) * want) != cudaSuccess) {
-    cudaGetLastError();
-    return false;
+  for (uint32_t*& l : s->list) {
+    cudaFree(l);  // waits for the work that reads it
+    l = nullptr;
+    if (cudaMalloc(&l, sizeof(uint32_t) * want) != cudaSuccess) {
+      cudaGetLastError();
+      return false;
+    }
   }
   s->list_cap = want;
   return true;
@@ -137,7 +169,7 @@ bbp_status launch_prime_form(bbp_plan p, uint64_t n, uint32_t W, uint32_t P, uin
   struct Span { uint64_t lo, hi; PrimeKernel k; };
   std::vector<Span> spans;
   {
-    const uint64_t cuts[] = {bottom, (1ull << 29) - 1, (1ull << 31) - 1, lim.A};
+    const uint64_t cuts[] = {bottom, (1ull << 29) - 1, (1ull << 31) - 1, kPrimeHalfMax, lim.A};
     std::vector<uint64_t> c(std::begin(cuts), std::end(cuts));
     std::sort(c.begin(), c.end());
     uint64_t lo = base_to;
@@ -146,15 +178,13 @@ bbp_status launch_prime_form(bbp_plan p, uint64_t n, uint32_t W, uint32_t P, uin
       if (hi <= lo) continue;
       PrimeKernel k;
       if (hi <= bottom) k = hi < (1ull << 31) ? kSums1 : kSums2;
-      else k = hi < (1ull << 29) ? kPrimes0 : hi < (1ull << 31) ? kPrimes3 : kPrimes1;
+      else k = hi < (1ull << 29) ? kPrimes0 : hi < (1ull << 31) ? kPrimes3 : hi <= kPrimeHalfMax ? kPrimesHalf : kPrimes1;
       spans.push_back(Span{lo, hi, k});
       lo = hi;
     }
   }
-  // segments: large enough that a base prime's first multiple is not most of its work
-  const uint32_t words = root < (1u << 16) ? 4096u : root < (1u << 17) ? 8192u : 16384u;
-  const uint64_t seg = 64ull * words;
-  const int sieve_blocks = sieve_occupancy(static_cast<int>(words)) * p->sm_count;
+  constexpr uint32_t entries = 64u << 10;
+  const uint64_t seg = 30ull * entries;
   struct List { uint64_t base, lo, hi; uint32_t segments; PrimeKernel k; };
   std::vector<List> lists;
   for (const Span& s : spans) {
@@ -164,7 +194,10 @@ bbp_status launch_prime_form(bbp_plan p, uint64_t n, uint32_t W, uint32_t P, uin
       // about 1 / ln x of the numbers are primes; a list that came out longer than the buffer
       // would be seen by the check
       const double room = 0.85 * S->list_cap * (std::log(static_cast<double>(std::max<uint64_t>(lo, 1000))) - 1.1);
-      const uint64_t nseg = std::max<uint64_t>(1, static_cast<uint64_t>(room) / seg);
+      uint64_t nseg = std::max<uint64_t>(1, static_cast<uint64_t>(room) / seg);
+      // whole waves of the sieve's CTAs, eight a segment, one an SM beside the primes' kernels
+      const uint64_t wave = std::max<uint64_t>(1, static_cast<uint64_t>(p->sm_count) / 8);
+      if (nseg > wave) nseg -= nseg % wave;
       const uint64_t hi = std::min(s.hi, base + nseg * seg - 1);
       lists.push_back(List{base, lo, hi, static_cast<uint32_t>((hi - base) / seg + 1), s.k});
       lo = hi;
@@ -172,42 +205,55 @@ bbp_status launch_prime_form(bbp_plan p, uint64_t n, uint32_t W, uint32_t P, uin
   }
   if (lists.size() > kMaxLists) return BBP_ERANGE;
 
-  chk(cudaMemsetAsync(S->counts, 0, sizeof(uint32_t) * (kCountHead + lists.size()), st));
-  chk(launch_base_primes(base_to, S->primes, S->inv, S->counts, S->counts + 1, st));
+  // The caller's stream runs the lists' kernels, the sieve runs one list ahead on its own
+  // stream, the prime powers (few, with long chains) run beside them on a third.
+  const size_t nl = lists.size();
+  uint32_t* const lengths = S->counts + kCountHead;
+  chk(cudaMemsetAsync(S->counts, 0, sizeof(uint32_t) * (kCountHead + 2 * nl), st));
+  chk(launch_base_primes(base_to, S->primes, S->sieve_primes, S->counts, S->counts + 1, st));
+  chk(cudaEventRecord(S->base, st));
+  chk(cudaStreamWaitEvent(S->sieve, S->base, 0));
+  chk(cudaStreamWaitEvent(S->sums, S->base, 0));
   a.list = S->primes;
   a.count = S->counts;
   a.cap = kBaseCap;
   a.base = 0;
   a.e = e;
-  chk(launch_prime(a, kPrimeWarps, lmax, p->sm_count, st));
-  chk(launch_prime(a, kPowers, lmax, p->sm_count, st));
+  chk(launch_prime(a, kPowers, lmax, p->sm_count, S->sums));
+  chk(launch_prime(a, kPrimeWarps, lmax, p->sm_count, S->sums));
+  chk(cudaEventRecord(S->done, S->sums));
   *launches += 3;
   SieveArgs v{};
-  v.words = words;
-  v.primes = S->primes + kSieveTinyPrimes;
-  v.inv = S->inv + kSieveTinyPrimes;
+  v.entries = entries;
+  v.primes = S->sieve_primes + kSieveTinyPrimes;
   v.nprimes = S->counts + 1;
-  v.list = S->list;
   v.cap = S->list_cap;
-  a.list = S->list;
   a.cap = S->list_cap;
-  for (size_t i = 0; i < lists.size(); ++i) {
+  for (size_t i = 0; i < nl; ++i) {
     const List& l = lists[i];
+    const size_t slot = i & 1;
+    if (i >= 2) chk(cudaStreamWaitEvent(S->sieve, S->used[slot], 0));  // the buffer's last list is done
+    v.list = S->list[slot];
     v.base = l.base;
     v.above = l.lo;
     v.upto = l.hi;
     v.segments = l.segments;
-    v.count = S->counts + kCountHead + i;
-    chk(launch_sieve(v, static_cast<int>(std::min<uint64_t>(l.segments, sieve_blocks)), st));
+    v.count = lengths + i;
+    chk(launch_sieve(v, p->sm_count, S->sieve));
+    chk(cudaEventRecord(S->ready[slot], S->sieve));
+    chk(cudaStreamWaitEvent(st, S->ready[slot], 0));
+    a.list = S->list[slot];
     a.base = l.base;
-    a.count = v.count;
-    // one-word products with H leave a factor 2^-64, two-word ladders start with 2^64, one-word ones with 2^32
-    a.e = l.k == kSums1 || l.k == kSums2 ? e : l.k == kPrimes1 ? e - kPrimeShift : e - kPrimeShift + 32;
+    a.count = lengths + i;
+    a.taken = lengths + nl + i;
+    a.e = l.k == kSums1 || l.k == kSums2 ? e : e - kPrimeShift + 64;  // the product with H leaves a factor 2^-64
     chk(launch_prime(a, l.k, lmax, p->sm_count, st));
-    *launches += 2;
+    chk(cudaEventRecord(S->used[slot], st));
+    *launches += 3;
   }
-  chk(launch_prime_check(slots, static_cast<int>(W / 32), P, bound, S->counts + kCountHead,
-                         static_cast<uint32_t>(lists.size()), S->list_cap, d_out, d_valid, S->counts + 2, st));
+  chk(cudaStreamWaitEvent(st, S->done, 0));
+  chk(launch_prime_check(slots, static_cast<int>(W / 32), P, bound, lengths, static_cast<uint32_t>(nl), S->list_cap,
+                         d_out, d_valid, S->counts + 2, st));
   *launches += 1;
   return err == cudaSuccess ? BBP_OK : BBP_ECUDA;
 }

@@ -24,23 +24,24 @@ namespace bbp {
 
 // ---------------------------------------------------------------- primes above A / 23
 
-// One prime's residue from the ladder: the exponent is reduced into
-//   V = e mod (p - 1) - (p - 1) - K,   K = (RB - l) 2^j,
-// so that its top, t = (V >> j) + RB, lies in [0, l): 2^t is below 2 p, needs no
-// reduction, and stands for 2^(t - RB) in Montgomery form.  The ladder then takes the
-// remaining j = l - 5 (two words) or l - 4 (one word) bits: no R mod p is needed and
-// the first five bits cost no squaring.  l is the warp's largest bit length;
-// p - 1 <= l 2^j = K' keeps every V of the warp in the window.
-template <int PATH>
-__device__ __forceinline__ uint64_t reduced_exponent(uint64_t e, uint64_t p1, int l, int j) {
-  constexpr int RB = PathTraits<PATH>::kRBits;
-  const uint64_t a = e + (static_cast<uint64_t>(RB - l) << j);
+// One prime's residue from the ladder.  Every factor in it is a power of two, so a value
+// is followed by its exponent f alone: start at x = 2^f with f = t in [0, l) (below 2 p, no
+// reduction), and each squaring with a reduction by 2^r and a window shift s takes f to
+// 2 f - r + s.  After j squarings f = t 2^j + S - OFF, S collecting the shifts (j bits) and
+// OFF the reductions, and this has to be e mod p - 1.  So t and S are the top and the low
+// j bits of u = e + OFF mod (p - 1), taken in the window [l 2^j - (p - 1), l 2^j): j = l - 5
+// (two words) or l - 4 (one word) makes l 2^j >= p - 1.  l is the warp's largest bit
+// length; no 2^64 mod p is needed, and the first five bits cost no squaring.
+//
+// `off` is OFF - l 2^j, `p1` is p - 1.
+__device__ __forceinline__ uint64_t reduced_exponent(uint64_t e, int64_t off, uint64_t p1, uint64_t top) {
+  const uint64_t a = e + static_cast<uint64_t>(off);
   // floor(a / (p - 1)), at most about 60: the single-precision quotient is off by at most one
   uint32_t q = static_cast<uint32_t>(__fdividef(static_cast<float>(a), static_cast<float>(p1)));
   int64_t rem = static_cast<int64_t>(a) - static_cast<int64_t>(q * p1);
   if (rem < 0) rem += static_cast<int64_t>(p1);
   if (rem >= static_cast<int64_t>(p1)) rem -= static_cast<int64_t>(p1);
-  return static_cast<uint64_t>(rem) + (static_cast<uint64_t>(l) << j) - p1;  // V + RB 2^j
+  return static_cast<uint64_t>(rem) + top - p1;
 }
 
 __device__ __forceinline__ uint32_t redc_den(uint64_t t, const PrimeClass& C) {  // < den for t < den 2^32
@@ -73,30 +74,57 @@ __device__ __forceinline__ uint64_t divide_by_den(uint64_t y, uint64_t p, const 
   return (y + p * t) * C.den_inv;  // exact, so the low 64 bits are enough
 }
 
-template <int PATH, int NT>
+// HALF (two words, p below kPrimeHalfMax): the ladder alternates a squaring with one
+// reduction step (r = 32) and one with two (r = 64) and a two-bit window.  With s <= 3 the
+// second leaves x < p + 2^35, the first then x^2 / 2^32 + p < 2^48, whose square still
+// fits three words.  A quarter of the reduction steps fall away: 25 multiply-pipe units for
+// two squarings in the place of 30 (2.0e7 primes near 1e10: 775 -> 717 us).
+template <int PATH, bool HALF, int NT>
 __device__ __forceinline__ void prime_residues(const uint64_t e, const uint64_t (&p)[NT], const bool (&valid)[NT],
                                                const PrimeClass* classes, uint32_t (&x0)[NT], uint32_t (&x1)[NT],
                                                uint32_t (&m0)[NT], uint32_t (&m1)[NT], uint32_t (&mp)[NT]) {
   constexpr bool WIDE = PathTraits<PATH>::kWide;
+  constexpr int RB = PathTraits<PATH>::kRBits;
   int l = 0;
 #pragma unroll
   for (int t = 0; t < NT; ++t) l = max(l, bitlen64(p[t]));
   l = static_cast<int>(__reduce_max_sync(0xffffffffu, static_cast<uint32_t>(l)));
   const int j = WIDE ? l - 5 : l - 4;
+  // OFF: RB (2^j - 1) with every reduction by RB; HALF: f -> 4 f - 128 + s for two squarings,
+  // after one of f -> 2 f - 64 + s if j is odd
+  const uint64_t two_j = 1ull << j;
+  const uint64_t off = HALF ? (j & 1 ? 32 * two_j : 0) + 128 * (((two_j >> (j & 1)) - 1) / 3) : RB * (two_j - 1);
+  const int64_t diff = static_cast<int64_t>(off) - static_cast<int64_t>(l * two_j);
   uint64_t rem[NT];
 #pragma unroll
   for (int t = 0; t < NT; ++t) {
     m0[t] = lo32(p[t]);
     m1[t] = hi32(p[t]);
     mp[t] = neg_inverse32(m0[t]);
-    const uint64_t u = reduced_exponent<PATH>(e, p[t] - 1, l, j);
+    const uint64_t u = reduced_exponent(e, diff, p[t] - 1, l * two_j);
     const uint64_t x = 1ull << static_cast<uint32_t>(u >> j);
     x0[t] = lo32(x);
     x1[t] = hi32(x);
-    rem[t] = u & ((1ull << j) - 1ull);
+    rem[t] = u & (two_j - 1);
   }
   int b = j;
-  if (WIDE) {
+  if (HALF) {
+    uint32_t sh[NT];
+    if (b & 1) {
+      --b;
+#pragma unroll
+      for (int t = 0; t < NT; ++t) sh[t] = static_cast<uint32_t>(rem[t] >> b);
+      square_all<PATH, NT>(x0, x1, m0, m1, mp, sh, true);
+    }
+    while (b > 0) {
+      b -= 2;
+#pragma unroll
+      for (int t = 0; t < NT; ++t) sh[t] = static_cast<uint32_t>(rem[t] >> b) & 3u;
+#pragma unroll
+      for (int t = 0; t < NT; ++t) sqr_half64_p1(x0[t], x1[t], Mod64{m0[t], m1[t], mp[t]});
+      square_all<PATH, NT>(x0, x1, m0, m1, mp, sh, true);
+    }
+  } else if (WIDE) {
     // groups of four bits from the bottom; the first one is short
     const int len = ((b - 1) & 3) + 1;
     b -= len;
@@ -133,7 +161,7 @@ __device__ __forceinline__ void prime_residues(const uint64_t e, const uint64_t 
     const uint32_t n0 = lo32(C.num), n1 = hi32(C.num);
     uint64_t y;
     if (WIDE) {
-      // x num / 2^64 mod p: x < 2 p < 2^47, num < 2^54, so the result is below 2 p
+      // x num / 2^64 mod p: x < 2 p < 2^47, num < 2^54, so the result is below 2 p (x = 2^(e + 64))
       const uint64_t a = static_cast<uint64_t>(x0[t]) * n0;
       const uint64_t b1 = static_cast<uint64_t>(x0[t]) * n1 + hi32(a);
       const uint64_t b2 = static_cast<uint64_t>(x1[t]) * n0 + lo32(b1);
@@ -191,9 +219,16 @@ __device__ __forceinline__ void flush_cta(uint32_t (&acc)[LMAX], uint32_t L, uns
   }
 }
 
+// Hands the next `n` primes of the list to the warp.
+__device__ __forceinline__ uint32_t take_primes(uint32_t* taken, uint32_t n, uint32_t lane) {
+  uint32_t at = 0;
+  if (lane == 0) at = atomicAdd(taken, n);
+  return __shfl_sync(0xffffffffu, at, 0);
+}
+
 constexpr int kPrimeNT = 4;  // primes per thread
 
-template <int LMAX, int PATH>
+template <int LMAX, int PATH, bool HALF>
 __global__ void __launch_bounds__(kHeadThreads) prime_kernel(const __grid_constant__ PrimeArgs A) {
   __shared__ PrimeClass classes[kMaxPrimeClasses];
   for (uint32_t i = threadIdx.x; i < A.nclasses * (sizeof(PrimeClass) / 4); i += blockDim.x)
@@ -201,13 +236,12 @@ __global__ void __launch_bounds__(kHeadThreads) prime_kernel(const __grid_consta
   __syncthreads();
   constexpr int NT = kPrimeNT;
   const uint32_t lane = threadIdx.x & 31u;
-  const uint32_t warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-  const uint32_t nwarps = (gridDim.x * blockDim.x) >> 5;
   const uint32_t count = min(*A.count, A.cap);
   uint32_t acc[LMAX];
 #pragma unroll
   for (int i = 0; i < LMAX; ++i) acc[i] = 0;
-  for (uint32_t at = warp * (32 * NT); at < count; at += nwarps * (32 * NT)) {
+  // warps take their primes as they come: other kernels share the SMs and delay some CTAs
+  for (uint32_t at; (at = take_primes(A.taken, 32 * NT, lane)) < count;) {
     uint64_t p[NT];
     bool valid[NT];
 #pragma unroll
@@ -217,7 +251,7 @@ __global__ void __launch_bounds__(kHeadThreads) prime_kernel(const __grid_consta
       p[t] = A.base + A.list[min(i, count - 1)];
     }
     uint32_t x0[NT], x1[NT], m0[NT], m1[NT], mp[NT];
-    prime_residues<PATH, NT>(A.e, p, valid, classes, x0, x1, m0, m1, mp);
+    prime_residues<PATH, HALF, NT>(A.e, p, valid, classes, x0, x1, m0, m1, mp);
     fold_digits<PathTraits<PATH>::kWide, false, NT, LMAX>(acc, x0, x1, m0, m1, mp);
   }
   flush_cta<LMAX>(acc, A.L, A.slots);
@@ -225,24 +259,24 @@ __global__ void __launch_bounds__(kHeadThreads) prime_kernel(const __grid_consta
 
 // ---------------------------------------------------------------- sums mod p
 
-// Residues mod m < 2^31 in one word, fully reduced.
+// Residues mod m < 2^31 in one word.  Between operations a residue is below m; `lazy`
+// ones are below 2 m.  t 2^-32 mod m is hi(t) - hi(u m) with u = lo(t) m^-1: the low
+// words of t and u m are equal, so nothing carries and m - hi(u m) + hi(t) is one
+// three-operand add.
 struct Arith1 {
   using T = uint32_t;
-  static constexpr int kBits = 32;
-  uint32_t m, mp;
-  __device__ explicit Arith1(uint64_t q) : m(lo32(q)), mp(neg_inverse32(lo32(q))) {}
-  __device__ __forceinline__ T redc(uint64_t t) const {  // t 2^-32 mod m, t < m 2^32
-    const uint32_t u = lo32(t) * mp;
-    const uint32_t r = hi32(t) + __umulhi(u, m) + (lo32(t) != 0u ? 1u : 0u);
-    return min(r, r - m);
+  uint32_t m, mp, minv;  // mp = -m^-1, minv = m^-1 mod 2^32
+  __device__ explicit Arith1(uint64_t q) : m(lo32(q)), mp(neg_inverse32(lo32(q))), minv(0u - mp) {}
+  __device__ __forceinline__ T lazy_redc(uint64_t t) const {  // t 2^-32, t < m 2^32 (or below 2 m for hi(t) < m)
+    return hi32(t) + m - __umulhi(lo32(t) * minv, m);
   }
+  __device__ __forceinline__ T lazy_redc_neg(uint64_t t) const {  // -t 2^-32
+    return __umulhi(lo32(t) * minv, m) + m - hi32(t);
+  }
+  __device__ __forceinline__ T fix(uint32_t r) const { return min(r, r - m); }  // r < 2 m
+  __device__ __forceinline__ T redc(uint64_t t) const { return fix(lazy_redc(t)); }
   __device__ __forceinline__ T mul(T a, T b) const { return redc(static_cast<uint64_t>(a) * b); }
-  // (a c + b) 2^-32 mod m for a word c < 2^32
-  __device__ __forceinline__ T mul_word(T a, uint32_t c, T b) const { return redc(static_cast<uint64_t>(a) * c + b); }
-  __device__ __forceinline__ T add(T a, T b) const {
-    const uint32_t r = a + b;
-    return min(r, r - m);
-  }
+  __device__ __forceinline__ T add(T a, T b) const { return fix(a + b); }
   __device__ __forceinline__ T neg(T a) const { return a != 0u ? m - a : 0u; }
   __device__ __forceinline__ T one() const { return static_cast<T>(r_mod_m_bitserial<32>(m).r); }
   __device__ __forceinline__ T plain(T a) const { return redc(a); }  // out of Montgomery form
@@ -319,14 +353,135 @@ __device__ __forceinline__ uint64_t exponent_mod(int64_t e, uint64_t phi) {
   return static_cast<uint64_t>(r < 0 ? r + static_cast<int64_t>(phi) : r);
 }
 
-// The sum over i0 <= i < i1 of s(i) h^-(i - i0) / c, c = 2 i + 1, as the fraction
-// h num / den, terms whose c is a multiple of p left out.  s(i) changes sign with bit
-// `flip` of i.  From the last term down: num <- c num + s den, den <- h c den, each
-// reduction leaving the same factor 2^-32 in both.  WORD: h is a word (a power of two
-// below 2^11 with h c < 2^32); else h is a residue in Montgomery form.
-template <class A, bool WORD, bool SKIP>
-__device__ __forceinline__ void sum_fraction(const A& M, uint64_t i0, uint64_t i1, uint32_t flip, uint64_t p,
-                                             typename A::T h, typename A::T& num, typename A::T& den) {
+// The three sums (0: A, 1: B, 2: C): the term at i is s(i) w^-i / c, c = 2 i + 1, with
+// w = 4, 1024, 32 for a prime; s(i) = (-1)^i for A and B, +, +, -, - for C.
+__device__ __forceinline__ constexpr uint32_t sum_weight_bits(int kind) { return kind == 0 ? 2u : kind == 1 ? 10u : 5u; }
+
+// Fractions of primes p < 2^31, one a lane: the sum over 0 <= i < n of s(i) w^-i / c as
+// w num / den.  Every lane of the warp must call it.
+//
+// From the last term down: num <- c num + den, den <- w c den, with s carried in den's
+// sign (den <- -w c den where s changes), so a step is two products by a word, two
+// reductions and no selection; each reduction leaves the same factor 2^-32 in both.  The
+// lanes of a warp walk i together from the largest n (c and the constants are uniform, no
+// lane waits for another's loop); until its own n a lane keeps num = den = 0 mod p.  A and C
+// take two terms at once where the constants allow: three products serve two terms.  In
+// multiply-pipe units (low half 1, high half or full product 2) a term costs 10 singly
+// and 6.3 in pairs.  (One term at a time, every lane with its own loop: the primes up to
+// A / 23 of n = 4e10 took 16.9 ms, now 10.)
+template <int KIND>
+__device__ __forceinline__ void prime_sum(const Arith1& M, uint32_t n, uint32_t& num, uint32_t& den) {
+  constexpr uint32_t kW = sum_weight_bits(KIND);
+  // pairs while w^2 c (c - 2) <= 2^31, which keeps every product below m 2^32
+  constexpr uint32_t kPairTop = KIND == 0 ? 11583u : KIND == 2 ? 1447u : 0u;
+  const uint32_t top = __reduce_max_sync(0xffffffffu, n);
+  uint32_t N = 0, D = 0;
+  auto step = [&](uint32_t i) {
+    const uint32_t c = 2u * i + 1u;
+    N = M.lazy_redc(static_cast<uint64_t>(N) * c + D);
+    const uint64_t t = static_cast<uint64_t>(D) * (c << kW);
+    D = KIND != 2 || (i & 1u) == 0u ? M.lazy_redc_neg(t) : M.lazy_redc(t);
+  };
+  uint32_t i = top;
+  while (i > 0 && (kPairTop == 0 || 2u * i - 1u > kPairTop || (i & 1u))) {
+    if (i == n) {
+      N = 0;
+      D = 1;
+    }
+    step(--i);
+  }
+  if (kPairTop != 0 && i > 0) {
+    // pairs (2h + 1, 2h), c c' = 16 h^2 + 16 h + 3:
+    //   A: num <- c c' num - (4 c - c') den, den <- 16 c c' den   (d = -den)
+    //   C: num <- c c' num + (32 c + c') den, den <- -1024 c c' den
+    // a lane whose n is odd starts with its last term, c = 2 n - 1, done: num = 1, den = -w c
+    if (n < i) {
+      N = 0;
+      D = 0;
+    }
+    const bool odd = (n & 1u) != 0u;
+    const uint32_t n0 = odd ? M.lazy_redc(1u) : 0u;
+    const uint32_t d0 = odd ? M.lazy_redc_neg(static_cast<uint64_t>(2u * n - 1u) << kW) : 1u;
+    const uint32_t start = n >> 1;
+    uint32_t d = KIND == 0 ? 2u * M.m - D : D;
+    const uint32_t d_start = KIND == 0 ? 2u * M.m - d0 : d0;
+    const bool late = n <= i;  // starts within the pairs
+    for (uint32_t h = i / 2; h > 0; --h) {
+      if (late && h == start) {
+        N = n0;
+        d = d_start;
+      }
+      const uint32_t g = h - 1u;
+      const uint32_t alpha = 16u * g * h + 3u;
+      const uint32_t beta = KIND == 0 ? 12u * g + 11u : 132u * g + 97u;
+      N = M.lazy_redc(static_cast<uint64_t>(N) * alpha + static_cast<uint64_t>(d) * beta);
+      const uint64_t t = static_cast<uint64_t>(d) * (alpha << (2u * kW));
+      d = KIND == 0 ? M.lazy_redc(t) : M.lazy_redc_neg(t);
+    }
+    D = KIND == 0 ? 2u * M.m - d : d;
+    if (late && start == 0u) {  // n = 1 (or none): no pair
+      N = n0;
+      D = d0;
+    }
+  } else if (n == 0) {
+    N = 0;
+    D = 1;
+  }
+  num = M.fix(N);
+  den = M.fix(D);
+  // den changed sign at every i (A, B) or every even i (C); the first term's own sign
+  const uint32_t flips = KIND != 2 ? n : (n + 1u) / 2u;
+  const uint32_t first = KIND != 2 ? n - 1u : (n - 1u) >> 1;
+  if (n != 0 && ((flips ^ first) & 1u)) num = M.neg(num);
+}
+
+// The same over lo <= i < hi, relative to the term at lo (w num / den with w^-(i - lo)), the
+// terms with c a multiple of p left out; the lanes walk their ranges in step.
+template <int KIND>
+__device__ __forceinline__ void prime_share(const Arith1& M, uint32_t lo, uint32_t hi, uint32_t p, uint32_t& num,
+                                            uint32_t& den) {
+  constexpr uint32_t kW = sum_weight_bits(KIND);
+  const uint32_t steps = __reduce_max_sync(0xffffffffu, hi > lo ? hi - lo : 0u);
+  uint32_t i = lo + steps, N = 0, D = 1;
+  uint32_t skip = hi > lo ? (2u * hi - 1u) / p : 0u;  // the last multiple of p: c = skip p, skip odd
+  skip = skip == 0u ? 0u : ((skip - 1u) | 1u) * p;
+  for (uint32_t k = steps; k > 0; --k) {
+    if (i == hi) {
+      N = 0;
+      D = 1;
+    }
+    --i;
+    uint32_t c = 2u * i + 1u, add = D;
+    if (c == skip) {
+      c = 1u;
+      add = 0u;
+      skip = skip > p ? skip - 2u * p : 0u;
+    }
+    N = M.lazy_redc(static_cast<uint64_t>(N) * c + add);
+    const uint64_t t = static_cast<uint64_t>(D) * (c << kW);
+    if (KIND != 2) {
+      D = M.lazy_redc_neg(t);
+    } else {
+      const uint32_t r = M.lazy_redc(t);
+      D = (i & 1u) ? r : 2u * M.m - r;
+    }
+  }
+  if (hi <= lo) {
+    N = 0;
+    D = 1;
+  }
+  num = M.fix(N);
+  den = M.fix(D);
+  const uint32_t flips = KIND != 2 ? hi - lo : (hi + 1u) / 2u - (lo + 1u) / 2u;
+  const uint32_t first = KIND != 2 ? hi - 1u : (hi - 1u) >> 1;
+  if (hi > lo && ((flips ^ first) & 1u)) num = M.neg(num);
+}
+
+// The same modulo q < 2^46, one term at a time: WORD: q = p and h = w; else q = p^a and
+// h = 2^(bits q) mod q in Montgomery form.  The sign of term i changes with bit `flip` of i.
+template <bool WORD, bool SKIP>
+__device__ __forceinline__ void power_sum(const Arith2& M, uint64_t i0, uint64_t i1, uint32_t flip, uint64_t p,
+                                          uint64_t h, uint64_t& num, uint64_t& den) {
   num = 0;
   den = 1;
   if (i0 >= i1) return;
@@ -337,16 +492,17 @@ __device__ __forceinline__ void sum_fraction(const A& M, uint64_t i0, uint64_t i
   }
   uint32_t c = static_cast<uint32_t>(2 * i1 - 1);
   const uint32_t c0 = static_cast<uint32_t>(2 * i0 + 1);
-  const uint32_t bit = 2 * flip;  // of c: bit `flip` of i is bit 2 flip of c
+  const uint32_t bit = 2 * flip;  // bit `flip` of i is bit 2 flip of c
   for (;;) {
+    uint32_t k = c;
     if (SKIP && c == static_cast<uint32_t>(skip)) {
       skip = skip > p ? skip - 2 * p : 0;
+      k = 1u;
       num = M.mul_word(num, 1u, 0);
-      den = WORD ? M.mul_word(den, static_cast<uint32_t>(h), 0) : M.mul(M.mul_word(den, 1u, 0), h);
     } else {
       num = M.mul_word(num, c, (c & bit) ? M.neg(den) : den);
-      den = WORD ? M.mul_word(den, c * static_cast<uint32_t>(h), 0) : M.mul(M.mul_word(den, c, 0), h);
     }
+    den = WORD ? M.mul_word(den, k * static_cast<uint32_t>(h), 0) : M.mul(M.mul_word(den, k, 0), h);
     if (c == c0) break;
     c -= 2;
   }
@@ -373,13 +529,22 @@ __global__ void __launch_bounds__(kHeadThreads) prime_sum_kernel(const __grid_co
 #pragma unroll
   for (int i = 0; i < LMAX; ++i) acc[i] = 0;
   using T = typename A::T;
-  for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < count; i += gridDim.x * blockDim.x) {
-    const uint64_t p = G.base + G.list[i];
+  const uint32_t lane = threadIdx.x & 31u;
+  for (uint32_t at; (at = take_primes(G.taken, 32, lane)) < count;) {
+    const uint32_t i = at + lane;  // a lane past the end repeats the last prime and adds nothing
+    const uint64_t p = G.base + G.list[min(i, count - 1)];
     const A M(p);
+    const uint64_t iA = (G.A / p + 1) / 2, iB = (G.B / p + 1) / 2, iC = (G.C / p + 1) / 2;
     T nA, dA, nB, dB, nC, dC;
-    sum_fraction<A, true, false>(M, 0, (G.A / p + 1) / 2, 1, p, 4, nA, dA);
-    sum_fraction<A, true, false>(M, 0, (G.B / p + 1) / 2, 1, p, 1024, nB, dB);
-    sum_fraction<A, true, false>(M, 0, (G.C / p + 1) / 2, 2, p, 32, nC, dC);
+    if constexpr (sizeof(T) == 4) {
+      prime_sum<0>(M, static_cast<uint32_t>(iA), nA, dA);
+      prime_sum<1>(M, static_cast<uint32_t>(iB), nB, dB);
+      prime_sum<2>(M, static_cast<uint32_t>(iC), nC, dC);
+    } else {
+      power_sum<true, false>(M, 0, iA, 1, p, 4, nA, dA);
+      power_sum<true, false>(M, 0, iB, 1, p, 1024, nB, dB);
+      power_sum<true, false>(M, 0, iC, 2, p, 32, nC, dC);
+    }
     const T bc = M.mul(dB, dC);
     const T b4 = M.add(nB, nB);
     T num = M.mul(nA, bc);
@@ -388,6 +553,7 @@ __global__ void __launch_bounds__(kHeadThreads) prime_sum_kernel(const __grid_co
     const T inv = inverse_times_power<A>(M, M.mul(dA, bc), p - 1, (G.e + 4) % (p - 1));
     T x = M.plain(M.mul(num, inv));
     if (p & 2u) x = M.neg(x);
+    if (i >= count) x = 0;
     fold_one<A, LMAX>(M, x, acc);
   }
   flush_cta<LMAX>(acc, G.L, G.slots);
@@ -409,75 +575,110 @@ __device__ typename A::T geometric(const A& M, typename A::T r, uint64_t n) {
   return s;
 }
 
+// What one lane adds of sum KIND to the part of q = p^a: its share of the summands
+// [lo, hi), `times` over, as a fraction added to num / den (all in Montgomery form).
+template <class A, int KIND>
+__device__ __forceinline__ void add_share(const A& M, uint64_t p, uint64_t q, uint64_t phi, int64_t e, uint64_t lo,
+                                          uint64_t hi, uint64_t period, uint64_t times, uint32_t lane,
+                                          typename A::T& num, typename A::T& den) {
+  using T = typename A::T;
+  const uint64_t share = (hi - lo + 31) / 32;
+  const uint64_t i0 = lo + min(hi - lo, lane * share), i1 = min(hi, i0 + share);
+  if (times == 0 || hi <= lo) return;  // the same for every lane
+  constexpr int64_t kRatio = sum_weight_bits(KIND);  // summand i carries 2^(-ratio q i)
+  const int64_t sq = static_cast<int64_t>(q);
+  T n_s, d_s;
+  if constexpr (sizeof(T) == 4) {
+    prime_share<KIND>(M, static_cast<uint32_t>(i0), static_cast<uint32_t>(i1), lo32(p), n_s, d_s);
+  } else {
+    const T h = power_of_two<A>(M, exponent_mod(kRatio * sq, phi));
+    power_sum<false, true>(M, i0, i1, KIND == 2 ? 2u : 1u, p, h, n_s, d_s);
+  }
+  // the first summand's power of 2, with the h that multiplies the fraction
+  const int64_t start = KIND == 0 ? e + 3 - sq : KIND == 1 ? e + 1 - 5 * sq : e - 1 - 5 * (sq - 1) / 2;
+  T k = power_of_two<A>(M, exponent_mod(start + kRatio * sq * (1 - static_cast<int64_t>(i0)), phi));
+  if (times > 1) {
+    T r = power_of_two<A>(M, exponent_mod(-kRatio * sq * static_cast<int64_t>(period), phi));
+    if (KIND != 2) r = M.neg(r);  // the period is odd for A and B
+    k = M.mul(k, geometric<A>(M, r, times));
+  }
+  const bool minus = KIND == 0 ? (q & 2u) != 0 : KIND == 1 ? (q & 2u) == 0 : (q & 4u) == 0;
+  k = M.mul(k, n_s);
+  num = M.add(M.mul(num, d_s), M.mul(minus ? M.neg(k) : k, den));
+  den = M.mul(den, d_s);
+}
+
+// Prime power of work item `unit`, 0 if there is none: for PRIME the primes in turn; else
+// p^2 of every prime, then p^3 and p^4 of the first 2560 (p up to 2^14.5 > A^(1/3)), then
+// p^5 ... p^28 of the first 128 (3^28 > A).
+template <bool PRIME>
+__device__ __forceinline__ uint64_t prime_power_of(const PrimeArgs& G, uint32_t unit, uint32_t count, uint64_t* p) {
+  uint32_t i = unit, a = 2;
+  if (!PRIME && unit >= count) {
+    const uint32_t first = min(count, 2560u), second = min(count, 128u);
+    i -= count;
+    if (i < 2 * first) {
+      a = 3 + i / first;
+      i %= first;
+    } else {
+      i -= 2 * first;
+      a = 5 + i / second;
+      i %= second;
+    }
+  }
+  *p = G.list[i];
+  if (PRIME) return *p <= G.A ? *p : 0;
+  uint64_t q = *p;
+  for (uint32_t k = 1; k < a; ++k) {
+    if (q > G.A / *p) return 0;
+    q *= *p;
+  }
+  return q;
+}
+
 // One warp per prime power q = p^a.  The summands of each sum repeat with a constant
-// ratio after `period` odd c (c^-1 mod q after q, the signs after 1 or 4 of those), so
-// at most `period` of them are added up, times a geometric sum: the lanes share them
-// evenly, each lane's part being its own fraction over q.  PRIME: a = 1 (p in the
-// list), else every a >= 2 with p^a <= A.
+// ratio after `period` odd c (c^-1 mod q after q of them, the signs after 1 or 4 times
+// that), so at most `period` of them are added up, times a geometric sum: the lanes
+// share them evenly, each lane's part being its own fraction over q.
 template <class A, bool PRIME, int LMAX>
 __global__ void __launch_bounds__(kHeadThreads) prime_power_kernel(const __grid_constant__ PrimeArgs G) {
   const uint32_t lane = threadIdx.x & 31u;
   const uint32_t warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   const uint32_t nwarps = (gridDim.x * blockDim.x) >> 5;
   const uint32_t count = min(*G.count, G.cap);
+  const uint32_t units = PRIME ? count : count + 2 * min(count, 2560u) + 24 * min(count, 128u);
   using T = typename A::T;
   uint32_t acc[LMAX];
 #pragma unroll
   for (int i = 0; i < LMAX; ++i) acc[i] = 0;
-  for (uint32_t at = warp; at < count; at += nwarps) {
-    const uint64_t p = G.base + G.list[at];
-    const uint64_t last = G.A / p;  // q p is another power up to A while q <= A / p
-    for (uint64_t q = PRIME ? p : p * p; q <= G.A; q *= p) {
-      const A M(q);
-      const uint64_t phi = q / p * (p - 1);
-      const int64_t sq = static_cast<int64_t>(q), e = static_cast<int64_t>(G.e);
-      const bool chi_neg = (q & 2u) != 0, psi_neg = (q & 4u) != 0;
-      const uint64_t limit[3] = {G.A, G.B, G.C};
-      uint64_t whole[3], rest[3], period[3];
-      bool repeats = false;
+  for (uint32_t unit = warp; unit < units; unit += nwarps) {
+    uint64_t p;
+    const uint64_t q = prime_power_of<PRIME>(G, unit, count, &p);
+    if (q == 0) continue;
+    const A M(q);
+    const uint64_t phi = q / p * (p - 1);
+    const int64_t e = static_cast<int64_t>(G.e);
+    const uint64_t limit[3] = {G.A, G.B, G.C};
+    uint64_t whole[3], rest[3], period[3];
 #pragma unroll
-      for (int s = 0; s < 3; ++s) {
-        const uint64_t n = (limit[s] / q + 1) / 2;  // odd c up to limit / q
-        period[s] = s == 2 ? 4 * q : q;
-        whole[s] = n / period[s];
-        rest[s] = n % period[s];
-        repeats |= whole[s] > 0;
-      }
-      for (int pass = 0; pass < (repeats ? 2 : 1); ++pass) {
-        // pass 0: the first `rest` summands, whole + 1 times; pass 1: the others, whole times
-        T num = 0, den = M.one();
-#pragma unroll
-        for (int s = 0; s < 3; ++s) {
-          const uint64_t lo = pass == 0 ? 0 : rest[s], hi = pass == 0 ? rest[s] : period[s];
-          const uint64_t times = whole[s] + (pass == 0 ? 1 : 0);
-          const uint64_t share = (hi - lo + 31) / 32;
-          const uint64_t i0 = lo + min(hi - lo, lane * share), i1 = min(hi, i0 + share);
-          if (times == 0 || i0 >= i1) continue;
-          constexpr uint32_t kRatio[3] = {2, 10, 5};  // summand i carries 2^(-ratio q i)
-          const int64_t ratio = kRatio[s];
-          const T h = PRIME ? static_cast<T>(1u << kRatio[s])
-                            : power_of_two<A>(M, exponent_mod(ratio * sq, phi));
-          T n_s, d_s;
-          sum_fraction<A, PRIME, true>(M, i0, i1, s == 2 ? 2 : 1, p, h, n_s, d_s);
-          // times 2^(e + const - (power at i0)), h of the fraction included
-          const int64_t start = s == 0 ? e + 3 - sq : s == 1 ? e + 1 - 5 * sq : e - 1 - 5 * (sq - 1) / 2;
-          T k = power_of_two<A>(M, exponent_mod(start + ratio * sq - ratio * sq * static_cast<int64_t>(i0), phi));
-          if (times > 1) {
-            const int64_t per = static_cast<int64_t>(period[s]);
-            T r = power_of_two<A>(M, exponent_mod(-ratio * sq * per, phi));
-            if (s != 2) r = M.neg(r);
-            k = M.mul(k, geometric<A>(M, r, times));
-          }
-          const bool minus = s == 0 ? chi_neg : s == 1 ? !chi_neg : !psi_neg;
-          k = M.mul(k, n_s);
-          // num / den + k / d_s
-          num = M.add(M.mul(num, d_s), M.mul(minus ? M.neg(k) : k, den));
-          den = M.mul(den, d_s);
-        }
+    for (int s = 0; s < 3; ++s) {
+      const uint64_t n = (limit[s] / q + 1) / 2;  // odd c up to limit / q
+      period[s] = s == 2 ? 4 * q : q;
+      whole[s] = n / period[s];
+      rest[s] = n % period[s];
+    }
+    const bool repeats = (whole[0] | whole[1] | whole[2]) != 0;
+    for (int pass = 0; pass < (repeats ? 2 : 1); ++pass) {
+      // pass 0: the first `rest` summands, whole + 1 times; pass 1: the others, whole times
+      T num = 0, den = M.one();
+      const bool f = pass == 0;
+      add_share<A, 0>(M, p, q, phi, e, f ? 0 : rest[0], f ? rest[0] : period[0], period[0], whole[0] + f, lane, num, den);
+      add_share<A, 1>(M, p, q, phi, e, f ? 0 : rest[1], f ? rest[1] : period[1], period[1], whole[1] + f, lane, num, den);
+      add_share<A, 2>(M, p, q, phi, e, f ? 0 : rest[2], f ? rest[2] : period[2], period[2], whole[2] + f, lane, num, den);
+      if (num != 0) {
         const T x = M.plain(M.mul(num, inverse_times_power<A>(M, den, phi, 0)));
         fold_one<A, LMAX>(M, x, acc);
       }
-      if (PRIME || q > last) break;
     }
   }
   flush_cta<LMAX>(acc, G.L, G.slots);

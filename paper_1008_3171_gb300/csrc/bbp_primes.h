@@ -42,6 +42,10 @@ PrimeLimits prime_limits(uint64_t d);
 // First k of series j (formula 0) that the prime form does not cover.
 uint64_t prime_first_k(const PrimeLimits& lim, uint32_t j);
 
+// Primes up to here take the half-reduced ladder: with x <= p + 2^35, x^2 / 2^32 + p stays
+// below 2^48.
+constexpr uint64_t kPrimeHalfMax = 1'020'000'000'000;
+
 // Primes with the same H = num / (den 2^kPrimeShift): those above `above`, up to the
 // previous class's `above`.
 constexpr int kPrimeShift = 24;   // every denominator of H up to kPrimeMaxC divides den 2^24
@@ -73,6 +77,6 @@ bool prime_form_serves(int formula, uint64_t n, uint32_t P, uint32_t W, uint64_t
 double prime_form_imad(const PrimeLimits& lim, int limbs);
 
 constexpr uint64_t kPrimeMinN = 100'000'000;  // below, the terms take no longer (1.4 ms each at 1e8, P = 64)
-constexpr uint64_t kPrimeMaxN = 1ull << 45;   // sieving primes below 2^23
+constexpr uint64_t kPrimeMaxN = 10'900'000'000'000;  // 1024 sqrt(0.4 n) < 2^31: word products of the sums
 
 }  // namespace bbp

@@ -9,31 +9,38 @@
 namespace bbp {
 
 constexpr int kSieveThreads = 512;
-constexpr int kSieveMaxWords = 1 << 14;  // 64 KB of odd numbers, 2^20 numbers a segment
+constexpr uint32_t kSieveMaxEntries = 192u << 10;  // bytes of shared memory
 
-// Primes p with `above` < p <= `upto` in the `segments` segments of 64 * words numbers
-// from `base` (a multiple of 64 * words), as offsets from `base`, ascending within a
-// segment, appended to list[0, cap) through *count.  *count counts all of them: a
-// count past `cap` says that some are missing.  The base primes are the `nprimes` odd
-// primes from 67 on, ascending, with inv[i] = floor((2^64 - 1) / primes[i]); they must
-// reach the square root of `upto`.
+// A base prime p as the sieve reads it.
+struct SievePrime {
+  uint32_t p;
+  uint32_t inv;    // floor((2^32 - 1) / p)
+  uint32_t inv30;  // 30^-1 mod p
+  uint32_t at;     // -base / 30 mod p for the list being sieved
+};
+
+// Primes p with `above` < p <= `upto` among the numbers prime to 30 of `segments`
+// segments of 30 * entries numbers (entries a multiple of 32; segments * entries < 2^28)
+// from `base` (a multiple of 30), as offsets from `base` in no particular order, appended
+// to list[0, cap) through *count.  *count counts all of them: a count past `cap` says that
+// some are missing.  The base primes are the *nprimes primes from 17 on (none above
+// `above`), ascending, up to at least the square root of `upto`; their `at` is set here.
 struct SieveArgs {
   uint64_t base, above, upto;
-  uint32_t segments, words;
-  const uint32_t* primes;
-  const uint64_t* inv;
+  uint32_t segments, entries;
+  SievePrime* primes;
   const uint32_t* nprimes;
   uint32_t* list;
   uint32_t* count;
   uint32_t cap;
 };
-cudaError_t launch_sieve(const SieveArgs& a, int blocks, cudaStream_t s);
-int sieve_occupancy(int words);
+cudaError_t launch_sieve(const SieveArgs& a, int sms, cudaStream_t s);
 
-// primes[0, *count) <- the odd primes up to `upto` (< 2^23) ascending, *count their number,
-// inv their reciprocals; the first kSieveTinyPrimes of them are below 67.
-constexpr int kSieveTinyPrimes = 17;
-cudaError_t launch_base_primes(uint32_t upto, uint32_t* primes, uint64_t* inv, uint32_t* count, uint32_t* nsieve,
+// primes[0, *count) <- the odd primes up to `upto` (below 2^23) ascending, *count their
+// number, *nsieve the number of those from 17 on, which are at sieve[kSieveTinyPrimes]
+// and after.
+constexpr int kSieveTinyPrimes = 5;
+cudaError_t launch_base_primes(uint32_t upto, uint32_t* primes, SievePrime* sieve, uint32_t* count, uint32_t* nsieve,
                                cudaStream_t s);
 
 // The prime form's sum S' and the term-by-term sum S both err by less than `bound`
