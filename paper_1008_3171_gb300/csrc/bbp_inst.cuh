@@ -70,10 +70,12 @@ cudaError_t BBP_CAT(launch_prime_l, BBP_LMAX)(const PrimeArgs& a, PrimeKernel k,
     case kPrimes1: return launch_prime_t(prime_kernel<BBP_LMAX, 1, false>, a, sms, s);
     case kPrimesHalf: return launch_prime_t(prime_kernel<BBP_LMAX, 1, true>, a, sms, s);
     case kPrimes3: return launch_prime_t(prime_kernel<BBP_LMAX, 3, false>, a, sms, s);
-    case kSums1: return launch_prime_t(prime_sum_kernel<Arith1, BBP_LMAX>, a, sms, s);
-    case kSums2: return launch_prime_t(prime_sum_kernel<Arith2, BBP_LMAX>, a, sms, s);
+    case kSums8: return launch_prime_t(prime_sum_kernel<Arith1, 8, BBP_LMAX>, a, sms, s);
+    case kSums1: return launch_prime_t(prime_sum_kernel<Arith1, 1, BBP_LMAX>, a, sms, s);
+    case kSums2: return launch_prime_t(prime_sum_kernel<Arith2, 1, BBP_LMAX>, a, sms, s);
     case kPrimeWarps: return launch_prime_t(prime_power_kernel<Arith1, true, BBP_LMAX>, a, sms, s);
-    case kPowers: return launch_prime_t(prime_power_kernel<Arith2, false, BBP_LMAX>, a, sms, s);
+    case kPowers1: return launch_prime_t(prime_power_kernel<Arith1, false, BBP_LMAX>, a, sms, s);
+    case kPowers2: return launch_prime_t(prime_power_kernel<Arith2, false, BBP_LMAX>, a, sms, s);
   }
   return cudaErrorInvalidValue;
 }

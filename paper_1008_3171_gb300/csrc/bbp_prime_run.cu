@@ -27,7 +27,8 @@ constexpr uint32_t kMaxBase = (1u << 23) - 1;       // base primes up to here: 5
 constexpr uint32_t kBaseCap = 565000;
 constexpr uint32_t kMaxListCap = 24u << 20;         // primes of one list (96 MB), two lists
 constexpr uint32_t kMaxLists = 1u << 16;
-constexpr uint64_t kLongSum = 16000;                // primes below A / this take a warp each
+constexpr uint64_t kLongSum = 32000;                // primes below A / this take a warp each,
+constexpr uint64_t kGroupSum = 1000;                // those below A / this eight lanes
 
 uint64_t isqrt(uint64_t v) {
   uint64_t r = static_cast<uint64_t>(std::sqrt(static_cast<double>(v)));
@@ -169,7 +170,8 @@ bbp_status launch_prime_form(bbp_plan p, uint64_t n, uint32_t W, uint32_t P, uin
   struct Span { uint64_t lo, hi; PrimeKernel k; };
   std::vector<Span> spans;
   {
-    const uint64_t cuts[] = {bottom, (1ull << 29) - 1, (1ull << 31) - 1, kPrimeHalfMax, lim.A};
+    const uint64_t grouped = std::min<uint64_t>(lim.A / kGroupSum, (1ull << 31) - 1);
+    const uint64_t cuts[] = {grouped, bottom, (1ull << 29) - 1, (1ull << 31) - 1, kPrimeHalfMax, lim.A};
     std::vector<uint64_t> c(std::begin(cuts), std::end(cuts));
     std::sort(c.begin(), c.end());
     uint64_t lo = base_to;
@@ -177,7 +179,7 @@ bbp_status launch_prime_form(bbp_plan p, uint64_t n, uint32_t W, uint32_t P, uin
       hi = std::min(hi, lim.A);
       if (hi <= lo) continue;
       PrimeKernel k;
-      if (hi <= bottom) k = hi < (1ull << 31) ? kSums1 : kSums2;
+      if (hi <= bottom) k = hi <= grouped ? kSums8 : hi < (1ull << 31) ? kSums1 : kSums2;
       else k = hi < (1ull << 29) ? kPrimes0 : hi < (1ull << 31) ? kPrimes3 : hi <= kPrimeHalfMax ? kPrimesHalf : kPrimes1;
       spans.push_back(Span{lo, hi, k});
       lo = hi;
@@ -219,10 +221,11 @@ bbp_status launch_prime_form(bbp_plan p, uint64_t n, uint32_t W, uint32_t P, uin
   a.cap = kBaseCap;
   a.base = 0;
   a.e = e;
-  chk(launch_prime(a, kPowers, lmax, p->sm_count, S->sums));
+  chk(launch_prime(a, kPowers1, lmax, p->sm_count, S->sums));
+  if (lim.A >= (1ull << 31)) chk(launch_prime(a, kPowers2, lmax, p->sm_count, S->sums));
   chk(launch_prime(a, kPrimeWarps, lmax, p->sm_count, S->sums));
   chk(cudaEventRecord(S->done, S->sums));
-  *launches += 3;
+  *launches += lim.A >= (1ull << 31) ? 4 : 3;
   SieveArgs v{};
   v.entries = entries;
   v.primes = S->sieve_primes + kSieveTinyPrimes;
@@ -246,7 +249,7 @@ bbp_status launch_prime_form(bbp_plan p, uint64_t n, uint32_t W, uint32_t P, uin
     a.base = l.base;
     a.count = lengths + i;
     a.taken = lengths + nl + i;
-    a.e = l.k == kSums1 || l.k == kSums2 ? e : e - kPrimeShift + 64;  // the product with H leaves a factor 2^-64
+    a.e = l.k == kSums1 || l.k == kSums2 || l.k == kSums8 ? e : e - kPrimeShift + 64;  // the product with H leaves a factor 2^-64
     chk(launch_prime(a, l.k, lmax, p->sm_count, st));
     chk(cudaEventRecord(S->used[slot], st));
     *launches += 3;

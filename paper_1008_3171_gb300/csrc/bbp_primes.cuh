@@ -3,7 +3,7 @@
 //
 //   prime_kernel       primes above A / 23: H is one of a few rational constants, so a
 //                      prime costs one modular power of 2, a product and W bits of quotient
-//   prime_sum_kernel   primes below: H summed mod p, one prime per thread
+//   prime_sum_kernel   primes below: H summed mod p, one prime per thread or eight threads
 //   prime_power_kernel primes and prime powers with long sums: one warp each
 //
 // Every part is a residue x = 2^W r mod q of a fraction r / q; its W bits are the
@@ -143,13 +143,29 @@ __device__ __forceinline__ void prime_residues(const uint64_t e, const uint64_t 
       square_all<PATH, NT>(x0, x1, m0, m1, mp, sh, true);
     }
   } else {
-    // one bit at a time: moduli of up to 29 (lazy) and 31 bits (reduced) allow a shift of one
+    // One bit at a time, the bit taken as a doubled operand of the square: x (2 x) stays below
+    // m 2^32 for a lazy x < 2 m of up to 29 bits (path 0) and a reduced x < m of up to 31 (path
+    // 3).  The reduction subtracts (Arith1): one three-operand add after the high product.
+    uint32_t bits[NT], inv[NT];
+#pragma unroll
+    for (int t = 0; t < NT; ++t) {
+      bits[t] = lo32(rem[t]);  // j <= 27
+      inv[t] = 0u - mp[t];
+    }
     while (b > 0) {
       --b;
-      uint32_t sh[NT];
+      const uint32_t mask = 1u << b;
 #pragma unroll
-      for (int t = 0; t < NT; ++t) sh[t] = static_cast<uint32_t>(rem[t] >> b) & 1u;
-      square_all<PATH, NT>(x0, x1, m0, m1, mp, sh, true);
+      for (int t = 0; t < NT; ++t) {
+        const uint64_t T = static_cast<uint64_t>(x0[t]) * ((bits[t] & mask) ? x0[t] + x0[t] : x0[t]);
+        const uint32_t h = __umulhi(lo32(T) * inv[t], m0[t]);
+        if (PATH == 3) {
+          const uint32_t r = hi32(T) - h;  // in (-m, m)
+          x0[t] = min(r, r + m0[t]);
+        } else {
+          x0[t] = hi32(T) + m0[t] - h;
+        }
+      }
     }
   }
   // times H, with p's sign
@@ -321,17 +337,41 @@ struct Arith2 {
   }
 };
 
+// a / p for quotients below 2^21 (a < 2^44): single precision is off by at most one
+__device__ __forceinline__ uint32_t small_quotient(uint64_t a, uint64_t p) {
+  uint32_t q = static_cast<uint32_t>(__fdividef(static_cast<float>(a), static_cast<float>(p)));
+  int64_t rem = static_cast<int64_t>(a) - static_cast<int64_t>(q * p);
+  if (rem < 0) --q;
+  if (rem >= static_cast<int64_t>(p)) ++q;
+  return q;
+}
+
 // den^-1 2^e (Montgomery form) for a unit `den` mod m whose group of units has
-// exponent phi: den^(phi - 1) and 2^e in one ladder.  0 <= e < phi.
+// exponent phi: den^(phi - 1) and 2^e in one ladder.  0 <= e < phi.  In one word two bits
+// at a time: the bits of e double an operand of the squares, those of phi - 1 choose
+// among 1, den, den^2, den^3.  Every lane of the warp must call it.
 template <class A>
 __device__ typename A::T inverse_times_power(const A& M, typename A::T den, uint64_t phi, uint64_t e) {
-  const typename A::T one = M.one();
-  typename A::T z = one;
-  const uint64_t f = phi - 1;
-  for (int b = bitlen64(phi) - 1; b >= 0; --b) {
-    z = M.mul(z, z);
-    if ((f >> b) & 1u) z = M.mul(z, den);
-    if ((e >> b) & 1u) z = M.add(z, z);
+  using T = typename A::T;
+  const T one = M.one();
+  T z = one;
+  if constexpr (sizeof(T) == 4) {
+    const uint32_t f = lo32(phi) - 1u, g = lo32(e);
+    const T den2 = M.mul(den, den), den3 = M.mul(den2, den);
+    const int bits = 32 - __clz(static_cast<int>(__reduce_max_sync(0xffffffffu, lo32(phi))));
+    for (int b = (bits - 1) & ~1; b >= 0; b -= 2) {
+      z = M.mul(z, (g >> (b + 1)) & 1u ? z + z : z);
+      z = M.mul(z, (g >> b) & 1u ? z + z : z);
+      const T lo = (f >> b) & 1u ? den : one, hi = (f >> b) & 1u ? den3 : den2;
+      z = M.mul(z, (f >> (b + 1)) & 1u ? hi : lo);
+    }
+  } else {
+    const uint64_t f = phi - 1;
+    for (int b = bitlen64(phi) - 1; b >= 0; --b) {
+      z = M.mul(z, z);
+      if ((f >> b) & 1u) z = M.mul(z, den);
+      if ((e >> b) & 1u) z = M.add(z, z);
+    }
   }
   return z;
 }
@@ -435,11 +475,102 @@ __device__ __forceinline__ void prime_sum(const Arith1& M, uint32_t n, uint32_t&
   if (n != 0 && ((flips ^ first) & 1u)) num = M.neg(num);
 }
 
-// The same over lo <= i < hi, relative to the term at lo (w num / den with w^-(i - lo)), the
-// terms with c a multiple of p left out; the lanes walk their ranges in step.
+// The same over lo <= i < hi, relative to the term at lo (w num / den with w^-(i - lo)), lo
+// even, each lane with its own range; the lanes walk them in step.
 template <int KIND>
-__device__ __forceinline__ void prime_share(const Arith1& M, uint32_t lo, uint32_t hi, uint32_t p, uint32_t& num,
-                                            uint32_t& den) {
+__device__ __forceinline__ void range_sum(const Arith1& M, uint32_t lo, uint32_t hi, uint32_t& num, uint32_t& den) {
+  constexpr uint32_t kW = sum_weight_bits(KIND);
+  constexpr uint32_t kPairTop = KIND == 0 ? 11583u : KIND == 2 ? 1447u : 0u;  // as in prime_sum
+  const uint32_t steps = __reduce_max_sync(0xffffffffu, hi - lo);
+  const bool pairs = kPairTop != 0u && __reduce_max_sync(0xffffffffu, 2u * hi) <= kPairTop;
+  uint32_t N = 0, D = 1;
+  if (pairs) {
+    const bool odd = (hi & 1u) != 0u;
+    const uint32_t n0 = odd ? M.lazy_redc(1u) : 0u;
+    const uint32_t d0 = odd ? M.lazy_redc_neg(static_cast<uint64_t>(2u * hi - 1u) << kW) : 1u;
+    uint32_t k = (steps + 1u) / 2u;
+    uint32_t h = lo / 2u + k;  // h - 1: the pair (2 h - 2, 2 h - 1)
+    uint32_t alpha = 16u * h * (h - 1u) + 3u, diff = 32u * (h - 1u);
+    uint32_t beta = KIND == 0 ? 12u * h - 1u : 132u * h - 35u;
+    uint32_t d = 1;
+    const uint32_t d_start = KIND == 0 ? 2u * M.m - d0 : d0, start = hi / 2u;
+    for (; k > 0u; --k, --h) {
+      if (h == start) {
+        N = n0;
+        d = d_start;
+      }
+      N = M.lazy_redc(static_cast<uint64_t>(N) * alpha + static_cast<uint64_t>(d) * beta);
+      const uint64_t t = static_cast<uint64_t>(d) * (alpha << (2u * kW));
+      d = KIND == 0 ? M.lazy_redc(t) : M.lazy_redc_neg(t);
+      alpha -= diff;
+      diff -= 32u;
+      beta -= KIND == 0 ? 12u : 132u;
+    }
+    D = KIND == 0 ? 2u * M.m - d : d;
+    if (start == lo / 2u) {  // one term, or none
+      N = n0;
+      D = d0;
+    }
+  } else {
+    uint32_t i = lo + steps;
+    for (uint32_t k = steps; k > 0u; --k) {
+      if (i == hi) {
+        N = 0;
+        D = 1;
+      }
+      --i;
+      const uint32_t c = 2u * i + 1u;
+      N = M.lazy_redc(static_cast<uint64_t>(N) * c + D);
+      const uint64_t t = static_cast<uint64_t>(D) * (c << kW);
+      if (KIND != 2) {
+        D = M.lazy_redc_neg(t);
+      } else {
+        const uint32_t r = M.lazy_redc(t);
+        D = (i & 1u) ? r : 2u * M.m - r;
+      }
+    }
+  }
+  if (hi <= lo) {
+    N = 0;
+    D = 1;
+  }
+  num = M.fix(N);
+  den = M.fix(D);
+  const uint32_t flips = KIND != 2 ? hi - lo : (hi + 1u) / 2u - (lo + 1u) / 2u;
+  const uint32_t first = KIND != 2 ? hi - 1u : (hi - 1u) >> 1;
+  if (hi > lo && ((flips ^ first) & 1u)) num = M.neg(num);
+}
+
+// The sum over 0 <= i < n shared by GROUP neighbouring lanes with the same prime: each takes
+// an even number s of terms, and the fractions are put together two by two,
+//   w num / den = w (num den' w^s + num' den) / (den den' w^s).
+// The group's first lane has the result.
+template <int KIND, int GROUP>
+__device__ __forceinline__ void group_sum(const Arith1& M, uint32_t n, uint32_t& num, uint32_t& den) {
+  constexpr uint32_t kW = sum_weight_bits(KIND);
+  const uint32_t share = ((n + GROUP - 1) / GROUP + 1u) & ~1u;
+  uint32_t lo = (threadIdx.x & (GROUP - 1)) * share, hi = min(n, lo + share);
+  if (lo >= n) lo = hi = 0;
+  range_sum<KIND>(M, lo, hi, num, den);
+  uint32_t z = M.one(), e = kW * share;  // w^s
+  const int bits = 32 - __clz(static_cast<int>(__reduce_max_sync(0xffffffffu, e)));
+  for (int b = bits - 1; b >= 0; --b) z = M.mul(z, (e >> b) & 1u ? z + z : z);
+#pragma unroll
+  for (int d = 1; d < GROUP; d <<= 1) {
+    const uint32_t num2 = __shfl_down_sync(0xffffffffu, num, d, GROUP);
+    const uint32_t den2 = __shfl_down_sync(0xffffffffu, den, d, GROUP);
+    num = M.add(M.mul(M.mul(num, z), den2), M.mul(den, num2));
+    den = M.mul(M.mul(den, z), den2);
+    z = M.mul(z, z);
+  }
+}
+
+// The same over lo <= i < hi, relative to the term at lo (w num / den with w^-(i - lo)), the
+// terms with c a multiple of p left out; the lanes walk their ranges in step.  WORD: modulo
+// p, with w a word; else modulo a power of p, with h (a residue in Montgomery form) for w.
+template <int KIND, bool WORD>
+__device__ __forceinline__ void prime_share(const Arith1& M, uint32_t lo, uint32_t hi, uint32_t p, uint32_t h,
+                                            uint32_t& num, uint32_t& den) {
   constexpr uint32_t kW = sum_weight_bits(KIND);
   const uint32_t steps = __reduce_max_sync(0xffffffffu, hi > lo ? hi - lo : 0u);
   uint32_t i = lo + steps, N = 0, D = 1;
@@ -458,7 +589,8 @@ __device__ __forceinline__ void prime_share(const Arith1& M, uint32_t lo, uint32
       skip = skip > p ? skip - 2u * p : 0u;
     }
     N = M.lazy_redc(static_cast<uint64_t>(N) * c + add);
-    const uint64_t t = static_cast<uint64_t>(D) * (c << kW);
+    const uint64_t t = WORD ? static_cast<uint64_t>(D) * (c << kW)
+                            : static_cast<uint64_t>(M.lazy_redc(static_cast<uint64_t>(D) * c)) * h;
     if (KIND != 2) {
       D = M.lazy_redc_neg(t);
     } else {
@@ -519,10 +651,12 @@ __device__ __forceinline__ void fold_one(const A& M, typename A::T x, uint32_t (
   }
 }
 
-// One prime per thread: num / den of the three sums with i0 = 0, one ladder for the
-// inverse of their denominators and the power of 2.
+// GROUP lanes per prime: num / den of the three sums, one ladder for the inverse of their
+// denominators and the power of 2.
 //   H = 16 (num_A / den_A - 4 num_B / den_B - num_C / den_C)
-template <class A, int LMAX>
+// One lane per prime walks up to 8000 terms in a row where the sums are long; eight lanes
+// bring n = 1e9's longest chain from 600 us (with the SM full) to a quarter.
+template <class A, int GROUP, int LMAX>
 __global__ void __launch_bounds__(kHeadThreads) prime_sum_kernel(const __grid_constant__ PrimeArgs G) {
   const uint32_t count = min(*G.count, G.cap);
   uint32_t acc[LMAX];
@@ -530,16 +664,21 @@ __global__ void __launch_bounds__(kHeadThreads) prime_sum_kernel(const __grid_co
   for (int i = 0; i < LMAX; ++i) acc[i] = 0;
   using T = typename A::T;
   const uint32_t lane = threadIdx.x & 31u;
-  for (uint32_t at; (at = take_primes(G.taken, 32, lane)) < count;) {
-    const uint32_t i = at + lane;  // a lane past the end repeats the last prime and adds nothing
+  for (uint32_t at; (at = take_primes(G.taken, 32 / GROUP, lane)) < count;) {
+    const uint32_t i = at + lane / GROUP;  // a lane past the end repeats the last prime and adds nothing
     const uint64_t p = G.base + G.list[min(i, count - 1)];
     const A M(p);
-    const uint64_t iA = (G.A / p + 1) / 2, iB = (G.B / p + 1) / 2, iC = (G.C / p + 1) / 2;
+    const uint32_t iA = (small_quotient(G.A, p) + 1) / 2, iB = (small_quotient(G.B, p) + 1) / 2,
+                   iC = (small_quotient(G.C, p) + 1) / 2;
     T nA, dA, nB, dB, nC, dC;
-    if constexpr (sizeof(T) == 4) {
-      prime_sum<0>(M, static_cast<uint32_t>(iA), nA, dA);
-      prime_sum<1>(M, static_cast<uint32_t>(iB), nB, dB);
-      prime_sum<2>(M, static_cast<uint32_t>(iC), nC, dC);
+    if constexpr (GROUP > 1) {
+      group_sum<0, GROUP>(M, iA, nA, dA);
+      group_sum<1, GROUP>(M, iB, nB, dB);
+      group_sum<2, GROUP>(M, iC, nC, dC);
+    } else if constexpr (sizeof(T) == 4) {
+      prime_sum<0>(M, iA, nA, dA);
+      prime_sum<1>(M, iB, nB, dB);
+      prime_sum<2>(M, iC, nC, dC);
     } else {
       power_sum<true, false>(M, 0, iA, 1, p, 4, nA, dA);
       power_sum<true, false>(M, 0, iB, 1, p, 1024, nB, dB);
@@ -550,10 +689,11 @@ __global__ void __launch_bounds__(kHeadThreads) prime_sum_kernel(const __grid_co
     T num = M.mul(nA, bc);
     num = M.add(num, M.neg(M.mul(M.mul(M.add(b4, b4), dA), dC)));
     num = M.add(num, M.neg(M.mul(M.mul(nC, dA), dB)));
-    const T inv = inverse_times_power<A>(M, M.mul(dA, bc), p - 1, (G.e + 4) % (p - 1));
+    const uint64_t e = G.e + 4 - small_quotient(G.e + 4, p - 1) * (p - 1);
+    const T inv = inverse_times_power<A>(M, M.mul(dA, bc), p - 1, e);
     T x = M.plain(M.mul(num, inv));
     if (p & 2u) x = M.neg(x);
-    if (i >= count) x = 0;
+    if (i >= count || (lane & (GROUP - 1)) != 0u) x = 0;
     fold_one<A, LMAX>(M, x, acc);
   }
   flush_cta<LMAX>(acc, G.L, G.slots);
@@ -577,7 +717,7 @@ __device__ typename A::T geometric(const A& M, typename A::T r, uint64_t n) {
 
 // What one lane adds of sum KIND to the part of q = p^a: its share of the summands
 // [lo, hi), `times` over, as a fraction added to num / den (all in Montgomery form).
-template <class A, int KIND>
+template <class A, int KIND, bool PRIME>
 __device__ __forceinline__ void add_share(const A& M, uint64_t p, uint64_t q, uint64_t phi, int64_t e, uint64_t lo,
                                           uint64_t hi, uint64_t period, uint64_t times, uint32_t lane,
                                           typename A::T& num, typename A::T& den) {
@@ -588,12 +728,11 @@ __device__ __forceinline__ void add_share(const A& M, uint64_t p, uint64_t q, ui
   constexpr int64_t kRatio = sum_weight_bits(KIND);  // summand i carries 2^(-ratio q i)
   const int64_t sq = static_cast<int64_t>(q);
   T n_s, d_s;
-  if constexpr (sizeof(T) == 4) {
-    prime_share<KIND>(M, static_cast<uint32_t>(i0), static_cast<uint32_t>(i1), lo32(p), n_s, d_s);
-  } else {
-    const T h = power_of_two<A>(M, exponent_mod(kRatio * sq, phi));
+  const T h = PRIME ? 0 : power_of_two<A>(M, exponent_mod(kRatio * sq, phi));
+  if constexpr (sizeof(T) == 4)
+    prime_share<KIND, PRIME>(M, static_cast<uint32_t>(i0), static_cast<uint32_t>(i1), lo32(p), h, n_s, d_s);
+  else
     power_sum<false, true>(M, i0, i1, KIND == 2 ? 2u : 1u, p, h, n_s, d_s);
-  }
   // the first summand's power of 2, with the h that multiplies the fraction
   const int64_t start = KIND == 0 ? e + 3 - sq : KIND == 1 ? e + 1 - 5 * sq : e - 1 - 5 * (sq - 1) / 2;
   T k = power_of_two<A>(M, exponent_mod(start + kRatio * sq * (1 - static_cast<int64_t>(i0)), phi));
@@ -636,7 +775,8 @@ __device__ __forceinline__ uint64_t prime_power_of(const PrimeArgs& G, uint32_t 
   return q;
 }
 
-// One warp per prime power q = p^a.  The summands of each sum repeat with a constant
+// One warp per prime power q = p^a: PRIME: a = 1; else a >= 2 and q below (Arith1) or from
+// (Arith2) 2^31 on.  The summands of each sum repeat with a constant
 // ratio after `period` odd c (c^-1 mod q after q of them, the signs after 1 or 4 times
 // that), so at most `period` of them are added up, times a geometric sum: the lanes
 // share them evenly, each lane's part being its own fraction over q.
@@ -654,7 +794,7 @@ __global__ void __launch_bounds__(kHeadThreads) prime_power_kernel(const __grid_
   for (uint32_t unit = warp; unit < units; unit += nwarps) {
     uint64_t p;
     const uint64_t q = prime_power_of<PRIME>(G, unit, count, &p);
-    if (q == 0) continue;
+    if (q == 0 || (!PRIME && (q < (1ull << 31)) != (sizeof(T) == 4))) continue;
     const A M(q);
     const uint64_t phi = q / p * (p - 1);
     const int64_t e = static_cast<int64_t>(G.e);
@@ -672,13 +812,11 @@ __global__ void __launch_bounds__(kHeadThreads) prime_power_kernel(const __grid_
       // pass 0: the first `rest` summands, whole + 1 times; pass 1: the others, whole times
       T num = 0, den = M.one();
       const bool f = pass == 0;
-      add_share<A, 0>(M, p, q, phi, e, f ? 0 : rest[0], f ? rest[0] : period[0], period[0], whole[0] + f, lane, num, den);
-      add_share<A, 1>(M, p, q, phi, e, f ? 0 : rest[1], f ? rest[1] : period[1], period[1], whole[1] + f, lane, num, den);
-      add_share<A, 2>(M, p, q, phi, e, f ? 0 : rest[2], f ? rest[2] : period[2], period[2], whole[2] + f, lane, num, den);
-      if (num != 0) {
-        const T x = M.plain(M.mul(num, inverse_times_power<A>(M, den, phi, 0)));
-        fold_one<A, LMAX>(M, x, acc);
-      }
+      add_share<A, 0, PRIME>(M, p, q, phi, e, f ? 0 : rest[0], f ? rest[0] : period[0], period[0], whole[0] + f, lane, num, den);
+      add_share<A, 1, PRIME>(M, p, q, phi, e, f ? 0 : rest[1], f ? rest[1] : period[1], period[1], whole[1] + f, lane, num, den);
+      add_share<A, 2, PRIME>(M, p, q, phi, e, f ? 0 : rest[2], f ? rest[2] : period[2], period[2], whole[2] + f, lane, num, den);
+      const T x = M.plain(M.mul(num, inverse_times_power<A>(M, den, phi, 0)));  // every lane: warp-wide
+      fold_one<A, LMAX>(M, x, acc);
     }
   }
   flush_cta<LMAX>(acc, G.L, G.slots);

@@ -76,7 +76,9 @@ bool prime_form_serves(int formula, uint64_t n, uint32_t P, uint32_t W, uint64_t
 // summand of its sums.
 double prime_form_imad(const PrimeLimits& lim, int limbs);
 
-constexpr uint64_t kPrimeMinN = 100'000'000;  // below, the terms take no longer (1.4 ms each at 1e8, P = 64)
+// P = 128, term by term and by primes: n = 2e7 334 and 217 us, 3e7 474 and 241, 1e8 1560 and 354.
+// About 200 us of the latter are launches and chains.
+constexpr uint64_t kPrimeMinN = 16'000'000;
 constexpr uint64_t kPrimeMaxN = 10'900'000'000'000;  // 1024 sqrt(0.4 n) < 2^31: word products of the sums
 
 }  // namespace bbp

@@ -49,8 +49,8 @@ def by_async(bbp, plan, n, P):
 # the smallest position that takes primes and its neighbours (n - 1 and n - 2 even and odd, A a
 # multiple of 5 or not), 2^27, 2^29 and 2^31 (word and path changes above and below the moduli),
 # A / 23 past 2^31 (sums in two words), several lists
-@pytest.mark.parametrize("n,P", [(10**8 - 1, 64), (10**8, 64), (10**8 + 1, 100), (10**8 + 3, 256), (10**8 + 4, 448),
-                                 (10**8 + 5, 1000), (2**27 + 1, 704), (2**29 - 1, 128), (2**29 + 3, 32),
+@pytest.mark.parametrize("n,P", [(16 * 10**6 - 1, 64), (16 * 10**6, 64), (16 * 10**6 + 1, 100),
+                                 (16 * 10**6 + 3, 256), (16 * 10**6 + 4, 448), (16 * 10**6 + 5, 1000), (10**8 + 6, 64), (2**27 + 1, 704), (2**29 - 1, 128), (2**29 + 3, 32),
                                  (2**31 - 1, 64), (2**31 + 2, 256), (23 * 2**29 + 7, 128), (23 * 2**31 + 11, 256)])
 def test_equals_the_terms(bbp, plans, n, P):
     assert plans[64].bits(n, P) == by_terms(bbp, plans[64], n, P)
