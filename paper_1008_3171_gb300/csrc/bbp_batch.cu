@@ -26,6 +26,7 @@
 #include "bbp.h"
 #include "bbp_kernels.cuh"
 #include "bbp_planner.h"
+#include "bbp_primes.h"
 #include "bbp_runtime.h"
 
 using namespace bbp;
@@ -33,6 +34,7 @@ using namespace bbp;
 namespace {
 
 constexpr int kVariants = kQueueVariants;
+constexpr int kPrimeLanes = 4;
 constexpr uint32_t kOutStride = kMaxWorkingBits / 8;  // bytes of output per query slot
 
 int lmax_index(int lmax) {
@@ -75,8 +77,8 @@ struct BatchState {
   // device buffers and their capacities (elements)
   HeadArgs* d_jobs = nullptr;               size_t c_jobs = 0;
   uint32_t* d_job_query = nullptr;          size_t c_job_query = 0;
-  uint64_t* d_job_tiles = nullptr;          size_t c_job_tiles = 0;
-  unsigned long long* d_job_ctr = nullptr;  size_t c_job_ctr = 0;  // taken[0..J) then done[0..J)
+  uint64_t* d_job_start = nullptr;          size_t c_job_start = 0;
+  unsigned long long* d_job_done = nullptr; size_t c_job_done = 0;
   TailArgs* d_tails = nullptr;              size_t c_tails = 0;
   uint32_t* d_tail_query = nullptr;         size_t c_tail_query = 0;
   QueryDesc* d_queries = nullptr;           size_t c_queries = 0;
@@ -85,11 +87,11 @@ struct BatchState {
   uint8_t* d_out = nullptr;                 size_t c_out = 0;
   uint32_t* d_valid = nullptr;              size_t c_valid = 0;
   unsigned long long* d_done = nullptr;     size_t c_done = 0;   // [0] = start time, [1 + q] = done
-  unsigned int* d_cursors = nullptr;        size_t c_cursors = 0;  // per wave: kVariants + 1 (tail)
+  unsigned long long* d_cursors = nullptr;  size_t c_cursors = 0;  // per wave: kVariants + 1 (tail)
   // pinned host staging
   HeadArgs* h_jobs = nullptr;               size_t hc_jobs = 0;
   uint32_t* h_job_query = nullptr;          size_t hc_job_query = 0;
-  uint64_t* h_job_tiles = nullptr;          size_t hc_job_tiles = 0;
+  uint64_t* h_job_start = nullptr;          size_t hc_job_start = 0;
   TailArgs* h_tails = nullptr;              size_t hc_tails = 0;
   uint32_t* h_tail_query = nullptr;         size_t hc_tail_query = 0;
   QueryDesc* h_queries = nullptr;           size_t hc_queries = 0;
@@ -97,6 +99,12 @@ struct BatchState {
   uint8_t* h_out = nullptr;                 size_t hc_out = 0;
   uint32_t* h_valid = nullptr;              size_t hc_valid = 0;
   unsigned long long* h_done = nullptr;     size_t hc_done = 0;
+  // prime forms: the check's verdict per query, and the workspaces with their streams
+  uint32_t* d_redo = nullptr;               size_t c_redo = 0;
+  uint32_t* h_redo = nullptr;               size_t hc_redo = 0;
+  PrimeState* lane[kPrimeLanes] = {};
+  cudaStream_t lane_stream[kPrimeLanes] = {};
+  cudaEvent_t lane_done[kPrimeLanes] = {};
   cudaGraphExec_t exec = nullptr;
   cudaStream_t stream = nullptr;  // capture needs a stream other than the legacy default stream
   cudaEvent_t ready = nullptr;
@@ -110,10 +118,17 @@ void release_batch_state(bbp_plan p) {
   if (b->exec) cudaGraphExecDestroy(b->exec);
   if (b->stream) cudaStreamDestroy(b->stream);
   if (b->ready) cudaEventDestroy(b->ready);
+  for (int i = 0; i < kPrimeLanes; ++i) {
+    release_prime_state(&b->lane[i]);
+    if (b->lane_stream[i]) cudaStreamDestroy(b->lane_stream[i]);
+    if (b->lane_done[i]) cudaEventDestroy(b->lane_done[i]);
+  }
+  cudaFree(b->d_redo);
+  cudaFreeHost(b->h_redo);
   cudaFree(b->d_jobs);
   cudaFree(b->d_job_query);
-  cudaFree(b->d_job_tiles);
-  cudaFree(b->d_job_ctr);
+  cudaFree(b->d_job_start);
+  cudaFree(b->d_job_done);
   cudaFree(b->d_tails);
   cudaFree(b->d_tail_query);
   cudaFree(b->d_queries);
@@ -125,7 +140,7 @@ void release_batch_state(bbp_plan p) {
   cudaFree(b->d_cursors);
   cudaFreeHost(b->h_jobs);
   cudaFreeHost(b->h_job_query);
-  cudaFreeHost(b->h_job_tiles);
+  cudaFreeHost(b->h_job_start);
   cudaFreeHost(b->h_tails);
   cudaFreeHost(b->h_tail_query);
   cudaFreeHost(b->h_queries);
@@ -146,10 +161,12 @@ struct BatchPlan {
   uint32_t tail_begin[kMaxWaves + 1] = {};               // tail jobs of a wave
   uint64_t terms = 0, head_terms = 0;
   double imad = 0;
+  struct Prime { uint32_t q, W; uint64_t n, bound; };
+  std::vector<Prime> primes;  // queries by the prime form, smallest first
 };
 
 static bbp_status plan_batch(bbp_plan p, int f, uint32_t count, const uint64_t* n, const uint32_t* P,
-                             BatchState* b, BatchPlan* bp) {
+                             BatchState* b, BatchPlan* bp, bool by_primes) {
   const FormulaDef& F = formula_def(f);
   std::vector<std::vector<HeadArgs>> vj(kVariants);
   std::vector<std::vector<uint32_t>> vq(kVariants);
@@ -179,10 +196,27 @@ static bbp_status plan_batch(bbp_plan p, int f, uint32_t count, const uint64_t* 
     for (const TermRange& r : ranges)
       if (!r.tail) qtiles += (r.count + tile_terms(p, r.path) - 1) / tile_terms(p, r.path);
     if (qtiles > kMaxQueueTiles) return BBP_ERANGE;  // carry-save limbs could pass 2^64
+    const uint64_t bound = N + F.count + 1;
+    const bool prime = by_primes && prime_form_serves(f, n[q], P[q], W, bound);
+    for (const TermRange& r : ranges) {
+      bp->terms += r.count;
+      if (!r.tail) bp->head_terms += r.count;
+      if (!r.tail && !prime) bp->imad += r.imad;
+    }
+    if (prime) {  // the queue takes what the prime form leaves
+      const PrimeLimits lim = prime_limits(n[q] - 1);
+      bp->imad += prime_form_imad(lim, static_cast<int>(L));
+      bp->primes.push_back(BatchPlan::Prime{q, W, n[q], bound});
+      ranges.clear();
+      for (uint32_t j = 0; j < F.count; ++j)
+        if (plan_series(F, j, n[q], W, static_cast<uint32_t>(lmax), prime_first_k(lim, j), UINT64_MAX, ranges,
+                        p->wide_min_bits) != 0)
+          return BBP_EINVAL;
+      jobs_left[q] = 1;  // held: the check writes the result
+    }
     for (const TermRange& r : ranges) {
       const SeriesDef& s = F.s[r.j];
       qterms[q] += r.count;
-      bp->terms += r.count;
       if (r.tail) {
         TailArgs a{};
         a.d = n[q] - 1;
@@ -212,7 +246,13 @@ static bbp_status plan_batch(bbp_plan p, int f, uint32_t count, const uint64_t* 
         a.L = L;
         a.alternating = F.alternating;
         a.negate = ((s.sign < 0) != (F.alternating && (r.k_begin & 1ull))) ? 1u : 0u;
-        a.run = static_cast<uint32_t>(p->run);
+        // Short ranges take fewer terms per stream: 64 tiles where they can, so that a range is not
+        // a few warps' long runs (but at least 8 terms: each run starts with a division).  With one
+        // tile counter for all jobs (queue_kernel), 164 queries up to 1.6e7: 12.6 -> 5.1 ms.
+        const uint64_t lanes = 32ull * static_cast<uint64_t>(head_streams(p, r.path));
+        uint32_t run = static_cast<uint32_t>(p->run);
+        while (run >= 16 && run % 4 == 0 && r.count < 64 * lanes * run) run /= 2;
+        a.run = run;
         a.window = r.window;
         a.first = r.first;
         a.first_max = r.first_max;
@@ -220,9 +260,7 @@ static bbp_status plan_batch(bbp_plan p, int f, uint32_t count, const uint64_t* 
         const int v = lmax_index(lmax) * kNumPaths + r.path;
         vj[v].push_back(a);
         vq[v].push_back(q);
-        vt[v].push_back((r.count + tile_terms(p, r.path) - 1) / tile_terms(p, r.path));
-        bp->head_terms += r.count;
-        bp->imad += r.imad;
+        vt[v].push_back((r.count + lanes * run - 1) / (lanes * run));
       }
       jobs_left[q]++;
     }
@@ -236,12 +274,17 @@ static bbp_status plan_batch(bbp_plan p, int f, uint32_t count, const uint64_t* 
       jobs_left[q] = 1;
     }
     QueryDesc& Q = queries[q];
-    Q.bound = N + F.count + 1;
+    Q.bound = bound;
     Q.P = P[q];
     Q.L = L;
     Q.out_offset = q * kOutStride;
   }
-  // waves: queries by size, each wave twice the work of the ones before it, at most 1/12 of the total
+  std::sort(bp->primes.begin(), bp->primes.end(),
+            [](const BatchPlan::Prime& x, const BatchPlan::Prime& y) { return x.n != y.n ? x.n < y.n : x.q < y.q; });
+  // waves: queries by size, each wave twice the work of the ones before it, at most 1/12 of the
+  // total -- but at least kWaveTerms, some milliseconds: a launch lasts no less than a tile's 50 us,
+  // whatever its size (164 queries up to 1.6e7, 2.5e8 terms: 19 ms in 24 waves, 12.6 in two)
+  constexpr uint64_t kWaveTerms = 200'000'000;
   std::vector<uint32_t> qorder(count);
   std::iota(qorder.begin(), qorder.end(), 0u);
   std::stable_sort(qorder.begin(), qorder.end(), [&](uint32_t x, uint32_t y) { return qterms[x] < qterms[y]; });
@@ -249,8 +292,8 @@ static bbp_status plan_batch(bbp_plan p, int f, uint32_t count, const uint64_t* 
   {
     uint64_t total = 0;
     for (uint64_t t : qterms) total += t;
-    const uint64_t first = std::max<uint64_t>(total / 4096, 1);  // the first wave: 1/4096 of the work
-    const uint64_t step_cap = std::max<uint64_t>(total / 12, 1);  // no wave beyond 1/12 of the work
+    const uint64_t first = std::max<uint64_t>(total / 4096, kWaveTerms);  // the first wave: 1/4096 of the work
+    const uint64_t step_cap = std::max<uint64_t>(total / 12, kWaveTerms);  // no wave beyond 1/12 of the work
     uint64_t done = 0, target = first;
     uint32_t w = 0;
     for (uint32_t i = 0; i < count; ++i) {
@@ -267,11 +310,12 @@ static bbp_status plan_batch(bbp_plan p, int f, uint32_t count, const uint64_t* 
   uint32_t nj = 0;
   for (int v = 0; v < kVariants; ++v) nj += static_cast<uint32_t>(vj[v].size());
   if (!grow_host(&b->h_jobs, &b->hc_jobs, nj) || !grow_host(&b->h_job_query, &b->hc_job_query, nj) ||
-      !grow_host(&b->h_job_tiles, &b->hc_job_tiles, nj) || !grow_host(&b->h_tails, &b->hc_tails, tails.size()) ||
+      !grow_host(&b->h_job_start, &b->hc_job_start, nj + 1) || !grow_host(&b->h_tails, &b->hc_tails, tails.size()) ||
       !grow_host(&b->h_tail_query, &b->hc_tail_query, tails.size()) ||
       !grow_host(&b->h_queries, &b->hc_queries, count) || !grow_host(&b->h_jobs_left, &b->hc_jobs_left, count))
     return BBP_ENOMEM;
   uint32_t at = 0;
+  b->h_job_start[0] = 0;
   for (uint32_t w = 0; w < bp->nwaves; ++w) {
     for (int v = 0; v < kVariants; ++v) {
       bp->group_begin[w * kVariants + v] = at;
@@ -283,7 +327,7 @@ static bbp_status plan_batch(bbp_plan p, int f, uint32_t count, const uint64_t* 
       for (uint32_t i : order) {
         b->h_jobs[at] = vj[v][i];
         b->h_job_query[at] = vq[v][i];
-        b->h_job_tiles[at] = vt[v][i];
+        b->h_job_start[at + 1] = b->h_job_start[at] + vt[v][i];
         ++at;
       }
     }
@@ -314,24 +358,28 @@ static bbp_status plan_batch(bbp_plan p, int f, uint32_t count, const uint64_t* 
     if ((expr) != cudaSuccess) return BBP_ECUDA;   \
   } while (0)
 
-extern "C" bbp_status bbp_bits_batch(bbp_plan p, bbp_formula f, uint32_t count, const uint64_t* n, const uint32_t* P,
-                                     uint8_t* out, uint32_t out_stride, uint32_t* valid_bits, double* latency_ms) {
-  if (!p || (f != BBP_BELLARD && f != BBP_BBP) || (count && (!n || !P || !out))) return BBP_EINVAL;
-  if (count == 0) return BBP_OK;
-  if (count > kMaxQueueQueries) return BBP_EINVAL;
-  uint32_t maxbytes = 0;
-  for (uint32_t q = 0; q < count; ++q) maxbytes = std::max(maxbytes, (P[q] + 7) / 8);
-  if (out_stride < maxbytes) return BBP_EINVAL;
-  BBP_TRY(cudaSetDevice(p->device));
-  if (!p->batch) {
-    p->batch = new (std::nothrow) BatchState();
-    if (!p->batch) return BBP_ENOMEM;
+namespace bbp {
+
+// The prime form's workspaces for positions up to n; false if they cannot be had.
+static bool prime_lanes(BatchState* b, uint64_t n, int lanes) {
+  for (int i = 0; i < lanes; ++i) {
+    if (!b->lane_stream[i] && cudaStreamCreateWithFlags(&b->lane_stream[i], cudaStreamNonBlocking) != cudaSuccess) return false;
+    if (!b->lane_done[i] && cudaEventCreateWithFlags(&b->lane_done[i], cudaEventDisableTiming) != cudaSuccess) return false;
+    if (!prime_workspace(&b->lane[i], n, kPrimeBatchListMax, b->lane_stream[i])) return false;
   }
+  return true;
+}
+
+// One pass over the queries; by_primes: with the prime form where it serves.
+static bbp_status run_batch(bbp_plan p, bbp_formula f, uint32_t count, const uint64_t* n, const uint32_t* P,
+                            uint8_t* out, uint32_t out_stride, uint32_t* valid_bits, double* latency_ms,
+                            bool by_primes) {
   BatchState* b = p->batch;
   // device buffers first (job descriptors hold accumulator addresses)
   if (!grow_device(&b->d_accum, &b->c_accum, static_cast<size_t>(count) * kMaxLimbs) ||
       !grow_device(&b->d_queries, &b->c_queries, count) || !grow_device(&b->d_jobs_left, &b->c_jobs_left, count) ||
       !grow_device(&b->d_out, &b->c_out, static_cast<size_t>(count) * kOutStride) ||
+      !grow_device(&b->d_redo, &b->c_redo, count) || !grow_host(&b->h_redo, &b->hc_redo, count) ||
       !grow_device(&b->d_valid, &b->c_valid, count) || !grow_device(&b->d_done, &b->c_done, count + 1ull) ||
       !grow_host(&b->h_out, &b->hc_out, static_cast<size_t>(count) * kOutStride) ||
       !grow_host(&b->h_valid, &b->hc_valid, count) || !grow_host(&b->h_done, &b->hc_done, count + 1ull))
@@ -339,20 +387,26 @@ extern "C" bbp_status bbp_bits_batch(bbp_plan p, bbp_formula f, uint32_t count, 
   if (!grow_device(&b->d_cursors, &b->c_cursors, static_cast<size_t>(kMaxWaves) * (kVariants + 1)))
     return BBP_ENOMEM;
   BatchPlan bp;
-  bbp_status st = plan_batch(p, f, count, n, P, b, &bp);
+  bbp_status st = plan_batch(p, f, count, n, P, b, &bp, by_primes);
   if (st != BBP_OK) return st;
+  const int lanes = static_cast<int>(std::min<size_t>(kPrimeLanes, bp.primes.size()));
+  if (lanes > 0 && !prime_lanes(b, bp.primes.back().n, lanes)) {  // no memory for it: everything through the queue
+    cudaGetLastError();
+    bp = BatchPlan{};
+    st = plan_batch(p, f, count, n, P, b, &bp, false);
+    if (st != BBP_OK) return st;
+  }
   if (!grow_device(&b->d_jobs, &b->c_jobs, bp.njobs) || !grow_device(&b->d_job_query, &b->c_job_query, bp.njobs) ||
-      !grow_device(&b->d_job_tiles, &b->c_job_tiles, bp.njobs) ||
-      !grow_device(&b->d_job_ctr, &b->c_job_ctr, 2ull * bp.njobs) ||
+      !grow_device(&b->d_job_start, &b->c_job_start, bp.njobs + 1ull) ||
+      !grow_device(&b->d_job_done, &b->c_job_done, bp.njobs) ||
       !grow_device(&b->d_tails, &b->c_tails, bp.ntails) || !grow_device(&b->d_tail_query, &b->c_tail_query, bp.ntails))
     return BBP_ENOMEM;
 
   BatchDev dev{};
   dev.jobs = b->d_jobs;
   dev.job_query = b->d_job_query;
-  dev.job_tiles = b->d_job_tiles;
-  dev.job_taken = b->d_job_ctr;
-  dev.job_done = b->d_job_ctr + bp.njobs;
+  dev.job_start = b->d_job_start;
+  dev.job_done = b->d_job_done;
   dev.tails = b->d_tails;
   dev.tail_query = b->d_tail_query;
   dev.grab = static_cast<uint32_t>(p->grab);
@@ -376,18 +430,18 @@ extern "C" bbp_status bbp_bits_batch(bbp_plan p, bbp_formula f, uint32_t count, 
   auto chk = [&](cudaError_t r) { if (e == cudaSuccess) e = r; };
   chk(cudaMemcpyAsync(b->d_jobs, b->h_jobs, sizeof(HeadArgs) * bp.njobs, cudaMemcpyHostToDevice, s));
   chk(cudaMemcpyAsync(b->d_job_query, b->h_job_query, sizeof(uint32_t) * bp.njobs, cudaMemcpyHostToDevice, s));
-  chk(cudaMemcpyAsync(b->d_job_tiles, b->h_job_tiles, sizeof(uint64_t) * bp.njobs, cudaMemcpyHostToDevice, s));
+  chk(cudaMemcpyAsync(b->d_job_start, b->h_job_start, sizeof(uint64_t) * (bp.njobs + 1ull), cudaMemcpyHostToDevice, s));
   chk(cudaMemcpyAsync(b->d_tails, b->h_tails, sizeof(TailArgs) * bp.ntails, cudaMemcpyHostToDevice, s));
   chk(cudaMemcpyAsync(b->d_tail_query, b->h_tail_query, sizeof(uint32_t) * bp.ntails, cudaMemcpyHostToDevice, s));
   chk(cudaMemcpyAsync(b->d_queries, b->h_queries, sizeof(QueryDesc) * count, cudaMemcpyHostToDevice, s));
   chk(cudaMemcpyAsync(b->d_jobs_left, b->h_jobs_left, sizeof(unsigned int) * count, cudaMemcpyHostToDevice, s));
-  chk(cudaMemsetAsync(b->d_job_ctr, 0, sizeof(unsigned long long) * 2 * bp.njobs, s));
-  chk(cudaMemsetAsync(b->d_cursors, 0, sizeof(unsigned int) * kMaxWaves * (kVariants + 1), s));
+  chk(cudaMemsetAsync(b->d_job_done, 0, sizeof(unsigned long long) * bp.njobs, s));
+  chk(cudaMemsetAsync(b->d_cursors, 0, sizeof(unsigned long long) * kMaxWaves * (kVariants + 1), s));
   chk(cudaMemsetAsync(b->d_accum, 0, sizeof(unsigned long long) * kMaxLimbs * count, s));
   chk(launch_timestamp(b->d_done, s));
   uint64_t launches = 1, head_launches = 0;
   for (uint32_t w = 0; w < bp.nwaves; ++w) {
-    unsigned int* cur = b->d_cursors + static_cast<size_t>(w) * (kVariants + 1);
+    unsigned long long* cur = b->d_cursors + static_cast<size_t>(w) * (kVariants + 1);
     if (bp.tail_begin[w] < bp.tail_begin[w + 1]) {
       chk(launch_queue_tail(dev, bp.tail_begin[w], bp.tail_begin[w + 1], cur + kVariants, p->sm_count * 4, s));
       ++launches;
@@ -402,9 +456,6 @@ extern "C" bbp_status bbp_bits_batch(bbp_plan p, bbp_formula f, uint32_t count, 
       ++head_launches;
     }
   }
-  chk(cudaMemcpyAsync(b->h_out, b->d_out, static_cast<size_t>(count) * kOutStride, cudaMemcpyDeviceToHost, s));
-  chk(cudaMemcpyAsync(b->h_valid, b->d_valid, sizeof(uint32_t) * count, cudaMemcpyDeviceToHost, s));
-  chk(cudaMemcpyAsync(b->h_done, b->d_done, sizeof(unsigned long long) * (count + 1ull), cudaMemcpyDeviceToHost, s));
   const cudaError_t ce = cudaStreamEndCapture(s, &graph);
   if (e != cudaSuccess || ce != cudaSuccess) {
     if (graph) cudaGraphDestroy(graph);
@@ -428,7 +479,31 @@ extern "C" bbp_status bbp_bits_batch(bbp_plan p, bbp_formula f, uint32_t count, 
   cudaGraphDestroy(graph);
   if (p->profile) BBP_TRY(cudaEventRecord(p->ev0, s));
   BBP_TRY(cudaGraphLaunch(b->exec, s));
+  if (!bp.primes.empty()) {
+    BBP_TRY(cudaEventRecord(b->ready, s));
+    const int used = static_cast<int>(std::min<size_t>(kPrimeLanes, bp.primes.size()));
+    for (int i = 0; i < used; ++i) BBP_TRY(cudaStreamWaitEvent(b->lane_stream[i], b->ready, 0));
+    for (size_t i = 0; i < bp.primes.size(); ++i) {
+      const BatchPlan::Prime& r = bp.primes[i];
+      const int k = static_cast<int>(i % kPrimeLanes);
+      const bbp_status ls = launch_prime_form(
+          b->lane[k], p->sm_count, r.n, r.W, P[r.q], r.bound, b->d_accum + static_cast<uint64_t>(r.q) * kMaxLimbs,
+          b->d_out + static_cast<size_t>(r.q) * kOutStride, b->d_valid + r.q, b->d_redo + r.q, b->lane_stream[k],
+          &launches);
+      if (ls != BBP_OK) return ls;
+      BBP_TRY(launch_timestamp(b->d_done + 1 + r.q, b->lane_stream[k]));
+      ++launches;
+    }
+    for (int i = 0; i < used; ++i) {
+      BBP_TRY(cudaEventRecord(b->lane_done[i], b->lane_stream[i]));
+      BBP_TRY(cudaStreamWaitEvent(s, b->lane_done[i], 0));
+    }
+    BBP_TRY(cudaMemcpyAsync(b->h_redo, b->d_redo, sizeof(uint32_t) * count, cudaMemcpyDeviceToHost, s));
+  }
   if (p->profile) BBP_TRY(cudaEventRecord(p->ev1, s));
+  BBP_TRY(cudaMemcpyAsync(b->h_out, b->d_out, static_cast<size_t>(count) * kOutStride, cudaMemcpyDeviceToHost, s));
+  BBP_TRY(cudaMemcpyAsync(b->h_valid, b->d_valid, sizeof(uint32_t) * count, cudaMemcpyDeviceToHost, s));
+  BBP_TRY(cudaMemcpyAsync(b->h_done, b->d_done, sizeof(unsigned long long) * (count + 1ull), cudaMemcpyDeviceToHost, s));
   BBP_TRY(cudaStreamSynchronize(s));
   p->stats = bbp_stats{};
   p->stats.terms = bp.terms;
@@ -441,14 +516,75 @@ extern "C" bbp_status bbp_bits_batch(bbp_plan p, bbp_formula f, uint32_t count, 
     BBP_TRY(cudaEventElapsedTime(&ms, p->ev0, p->ev1));
     p->stats.head_ms = ms;
   }
+  double last_ms = 0;
   for (uint32_t q = 0; q < count; ++q) {
     std::memcpy(out + static_cast<size_t>(q) * out_stride, b->h_out + static_cast<size_t>(q) * kOutStride,
                 (P[q] + 7) / 8);
-    if (valid_bits) valid_bits[q] = b->h_valid[q];
-    if (latency_ms) latency_ms[q] = static_cast<double>(b->h_done[1 + q] - b->h_done[0]) * 1e-6;
+    valid_bits[q] = b->h_valid[q];
+    latency_ms[q] = static_cast<double>(b->h_done[1 + q] - b->h_done[0]) * 1e-6;
+    last_ms = std::max(last_ms, latency_ms[q]);
   }
-  if (p->strict)
-    for (uint32_t q = 0; q < count; ++q)
-      if (b->h_valid[q] < P[q]) return BBP_EINVALID_BITS;
+  // queries that the check sends back to the terms: a second pass
+  std::vector<uint32_t> again;
+  for (const BatchPlan::Prime& r : bp.primes)
+    if (b->h_redo[r.q]) again.push_back(r.q);
+  if (!again.empty()) {
+    const uint32_t m = static_cast<uint32_t>(again.size());
+    std::vector<uint64_t> n2(m);
+    std::vector<uint32_t> P2(m), valid2(m);
+    std::vector<uint8_t> out2(static_cast<size_t>(m) * out_stride);
+    std::vector<double> ms2(m);
+    for (uint32_t i = 0; i < m; ++i) {
+      n2[i] = n[again[i]];
+      P2[i] = P[again[i]];
+    }
+    const bbp_stats first = p->stats;
+    const bbp_status rs = run_batch(p, f, m, n2.data(), P2.data(), out2.data(), out_stride, valid2.data(), ms2.data(), false);
+    if (rs != BBP_OK) return rs;
+    const bbp_stats second = p->stats;
+    p->stats = first;
+    p->stats.head_launches += second.head_launches;
+    p->stats.kernel_launches += second.kernel_launches;
+    p->stats.imad_model += second.imad_model;
+    p->stats.head_ms += second.head_ms;
+    for (uint32_t i = 0; i < m; ++i) {
+      const uint32_t q = again[i];
+      std::memcpy(out + static_cast<size_t>(q) * out_stride, out2.data() + static_cast<size_t>(i) * out_stride,
+                  (P[q] + 7) / 8);
+      valid_bits[q] = valid2[i];
+      latency_ms[q] = last_ms + ms2[i];
+    }
+  }
+  return BBP_OK;
+}
+
+}  // namespace bbp
+
+extern "C" bbp_status bbp_bits_batch(bbp_plan p, bbp_formula f, uint32_t count, const uint64_t* n, const uint32_t* P,
+                                     uint8_t* out, uint32_t out_stride, uint32_t* valid_bits, double* latency_ms) {
+  if (!p || (f != BBP_BELLARD && f != BBP_BBP) || (count && (!n || !P || !out))) return BBP_EINVAL;
+  if (count == 0) return BBP_OK;
+  if (count > kMaxQueueQueries) return BBP_EINVAL;
+  uint32_t maxbytes = 0;
+  for (uint32_t q = 0; q < count; ++q) maxbytes = std::max(maxbytes, (P[q] + 7) / 8);
+  if (out_stride < maxbytes) return BBP_EINVAL;
+  BBP_TRY(cudaSetDevice(p->device));
+  if (!p->batch) {
+    p->batch = new (std::nothrow) BatchState();
+    if (!p->batch) return BBP_ENOMEM;
+  }
+  try {
+    std::vector<uint32_t> valid(count);
+    std::vector<double> ms(count);
+    const bbp_status st = run_batch(p, f, count, n, P, out, out_stride, valid.data(), ms.data(), true);
+    if (st != BBP_OK) return st;
+    if (valid_bits) std::copy(valid.begin(), valid.end(), valid_bits);
+    if (latency_ms) std::copy(ms.begin(), ms.end(), latency_ms);
+    if (p->strict)
+      for (uint32_t q = 0; q < count; ++q)
+        if (valid[q] < P[q]) return BBP_EINVALID_BITS;
+  } catch (const std::bad_alloc&) {
+    return BBP_ENOMEM;
+  }
   return BBP_OK;
 }

@@ -35,7 +35,7 @@ int head_occupancy_t(int threads) {
 }
 
 template <int PATH, int S>
-cudaError_t launch_queue_t(const BatchDev& b, uint32_t jb, uint32_t je, unsigned int* cursor, int blocks,
+cudaError_t launch_queue_t(const BatchDev& b, uint32_t jb, uint32_t je, unsigned long long* cursor, int blocks,
                            cudaStream_t s) {
   queue_kernel<BBP_LMAX, PATH, S><<<blocks, kHeadThreads, 0, s>>>(b, jb, je, cursor);
   return cudaGetLastError();
@@ -104,7 +104,7 @@ int BBP_CAT(head_occupancy_l, BBP_LMAX)(int path, int streams, int threads) {
   }
 }
 
-cudaError_t BBP_CAT(launch_queue_l, BBP_LMAX)(const BatchDev& b, uint32_t jb, uint32_t je, unsigned int* cursor,
+cudaError_t BBP_CAT(launch_queue_l, BBP_LMAX)(const BatchDev& b, uint32_t jb, uint32_t je, unsigned long long* cursor,
                                               int path, int streams, int blocks, cudaStream_t s) {
   const bool two = streams == 2;
   switch (path) {

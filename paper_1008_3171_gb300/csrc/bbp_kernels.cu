@@ -125,11 +125,11 @@ __global__ void timestamp_kernel(unsigned long long* where) {
 
 // Tail jobs: one warp per job, one term per lane at a time.
 __global__ void queue_tail_kernel(const BatchDev B, const uint32_t tail_begin, const uint32_t tail_end,
-                                  unsigned int* cursor) {
+                                  unsigned long long* cursor) {
   const uint32_t lane = threadIdx.x & 31u;
   for (;;) {
     uint32_t j = 0;
-    if (lane == 0) j = tail_begin + atomicAdd(cursor, 1u);
+    if (lane == 0) j = tail_begin + static_cast<uint32_t>(atomicAdd(cursor, 1ull));
     j = __shfl_sync(0xffffffffu, j, 0);
     if (j >= tail_end) break;
     const TailArgs A = B.tails[j];
@@ -237,7 +237,7 @@ int queue_occupancy(int path, int streams, int lmax) {
   }
 }
 
-cudaError_t launch_queue(const BatchDev& b, uint32_t job_begin, uint32_t job_end, unsigned int* cursor, int path,
+cudaError_t launch_queue(const BatchDev& b, uint32_t job_begin, uint32_t job_end, unsigned long long* cursor, int path,
                          int streams, int lmax, int blocks, cudaStream_t s) {
   switch (lmax) {
 #define BBP_CASE(L) \
@@ -274,7 +274,7 @@ cudaError_t launch_timestamp(unsigned long long* where, cudaStream_t s) {
   return cudaGetLastError();
 }
 
-cudaError_t launch_queue_tail(const BatchDev& b, uint32_t tail_begin, uint32_t tail_end, unsigned int* cursor,
+cudaError_t launch_queue_tail(const BatchDev& b, uint32_t tail_begin, uint32_t tail_end, unsigned long long* cursor,
                               int blocks, cudaStream_t s) {
   if (tail_begin >= tail_end) return cudaSuccess;
   queue_tail_kernel<<<blocks, 128, 0, s>>>(b, tail_begin, tail_end, cursor);

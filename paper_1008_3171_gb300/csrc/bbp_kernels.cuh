@@ -70,8 +70,8 @@ constexpr int kQueueVariants = kNumLmaxClasses * kNumPaths;  // limb class x mod
 //
 // A batch of queries is a list of jobs: head jobs (one HeadArgs each: a range of
 // head terms of one series of one query, whose `slots` point at that query's
-// accumulators) grouped by kernel variant, plus tail jobs.  Persistent warps hand
-// out `grab` tiles of the current job at a time; the warp that finishes a query's
+// accumulators) grouped by kernel variant, plus tail jobs.  Persistent warps take
+// `grab` tiles of the jobs laid end to end at a time; the warp that finishes a query's
 // last job finalizes the query.
 struct QueryDesc {
   uint64_t bound;       // N + J + 1: |S - exact| < bound units
@@ -84,8 +84,7 @@ struct QueryDesc {
 struct BatchDev {
   const HeadArgs* jobs;            // head jobs, grouped by kernel variant
   const uint32_t* job_query;       // query index of each head job
-  const uint64_t* job_tiles;       // warp tiles of each head job
-  unsigned long long* job_taken;   // tiles handed out so far (atomic)
+  const uint64_t* job_start;       // warp tiles of the head jobs before each (and after the last)
   unsigned long long* job_done;    // tiles finished so far (atomic)
   const TailArgs* tails;           // tail jobs
   const uint32_t* tail_query;
@@ -130,11 +129,11 @@ cudaError_t launch_finalize_bits(const unsigned long long* slots, int L, uint32_
                                  uint8_t* out_bytes, uint32_t* valid_bits, uint32_t* out_limbs, cudaStream_t s,
                                  const uint32_t* gate = nullptr);
 // One persistent launch over the head jobs [job_begin, job_end) of one variant;
-// *cursor (relative to job_begin) must be 0.  blocks = resident CTAs.
-cudaError_t launch_queue(const BatchDev& b, uint32_t job_begin, uint32_t job_end, unsigned int* cursor, int path,
+// *cursor (tiles handed out) must be 0.  blocks = resident CTAs.
+cudaError_t launch_queue(const BatchDev& b, uint32_t job_begin, uint32_t job_end, unsigned long long* cursor, int path,
                          int streams, int lmax, int blocks, cudaStream_t s);
-// Tail jobs [tail_begin, tail_end); *cursor (relative to tail_begin) must be 0.
-cudaError_t launch_queue_tail(const BatchDev& b, uint32_t tail_begin, uint32_t tail_end, unsigned int* cursor,
+// Tail jobs [tail_begin, tail_end); *cursor (jobs handed out) must be 0.
+cudaError_t launch_queue_tail(const BatchDev& b, uint32_t tail_begin, uint32_t tail_end, unsigned long long* cursor,
                               int blocks, cudaStream_t s);
 cudaError_t launch_timestamp(unsigned long long* where, cudaStream_t s);
 int queue_occupancy(int path, int streams, int lmax);
@@ -153,7 +152,7 @@ cudaError_t launch_prime(const PrimeArgs& a, PrimeKernel k, int lmax, int sms, c
 #define BBP_DECLARE_LMAX(L)                                                                                    \
   cudaError_t launch_head_l##L(const HeadArgs& a, int path, int streams, int blocks, int threads, cudaStream_t s); \
   int head_occupancy_l##L(int path, int streams, int threads);                                                 \
-  cudaError_t launch_queue_l##L(const BatchDev& b, uint32_t jb, uint32_t je, unsigned int* cursor, int path,      \
+  cudaError_t launch_queue_l##L(const BatchDev& b, uint32_t jb, uint32_t je, unsigned long long* cursor, int path,      \
                                 int streams, int blocks, cudaStream_t s);                                      \
   int queue_occupancy_l##L(int path, int streams);                                                             \
   cudaError_t launch_prime_l##L(const PrimeArgs& a, PrimeKernel k, int sms, cudaStream_t s);

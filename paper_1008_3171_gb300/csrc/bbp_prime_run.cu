@@ -25,7 +25,6 @@ namespace {
 
 constexpr uint32_t kMaxBase = (1u << 23) - 1;       // base primes up to here: 564,162 odd ones
 constexpr uint32_t kBaseCap = 565000;
-constexpr uint32_t kMaxListCap = 24u << 20;         // primes of one list (96 MB), two lists
 constexpr uint32_t kMaxLists = 1u << 16;
 constexpr uint64_t kLongSum = 32000;                // primes below A / this take a warp each,
 constexpr uint64_t kGroupSum = 1000;                // those below A / this eight lanes
@@ -41,13 +40,14 @@ uint64_t isqrt(uint64_t v) {
 
 }  // namespace bbp
 
+// Device memory, streams and events of one query at a time.
 struct PrimeState {
   uint32_t* list[2] = {};
   uint32_t list_cap = 0;
   uint32_t* primes = nullptr;  // base primes
   bbp::SievePrime* sieve_primes = nullptr;
-  // [0] base primes, [1] those from 17 on, [2] redo; then the length of each list, then the
-  // primes of each handed out so far
+  // [0] base primes, [1] those from 17 on; then the length of each list, then the primes of
+  // each handed out so far
   uint32_t* counts = nullptr;
   cudaStream_t sieve = nullptr, sums = nullptr;  // beside the caller's stream
   cudaEvent_t ready[2] = {}, used[2] = {}, base = nullptr, done = nullptr;
@@ -57,12 +57,6 @@ namespace bbp {
 
 namespace {
 constexpr size_t kCountHead = 4;
-
-// Primes of one list for a query at position n: all of them up to the limit.
-uint32_t list_length(uint64_t n) {
-  const double x = static_cast<double>(n);
-  return static_cast<uint32_t>(std::min<double>(kMaxListCap, 1.2 * x / std::log(x) + 4096.0));
-}
 
 bool make_state(PrimeState* s) {
   int low = 0, high = 0;
@@ -83,8 +77,8 @@ bool make_state(PrimeState* s) {
 }
 }  // namespace
 
-void release_prime_state(bbp_plan p) {
-  PrimeState* s = p->primes;
+void release_prime_state(PrimeState** state) {
+  PrimeState* s = *state;
   if (!s) return;
   if (s->sieve) cudaStreamSynchronize(s->sieve);
   if (s->sums) cudaStreamSynchronize(s->sums);
@@ -101,29 +95,29 @@ void release_prime_state(bbp_plan p) {
   cudaFree(s->sieve_primes);
   cudaFree(s->counts);
   delete s;
-  p->primes = nullptr;
+  *state = nullptr;
 }
 
-// The workspace for position n; false if it is not there and cannot be made now (a
-// stream capture is going on, or memory is short): the caller then runs term by term.
-bool prime_workspace(bbp_plan p, uint64_t n, cudaStream_t st) {
-  const uint32_t want = list_length(n);
-  if (p->primes && p->primes->list_cap >= want) return true;
+bool prime_workspace(PrimeState** state, uint64_t n, uint32_t max_list, cudaStream_t st) {
+  // primes of one list: all of them up to the limit
+  const double x = static_cast<double>(n);
+  const uint32_t want = static_cast<uint32_t>(std::min<double>(max_list, 1.2 * x / std::log(x) + 4096.0));
+  if (*state && (*state)->list_cap >= want) return true;
   cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
   if (cudaStreamIsCapturing(st, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone) {
     cudaGetLastError();
     return false;
   }
-  if (!p->primes) {
-    p->primes = new (std::nothrow) PrimeState();
-    if (!p->primes) return false;
-    if (!make_state(p->primes)) {
+  if (!*state) {
+    *state = new (std::nothrow) PrimeState();
+    if (!*state) return false;
+    if (!make_state(*state)) {
       cudaGetLastError();
-      release_prime_state(p);
+      release_prime_state(state);
       return false;
     }
   }
-  PrimeState* s = p->primes;
+  PrimeState* s = *state;
   s->list_cap = 0;
   for (uint32_t*& l : s->list) {
     cudaFree(l);  // waits for the work that reads it
@@ -137,15 +131,9 @@ bool prime_workspace(bbp_plan p, uint64_t n, cudaStream_t st) {
   return true;
 }
 
-uint32_t* prime_redo_flag(bbp_plan p) { return p->primes->counts + 2; }
-
-// Adds the prime form of the head terms covered by prime_limits(n - 1) to `slots`, and
-// enqueues the check of the finished sum (the terms it does not cover must be in `slots`
-// already).  *launches counts the kernels.
-bbp_status launch_prime_form(bbp_plan p, uint64_t n, uint32_t W, uint32_t P, uint64_t bound,
-                             unsigned long long* slots, uint8_t* d_out, uint32_t* d_valid, cudaStream_t st,
-                             uint64_t* launches) {
-  PrimeState* S = p->primes;
+bbp_status launch_prime_form(PrimeState* S, int sm_count, uint64_t n, uint32_t W, uint32_t P, uint64_t bound,
+                             unsigned long long* slots, uint8_t* d_out, uint32_t* d_valid, uint32_t* d_redo,
+                             cudaStream_t st, uint64_t* launches) {
   const int lmax = head_lmax_for(static_cast<int>(W / 32));
   if (lmax == 0) return BBP_EINVAL;
   const PrimeLimits lim = prime_limits(n - 1);
@@ -198,7 +186,7 @@ bbp_status launch_prime_form(bbp_plan p, uint64_t n, uint32_t W, uint32_t P, uin
       const double room = 0.85 * S->list_cap * (std::log(static_cast<double>(std::max<uint64_t>(lo, 1000))) - 1.1);
       uint64_t nseg = std::max<uint64_t>(1, static_cast<uint64_t>(room) / seg);
       // whole waves of the sieve's CTAs, eight a segment, one an SM beside the primes' kernels
-      const uint64_t wave = std::max<uint64_t>(1, static_cast<uint64_t>(p->sm_count) / 8);
+      const uint64_t wave = std::max<uint64_t>(1, static_cast<uint64_t>(sm_count) / 8);
       if (nseg > wave) nseg -= nseg % wave;
       const uint64_t hi = std::min(s.hi, base + nseg * seg - 1);
       lists.push_back(List{base, lo, hi, static_cast<uint32_t>((hi - base) / seg + 1), s.k});
@@ -221,9 +209,9 @@ bbp_status launch_prime_form(bbp_plan p, uint64_t n, uint32_t W, uint32_t P, uin
   a.cap = kBaseCap;
   a.base = 0;
   a.e = e;
-  chk(launch_prime(a, kPowers1, lmax, p->sm_count, S->sums));
-  if (lim.A >= (1ull << 31)) chk(launch_prime(a, kPowers2, lmax, p->sm_count, S->sums));
-  chk(launch_prime(a, kPrimeWarps, lmax, p->sm_count, S->sums));
+  chk(launch_prime(a, kPowers1, lmax, sm_count, S->sums));
+  if (lim.A >= (1ull << 31)) chk(launch_prime(a, kPowers2, lmax, sm_count, S->sums));
+  chk(launch_prime(a, kPrimeWarps, lmax, sm_count, S->sums));
   chk(cudaEventRecord(S->done, S->sums));
   *launches += lim.A >= (1ull << 31) ? 4 : 3;
   SieveArgs v{};
@@ -242,7 +230,7 @@ bbp_status launch_prime_form(bbp_plan p, uint64_t n, uint32_t W, uint32_t P, uin
     v.upto = l.hi;
     v.segments = l.segments;
     v.count = lengths + i;
-    chk(launch_sieve(v, p->sm_count, S->sieve));
+    chk(launch_sieve(v, sm_count, S->sieve));
     chk(cudaEventRecord(S->ready[slot], S->sieve));
     chk(cudaStreamWaitEvent(st, S->ready[slot], 0));
     a.list = S->list[slot];
@@ -250,13 +238,13 @@ bbp_status launch_prime_form(bbp_plan p, uint64_t n, uint32_t W, uint32_t P, uin
     a.count = lengths + i;
     a.taken = lengths + nl + i;
     a.e = l.k == kSums1 || l.k == kSums2 || l.k == kSums8 ? e : e - kPrimeShift + 64;  // the product with H leaves a factor 2^-64
-    chk(launch_prime(a, l.k, lmax, p->sm_count, st));
+    chk(launch_prime(a, l.k, lmax, sm_count, st));
     chk(cudaEventRecord(S->used[slot], st));
     *launches += 3;
   }
   chk(cudaStreamWaitEvent(st, S->done, 0));
   chk(launch_prime_check(slots, static_cast<int>(W / 32), P, bound, lengths, static_cast<uint32_t>(nl), S->list_cap,
-                         d_out, d_valid, S->counts + 2, st));
+                         d_out, d_valid, d_redo, st));
   *launches += 1;
   return err == cudaSuccess ? BBP_OK : BBP_ECUDA;
 }

@@ -115,6 +115,7 @@ bbp_status bbp_plan_create(bbp_plan* out, const bbp_plan_opts* opts) {
             cudaMalloc(&p->d_limbs, sizeof(uint32_t) * kMaxLimbs) == cudaSuccess &&
             cudaMalloc(&p->d_bytes, kMaxWorkingBits / 8) == cudaSuccess &&
             cudaMalloc(&p->d_valid, sizeof(uint32_t)) == cudaSuccess &&
+            cudaMalloc(&p->d_redo, sizeof(uint32_t)) == cudaSuccess &&
             cudaMallocHost(&p->h_stage, 4096) == cudaSuccess &&
             cudaEventCreate(&p->ev0) == cudaSuccess && cudaEventCreate(&p->ev1) == cudaSuccess &&
             cudaEventCreate(&p->ev2) == cudaSuccess;
@@ -133,11 +134,12 @@ bbp_status bbp_plan_destroy(bbp_plan p) {
   release_serve_state(p);
   if (p->stream) cudaStreamSynchronize(p->stream);
   release_batch_state(p);
-  release_prime_state(p);
+  release_prime_state(&p->primes);
   cudaFree(p->d_slots);
   cudaFree(p->d_limbs);
   cudaFree(p->d_bytes);
   cudaFree(p->d_valid);
+  cudaFree(p->d_redo);
   cudaFreeHost(p->h_stage);
   if (p->ev0) cudaEventDestroy(p->ev0);
   if (p->ev1) cudaEventDestroy(p->ev1);
@@ -308,7 +310,7 @@ bbp_status enqueue_bits(bbp_plan p, int f, uint64_t n, uint32_t P, uint32_t W, u
   uint64_t prime_launches = 0;
   float prime_ms = 0;
   p->stats = bbp_stats{};
-  if (form != kTerms && !d_limbs && prime_form_serves(f, n, P, W, bound) && prime_workspace(p, n, s)) {
+  if (form != kTerms && !d_limbs && prime_form_serves(f, n, P, W, bound) && prime_workspace(&p->primes, n, kPrimeListMax, s)) {
     const PrimeLimits lim = prime_limits(n - 1);
     std::vector<TermRange> rest;  // tails, and a head term past the limits
     for (uint32_t j = 0; j < F.count; ++j) {
@@ -319,7 +321,8 @@ bbp_status enqueue_bits(bbp_plan p, int f, uint64_t n, uint32_t P, uint32_t W, u
     BBP_CUDA(launch_zero_slots(p->d_slots, L, s));
     const bbp_status ls = launch_ranges(p, f, n, W, rest, p->d_slots, s);
     if (ls != BBP_OK) return ls;
-    const bbp_status ps = launch_prime_form(p, n, W, P, bound, p->d_slots, d_out, d_valid, s, &prime_launches);
+    const bbp_status ps = launch_prime_form(p->primes, p->sm_count, n, W, P, bound, p->d_slots, d_out, d_valid, p->d_redo,
+                                           s, &prime_launches);
     if (ps != BBP_OK) return ps;
     if (p->profile) {
       BBP_CUDA(cudaEventRecord(p->ev1, s));
@@ -327,7 +330,7 @@ bbp_status enqueue_bits(bbp_plan p, int f, uint64_t n, uint32_t P, uint32_t W, u
       BBP_CUDA(cudaEventElapsedTime(&prime_ms, p->ev2, p->ev1));
     }
     prime_launches += p->stats.kernel_launches + 1;
-    gate = prime_redo_flag(p);
+    gate = p->d_redo;
     if (by_primes) *by_primes = true;
   }
   if (gate && form == kPrimeOnly) {
@@ -498,7 +501,7 @@ bbp_status bbp_bits_formula(bbp_plan p, bbp_formula f, uint64_t n, uint32_t P, u
     BBP_CUDA(cudaMemcpyAsync(h, p->d_bytes, nbytes, cudaMemcpyDeviceToHost, p->stream));
     BBP_CUDA(cudaMemcpyAsync(h + 2048, p->d_valid, sizeof(uint32_t), cudaMemcpyDeviceToHost, p->stream));
     if (by_primes)
-      BBP_CUDA(cudaMemcpyAsync(h + 2052, prime_redo_flag(p), sizeof(uint32_t), cudaMemcpyDeviceToHost, p->stream));
+      BBP_CUDA(cudaMemcpyAsync(h + 2052, p->d_redo, sizeof(uint32_t), cudaMemcpyDeviceToHost, p->stream));
     BBP_CUDA(cudaStreamSynchronize(p->stream));
     uint32_t redo = 0;
     if (by_primes) std::memcpy(&redo, h + 2052, sizeof(redo));

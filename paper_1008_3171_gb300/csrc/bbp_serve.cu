@@ -113,7 +113,7 @@ struct Query {
 struct HostStage {
   HeadArgs* jobs = nullptr;          size_t c_jobs = 0;
   uint32_t* job_query = nullptr;     size_t c_job_query = 0;
-  uint64_t* job_tiles = nullptr;     size_t c_job_tiles = 0;
+  uint64_t* job_start = nullptr;     size_t c_job_start = 0;
   TailArgs* tails = nullptr;         size_t c_tails = 0;
   uint32_t* tail_query = nullptr;    size_t c_tail_query = 0;
   QueryDesc* queries = nullptr;      // one per slot
@@ -148,11 +148,11 @@ struct ServeEngine {
   uint8_t* d_out = nullptr;
   uint32_t* d_valid = nullptr;
   unsigned long long* d_done = nullptr;
-  unsigned int* d_cursors = nullptr;
+  unsigned long long* d_cursors = nullptr;
   HeadArgs* d_jobs = nullptr;            size_t c_jobs = 0;
   uint32_t* d_job_query = nullptr;       size_t c_job_query = 0;
-  uint64_t* d_job_tiles = nullptr;       size_t c_job_tiles = 0;
-  unsigned long long* d_job_ctr = nullptr; size_t c_job_ctr = 0;
+  uint64_t* d_job_start = nullptr;       size_t c_job_start = 0;
+  unsigned long long* d_job_done = nullptr; size_t c_job_done = 0;
   TailArgs* d_tails = nullptr;           size_t c_tails = 0;
   uint32_t* d_tail_query = nullptr;      size_t c_tail_query = 0;
   HostStage stage;
@@ -302,7 +302,7 @@ bool alloc_engine(ServeEngine* E) {
             cudaMalloc(&E->d_out, static_cast<size_t>(kOutStride) * S) == cudaSuccess &&
             cudaMalloc(&E->d_valid, sizeof(uint32_t) * S) == cudaSuccess &&
             cudaMalloc(&E->d_done, sizeof(unsigned long long) * S) == cudaSuccess &&
-            cudaMalloc(&E->d_cursors, sizeof(unsigned int) * (kVariants + 1)) == cudaSuccess;
+            cudaMalloc(&E->d_cursors, sizeof(unsigned long long) * (kVariants + 1)) == cudaSuccess;
   {
     HostStage& h = E->stage;
     ok = ok && cudaMallocHost(&h.queries, sizeof(QueryDesc) * S) == cudaSuccess &&
@@ -329,15 +329,15 @@ void free_engine(ServeEngine* E) {
   cudaFree(E->d_cursors);
   cudaFree(E->d_jobs);
   cudaFree(E->d_job_query);
-  cudaFree(E->d_job_tiles);
-  cudaFree(E->d_job_ctr);
+  cudaFree(E->d_job_start);
+  cudaFree(E->d_job_done);
   cudaFree(E->d_tails);
   cudaFree(E->d_tail_query);
   {
     HostStage& h = E->stage;
     cudaFreeHost(h.jobs);
     cudaFreeHost(h.job_query);
-    cudaFreeHost(h.job_tiles);
+    cudaFreeHost(h.job_start);
     cudaFreeHost(h.tails);
     cudaFreeHost(h.tail_query);
     cudaFreeHost(h.queries);
@@ -383,16 +383,17 @@ bool enqueue_iteration(ServeEngine* E, HostStage& H, std::vector<Query*>& batch,
     if (pc.tail) tails.push_back(&pc);
   const size_t nh = heads.size(), nt = tails.size();
   if (!grow_pinned(&H.jobs, &H.c_jobs, nh) || !grow_pinned(&H.job_query, &H.c_job_query, nh) ||
-      !grow_pinned(&H.job_tiles, &H.c_job_tiles, nh) || !grow_pinned(&H.tails, &H.c_tails, nt) ||
+      !grow_pinned(&H.job_start, &H.c_job_start, nh + 1) || !grow_pinned(&H.tails, &H.c_tails, nt) ||
       !grow_pinned(&H.tail_query, &H.c_tail_query, nt) || !grow_dev(&E->d_jobs, &E->c_jobs, nh) ||
-      !grow_dev(&E->d_job_query, &E->c_job_query, nh) || !grow_dev(&E->d_job_tiles, &E->c_job_tiles, nh) ||
-      !grow_dev(&E->d_job_ctr, &E->c_job_ctr, 2 * nh) || !grow_dev(&E->d_tails, &E->c_tails, nt) ||
+      !grow_dev(&E->d_job_query, &E->c_job_query, nh) || !grow_dev(&E->d_job_start, &E->c_job_start, nh + 1) ||
+      !grow_dev(&E->d_job_done, &E->c_job_done, nh) || !grow_dev(&E->d_tails, &E->c_tails, nt) ||
       !grow_dev(&E->d_tail_query, &E->c_tail_query, nt))
     return false;
+  H.job_start[0] = 0;
   for (size_t i = 0; i < nh; ++i) {
     H.jobs[i] = heads[i]->head;
     H.job_query[i] = heads[i]->slot;
-    H.job_tiles[i] = heads[i]->tiles;
+    H.job_start[i + 1] = H.job_start[i] + heads[i]->tiles;
   }
   for (size_t i = 0; i < nt; ++i) {
     H.tails[i] = tails[i]->tailargs;
@@ -419,17 +420,16 @@ bool enqueue_iteration(ServeEngine* E, HostStage& H, std::vector<Query*>& batch,
   chk(cudaMemcpyAsync(E->d_jobs_left, H.jobs_left, sizeof(unsigned int) * E->max_slots, cudaMemcpyHostToDevice, s));
   chk(cudaMemcpyAsync(E->d_jobs, H.jobs, sizeof(HeadArgs) * nh, cudaMemcpyHostToDevice, s));
   chk(cudaMemcpyAsync(E->d_job_query, H.job_query, sizeof(uint32_t) * nh, cudaMemcpyHostToDevice, s));
-  chk(cudaMemcpyAsync(E->d_job_tiles, H.job_tiles, sizeof(uint64_t) * nh, cudaMemcpyHostToDevice, s));
+  chk(cudaMemcpyAsync(E->d_job_start, H.job_start, sizeof(uint64_t) * (nh + 1), cudaMemcpyHostToDevice, s));
   chk(cudaMemcpyAsync(E->d_tails, H.tails, sizeof(TailArgs) * nt, cudaMemcpyHostToDevice, s));
   chk(cudaMemcpyAsync(E->d_tail_query, H.tail_query, sizeof(uint32_t) * nt, cudaMemcpyHostToDevice, s));
-  chk(cudaMemsetAsync(E->d_job_ctr, 0, sizeof(unsigned long long) * 2 * std::max<size_t>(nh, 1), s));
-  chk(cudaMemsetAsync(E->d_cursors, 0, sizeof(unsigned int) * (kVariants + 1), s));
+  chk(cudaMemsetAsync(E->d_job_done, 0, sizeof(unsigned long long) * std::max<size_t>(nh, 1), s));
+  chk(cudaMemsetAsync(E->d_cursors, 0, sizeof(unsigned long long) * (kVariants + 1), s));
   BatchDev dev{};
   dev.jobs = E->d_jobs;
   dev.job_query = E->d_job_query;
-  dev.job_tiles = E->d_job_tiles;
-  dev.job_taken = E->d_job_ctr;
-  dev.job_done = E->d_job_ctr + nh;
+  dev.job_start = E->d_job_start;
+  dev.job_done = E->d_job_done;
   dev.tails = E->d_tails;
   dev.tail_query = E->d_tail_query;
   dev.grab = 1;  // short iterations: hand out single tiles so every launch ends evenly

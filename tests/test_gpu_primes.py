@@ -60,16 +60,33 @@ def test_check_sends_uncertain_positions_to_the_terms(bbp, plans):
     """G = 32 and P = 60: 36 bits below the output for a bound of 2^26.1 units, so about one
     position in 160 lies within three bounds of a carry.  Those and the others agree."""
     plan, P = plans[32], 60
-    redone = 0
+    redone, checked = 0, {}
     for n in range(10**8 + 1, 10**8 + 801):
         got = plan.bits(n, P)
         terms_run = plan.stats()["imad_model"] > 4e9   # 7.5e9 for the terms, about 1e9 for the primes
         redone += terms_run
         if terms_run or n % 64 == 0:
-            want = by_terms(bbp, plan, n, P)
-            assert got == want, n
-            assert by_async(bbp, plan, n, P) == want, n
+            checked[n] = by_terms(bbp, plan, n, P)
+            assert got == checked[n], n
+            assert by_async(bbp, plan, n, P) == checked[n], n
     assert 0 < redone < 40   # 5 expected
+    # in one batch, some of them through its second pass
+    ns = list(checked)
+    vals, valid, lat = bbp.bbp_bits_batch(plan.handle, 0, ns, [P] * len(ns))
+    assert dict(zip(ns, zip(vals, valid))) == checked
+    assert all(v > 0 for v in lat)
+
+
+def test_batch_of_both_kinds(bbp, plans):
+    """Queries of both kinds around the smallest position that takes primes, and the same batch
+    again: each as alone, term by term."""
+    plan = plans[64]
+    ns = [10**4, 16 * 10**6 + 9, 12_345, 16 * 10**6 - 1, 10**8 + 21, 1, 3 * 10**7 + 2, 16 * 10**6, 10**6 + 1]
+    Ps = [64, 128, 256, 64, 448, 8, 100, 256, 1000]
+    want = [by_terms(bbp, plan, n, P) for n, P in zip(ns, Ps)]
+    for _ in range(2):
+        vals, valid, _ = bbp.bbp_bits_batch(plan.handle, 0, ns, Ps)
+        assert list(zip(vals, valid)) == want
 
 
 def test_async_on_a_stream_and_under_capture(bbp, plans):
