@@ -26,6 +26,7 @@
 #include "bbp.h"
 #include "bbp_kernels.cuh"
 #include "bbp_planner.h"
+#include "bbp_prime_run.h"
 #include "bbp_primes.h"
 #include "bbp_runtime.h"
 
@@ -365,7 +366,7 @@ static bool prime_lanes(BatchState* b, uint64_t n, int lanes) {
   for (int i = 0; i < lanes; ++i) {
     if (!b->lane_stream[i] && cudaStreamCreateWithFlags(&b->lane_stream[i], cudaStreamNonBlocking) != cudaSuccess) return false;
     if (!b->lane_done[i] && cudaEventCreateWithFlags(&b->lane_done[i], cudaEventDisableTiming) != cudaSuccess) return false;
-    if (!prime_workspace(&b->lane[i], n, kPrimeBatchListMax, b->lane_stream[i])) return false;
+    if (!prime_workspace(&b->lane[i], n, kPrimeLaneListMax, b->lane_stream[i])) return false;
   }
   return true;
 }
@@ -486,10 +487,15 @@ static bbp_status run_batch(bbp_plan p, bbp_formula f, uint32_t count, const uin
     for (size_t i = 0; i < bp.primes.size(); ++i) {
       const BatchPlan::Prime& r = bp.primes[i];
       const int k = static_cast<int>(i % kPrimeLanes);
-      const bbp_status ls = launch_prime_form(
-          b->lane[k], p->sm_count, r.n, r.W, P[r.q], r.bound, b->d_accum + static_cast<uint64_t>(r.q) * kMaxLimbs,
-          b->d_out + static_cast<size_t>(r.q) * kOutStride, b->d_valid + r.q, b->d_redo + r.q, b->lane_stream[k],
-          &launches);
+      const cudaStream_t to = b->lane_stream[k];
+      PrimeRun run;
+      bbp_status ls = run.plan(b->lane[k], p->sm_count, r.n, r.W, b->d_accum + static_cast<uint64_t>(r.q) * kMaxLimbs);
+      if (ls == BBP_OK) ls = run.begin(to);
+      if (ls == BBP_OK) ls = run.run(0, run.lists(), to);
+      if (ls == BBP_OK)
+        ls = run.finish(P[r.q], r.bound, b->d_out + static_cast<size_t>(r.q) * kOutStride, b->d_valid + r.q,
+                        b->d_redo + r.q, to);
+      launches += run.launches();
       if (ls != BBP_OK) return ls;
       BBP_TRY(launch_timestamp(b->d_done + 1 + r.q, b->lane_stream[k]));
       ++launches;

@@ -14,9 +14,8 @@
 #include <new>
 #include <vector>
 
-#include "bbp_kernels.cuh"
 #include "bbp_planner.h"
-#include "bbp_runtime.h"
+#include "bbp_prime_run.h"
 #include "bbp_sieve.cuh"
 
 namespace bbp {
@@ -25,7 +24,8 @@ namespace {
 
 constexpr uint32_t kMaxBase = (1u << 23) - 1;       // base primes up to here: 564,162 odd ones
 constexpr uint32_t kBaseCap = 565000;
-constexpr uint32_t kMaxLists = 1u << 16;
+constexpr uint32_t kMaxLists = 1u << 17;            // 7.6e4 lists of 6 M primes at the largest position
+constexpr uint32_t kSieveEntries = 64u << 10;       // of a sieve segment: three CTAs an SM
 constexpr uint64_t kLongSum = 32000;                // primes below A / this take a warp each,
 constexpr uint64_t kGroupSum = 1000;                // those below A / this eight lanes
 
@@ -131,15 +131,18 @@ bool prime_workspace(PrimeState** state, uint64_t n, uint32_t max_list, cudaStre
   return true;
 }
 
-bbp_status launch_prime_form(PrimeState* S, int sm_count, uint64_t n, uint32_t W, uint32_t P, uint64_t bound,
-                             unsigned long long* slots, uint8_t* d_out, uint32_t* d_valid, uint32_t* d_redo,
-                             cudaStream_t st, uint64_t* launches) {
-  const int lmax = head_lmax_for(static_cast<int>(W / 32));
-  if (lmax == 0) return BBP_EINVAL;
+bbp_status PrimeRun::plan(PrimeState* state, int sm_count, uint64_t n, uint32_t W, unsigned long long* slots) {
+  state_ = state;
+  sms_ = sm_count;
+  launches_ = 0;
+  lists_.clear();
+  lmax_ = head_lmax_for(static_cast<int>(W / 32));
+  if (lmax_ == 0) return BBP_EINVAL;
   const PrimeLimits lim = prime_limits(n - 1);
   const std::vector<PrimeClass> classes = prime_classes(lim);
   if (classes.empty() || classes.size() > static_cast<size_t>(kMaxPrimeClasses)) return BBP_EINVAL;
-  PrimeArgs a{};
+  PrimeArgs& a = args_;
+  a = PrimeArgs{};
   a.L = W / 32;
   a.A = lim.A;
   a.B = lim.B;
@@ -147,12 +150,9 @@ bbp_status launch_prime_form(PrimeState* S, int sm_count, uint64_t n, uint32_t W
   a.slots = slots;
   a.nclasses = static_cast<uint32_t>(classes.size());
   std::copy(classes.begin(), classes.end(), a.classes);
-  const uint64_t e = n - 1 + W;
-  cudaError_t err = cudaSuccess;
-  auto chk = [&](cudaError_t r) { if (err == cudaSuccess) err = r; };
-
+  e_ = n - 1 + W;
   const uint64_t root = isqrt(lim.A);
-  const uint32_t base_to = static_cast<uint32_t>(std::min<uint64_t>(kMaxBase, std::max(root, lim.A / kLongSum)));
+  base_to_ = static_cast<uint32_t>(std::min<uint64_t>(kMaxBase, std::max(root, lim.A / kLongSum)));
   const uint64_t bottom = classes.back().above;
   // lists: primes in (base_to, A], cut where their kernel changes
   struct Span { uint64_t lo, hi; PrimeKernel k; };
@@ -162,7 +162,7 @@ bbp_status launch_prime_form(PrimeState* S, int sm_count, uint64_t n, uint32_t W
     const uint64_t cuts[] = {grouped, bottom, (1ull << 29) - 1, (1ull << 31) - 1, kPrimeHalfMax, lim.A};
     std::vector<uint64_t> c(std::begin(cuts), std::end(cuts));
     std::sort(c.begin(), c.end());
-    uint64_t lo = base_to;
+    uint64_t lo = base_to_;
     for (uint64_t hi : c) {
       hi = std::min(hi, lim.A);
       if (hi <= lo) continue;
@@ -173,55 +173,69 @@ bbp_status launch_prime_form(PrimeState* S, int sm_count, uint64_t n, uint32_t W
       lo = hi;
     }
   }
-  constexpr uint32_t entries = 64u << 10;
-  const uint64_t seg = 30ull * entries;
-  struct List { uint64_t base, lo, hi; uint32_t segments; PrimeKernel k; };
-  std::vector<List> lists;
+  constexpr uint64_t seg = 30ull * kSieveEntries;
   for (const Span& s : spans) {
     uint64_t lo = s.lo;
     while (lo < s.hi) {
       const uint64_t base = (lo + 1) / seg * seg;
       // about 1 / ln x of the numbers are primes; a list that came out longer than the buffer
       // would be seen by the check
-      const double room = 0.85 * S->list_cap * (std::log(static_cast<double>(std::max<uint64_t>(lo, 1000))) - 1.1);
+      const double room = 0.85 * state_->list_cap * (std::log(static_cast<double>(std::max<uint64_t>(lo, 1000))) - 1.1);
       uint64_t nseg = std::max<uint64_t>(1, static_cast<uint64_t>(room) / seg);
       // whole waves of the sieve's CTAs, eight a segment, one an SM beside the primes' kernels
-      const uint64_t wave = std::max<uint64_t>(1, static_cast<uint64_t>(sm_count) / 8);
+      const uint64_t wave = std::max<uint64_t>(1, static_cast<uint64_t>(sms_) / 8);
       if (nseg > wave) nseg -= nseg % wave;
       const uint64_t hi = std::min(s.hi, base + nseg * seg - 1);
-      lists.push_back(List{base, lo, hi, static_cast<uint32_t>((hi - base) / seg + 1), s.k});
+      lists_.push_back(List{base, lo, hi, static_cast<uint32_t>((hi - base) / seg + 1), s.k});
       lo = hi;
     }
   }
-  if (lists.size() > kMaxLists) return BBP_ERANGE;
+  return lists_.size() > kMaxLists ? BBP_ERANGE : BBP_OK;
+}
 
-  // The caller's stream runs the lists' kernels, the sieve runs one list ahead on its own
-  // stream, the prime powers (few, with long chains) run beside them on a third.
-  const size_t nl = lists.size();
-  uint32_t* const lengths = S->counts + kCountHead;
-  chk(cudaMemsetAsync(S->counts, 0, sizeof(uint32_t) * (kCountHead + 2 * nl), st));
-  chk(launch_base_primes(base_to, S->primes, S->sieve_primes, S->counts, S->counts + 1, st));
+double PrimeRun::share(size_t i) const {
+  return static_cast<double>(lists_[i].hi - lists_[i].lo) / static_cast<double>(args_.A);
+}
+
+// The caller's stream runs the lists' kernels, the sieve runs one list ahead on its own
+// stream, the prime powers (few, with long chains) run beside them on a third.
+bbp_status PrimeRun::begin(cudaStream_t st) {
+  PrimeState* const S = state_;
+  cudaError_t err = cudaSuccess;
+  auto chk = [&](cudaError_t r) { if (err == cudaSuccess) err = r; };
+  chk(cudaMemsetAsync(S->counts, 0, sizeof(uint32_t) * (kCountHead + 2 * lists_.size()), st));
+  chk(launch_base_primes(base_to_, S->primes, S->sieve_primes, S->counts, S->counts + 1, st));
   chk(cudaEventRecord(S->base, st));
   chk(cudaStreamWaitEvent(S->sieve, S->base, 0));
   chk(cudaStreamWaitEvent(S->sums, S->base, 0));
+  PrimeArgs a = args_;
   a.list = S->primes;
   a.count = S->counts;
   a.cap = kBaseCap;
-  a.base = 0;
-  a.e = e;
-  chk(launch_prime(a, kPowers1, lmax, sm_count, S->sums));
-  if (lim.A >= (1ull << 31)) chk(launch_prime(a, kPowers2, lmax, sm_count, S->sums));
-  chk(launch_prime(a, kPrimeWarps, lmax, sm_count, S->sums));
+  a.e = e_;
+  const bool above_word = a.A >= (1ull << 31);
+  chk(launch_prime(a, kPowers1, lmax_, sms_, S->sums));
+  if (above_word) chk(launch_prime(a, kPowers2, lmax_, sms_, S->sums));
+  chk(launch_prime(a, kPrimeWarps, lmax_, sms_, S->sums));
   chk(cudaEventRecord(S->done, S->sums));
-  *launches += lim.A >= (1ull << 31) ? 4 : 3;
+  launches_ += above_word ? 4 : 3;
+  return err == cudaSuccess ? BBP_OK : BBP_ECUDA;
+}
+
+bbp_status PrimeRun::run(size_t first, size_t last, cudaStream_t st) {
+  PrimeState* const S = state_;
+  cudaError_t err = cudaSuccess;
+  auto chk = [&](cudaError_t r) { if (err == cudaSuccess) err = r; };
+  uint32_t* const lengths = S->counts + kCountHead;
   SieveArgs v{};
-  v.entries = entries;
+  v.entries = kSieveEntries;
   v.primes = S->sieve_primes + kSieveTinyPrimes;
   v.nprimes = S->counts + 1;
   v.cap = S->list_cap;
+  PrimeArgs a = args_;
   a.cap = S->list_cap;
-  for (size_t i = 0; i < nl; ++i) {
-    const List& l = lists[i];
+  for (size_t i = first; i < last; ++i) {
+    const List& l = lists_[i];
     const size_t slot = i & 1;
     if (i >= 2) chk(cudaStreamWaitEvent(S->sieve, S->used[slot], 0));  // the buffer's last list is done
     v.list = S->list[slot];
@@ -230,22 +244,29 @@ bbp_status launch_prime_form(PrimeState* S, int sm_count, uint64_t n, uint32_t W
     v.upto = l.hi;
     v.segments = l.segments;
     v.count = lengths + i;
-    chk(launch_sieve(v, sm_count, S->sieve));
+    chk(launch_sieve(v, sms_, S->sieve));
     chk(cudaEventRecord(S->ready[slot], S->sieve));
     chk(cudaStreamWaitEvent(st, S->ready[slot], 0));
     a.list = S->list[slot];
     a.base = l.base;
     a.count = lengths + i;
-    a.taken = lengths + nl + i;
-    a.e = l.k == kSums1 || l.k == kSums2 || l.k == kSums8 ? e : e - kPrimeShift + 64;  // the product with H leaves a factor 2^-64
-    chk(launch_prime(a, l.k, lmax, sm_count, st));
+    a.taken = lengths + lists_.size() + i;
+    const bool sums = l.kernel == kSums1 || l.kernel == kSums2 || l.kernel == kSums8;
+    a.e = sums ? e_ : e_ - kPrimeShift + 64;  // the product with H leaves a factor 2^-64
+    chk(launch_prime(a, l.kernel, lmax_, sms_, st));
     chk(cudaEventRecord(S->used[slot], st));
-    *launches += 3;
+    launches_ += 3;
   }
-  chk(cudaStreamWaitEvent(st, S->done, 0));
-  chk(launch_prime_check(slots, static_cast<int>(W / 32), P, bound, lengths, static_cast<uint32_t>(nl), S->list_cap,
-                         d_out, d_valid, d_redo, st));
-  *launches += 1;
+  return err == cudaSuccess ? BBP_OK : BBP_ECUDA;
+}
+
+bbp_status PrimeRun::finish(uint32_t P, uint64_t bound, uint8_t* d_out, uint32_t* d_valid, uint32_t* d_redo,
+                            cudaStream_t st) {
+  cudaError_t err = cudaStreamWaitEvent(st, state_->done, 0);
+  if (err == cudaSuccess)
+    err = launch_prime_check(args_.slots, static_cast<int>(args_.L), P, bound, state_->counts + kCountHead,
+                             static_cast<uint32_t>(lists_.size()), state_->list_cap, d_out, d_valid, d_redo, st);
+  ++launches_;
   return err == cudaSuccess ? BBP_OK : BBP_ECUDA;
 }
 

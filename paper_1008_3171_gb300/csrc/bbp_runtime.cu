@@ -18,6 +18,7 @@
 #include "bbp.h"
 #include "bbp_kernels.cuh"
 #include "bbp_planner.h"
+#include "bbp_prime_run.h"
 #include "bbp_primes.h"
 #include "bbp_runtime.h"
 
@@ -321,8 +322,12 @@ bbp_status enqueue_bits(bbp_plan p, int f, uint64_t n, uint32_t P, uint32_t W, u
     BBP_CUDA(launch_zero_slots(p->d_slots, L, s));
     const bbp_status ls = launch_ranges(p, f, n, W, rest, p->d_slots, s);
     if (ls != BBP_OK) return ls;
-    const bbp_status ps = launch_prime_form(p->primes, p->sm_count, n, W, P, bound, p->d_slots, d_out, d_valid, p->d_redo,
-                                           s, &prime_launches);
+    PrimeRun run;
+    bbp_status ps = run.plan(p->primes, p->sm_count, n, W, p->d_slots);
+    if (ps == BBP_OK) ps = run.begin(s);
+    if (ps == BBP_OK) ps = run.run(0, run.lists(), s);
+    if (ps == BBP_OK) ps = run.finish(P, bound, d_out, d_valid, p->d_redo, s);
+    prime_launches = run.launches();
     if (ps != BBP_OK) return ps;
     if (p->profile) {
       BBP_CUDA(cudaEventRecord(p->ev1, s));

@@ -57,22 +57,6 @@ bbp_status plan_query(bbp_plan p, int f, uint64_t n, uint32_t W, int j_only, uin
                       std::vector<TermRange>& ranges, uint64_t* n_terms);
 bbp_status launch_ranges(bbp_plan p, int f, uint64_t n, uint32_t W, const std::vector<TermRange>& ranges,
                          unsigned long long* slots, cudaStream_t st, const uint32_t* gate = nullptr);
-// Prime form of a query's head sum (bbp_prime_run.cu).
-//
-// The workspace for position n, made or enlarged to lists of up to `max_list` primes;
-// false if it is not there and cannot be made now (a stream capture is going on on `st`,
-// or memory is short): the caller then sums the terms.
-constexpr uint32_t kPrimeListMax = 24u << 20;       // single queries: two lists of 96 MB
-constexpr uint32_t kPrimeBatchListMax = 6u << 20;   // each of a batch's workspaces: two of 24 MB
-bool prime_workspace(PrimeState** state, uint64_t n, uint32_t max_list, cudaStream_t st);
-void release_prime_state(PrimeState** state);
-// Adds the prime form of the head terms covered by prime_limits(n - 1) to `slots` and
-// enqueues the check of the finished sum (the terms it does not cover must be in `slots`
-// already): d_out and d_valid (may be NULL) are written and *d_redo = 0, or *d_redo = 1.
-// *launches counts the kernels.
-bbp_status launch_prime_form(PrimeState* state, int sm_count, uint64_t n, uint32_t W, uint32_t P, uint64_t bound,
-                             unsigned long long* slots, uint8_t* d_out, uint32_t* d_valid, uint32_t* d_redo,
-                             cudaStream_t st, uint64_t* launches);
 void load_tune_table(bbp_plan p, const char* path);
 void release_batch_state(bbp_plan p);
 void release_serve_state(bbp_plan p);

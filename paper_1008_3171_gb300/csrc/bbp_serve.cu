@@ -11,7 +11,16 @@
 // slot between iterations.  A query's job counter carries one extra hold while it
 // has work left, so the device finalizes it (bits, certified count) exactly in the
 // iteration that runs its last piece; the host then publishes the result to
-// bbp_poll and frees the slot.  Iterations run one at a time: a query that
+// bbp_poll and frees the slot.
+//
+// Queries that the prime form serves (bbp_primes.h) run it instead: their tails go through
+// the queue in their first iteration, their lists of primes through kServeLanes
+// workspaces.  One that fits an iteration runs as a whole on the next free workspace; a
+// longer one keeps a workspace, up to all but one of them, and runs some lists in each
+// iteration.  A query whose check asks for the terms goes back to them.  48 queries of
+// n = 10^6 ... 10^9 submitted together: 96 -> 14.4 ms.
+//
+// Iterations run one at a time: a query that
 // arrives while one runs joins the next.  (Planning iteration i+1 while i runs was
 // measured on the serving workload: the same terms/s, and every arrival waits one
 // iteration longer, so the median latency rose from 46 to 72 ms.)
@@ -22,6 +31,7 @@
 #include <cstdint>
 #include <cstring>
 #include <deque>
+#include <memory>
 #include <mutex>
 #include <new>
 #include <thread>
@@ -31,6 +41,8 @@
 #include "bbp.h"
 #include "bbp_kernels.cuh"
 #include "bbp_planner.h"
+#include "bbp_prime_run.h"
+#include "bbp_primes.h"
 #include "bbp_runtime.h"
 
 using namespace bbp;
@@ -41,6 +53,10 @@ constexpr int kVariants = kQueueVariants;
 constexpr uint32_t kOutStride = kMaxWorkingBits / 8;
 constexpr double kIterTargetSeconds = 0.025;  // target duration of one iteration
 constexpr double kInitialRate = 2.0e10;       // terms/s before the first measurement
+constexpr int kServeLanes = 4;
+// The work of a prime form in terms of the queue kernels: an eighth of its terms, and some
+// 0.15 ms of launches and chains.
+constexpr uint64_t kPrimeTermsPerTerm = 8, kPrimeFixedTerms = 6'000'000;
 
 int lmax_index(int lmax) {
   for (int i = 0; i < kNumLmaxClasses; ++i)
@@ -101,6 +117,12 @@ struct Query {
   uint64_t tile_off = 0;   // tiles of work[next] already handed out
   uint64_t bound = 0;      // N + J + 1
   uint64_t total_terms = 0;
+  // prime form: `work` holds what it does not cover
+  bool prime = false;
+  std::unique_ptr<PrimeRun> run;  // once begun
+  int lane = -1;                  // workspace kept between iterations
+  size_t next_list = 0;
+  uint64_t terms_done = 0;
   bool final_in_flight = false;
   std::vector<uint8_t> out;
   uint32_t valid = 0;
@@ -120,9 +142,11 @@ struct HostStage {
   unsigned int* jobs_left = nullptr; // one per slot
   uint8_t* out = nullptr;            // kOutStride bytes per slot
   uint32_t* valid = nullptr;         // one per slot
+  uint32_t* redo = nullptr;          // one per slot (prime forms)
   cudaEvent_t start = nullptr, done = nullptr;
   std::vector<Query*> finishing;     // queries whose last piece runs in this iteration
-  uint64_t terms = 0;
+  uint64_t terms = 0;                // terms of the iteration,
+  uint64_t cost = 0;                 // and their work as queue terms
   bool in_flight = false;
 };
 
@@ -139,9 +163,19 @@ struct ServeEngine {
   std::unordered_map<uint64_t, Query*> tickets;
   std::vector<int> free_slots;
   uint32_t max_slots = 0;
-  double rate = kInitialRate;  // measured terms/s
+  double rate = kInitialRate;  // measured work, queue terms/s
+  double terms_rate = kInitialRate;  // measured terms/s
+  // prime forms
+  PrimeState* lane[kServeLanes] = {};
+  cudaStream_t lane_stream[kServeLanes] = {};
+  cudaEvent_t lane_done[kServeLanes] = {};
+  Query* lane_owner[kServeLanes] = {};
+  bool no_lanes = false;             // workspaces could not be had: everything term by term
+  uint32_t* d_redo = nullptr;
+  std::vector<int> rezero;           // slots of queries that start again with their terms
   // device state (shared by consecutive iterations: stream order separates them)
   cudaStream_t stream = nullptr;
+  cudaEvent_t queued = nullptr;      // the iteration's queue part, before its prime forms
   unsigned long long* d_accum = nullptr;
   QueryDesc* d_queries = nullptr;
   unsigned int* d_jobs_left = nullptr;
@@ -163,8 +197,9 @@ struct ServeEngine {
 
 namespace {
 
-// Host planning of one query into work items (the same ranges as bbp_bits).
-bbp_status plan_query_work(bbp_plan p, uint64_t n, uint32_t P, Query* q) {
+// Host planning of one query into work items (the same ranges as bbp_bits); by_primes: only
+// what the prime form leaves, where that serves.
+bbp_status plan_query_work(bbp_plan p, uint64_t n, uint32_t P, Query* q, bool by_primes) {
   uint32_t W;
   if (n == 0 || !working_bits(P, p->guard, &W)) return BBP_EINVAL;
   const uint32_t L = W / 32;
@@ -184,11 +219,27 @@ bbp_status plan_query_work(bbp_plan p, uint64_t n, uint32_t P, Query* q) {
   q->W = W;
   q->L = L;
   q->bound = N + F.count + 1;
+  q->total_terms = 0;
+  q->work.clear();
+  uint64_t tiles = 0;
+  for (const TermRange& r : ranges) {
+    q->total_terms += r.count;
+    if (!r.tail) tiles += (r.count + tile_terms(p, r.path) - 1) / tile_terms(p, r.path);
+  }
+  if (tiles > kMaxQueueTiles) return BBP_ERANGE;  // carry-save limbs could pass 2^64
+  q->prime = by_primes && prime_form_serves(BBP_BELLARD, n, P, W, q->bound);
+  if (q->prime) {
+    const PrimeLimits lim = prime_limits(n - 1);
+    ranges.clear();
+    for (uint32_t j = 0; j < F.count; ++j)
+      if (plan_series(F, j, n, W, static_cast<uint32_t>(lmax), prime_first_k(lim, j), UINT64_MAX, ranges,
+                      p->wide_min_bits) != 0)
+        return BBP_EINVAL;
+  }
   for (const TermRange& r : ranges) {
     const SeriesDef& s = F.s[r.j];
     Work w{};
     w.tail = r.tail != 0;
-    q->total_terms += r.count;
     if (w.tail) {
       TailArgs& a = w.tailargs;
       a.d = n - 1;
@@ -225,10 +276,6 @@ bbp_status plan_query_work(bbp_plan p, uint64_t n, uint32_t P, Query* q) {
     }
     q->work.push_back(w);
   }
-  uint64_t tiles = 0;
-  for (const Work& w : q->work)
-    if (!w.tail) tiles += w.tiles;
-  if (tiles > kMaxQueueTiles) return BBP_ERANGE;  // carry-save limbs could pass 2^64
   if (q->work.empty()) {  // nothing to sum: a zero-length tail still retires the query
     Work w{};
     w.tail = true;
@@ -296,11 +343,13 @@ void take_pieces(ServeEngine* E, Query* q, uint64_t budget_terms, std::vector<Pi
 bool alloc_engine(ServeEngine* E) {
   const size_t S = E->max_slots;
   bool ok = cudaStreamCreateWithFlags(&E->stream, cudaStreamNonBlocking) == cudaSuccess &&
+            cudaEventCreateWithFlags(&E->queued, cudaEventDisableTiming) == cudaSuccess &&
             cudaMalloc(&E->d_accum, sizeof(unsigned long long) * kMaxLimbs * S) == cudaSuccess &&
             cudaMalloc(&E->d_queries, sizeof(QueryDesc) * S) == cudaSuccess &&
             cudaMalloc(&E->d_jobs_left, sizeof(unsigned int) * S) == cudaSuccess &&
             cudaMalloc(&E->d_out, static_cast<size_t>(kOutStride) * S) == cudaSuccess &&
             cudaMalloc(&E->d_valid, sizeof(uint32_t) * S) == cudaSuccess &&
+            cudaMalloc(&E->d_redo, sizeof(uint32_t) * S) == cudaSuccess &&
             cudaMalloc(&E->d_done, sizeof(unsigned long long) * S) == cudaSuccess &&
             cudaMalloc(&E->d_cursors, sizeof(unsigned long long) * (kVariants + 1)) == cudaSuccess;
   {
@@ -309,6 +358,7 @@ bool alloc_engine(ServeEngine* E) {
          cudaMallocHost(&h.jobs_left, sizeof(unsigned int) * S) == cudaSuccess &&
          cudaMallocHost(&h.out, static_cast<size_t>(kOutStride) * S) == cudaSuccess &&
          cudaMallocHost(&h.valid, sizeof(uint32_t) * S) == cudaSuccess &&
+         cudaMallocHost(&h.redo, sizeof(uint32_t) * S) == cudaSuccess &&
          cudaEventCreate(&h.start) == cudaSuccess && cudaEventCreate(&h.done) == cudaSuccess;
     if (ok) {
       std::memset(h.queries, 0, sizeof(QueryDesc) * S);
@@ -320,6 +370,13 @@ bool alloc_engine(ServeEngine* E) {
 
 void free_engine(ServeEngine* E) {
   if (E->stream) cudaStreamSynchronize(E->stream);
+  for (int i = 0; i < kServeLanes; ++i) {
+    if (E->lane_stream[i]) cudaStreamSynchronize(E->lane_stream[i]);
+    release_prime_state(&E->lane[i]);
+    if (E->lane_stream[i]) cudaStreamDestroy(E->lane_stream[i]);
+    if (E->lane_done[i]) cudaEventDestroy(E->lane_done[i]);
+  }
+  cudaFree(E->d_redo);
   cudaFree(E->d_accum);
   cudaFree(E->d_queries);
   cudaFree(E->d_jobs_left);
@@ -344,10 +401,94 @@ void free_engine(ServeEngine* E) {
     cudaFreeHost(h.jobs_left);
     cudaFreeHost(h.out);
     cudaFreeHost(h.valid);
+    cudaFreeHost(h.redo);
     if (h.start) cudaEventDestroy(h.start);
     if (h.done) cudaEventDestroy(h.done);
   }
+  if (E->queued) cudaEventDestroy(E->queued);
   if (E->stream) cudaStreamDestroy(E->stream);
+}
+
+uint64_t prime_cost(const Query* q) { return q->total_terms / kPrimeTermsPerTerm + kPrimeFixedTerms; }
+
+// All workspaces, made when the first query needs one.
+bool make_lanes(ServeEngine* E) {
+  if (E->no_lanes) return false;
+  for (int i = 0; i < kServeLanes; ++i) {
+    if ((!E->lane_stream[i] && cudaStreamCreateWithFlags(&E->lane_stream[i], cudaStreamNonBlocking) != cudaSuccess) ||
+        (!E->lane_done[i] && cudaEventCreateWithFlags(&E->lane_done[i], cudaEventDisableTiming) != cudaSuccess) ||
+        !prime_workspace(&E->lane[i], kPrimeMaxN, kPrimeLaneListMax, E->lane_stream[i])) {
+      cudaGetLastError();
+      E->no_lanes = true;
+      return false;
+    }
+  }
+  return true;
+}
+
+// What an iteration does for one query by primes: its lists [first, last) on a workspace.
+struct PrimePart {
+  Query* q;
+  int lane;
+  size_t first, last;
+};
+
+// Chooses the iteration's parts, in the order of the active queries, for about
+// `budget` queue terms; sets what it takes in each query.
+void take_primes(ServeEngine* E, std::vector<Query*>& batch, uint64_t budget, std::vector<PrimePart>& parts,
+                 std::vector<Query*>& begun, uint64_t* terms, uint64_t* cost) {
+  uint64_t taken = 0;
+  int turn = 0;
+  for (Query* q : batch) {
+    if (!q->prime) continue;
+    const uint64_t whole = prime_cost(q);
+    const bool is_long = whole > budget;
+    if (q->lane < 0) {
+      if (taken >= budget && !parts.empty()) continue;  // waits for the next iteration
+      int free_lane = -1, held = 0;
+      for (int k = 0; k < kServeLanes; ++k) {
+        const int i = (turn + k) % kServeLanes;
+        if (E->lane_owner[i]) ++held;
+        else if (free_lane < 0) free_lane = i;
+      }
+      if (free_lane < 0 || (is_long && held >= kServeLanes - 1)) continue;
+      q->run.reset(new (std::nothrow) PrimeRun());
+      const uint64_t slot = static_cast<uint64_t>(q->slot);
+      if (!q->run || q->run->plan(E->lane[free_lane], E->plan->sm_count, q->n, q->W,
+                                  E->d_accum + slot * kMaxLimbs) != BBP_OK) {
+        q->run.reset();
+        if (plan_query_work(E->plan, q->n, q->P, q, false) != BBP_OK) q->prime = false;  // by its terms instead
+        continue;
+      }
+      q->next_list = 0;
+      turn = free_lane + 1;
+      begun.push_back(q);
+      if (is_long) {
+        q->lane = free_lane;
+        E->lane_owner[free_lane] = q;
+      } else {
+        parts.push_back(PrimePart{q, free_lane, 0, q->run->lists()});
+        q->next_list = q->run->lists();
+        *terms += q->total_terms;
+        *cost += whole;
+        taken += whole;
+        continue;
+      }
+    }
+    // some lists of a long query
+    const size_t first = q->next_list;
+    uint64_t part = 0;
+    while (q->next_list < q->run->lists() && (part == 0 || part < budget / kServeLanes))
+      part += std::max<uint64_t>(1, static_cast<uint64_t>(q->run->share(q->next_list++) * static_cast<double>(whole)));
+    parts.push_back(PrimePart{q, q->lane, first, q->next_list});
+    const uint64_t done = q->next_list == q->run->lists()
+                              ? q->total_terms
+                              : std::min(q->total_terms, q->terms_done + part * kPrimeTermsPerTerm);
+    *terms += done - q->terms_done;
+    q->terms_done = done;
+    *cost += part;
+    taken += part;
+  }
 }
 
 // Plans one iteration over the active queries into staging H and enqueues it
@@ -356,20 +497,38 @@ void free_engine(ServeEngine* E) {
 bool enqueue_iteration(ServeEngine* E, HostStage& H, std::vector<Query*>& batch, std::vector<int>& fresh_slots) {
   bbp_plan p = E->plan;
   const uint64_t budget_terms = std::max<uint64_t>(1, static_cast<uint64_t>(E->rate * kIterTargetSeconds));
-  const uint64_t share = std::max<uint64_t>(1, budget_terms / std::max<size_t>(1, batch.size()));
   std::vector<Piece> pieces;
-  uint64_t terms = 0;
+  std::vector<PrimePart> parts;
+  std::vector<Query*> begun;
+  uint64_t terms = 0, cost = 0, prime_terms = 0;
   std::vector<uint32_t> npieces(batch.size(), 0);
   H.finishing.clear();
+  bool primes = false;
+  for (Query* q : batch) primes |= q->prime;
+  if (primes && !make_lanes(E))
+    for (Query* q : batch)
+      if (q->prime && plan_query_work(p, q->n, q->P, q, false) != BBP_OK) return false;
+  size_t by_terms = 0;
+  for (Query* q : batch) by_terms += q->prime ? 0 : 1;
+  // half of an iteration for either kind while there are both
+  take_primes(E, batch, by_terms ? budget_terms / 2 : budget_terms, parts, begun, &prime_terms, &cost);
+  const uint64_t share = std::max<uint64_t>(1, (budget_terms - std::min(cost, budget_terms / 2)) / std::max<size_t>(1, by_terms));
   for (size_t i = 0; i < batch.size(); ++i) {
     Query* q = batch[i];
     const size_t before = pieces.size();
-    take_pieces(E, q, share, pieces, &terms);
+    if (q->prime) {  // its few other terms with its first lists
+      uint64_t few = 0;
+      if (std::find(begun.begin(), begun.end(), q) != begun.end()) take_pieces(E, q, UINT64_MAX, pieces, &few);
+      q->final_in_flight = q->run && q->next_list == q->run->lists();
+    } else {
+      take_pieces(E, q, share, pieces, &terms);
+      q->final_in_flight = q->next >= q->work.size();
+    }
     npieces[i] = static_cast<uint32_t>(pieces.size() - before);
-    q->final_in_flight = q->next >= q->work.size();
     if (q->final_in_flight) H.finishing.push_back(q);
   }
-  H.terms = terms;
+  H.terms = terms + prime_terms;
+  H.cost = terms + cost;
   // group head pieces by variant, tails apart
   std::vector<uint32_t> vb(kVariants + 1, 0);
   std::vector<const Piece*> heads, tails;
@@ -406,7 +565,8 @@ bool enqueue_iteration(ServeEngine* E, HostStage& H, std::vector<Query*>& batch,
     Q.P = q->P;
     Q.L = q->L;
     Q.out_offset = static_cast<uint32_t>(q->slot) * kOutStride;
-    H.jobs_left[q->slot] = npieces[i] + (q->final_in_flight ? 0u : 1u);  // hold while work remains
+    // held while work remains, and for a prime form, whose check writes the result
+    H.jobs_left[q->slot] = npieces[i] + (q->final_in_flight && !q->prime ? 0u : 1u);
   }
   cudaStream_t s = E->stream;
   cudaError_t e = cudaSuccess;
@@ -446,6 +606,29 @@ bool enqueue_iteration(ServeEngine* E, HostStage& H, std::vector<Query*>& batch,
     const int blocks = queue_occupancy(path, head_streams(p, path), lmax) * p->sm_count;
     chk(launch_queue(dev, vb[v], vb[v + 1], E->d_cursors + v, path, head_streams(p, path), lmax, blocks, s));
   }
+  if (!parts.empty()) {
+    bool used[kServeLanes] = {};
+    chk(cudaEventRecord(E->queued, s));
+    for (const PrimePart& part : parts) {
+      const cudaStream_t to = E->lane_stream[part.lane];
+      const size_t slot = static_cast<size_t>(part.q->slot);
+      PrimeRun& run = *part.q->run;
+      if (!used[part.lane]) chk(cudaStreamWaitEvent(to, E->queued, 0));
+      used[part.lane] = true;
+      bool ok = part.first != 0 || run.begin(to) == BBP_OK;
+      ok = ok && run.run(part.first, part.last, to) == BBP_OK;
+      if (part.last == run.lists())
+        ok = ok && run.finish(part.q->P, part.q->bound, E->d_out + slot * kOutStride, E->d_valid + slot,
+                              E->d_redo + slot, to) == BBP_OK;
+      if (!ok) chk(cudaErrorUnknown);
+    }
+    for (int i = 0; i < kServeLanes; ++i) {
+      if (!used[i]) continue;
+      chk(cudaEventRecord(E->lane_done[i], E->lane_stream[i]));
+      chk(cudaStreamWaitEvent(s, E->lane_done[i], 0));
+    }
+    chk(cudaMemcpyAsync(H.redo, E->d_redo, sizeof(uint32_t) * E->max_slots, cudaMemcpyDeviceToHost, s));
+  }
   if (!H.finishing.empty()) {  // results of the queries that finish in this iteration
     chk(cudaMemcpyAsync(H.out, E->d_out, static_cast<size_t>(kOutStride) * E->max_slots, cudaMemcpyDeviceToHost, s));
     chk(cudaMemcpyAsync(H.valid, E->d_valid, sizeof(uint32_t) * E->max_slots, cudaMemcpyDeviceToHost, s));
@@ -464,10 +647,35 @@ bool finish_iteration(ServeEngine* E, HostStage& H) {
   float ms = 0;
   const bool timed = cudaEventElapsedTime(&ms, H.start, H.done) == cudaSuccess && ms > 0.1f && H.terms > 0;
   std::lock_guard<std::mutex> lock(E->mu);
-  if (timed) E->rate = 0.7 * E->rate + 0.3 * (static_cast<double>(H.terms) / (1e-3 * ms));
+  if (timed) {
+    // a short iteration is mostly launches: it says little about the rate of a full one
+    const double w = 0.3 * std::min(1.0, ms / 5.0);
+    E->rate = (1.0 - w) * E->rate + w * (static_cast<double>(H.cost) / (1e-3 * ms));
+    E->terms_rate = 0.7 * E->terms_rate + 0.3 * (static_cast<double>(H.terms) / (1e-3 * ms));
+  }
   E->iterations++;
   E->terms_done += H.terms;
   for (Query* q : H.finishing) {
+    if (q->lane >= 0) E->lane_owner[q->lane] = nullptr;
+    q->lane = -1;
+    q->run.reset();
+    if (q->prime && H.redo[q->slot] != 0) {  // too close to a carry: the terms decide
+      E->terms_done -= q->total_terms;
+      q->next = 0;
+      q->tile_off = 0;
+      q->final_in_flight = false;
+      const bbp_status ps = plan_query_work(E->plan, q->n, q->P, q, false);
+      if (ps == BBP_OK) {
+        E->rezero.push_back(q->slot);
+        E->active.push_back(q);
+        continue;
+      }
+      q->state = kFailed;
+      q->error = ps;
+      E->free_slots.push_back(q->slot);
+      q->slot = -1;
+      continue;
+    }
     q->out.assign(H.out + static_cast<size_t>(q->slot) * kOutStride,
                   H.out + static_cast<size_t>(q->slot) * kOutStride + (q->P + 7) / 8);
     q->valid = H.valid[q->slot];
@@ -491,6 +699,9 @@ void fail_all(ServeEngine* E) {
     q->error = BBP_ECUDA;
     if (q->slot >= 0) E->free_slots.push_back(q->slot);
     q->slot = -1;
+    if (q->lane >= 0) E->lane_owner[q->lane] = nullptr;
+    q->lane = -1;
+    q->run.reset();
     q->work.clear();
   };
   for (Query* q : E->stage.finishing) fail(q);
@@ -518,6 +729,8 @@ void engine_main(ServeEngine* E) {
         E->active.push_back(q);
         fresh.push_back(q->slot);
       }
+      fresh.insert(fresh.end(), E->rezero.begin(), E->rezero.end());
+      E->rezero.clear();
       batch = E->active;
     }
     bool ok = enqueue_iteration(E, E->stage, batch, fresh);
@@ -587,7 +800,7 @@ bbp_status bbp_submit(bbp_plan p, uint64_t n, uint32_t P, bbp_ticket* t) {
   if (!p || !t) return BBP_EINVAL;
   Query* q = new (std::nothrow) Query();
   if (!q) return BBP_ENOMEM;
-  const bbp_status ps = plan_query_work(p, n, P, q);
+  const bbp_status ps = plan_query_work(p, n, P, q, true);
   if (ps != BBP_OK) {
     delete q;
     return ps;
@@ -644,7 +857,7 @@ bbp_status bbp_serve_stats(bbp_plan p, bbp_serve_info* info) {
   info->slots = E->max_slots;
   info->iterations = E->iterations;
   info->terms = E->terms_done;
-  info->terms_per_s = E->rate;
+  info->terms_per_s = E->terms_rate;
   return BBP_OK;
 }
 

@@ -3,6 +3,8 @@ term-by-term kernels (bbp_accumulate_async + bbp_finalize_async): the same bits 
 certified count, tolerance 0, at positions where the prime form's limits, classes, lists and
 words change, and where its check sends the query back to the terms."""
 
+import time
+
 import pytest
 
 pytestmark = pytest.mark.gpu
@@ -75,6 +77,17 @@ def test_check_sends_uncertain_positions_to_the_terms(bbp, plans):
     vals, valid, lat = bbp.bbp_bits_batch(plan.handle, 0, ns, [P] * len(ns))
     assert dict(zip(ns, zip(vals, valid))) == checked
     assert all(v > 0 for v in lat)
+    # and through the serving engine, where they go back to its queue
+    tickets = {n: bbp.bbp_submit(plan.handle, n, P) for n in ns}
+    got, t_end = {}, time.time() + 60
+    while len(got) < len(ns) and time.time() < t_end:
+        for n in ns:
+            if n not in got:
+                r = bbp.bbp_poll(plan.handle, tickets[n], P)
+                if r is not None:
+                    got[n] = r
+        time.sleep(0.001)
+    assert got == checked
 
 
 def test_batch_of_both_kinds(bbp, plans):
