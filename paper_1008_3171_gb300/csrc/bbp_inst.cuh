@@ -50,6 +50,12 @@ int queue_occupancy_t() {
   return n > 0 ? n : 1;
 }
 
+template <int S>
+cudaError_t launch_query_t(const QuerySet& q, int blocks, int threads, cudaStream_t s) {
+  query_kernel<BBP_LMAX, S><<<q.tail_blocks + blocks, threads, 0, s>>>(q);
+  return cudaGetLastError();
+}
+
 template <typename K>
 cudaError_t launch_prime_t(K kernel, const PrimeArgs& a, int sms, cudaStream_t s) {
   // the sieve's CTAs need the SM's shared memory while these run
@@ -78,6 +84,18 @@ cudaError_t BBP_CAT(launch_prime_l, BBP_LMAX)(const PrimeArgs& a, PrimeKernel k,
     case kPowers2: return launch_prime_t(prime_power_kernel<Arith2, false, BBP_LMAX>, a, sms, s);
   }
   return cudaErrorInvalidValue;
+}
+
+cudaError_t BBP_CAT(launch_query_l, BBP_LMAX)(const QuerySet& q, int streams, int blocks, int threads, cudaStream_t s) {
+  return streams == 2 ? launch_query_t<2>(q, blocks, threads, s) : launch_query_t<1>(q, blocks, threads, s);
+}
+
+int BBP_CAT(query_occupancy_l, BBP_LMAX)(int streams, int threads) {
+  int n = 0;
+  const cudaError_t e =
+      streams == 2 ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, query_kernel<BBP_LMAX, 2>, threads, 0)
+                   : cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, query_kernel<BBP_LMAX, 1>, threads, 0);
+  return e == cudaSuccess && n > 0 ? n : 1;
 }
 
 // path 0..3 (kNumPaths), streams 1 or 2 (anything else runs 1)

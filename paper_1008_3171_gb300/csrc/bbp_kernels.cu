@@ -14,57 +14,10 @@
 #include "bbp_device.cuh"
 #include "bbp_finalize.cuh"
 #include "bbp_kernels.cuh"
+#include "bbp_tail.cuh"
 
 namespace bbp {
 namespace {
-
-// ---------------------------------------------------------------- tail terms
-//
-// A tail term is B_k = 2^e / m with e < 0 (Eq. 5); its W-bit value is
-// floor(2^(W+e)/m) = floor(floor(2^W/m) / 2^-e): the fraction of 1/m, shifted
-// (Sec. 4.3: shift by b bits, then divide to W - b bits).  There are only about
-// W/step of them per series, so one thread per term with plain loops.
-// t (W/32 limbs, signed by (-1)^k and the series sign, mod 2^W) of tail term k.
-__device__ void tail_term(const TailArgs& A, const uint64_t k, uint32_t* t) {
-  const int64_t e = static_cast<int64_t>(A.d) + A.c - static_cast<int64_t>(A.step) * static_cast<int64_t>(k);
-  const uint32_t L = A.L;
-  const int64_t bshift = -e;  // 1 <= bshift <= W
-  const uint64_t m = static_cast<uint64_t>(A.a) * k + A.b;
-  uint32_t q[kMaxLimbs];
-  for (uint32_t i = 0; i < L; ++i) { q[i] = 0; t[i] = 0; }
-  if (e >= 0 || bshift > static_cast<int64_t>(A.W)) return;
-  const uint32_t b = static_cast<uint32_t>(bshift);
-  if (m == 1) {
-    const uint32_t bit = A.W - b;  // floor(2^(W-b) / 1), below 2^W since b >= 1
-    t[bit >> 5] = 1u << (bit & 31u);
-  } else {
-    uint64_t x = 1;  // 2^W mod m by doubling; m < 2^62
-    for (uint32_t i = 0; i < A.W; ++i) {
-      x <<= 1;
-      if (x >= m) x -= m;
-    }
-    Mod64 M{lo32(m), hi32(m), neg_inverse32(lo32(m))};
-    uint32_t x0 = lo32(x), x1 = hi32(x);
-    for (uint32_t i = 0; i < L; ++i) q[i] = hensel_step64(x0, x1, M);
-    // t = q >> b
-    const uint32_t bl = b >> 5, bb = b & 31u;
-    for (uint32_t i = 0; i < L; ++i) {
-      const uint32_t src = i + bl;
-      uint32_t lo = src < L ? q[src] : 0u;
-      uint32_t hi = src + 1 < L ? q[src + 1] : 0u;
-      t[i] = bb ? ((lo >> bb) | (hi << (32u - bb))) : lo;
-    }
-  }
-  const bool neg = ((A.alternating && (k & 1ull)) ? 1u : 0u) ^ A.negate;
-  if (neg) {
-    uint64_t carry = 1;
-    for (uint32_t i = 0; i < L; ++i) {
-      const uint64_t s = static_cast<uint64_t>(~t[i]) + carry;
-      t[i] = static_cast<uint32_t>(s);
-      carry = s >> 32;
-    }
-  }
-}
 
 __global__ void tail_kernel(const TailArgs A) {
   const uint64_t tid = static_cast<uint64_t>(blockIdx.x) * blockDim.x + threadIdx.x;
@@ -79,15 +32,7 @@ __global__ void tail_kernel(const TailArgs A) {
 // the ranges laid end to end.
 __global__ void tail_set_kernel(const TailSet S) {
   if (S.gate && *S.gate == 0u) return;
-  uint64_t i = static_cast<uint64_t>(blockIdx.x) * blockDim.x + threadIdx.x;
-  uint32_t r = 0;
-  while (r < S.n && i >= S.a[r].count) i -= S.a[r++].count;
-  if (r >= S.n) return;
-  const TailArgs& A = S.a[r];
-  uint32_t t[kMaxLimbs];
-  tail_term(A, A.k_begin + i, t);
-  for (uint32_t l = 0; l < A.L; ++l)
-    if (t[l]) atomicAdd(A.slots + l, static_cast<unsigned long long>(t[l]));
+  add_tail_term(S, static_cast<uint64_t>(blockIdx.x) * blockDim.x + threadIdx.x);
 }
 
 // ---------------------------------------------------------------- fold / finalize
@@ -263,6 +208,28 @@ cudaError_t launch_prime(const PrimeArgs& a, PrimeKernel k, int lmax, int sms, c
   switch (lmax) {
 #define BBP_CASE(L) \
   case L: return launch_prime_l##L(a, k, sms, s);
+    BBP_LMAX_CASES(BBP_CASE)
+#undef BBP_CASE
+    default: return cudaErrorInvalidValue;
+  }
+}
+
+int query_occupancy(int streams, int lmax, int threads) {
+  if (!valid_head_threads(threads)) return 1;
+  switch (lmax) {
+#define BBP_CASE(L) \
+  case L: return query_occupancy_l##L(streams, threads);
+    BBP_LMAX_CASES(BBP_CASE)
+#undef BBP_CASE
+    default: return 1;
+  }
+}
+
+cudaError_t launch_query(const QuerySet& q, int streams, int lmax, int blocks, int threads, cudaStream_t s) {
+  if (!valid_head_threads(threads)) return cudaErrorInvalidValue;
+  switch (lmax) {
+#define BBP_CASE(L) \
+  case L: return launch_query_l##L(q, streams, blocks, threads, s);
     BBP_LMAX_CASES(BBP_CASE)
 #undef BBP_CASE
     default: return cudaErrorInvalidValue;

@@ -54,6 +54,24 @@ struct TailSet {
   const uint32_t* gate;  // as in HeadArgs
 };
 
+// A whole query in one launch (query_kernel): head ranges on modulus path 0, tails and the
+// result.
+constexpr int kMaxQueryRanges = 32;
+struct QuerySet {
+  HeadArgs head[kMaxQueryRanges];       // `slots` and `gate` not used
+  uint64_t start[kMaxQueryRanges + 1];  // warp tiles before each range, and of all
+  uint32_t n;                           // ranges in use
+  uint32_t tail_blocks;                 // CTAs of tail terms, one term a thread
+  uint64_t bound;
+  uint32_t L, P;
+  TailSet tails;
+  unsigned long long* slots;  // L accumulators, 0 at the start
+  unsigned int* finished;     // CTAs that are done, 0 at the start
+  uint8_t* out;               // device or pinned host memory
+  uint32_t* valid;            // may be NULL
+  uint32_t* limbs;            // may be NULL
+};
+
 constexpr int kMaxLimbs = 40;    // W <= 1280 bits
 constexpr int kHeadThreads = 256;
 // Compiled accumulator capacities (limbs per thread) of the head and queue
@@ -148,6 +166,9 @@ int head_occupancy(int path, int streams, int lmax, int threads = kHeadThreads);
 // below 2^31 or from there on.
 enum PrimeKernel { kPrimes0, kPrimes1, kPrimesHalf, kPrimes3, kSums8, kSums1, kSums2, kPrimeWarps, kPowers1, kPowers2 };
 cudaError_t launch_prime(const PrimeArgs& a, PrimeKernel k, int lmax, int sms, cudaStream_t s);
+// blocks: CTAs for the head ranges, besides q.tail_blocks; both together at least 1.
+cudaError_t launch_query(const QuerySet& q, int streams, int lmax, int blocks, int threads, cudaStream_t s);
+int query_occupancy(int streams, int lmax, int threads);
 // Per accumulator class (bbp_lmax*.cu): the launchers the dispatchers above call.
 #define BBP_DECLARE_LMAX(L)                                                                                    \
   cudaError_t launch_head_l##L(const HeadArgs& a, int path, int streams, int blocks, int threads, cudaStream_t s); \
@@ -155,7 +176,9 @@ cudaError_t launch_prime(const PrimeArgs& a, PrimeKernel k, int lmax, int sms, c
   cudaError_t launch_queue_l##L(const BatchDev& b, uint32_t jb, uint32_t je, unsigned long long* cursor, int path,      \
                                 int streams, int blocks, cudaStream_t s);                                      \
   int queue_occupancy_l##L(int path, int streams);                                                             \
-  cudaError_t launch_prime_l##L(const PrimeArgs& a, PrimeKernel k, int sms, cudaStream_t s);
+  cudaError_t launch_prime_l##L(const PrimeArgs& a, PrimeKernel k, int sms, cudaStream_t s);                   \
+  cudaError_t launch_query_l##L(const QuerySet& q, int streams, int blocks, int threads, cudaStream_t s);      \
+  int query_occupancy_l##L(int streams, int threads);
 BBP_DECLARE_LMAX(3)
 BBP_DECLARE_LMAX(4)
 BBP_DECLARE_LMAX(6)

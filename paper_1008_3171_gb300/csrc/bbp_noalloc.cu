@@ -124,15 +124,18 @@ extern "C" bbp_status bbp_partial_sum_noalloc(bbp_formula f, uint32_t denominato
       a.L = L;
       a.alternating = F.alternating;
       a.negate = ((s.sign < 0) != (F.alternating && (kb & 1ull))) ? 1u : 0u;
-      a.run = kRun;
       a.window = window;
       a.first = first;
       a.first_max = first_max;
       a.slots = slots;
-      const uint64_t tile = 32ull * static_cast<uint64_t>(streams) * kRun;
-      const uint64_t ntiles = (a.count + tile - 1) / tile;
-      const uint64_t want = (ntiles + kHeadThreads / 32 - 1) / (kHeadThreads / 32);
       const uint64_t cap = static_cast<uint64_t>(head_occupancy(path, streams, lmax)) * static_cast<uint64_t>(sms);
+      // a short range takes fewer terms per stream, so that its tiles fill the resident warps
+      // (150,001 terms: 57.4 us with runs of 64 on 74 warps, 12.5 with runs of 2)
+      const uint64_t warps = kHeadThreads / 32, lanes = 32ull * static_cast<uint64_t>(streams);
+      a.run = kRun;
+      while (a.run % 4 == 0 && (a.count + lanes * a.run - 1) / (lanes * a.run) < cap * warps) a.run /= 2;
+      const uint64_t ntiles = (a.count + lanes * a.run - 1) / (lanes * a.run);
+      const uint64_t want = (ntiles + warps - 1) / warps;
       const int blocks = static_cast<int>(std::max<uint64_t>(1, std::min(want, cap)));
       if (launch_head(a, path, streams, lmax, blocks, st) != cudaSuccess) return BBP_ECUDA;
     }

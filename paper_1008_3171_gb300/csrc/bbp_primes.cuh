@@ -207,34 +207,6 @@ __device__ __forceinline__ void prime_residues(const uint64_t e, const uint64_t 
   }
 }
 
-// Sums every thread's LMAX-limb value over the CTA and adds it to the carry-save slots.
-template <int LMAX>
-__device__ __forceinline__ void flush_cta(uint32_t (&acc)[LMAX], uint32_t L, unsigned long long* slots) {
-  const uint32_t lane = threadIdx.x & 31u;
-  const uint32_t wid = threadIdx.x >> 5;
-#pragma unroll
-  for (int i = 0; i < LMAX; ++i)
-    if (i >= static_cast<int>(L)) acc[i] = 0;
-  __shared__ uint32_t red[kHeadThreads / 32][LMAX];
-  warp_sum_limbs<LMAX>(acc);
-  if (lane == 0) {
-#pragma unroll
-    for (int i = 0; i < LMAX; ++i) red[wid][i] = acc[i];
-  }
-  __syncthreads();
-  if (wid == 0) {
-    const uint32_t nw = blockDim.x >> 5;
-#pragma unroll
-    for (int i = 0; i < LMAX; ++i) acc[i] = lane < nw ? red[lane][i] : 0u;
-    warp_sum_limbs<LMAX>(acc);
-    if (lane == 0) {
-#pragma unroll
-      for (int i = 0; i < LMAX; ++i)
-        if (i < static_cast<int>(L) && acc[i]) atomicAdd(slots + i, static_cast<unsigned long long>(acc[i]));
-    }
-  }
-}
-
 // Hands the next `n` primes of the list to the warp.
 __device__ __forceinline__ uint32_t take_primes(uint32_t* taken, uint32_t n, uint32_t lane) {
   uint32_t at = 0;

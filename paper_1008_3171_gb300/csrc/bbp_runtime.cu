@@ -114,8 +114,7 @@ bbp_status bbp_plan_create(bbp_plan* out, const bbp_plan_opts* opts) {
   }
   bool ok = cudaMalloc(&p->d_slots, sizeof(unsigned long long) * kMaxLimbs) == cudaSuccess &&
             cudaMalloc(&p->d_limbs, sizeof(uint32_t) * kMaxLimbs) == cudaSuccess &&
-            cudaMalloc(&p->d_bytes, kMaxWorkingBits / 8) == cudaSuccess &&
-            cudaMalloc(&p->d_valid, sizeof(uint32_t)) == cudaSuccess &&
+            cudaMalloc(&p->d_query, sizeof(unsigned long long) * (kMaxLimbs + 1)) == cudaSuccess &&
             cudaMalloc(&p->d_redo, sizeof(uint32_t)) == cudaSuccess &&
             cudaMallocHost(&p->h_stage, 4096) == cudaSuccess &&
             cudaEventCreate(&p->ev0) == cudaSuccess && cudaEventCreate(&p->ev1) == cudaSuccess &&
@@ -138,8 +137,7 @@ bbp_status bbp_plan_destroy(bbp_plan p) {
   release_prime_state(&p->primes);
   cudaFree(p->d_slots);
   cudaFree(p->d_limbs);
-  cudaFree(p->d_bytes);
-  cudaFree(p->d_valid);
+  cudaFree(p->d_query);
   cudaFree(p->d_redo);
   cudaFreeHost(p->h_stage);
   if (p->ev0) cudaEventDestroy(p->ev0);
@@ -176,34 +174,137 @@ bbp_status bbp_plan_stats(bbp_plan p, bbp_stats* out) {
 
 namespace bbp {
 
+namespace {
+
+HeadArgs head_args(const FormulaDef& F, const TermRange& r, uint64_t n, uint32_t W) {
+  const SeriesDef& s = F.s[r.j];
+  HeadArgs a{};
+  a.d = n - 1;
+  a.k_begin = r.k_begin;
+  a.count = r.count;
+  a.a = s.a;
+  a.b = s.b;
+  a.c = s.c;
+  a.step = F.step;
+  a.W = W;
+  a.L = W / 32;
+  a.alternating = F.alternating;
+  a.negate = ((s.sign < 0) != (F.alternating && (r.k_begin & 1ull))) ? 1u : 0u;
+  a.window = r.window;
+  a.first = r.first;
+  a.first_max = r.first_max;
+  return a;
+}
+
+TailArgs tail_args(const FormulaDef& F, const TermRange& r, uint64_t n, uint32_t W, unsigned long long* slots) {
+  const SeriesDef& s = F.s[r.j];
+  TailArgs a{};
+  a.d = n - 1;
+  a.k_begin = r.k_begin;
+  a.count = r.count;
+  a.a = s.a;
+  a.b = s.b;
+  a.c = s.c;
+  a.step = F.step;
+  a.W = W;
+  a.L = W / 32;
+  a.alternating = F.alternating;
+  a.negate = s.sign < 0 ? 1u : 0u;
+  a.slots = slots;
+  return a;
+}
+
+// Consecutive terms per stream: the plan's, less while `count_tiles(run)` tiles would not
+// fill the resident warps.
+template <typename F>
+uint32_t run_for(uint32_t run, uint64_t resident_warps, F count_tiles) {
+  while (run % 4 == 0 && count_tiles(run) < resident_warps) run /= 2;
+  return run;
+}
+
+}  // namespace
+
+// Queues a whole query as one launch if all its head ranges are on modulus path 0 (n up
+// to 2^29); *done says whether it did.
+bbp_status launch_one(bbp_plan p, int f, uint64_t n, uint32_t W, uint32_t P, const std::vector<TermRange>& ranges,
+                      uint64_t bound, uint8_t* out, uint32_t* valid, uint32_t* limbs, cudaStream_t st, bool* done) {
+  *done = false;
+  const FormulaDef& F = formula_def(f);
+  const int lmax = pick_lmax(W, p->limb_bump);
+  if (lmax == 0) return BBP_EINVAL;
+  uint32_t heads = 0, tails = 0;
+  for (const TermRange& r : ranges) {
+    if (!r.tail && r.path != 0) return BBP_OK;
+    ++(r.tail ? tails : heads);
+  }
+  if (heads > static_cast<uint32_t>(kMaxQueryRanges) || tails > static_cast<uint32_t>(kMaxTailSet)) return BBP_OK;
+  QuerySet q{};
+  q.slots = p->d_query;
+  q.finished = reinterpret_cast<unsigned int*>(p->d_query + kMaxLimbs);
+  q.bound = bound;
+  q.L = W / 32;
+  q.P = P;
+  q.out = out;
+  q.valid = valid;
+  q.limbs = limbs;
+  const int streams = head_streams(p, 0);
+  const int warps_per_block = p->cta / 32;
+  const uint64_t cap = static_cast<uint64_t>(query_occupancy(streams, lmax, p->cta)) * p->sm_count;
+  auto tiles_of = [&](uint64_t count, uint32_t run) { return (count + 32ull * streams * run - 1) / (32ull * streams * run); };
+  auto count_tiles = [&](uint32_t run) {
+    uint64_t total = 0;
+    for (const TermRange& r : ranges) total += r.tail ? 0 : tiles_of(r.count, run);
+    return total;
+  };
+  const uint32_t run = run_for(static_cast<uint32_t>(p->run), cap * warps_per_block, count_tiles);
+  uint64_t tail_terms = 0;
+  p->stats = bbp_stats{};
+  for (const TermRange& r : ranges) {
+    p->stats.terms += r.count;
+    if (r.tail) {
+      q.tails.a[q.tails.n++] = tail_args(F, r, n, W, q.slots);
+      tail_terms += r.count;
+    } else {
+      HeadArgs& a = q.head[q.n];
+      a = head_args(F, r, n, W);
+      a.run = run;
+      q.start[q.n + 1] = q.start[q.n] + tiles_of(r.count, run);
+      ++q.n;
+      p->stats.head_terms += r.count;
+      p->stats.imad_model += r.imad;
+    }
+  }
+  q.tail_blocks = static_cast<uint32_t>((tail_terms + p->cta - 1) / p->cta);
+  const uint64_t want = (q.start[q.n] + warps_per_block - 1) / warps_per_block;
+  const int blocks = static_cast<int>(std::max<uint64_t>(q.tail_blocks ? 0 : 1, std::min(want, cap)));
+  BBP_CUDA(cudaMemsetAsync(p->d_query, 0, sizeof(unsigned long long) * (kMaxLimbs + 1), st));
+  if (p->profile) BBP_CUDA(cudaEventRecord(p->ev0, st));
+  BBP_CUDA(launch_query(q, streams, lmax, blocks, p->cta, st));
+  p->stats.kernel_launches = 1;
+  p->stats.head_launches = 1;
+  if (p->profile) {
+    BBP_CUDA(cudaEventRecord(p->ev1, st));
+    BBP_CUDA(cudaEventSynchronize(p->ev1));
+    float ms = 0;
+    BBP_CUDA(cudaEventElapsedTime(&ms, p->ev0, p->ev1));
+    p->stats.head_ms = ms;
+  }
+  *done = true;
+  return BBP_OK;
+}
+
 // Launches every range of `ranges` (all of one query, same W) into `slots`.
 bbp_status launch_ranges(bbp_plan p, int f, uint64_t n, uint32_t W, const std::vector<TermRange>& ranges,
                          unsigned long long* slots, cudaStream_t st, const uint32_t* gate) {
   const FormulaDef& F = formula_def(f);
-  const uint32_t L = W / 32;
   const int lmax = pick_lmax(W, p->limb_bump);
   if (lmax == 0) return BBP_EINVAL;
   float total_ms = 0;
   TailSet tails{};
   tails.gate = gate;
   for (const TermRange& r : ranges) {
-    const SeriesDef& s = F.s[r.j];
-    const bool odd_start = F.alternating && (r.k_begin & 1ull);
     if (r.tail) {  // collected, and launched together once the set is full or the ranges end
-      TailArgs& a = tails.a[tails.n++];
-      a = TailArgs{};
-      a.d = n - 1;
-      a.k_begin = r.k_begin;
-      a.count = r.count;
-      a.a = s.a;
-      a.b = s.b;
-      a.c = s.c;
-      a.step = F.step;
-      a.W = W;
-      a.L = L;
-      a.alternating = F.alternating;
-      a.negate = s.sign < 0 ? 1u : 0u;
-      a.slots = slots;
+      tails.a[tails.n++] = tail_args(F, r, n, W, slots);
       p->stats.terms += r.count;
       if (tails.n == kMaxTailSet) {
         BBP_CUDA(launch_tail_set(tails, st));
@@ -212,21 +313,7 @@ bbp_status launch_ranges(bbp_plan p, int f, uint64_t n, uint32_t W, const std::v
       }
       continue;
     }
-    HeadArgs a{};
-    a.d = n - 1;
-    a.k_begin = r.k_begin;
-    a.count = r.count;
-    a.a = s.a;
-    a.b = s.b;
-    a.c = s.c;
-    a.step = F.step;
-    a.W = W;
-    a.L = L;
-    a.alternating = F.alternating;
-    a.negate = ((s.sign < 0) != odd_start) ? 1u : 0u;
-    a.window = r.window;
-    a.first = r.first;
-    a.first_max = r.first_max;
+    HeadArgs a = head_args(F, r, n, W);
     a.slots = slots;
     a.gate = gate;
     const int streams = head_streams(p, r.path);
@@ -235,9 +322,8 @@ bbp_status launch_ranges(bbp_plan p, int f, uint64_t n, uint32_t W, const std::v
     const uint64_t resident_warps = static_cast<uint64_t>(occ) * p->sm_count * warps_per_block;
     // a short range takes fewer consecutive terms per stream, so that its tiles
     // spread over the GPU's resident warps instead of a few warps running long runs
-    uint32_t run = static_cast<uint32_t>(p->run);
     auto tiles_for = [&](uint32_t rn) { return (r.count + 32ull * streams * rn - 1) / (32ull * streams * rn); };
-    while (run % 4 == 0 && tiles_for(run) < resident_warps) run /= 2;
+    const uint32_t run = run_for(static_cast<uint32_t>(p->run), resident_warps, tiles_for);
     a.run = run;
     const uint64_t ntiles = tiles_for(run);
     const uint64_t want = (ntiles + warps_per_block - 1) / warps_per_block;
@@ -294,10 +380,11 @@ namespace {
 // queued behind it, which do nothing unless the check asks for them.
 enum Form { kTerms, kPrimeOnly, kPrimeOrTerms };
 
-// Queues a whole query.  *by_primes (may be NULL): whether the prime form runs.
+// Queues a whole query.  kPrimeOnly: *redo says whether the terms are wanted, 0 unless
+// the prime form runs.  Outputs may be in pinned host memory.
 bbp_status enqueue_bits(bbp_plan p, int f, uint64_t n, uint32_t P, uint32_t W, uint8_t* d_out, uint32_t* d_valid,
-                        uint32_t* d_limbs, cudaStream_t s, Form form, bool* by_primes) {
-  if (by_primes) *by_primes = false;
+                        uint32_t* d_limbs, cudaStream_t s, Form form, uint32_t* redo) {
+  if (!redo) redo = p->d_redo;
   const FormulaDef& F = formula_def(f);
   std::vector<TermRange> ranges;
   uint64_t N = 0;
@@ -326,7 +413,7 @@ bbp_status enqueue_bits(bbp_plan p, int f, uint64_t n, uint32_t P, uint32_t W, u
     bbp_status ps = run.plan(p->primes, p->sm_count, n, W, p->d_slots);
     if (ps == BBP_OK) ps = run.begin(s);
     if (ps == BBP_OK) ps = run.run(0, run.lists(), s);
-    if (ps == BBP_OK) ps = run.finish(P, bound, d_out, d_valid, p->d_redo, s);
+    if (ps == BBP_OK) ps = run.finish(P, bound, d_out, d_valid, redo, s);
     prime_launches = run.launches();
     if (ps != BBP_OK) return ps;
     if (p->profile) {
@@ -335,8 +422,11 @@ bbp_status enqueue_bits(bbp_plan p, int f, uint64_t n, uint32_t P, uint32_t W, u
       BBP_CUDA(cudaEventElapsedTime(&prime_ms, p->ev2, p->ev1));
     }
     prime_launches += p->stats.kernel_launches + 1;
-    gate = p->d_redo;
-    if (by_primes) *by_primes = true;
+    gate = redo;
+  } else {
+    bool done = false;
+    const bbp_status os = launch_one(p, f, n, W, P, ranges, bound, d_out, d_valid, d_limbs, s, &done);
+    if (os != BBP_OK || done) return os;
   }
   if (gate && form == kPrimeOnly) {
     p->stats = bbp_stats{};
@@ -496,24 +586,19 @@ bbp_status bbp_bits_formula(bbp_plan p, bbp_formula f, uint64_t n, uint32_t P, u
   if (!p || !out) return BBP_EINVAL;
   uint32_t W;
   if (!valid_formula(f) || n == 0 || P == 0 || !working_bits(P, p->guard, &W)) return BBP_EINVAL;
-  const uint32_t nbytes = (P + 7) / 8;
+  // the kernels write their results to pinned host memory: no copies behind them
   uint8_t* h = static_cast<uint8_t*>(p->h_stage);
-  uint32_t valid = 0;
+  uint32_t* h_valid = reinterpret_cast<uint32_t*>(h + 2048);
+  uint32_t* h_redo = h_valid + 1;
   for (Form form = kPrimeOnly;; form = kTerms) {
-    bool by_primes = false;
-    const bbp_status st = enqueue_bits(p, f, n, P, W, p->d_bytes, p->d_valid, nullptr, p->stream, form, &by_primes);
+    *h_redo = 0;
+    const bbp_status st = enqueue_bits(p, f, n, P, W, h, h_valid, nullptr, p->stream, form, h_redo);
     if (st != BBP_OK) return st;
-    BBP_CUDA(cudaMemcpyAsync(h, p->d_bytes, nbytes, cudaMemcpyDeviceToHost, p->stream));
-    BBP_CUDA(cudaMemcpyAsync(h + 2048, p->d_valid, sizeof(uint32_t), cudaMemcpyDeviceToHost, p->stream));
-    if (by_primes)
-      BBP_CUDA(cudaMemcpyAsync(h + 2052, p->d_redo, sizeof(uint32_t), cudaMemcpyDeviceToHost, p->stream));
     BBP_CUDA(cudaStreamSynchronize(p->stream));
-    uint32_t redo = 0;
-    if (by_primes) std::memcpy(&redo, h + 2052, sizeof(redo));
-    if (redo == 0) break;
+    if (*reinterpret_cast<volatile uint32_t*>(h_redo) == 0) break;
   }
-  std::memcpy(out, h, nbytes);
-  std::memcpy(&valid, h + 2048, sizeof(valid));
+  std::memcpy(out, h, (P + 7) / 8);
+  const uint32_t valid = *reinterpret_cast<volatile uint32_t*>(h_valid);
   if (valid_bits) *valid_bits = valid;
   if (p->strict && valid < P) return BBP_EINVALID_BITS;
   return BBP_OK;

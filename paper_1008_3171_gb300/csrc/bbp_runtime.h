@@ -28,9 +28,8 @@ struct bbp_plan_s {
   int wide_min_bits = bbp::kWideMinBits;  // moduli of at least this many bits take the 64-bit Montgomery path
   // single-query buffers
   unsigned long long* d_slots = nullptr;  // kMaxLimbs carry-save accumulators
+  unsigned long long* d_query = nullptr;  // the same for one-launch queries, and their CTA counter
   uint32_t* d_limbs = nullptr;
-  uint8_t* d_bytes = nullptr;
-  uint32_t* d_valid = nullptr;
   void* h_stage = nullptr;  // 4 KiB pinned staging
   cudaEvent_t ev0 = nullptr, ev1 = nullptr, ev2 = nullptr;
   bbp_stats stats{};
