@@ -126,7 +126,7 @@ bbp_status bbp_partial_sum_async(bbp_plan p, bbp_formula f, uint32_t denominator
                                  uint64_t k_end, uint64_t n, uint32_t P, uint32_t* d_out_limbs,
                                  void* stream);
 
-/* Bits n .. n+P-1 of pi by Eq. 2.  Whole queries by Eq. 2 with 1.6e7 <= n <= 1.09e13 and guard
+/* Bits n .. n+P-1 of pi by Eq. 2.  Whole queries by either formula with 1.6e7 <= n <= 1.09e13 and guard
  * bits to spare are summed over the primes up to n instead of over the terms (partial
  * fractions of the moduli); the sum is checked on the device, and where it is too close
  * to a carry to have the term-by-term sum's bits for certain, the terms are summed.  The

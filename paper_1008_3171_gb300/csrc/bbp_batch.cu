@@ -205,12 +205,12 @@ static bbp_status plan_batch(bbp_plan p, int f, uint32_t count, const uint64_t* 
       if (!r.tail && !prime) bp->imad += r.imad;
     }
     if (prime) {  // the queue takes what the prime form leaves
-      const PrimeLimits lim = prime_limits(n[q] - 1);
+      const PrimeLimits lim = prime_limits(f, n[q] - 1);
       bp->imad += prime_form_imad(lim, static_cast<int>(L));
       bp->primes.push_back(BatchPlan::Prime{q, W, n[q], bound});
       ranges.clear();
       for (uint32_t j = 0; j < F.count; ++j)
-        if (plan_series(F, j, n[q], W, static_cast<uint32_t>(lmax), prime_first_k(lim, j), UINT64_MAX, ranges,
+        if (plan_series(F, j, n[q], W, static_cast<uint32_t>(lmax), prime_first_k(lim, j, n[q] - 1), UINT64_MAX, ranges,
                         p->wide_min_bits) != 0)
           return BBP_EINVAL;
       jobs_left[q] = 1;  // held: the check writes the result
@@ -489,7 +489,7 @@ static bbp_status run_batch(bbp_plan p, bbp_formula f, uint32_t count, const uin
       const int k = static_cast<int>(i % kPrimeLanes);
       const cudaStream_t to = b->lane_stream[k];
       PrimeRun run;
-      bbp_status ls = run.plan(b->lane[k], p->sm_count, r.n, r.W, b->d_accum + static_cast<uint64_t>(r.q) * kMaxLimbs);
+      bbp_status ls = run.plan(b->lane[k], p->sm_count, f, r.n, r.W, b->d_accum + static_cast<uint64_t>(r.q) * kMaxLimbs);
       if (ls == BBP_OK) ls = run.begin(to);
       if (ls == BBP_OK) ls = run.run(0, run.lists(), to);
       if (ls == BBP_OK)

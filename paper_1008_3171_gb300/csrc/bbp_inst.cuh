@@ -70,18 +70,20 @@ cudaError_t launch_prime_t(K kernel, const PrimeArgs& a, int sms, cudaStream_t s
 
 }  // namespace
 
-cudaError_t BBP_CAT(launch_prime_l, BBP_LMAX)(const PrimeArgs& a, PrimeKernel k, int sms, cudaStream_t s) {
+cudaError_t BBP_CAT(launch_prime_l, BBP_LMAX)(const PrimeArgs& a, PrimeKernel k, int formula, int sms,
+                                              cudaStream_t s) {
+  const bool f = formula != 0;
   switch (k) {
     case kPrimes0: return launch_prime_t(prime_kernel<BBP_LMAX, 0, false>, a, sms, s);
     case kPrimes1: return launch_prime_t(prime_kernel<BBP_LMAX, 1, false>, a, sms, s);
     case kPrimesHalf: return launch_prime_t(prime_kernel<BBP_LMAX, 1, true>, a, sms, s);
     case kPrimes3: return launch_prime_t(prime_kernel<BBP_LMAX, 3, false>, a, sms, s);
-    case kSums8: return launch_prime_t(prime_sum_kernel<Arith1, 8, BBP_LMAX>, a, sms, s);
-    case kSums1: return launch_prime_t(prime_sum_kernel<Arith1, 1, BBP_LMAX>, a, sms, s);
-    case kSums2: return launch_prime_t(prime_sum_kernel<Arith2, 1, BBP_LMAX>, a, sms, s);
-    case kPrimeWarps: return launch_prime_t(prime_power_kernel<Arith1, true, BBP_LMAX>, a, sms, s);
-    case kPowers1: return launch_prime_t(prime_power_kernel<Arith1, false, BBP_LMAX>, a, sms, s);
-    case kPowers2: return launch_prime_t(prime_power_kernel<Arith2, false, BBP_LMAX>, a, sms, s);
+    case kSums8: return launch_prime_t(f ? prime_sum_kernel<Arith1, 1, 8, BBP_LMAX> : prime_sum_kernel<Arith1, 0, 8, BBP_LMAX>, a, sms, s);
+    case kSums1: return launch_prime_t(f ? prime_sum_kernel<Arith1, 1, 1, BBP_LMAX> : prime_sum_kernel<Arith1, 0, 1, BBP_LMAX>, a, sms, s);
+    case kSums2: return launch_prime_t(f ? prime_sum_kernel<Arith2, 1, 1, BBP_LMAX> : prime_sum_kernel<Arith2, 0, 1, BBP_LMAX>, a, sms, s);
+    case kPrimeWarps: return launch_prime_t(f ? prime_power_kernel<Arith1, 1, true, BBP_LMAX> : prime_power_kernel<Arith1, 0, true, BBP_LMAX>, a, sms, s);
+    case kPowers1: return launch_prime_t(f ? prime_power_kernel<Arith1, 1, false, BBP_LMAX> : prime_power_kernel<Arith1, 0, false, BBP_LMAX>, a, sms, s);
+    case kPowers2: return launch_prime_t(f ? prime_power_kernel<Arith2, 1, false, BBP_LMAX> : prime_power_kernel<Arith2, 0, false, BBP_LMAX>, a, sms, s);
   }
   return cudaErrorInvalidValue;
 }

@@ -204,10 +204,10 @@ cudaError_t launch_head(const HeadArgs& a, int path, int streams, int lmax, int 
   }
 }
 
-cudaError_t launch_prime(const PrimeArgs& a, PrimeKernel k, int lmax, int sms, cudaStream_t s) {
+cudaError_t launch_prime(const PrimeArgs& a, PrimeKernel k, int formula, int lmax, int sms, cudaStream_t s) {
   switch (lmax) {
 #define BBP_CASE(L) \
-  case L: return launch_prime_l##L(a, k, sms, s);
+  case L: return launch_prime_l##L(a, k, formula, sms, s);
     BBP_LMAX_CASES(BBP_CASE)
 #undef BBP_CASE
     default: return cudaErrorInvalidValue;

@@ -165,7 +165,7 @@ int head_occupancy(int path, int streams, int lmax, int threads = kHeadThreads);
 // words, kSums8 in one word with eight lanes a prime; kPrimeWarps: prime_power_kernel, a = 1 (p < 2^31); kPowers1, kPowers2: a >= 2 (p < 2^23), p^a
 // below 2^31 or from there on.
 enum PrimeKernel { kPrimes0, kPrimes1, kPrimesHalf, kPrimes3, kSums8, kSums1, kSums2, kPrimeWarps, kPowers1, kPowers2 };
-cudaError_t launch_prime(const PrimeArgs& a, PrimeKernel k, int lmax, int sms, cudaStream_t s);
+cudaError_t launch_prime(const PrimeArgs& a, PrimeKernel k, int formula, int lmax, int sms, cudaStream_t s);
 // blocks: CTAs for the head ranges, besides q.tail_blocks; both together at least 1.
 cudaError_t launch_query(const QuerySet& q, int streams, int lmax, int blocks, int threads, cudaStream_t s);
 int query_occupancy(int streams, int lmax, int threads);
@@ -176,7 +176,7 @@ int query_occupancy(int streams, int lmax, int threads);
   cudaError_t launch_queue_l##L(const BatchDev& b, uint32_t jb, uint32_t je, unsigned long long* cursor, int path,      \
                                 int streams, int blocks, cudaStream_t s);                                      \
   int queue_occupancy_l##L(int path, int streams);                                                             \
-  cudaError_t launch_prime_l##L(const PrimeArgs& a, PrimeKernel k, int sms, cudaStream_t s);                   \
+  cudaError_t launch_prime_l##L(const PrimeArgs& a, PrimeKernel k, int formula, int sms, cudaStream_t s);      \
   cudaError_t launch_query_l##L(const QuerySet& q, int streams, int blocks, int threads, cudaStream_t s);      \
   int query_occupancy_l##L(int streams, int threads);
 BBP_DECLARE_LMAX(3)

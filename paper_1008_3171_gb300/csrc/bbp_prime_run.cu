@@ -4,9 +4,10 @@
 // next is sieved.
 //
 // Measured on a GB300, whole bbp_bits calls, term by term -> by primes: n = 1e9, P = 128:
-// 15.6 -> 2.05 ms; n = 3e8, P = 1000: 7.89 -> 1.20 ms; n = 4e10, P = 256: 1005 -> 89.7 ms;
-// n = 1e12, P = 256: 27.1 -> 2.86 s.  At 4e10 the kernels alone take 52 ms (primes above
-// A / 23), 10 (below), 11 and 2 (prime powers) and 20 (sieve).
+// 15.6 -> 1.79 ms; n = 1e9, P = 64 by Eq. 1: 20.5 -> 2.56 ms; n = 3e8, P = 1000:
+// 7.89 -> 0.93 ms; n = 4e10, P = 256: 1007 -> 89.5 ms; n = 1e12, P = 256: 27.1 -> 2.86 s.
+// At 4e10 the kernels alone take 52 ms (primes above A / 23), 10 (below), 11 and 2 (prime
+// powers) and 20 (sieve).
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -131,14 +132,16 @@ bool prime_workspace(PrimeState** state, uint64_t n, uint32_t max_list, cudaStre
   return true;
 }
 
-bbp_status PrimeRun::plan(PrimeState* state, int sm_count, uint64_t n, uint32_t W, unsigned long long* slots) {
+bbp_status PrimeRun::plan(PrimeState* state, int sm_count, int formula, uint64_t n, uint32_t W,
+                          unsigned long long* slots) {
   state_ = state;
   sms_ = sm_count;
+  formula_ = formula;
   launches_ = 0;
   lists_.clear();
   lmax_ = head_lmax_for(static_cast<int>(W / 32));
   if (lmax_ == 0) return BBP_EINVAL;
-  const PrimeLimits lim = prime_limits(n - 1);
+  const PrimeLimits lim = prime_limits(formula, n - 1);
   const std::vector<PrimeClass> classes = prime_classes(lim);
   if (classes.empty() || classes.size() > static_cast<size_t>(kMaxPrimeClasses)) return BBP_EINVAL;
   PrimeArgs& a = args_;
@@ -159,7 +162,8 @@ bbp_status PrimeRun::plan(PrimeState* state, int sm_count, uint64_t n, uint32_t 
   std::vector<Span> spans;
   {
     const uint64_t grouped = std::min<uint64_t>(lim.A / kGroupSum, (1ull << 31) - 1);
-    const uint64_t cuts[] = {grouped, bottom, (1ull << 29) - 1, (1ull << 31) - 1, kPrimeHalfMax, lim.A};
+    const uint64_t cuts[] = {grouped, bottom, (1ull << 29) - 1, (1ull << 31) - 1, kPrimeHalfMax,
+                             formula == 1 ? lim.B : lim.A, lim.A};
     std::vector<uint64_t> c(std::begin(cuts), std::end(cuts));
     std::sort(c.begin(), c.end());
     uint64_t lo = base_to_;
@@ -186,7 +190,9 @@ bbp_status PrimeRun::plan(PrimeState* state, int sm_count, uint64_t n, uint32_t 
       const uint64_t wave = std::max<uint64_t>(1, static_cast<uint64_t>(sms_) / 8);
       if (nseg > wave) nseg -= nseg % wave;
       const uint64_t hi = std::min(s.hi, base + nseg * seg - 1);
-      lists_.push_back(List{base, lo, hi, static_cast<uint32_t>((hi - base) / seg + 1), s.k});
+      // Eq. 1 above B: c = 1 alone, which only p = 1 mod 4 has
+      lists_.push_back(List{base, lo, hi, static_cast<uint32_t>((hi - base) / seg + 1), s.k,
+                            formula == 1 && lo >= lim.B ? 1u : 0u});
       lo = hi;
     }
   }
@@ -214,9 +220,9 @@ bbp_status PrimeRun::begin(cudaStream_t st) {
   a.cap = kBaseCap;
   a.e = e_;
   const bool above_word = a.A >= (1ull << 31);
-  chk(launch_prime(a, kPowers1, lmax_, sms_, S->sums));
-  if (above_word) chk(launch_prime(a, kPowers2, lmax_, sms_, S->sums));
-  chk(launch_prime(a, kPrimeWarps, lmax_, sms_, S->sums));
+  chk(launch_prime(a, kPowers1, formula_, lmax_, sms_, S->sums));
+  if (above_word) chk(launch_prime(a, kPowers2, formula_, lmax_, sms_, S->sums));
+  chk(launch_prime(a, kPrimeWarps, formula_, lmax_, sms_, S->sums));
   chk(cudaEventRecord(S->done, S->sums));
   launches_ += above_word ? 4 : 3;
   return err == cudaSuccess ? BBP_OK : BBP_ECUDA;
@@ -243,6 +249,7 @@ bbp_status PrimeRun::run(size_t first, size_t last, cudaStream_t st) {
     v.above = l.lo;
     v.upto = l.hi;
     v.segments = l.segments;
+    v.one_mod_4 = l.one_mod_4;
     v.count = lengths + i;
     chk(launch_sieve(v, sms_, S->sieve));
     chk(cudaEventRecord(S->ready[slot], S->sieve));
@@ -253,7 +260,7 @@ bbp_status PrimeRun::run(size_t first, size_t last, cudaStream_t st) {
     a.taken = lengths + lists_.size() + i;
     const bool sums = l.kernel == kSums1 || l.kernel == kSums2 || l.kernel == kSums8;
     a.e = sums ? e_ : e_ - kPrimeShift + 64;  // the product with H leaves a factor 2^-64
-    chk(launch_prime(a, l.kernel, lmax_, sms_, st));
+    chk(launch_prime(a, l.kernel, formula_, lmax_, sms_, st));
     chk(cudaEventRecord(S->used[slot], st));
     launches_ += 3;
   }

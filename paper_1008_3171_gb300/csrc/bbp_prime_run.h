@@ -28,7 +28,7 @@ class PrimeRun {
  public:
   // The query at position n, W working bits, into `slots` (to which the terms that the
   // prime form does not cover are added by the caller).
-  bbp_status plan(PrimeState* state, int sm_count, uint64_t n, uint32_t W, unsigned long long* slots);
+  bbp_status plan(PrimeState* state, int sm_count, int formula, uint64_t n, uint32_t W, unsigned long long* slots);
   size_t lists() const { return lists_.size(); }
   double share(size_t i) const;  // list i's part of the numbers up to n
   // Base primes and prime powers.
@@ -45,9 +45,10 @@ class PrimeRun {
     uint64_t base, lo, hi;
     uint32_t segments;
     PrimeKernel kernel;
+    uint32_t one_mod_4;  // only primes 1 mod 4 matter
   };
   PrimeState* state_ = nullptr;
-  int sms_ = 0, lmax_ = 0;
+  int sms_ = 0, lmax_ = 0, formula_ = 0;
   uint32_t base_to_ = 0;
   uint64_t e_ = 0, launches_ = 0;
   PrimeArgs args_{};

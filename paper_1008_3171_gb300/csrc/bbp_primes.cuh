@@ -174,7 +174,8 @@ __device__ __forceinline__ void prime_residues(const uint64_t e, const uint64_t 
     int c = 0;
     while (p[t] <= classes[c].above) ++c;
     const PrimeClass& C = classes[c];
-    const uint32_t n0 = lo32(C.num), n1 = hi32(C.num);
+    const uint32_t mod4 = (m0[t] >> 1) & 1u;  // 0: p = 1 mod 4, 1: p = 3
+    const uint32_t n0 = lo32(C.num[mod4]), n1 = hi32(C.num[mod4]);
     uint64_t y;
     if (WIDE) {
       // x num / 2^64 mod p: x < 2 p < 2^47, num < 2^54, so the result is below 2 p (x = 2^(e + 64))
@@ -200,7 +201,7 @@ __device__ __forceinline__ void prime_residues(const uint64_t e, const uint64_t 
     }
     if (y >= p[t]) y -= p[t];
     if (C.den > 1u) y = divide_by_den(y, p[t], C);
-    if ((m0[t] & 2u) && y != 0) y = p[t] - y;  // chi(p) = -1 for p = 3 mod 4
+    if (((C.negative >> mod4) & 1u) && y != 0) y = p[t] - y;
     if (!valid[t]) y = 0;
     x0[t] = lo32(y);
     x1[t] = hi32(y);
@@ -365,72 +366,125 @@ __device__ __forceinline__ uint64_t exponent_mod(int64_t e, uint64_t phi) {
   return static_cast<uint64_t>(r < 0 ? r + static_cast<int64_t>(phi) : r);
 }
 
-// The three sums (0: A, 1: B, 2: C): the term at i is s(i) w^-i / c, c = 2 i + 1, with
-// w = 4, 1024, 32 for a prime; s(i) = (-1)^i for A and B, +, +, -, - for C.
-__device__ __forceinline__ constexpr uint32_t sum_weight_bits(int kind) { return kind == 0 ? 2u : kind == 1 ? 10u : 5u; }
+// The sums mod p, three of each formula: the term at i is s(i) w^-i / c, c = stride i + c0, with
+// w a power of two for a prime p.
+//
+//   kind       w     c        s(i)
+//   0 A      2^2    2 i + 1   (-1)^i
+//   1 B      2^10   2 i + 1   (-1)^i
+//   2 C      2^5    2 i + 1   + + - -
+//   3 D      2^2    4 i + c0  (-1)^i   c0 = p mod 4
+//   4 E      2^4    4 i + c0  +        c0 = 4 - p mod 4
+//   5 F      2^4    2 i + 1   +
+template <int KIND>
+struct SumKind {
+  static constexpr uint32_t kW = KIND == 1 ? 10u : KIND == 2 ? 5u : KIND >= 4 ? 4u : 2u;  // log2 w
+  static constexpr uint32_t kStride = KIND == 3 || KIND == 4 ? 4u : 2u;
+  static constexpr bool kAlternates = KIND == 0 || KIND == 1 || KIND == 3;
+  static constexpr bool kInTwos = KIND == 2;  // the signs + + - -
+  // two terms at once while w^2 c (c - stride) <= 2^31, which keeps every product below m 2^32
+  static constexpr uint32_t kPairTop = KIND == 0 || KIND == 3 ? 11583u : KIND == 2 ? 1447u : KIND >= 4 ? 2896u : 0u;
+
+  // Whether den changes sign after term i (s(i - 1) is not s(i)).
+  __device__ static __forceinline__ bool flips(uint32_t i) { return kAlternates || (kInTwos && (i & 1u) == 0u); }
+  // s(i) of the last term, times the sign that den has collected over [lo, hi): num's sign.
+  __device__ static __forceinline__ bool negative(uint32_t lo, uint32_t hi) {
+    if (kAlternates) return ((hi - lo) ^ (hi - 1u)) & 1u;
+    if (kInTwos) return (((hi + 1u) / 2u - (lo + 1u) / 2u) ^ ((hi - 1u) >> 1)) & 1u;
+    return false;
+  }
+};
+
+// One term, from the last down: num <- c num + den, den <- w c den, with s carried in den's
+// sign (den <- -w c den where s changes), so a step is two products by a word, two
+// reductions and no selection; each reduction leaves the same factor 2^-32 in both.
+template <int KIND>
+__device__ __forceinline__ void sum_step(const Arith1& M, uint32_t i, uint32_t c, uint32_t& N, uint32_t& D) {
+  using K = SumKind<KIND>;
+  N = M.lazy_redc(static_cast<uint64_t>(N) * c + D);
+  const uint64_t t = static_cast<uint64_t>(D) * (c << K::kW);
+  if (K::kInTwos) {
+    const uint32_t r = M.lazy_redc(t);
+    D = (i & 1u) ? r : 2u * M.m - r;
+  } else {
+    D = K::kAlternates ? M.lazy_redc_neg(t) : M.lazy_redc(t);
+  }
+}
+
+// Two terms, i odd at c and i - 1 at c' = c - stride: three products serve both.
+//   signs alternate:  num <- c c' num - (w c - c') den, den <- w^2 c c' den   (d = -den)
+//   + +, then - -:    num <- c c' num + (w c + c') den, den <- -w^2 c c' den
+//   no change:        num <- c c' num + (w c + c') den, den <- w^2 c c' den
+template <int KIND>
+__device__ __forceinline__ void sum_pair(const Arith1& M, uint32_t c, uint32_t& N, uint32_t& d) {
+  using K = SumKind<KIND>;
+  const uint32_t c2 = c - K::kStride, alpha = c * c2;
+  const uint32_t beta = K::kAlternates ? (c << K::kW) - c2 : (c << K::kW) + c2;
+  N = M.lazy_redc(static_cast<uint64_t>(N) * alpha + static_cast<uint64_t>(d) * beta);
+  const uint64_t t = static_cast<uint64_t>(d) * (alpha << (2u * K::kW));
+  d = K::kInTwos ? M.lazy_redc_neg(t) : M.lazy_redc(t);
+}
+
+// Where a lane starts among the pairs: nothing done yet, or its last term done if that
+// is the first of a pair.
+template <int KIND>
+__device__ __forceinline__ void pair_start(const Arith1& M, uint32_t hi, uint32_t c0, uint32_t& N, uint32_t& D) {
+  using K = SumKind<KIND>;
+  N = 0;
+  D = 1;
+  if (hi & 1u) {
+    const uint64_t wc = static_cast<uint64_t>(K::kStride * (hi - 1u) + c0) << K::kW;
+    N = M.lazy_redc(1u);
+    D = K::kAlternates || K::kInTwos ? M.lazy_redc_neg(wc) : M.lazy_redc(wc);
+  }
+}
+
+template <int KIND>
+__device__ __forceinline__ uint32_t pair_sign(const Arith1& M, uint32_t d) {  // den <-> the pairs' d
+  return SumKind<KIND>::kAlternates ? 2u * M.m - d : d;
+}
 
 // Fractions of primes p < 2^31, one a lane: the sum over 0 <= i < n of s(i) w^-i / c as
 // w num / den.  Every lane of the warp must call it.
 //
-// From the last term down: num <- c num + den, den <- w c den, with s carried in den's
-// sign (den <- -w c den where s changes), so a step is two products by a word, two
-// reductions and no selection; each reduction leaves the same factor 2^-32 in both.  The
-// lanes of a warp walk i together from the largest n (c and the constants are uniform, no
-// lane waits for another's loop); until its own n a lane keeps num = den = 0 mod p.  A and C
-// take two terms at once where the constants allow: three products serve two terms.  In
-// multiply-pipe units (low half 1, high half or full product 2) a term costs 10 singly
+// The lanes of a warp walk i together from the largest n, so no lane waits for another's
+// loop (and c is uniform where c0 is 1); until its own n a lane keeps num = den = 0 mod p.
+// In multiply-pipe units (low half 1, high half or full product 2) a term costs 10 singly
 // and 6.3 in pairs.  (One term at a time, every lane with its own loop: the primes up to
 // A / 23 of n = 4e10 took 16.9 ms, now 10.)
 template <int KIND>
-__device__ __forceinline__ void prime_sum(const Arith1& M, uint32_t n, uint32_t& num, uint32_t& den) {
-  constexpr uint32_t kW = sum_weight_bits(KIND);
-  // pairs while w^2 c (c - 2) <= 2^31, which keeps every product below m 2^32
-  constexpr uint32_t kPairTop = KIND == 0 ? 11583u : KIND == 2 ? 1447u : 0u;
+__device__ __forceinline__ void prime_sum(const Arith1& M, uint32_t n, uint32_t c0, uint32_t& num, uint32_t& den) {
+  using K = SumKind<KIND>;
   const uint32_t top = __reduce_max_sync(0xffffffffu, n);
+  const uint32_t first = K::kStride == 2u ? 1u : c0;
   uint32_t N = 0, D = 0;
-  auto step = [&](uint32_t i) {
-    const uint32_t c = 2u * i + 1u;
-    N = M.lazy_redc(static_cast<uint64_t>(N) * c + D);
-    const uint64_t t = static_cast<uint64_t>(D) * (c << kW);
-    D = KIND != 2 || (i & 1u) == 0u ? M.lazy_redc_neg(t) : M.lazy_redc(t);
-  };
   uint32_t i = top;
-  while (i > 0 && (kPairTop == 0 || 2u * i - 1u > kPairTop || (i & 1u))) {
+  while (i > 0 && (K::kPairTop == 0 || K::kStride * i > K::kPairTop || (i & 1u))) {
     if (i == n) {
       N = 0;
       D = 1;
     }
-    step(--i);
+    --i;
+    sum_step<KIND>(M, i, K::kStride * i + first, N, D);
   }
-  if (kPairTop != 0 && i > 0) {
-    // pairs (2h + 1, 2h), c c' = 16 h^2 + 16 h + 3:
-    //   A: num <- c c' num - (4 c - c') den, den <- 16 c c' den   (d = -den)
-    //   C: num <- c c' num + (32 c + c') den, den <- -1024 c c' den
-    // a lane whose n is odd starts with its last term, c = 2 n - 1, done: num = 1, den = -w c
+  if (K::kPairTop != 0 && i > 0) {
     if (n < i) {
       N = 0;
       D = 0;
     }
-    const bool odd = (n & 1u) != 0u;
-    const uint32_t n0 = odd ? M.lazy_redc(1u) : 0u;
-    const uint32_t d0 = odd ? M.lazy_redc_neg(static_cast<uint64_t>(2u * n - 1u) << kW) : 1u;
-    const uint32_t start = n >> 1;
-    uint32_t d = KIND == 0 ? 2u * M.m - D : D;
-    const uint32_t d_start = KIND == 0 ? 2u * M.m - d0 : d0;
+    uint32_t n0, d0;
+    pair_start<KIND>(M, n, first, n0, d0);
+    const uint32_t start = n >> 1, d_start = pair_sign<KIND>(M, d0);
+    uint32_t d = pair_sign<KIND>(M, D);
     const bool late = n <= i;  // starts within the pairs
     for (uint32_t h = i / 2; h > 0; --h) {
       if (late && h == start) {
         N = n0;
         d = d_start;
       }
-      const uint32_t g = h - 1u;
-      const uint32_t alpha = 16u * g * h + 3u;
-      const uint32_t beta = KIND == 0 ? 12u * g + 11u : 132u * g + 97u;
-      N = M.lazy_redc(static_cast<uint64_t>(N) * alpha + static_cast<uint64_t>(d) * beta);
-      const uint64_t t = static_cast<uint64_t>(d) * (alpha << (2u * kW));
-      d = KIND == 0 ? M.lazy_redc(t) : M.lazy_redc_neg(t);
+      sum_pair<KIND>(M, K::kStride * (2u * h - 1u) + first, N, d);
     }
-    D = KIND == 0 ? 2u * M.m - d : d;
+    D = pair_sign<KIND>(M, d);
     if (late && start == 0u) {  // n = 1 (or none): no pair
       N = n0;
       D = d0;
@@ -441,44 +495,35 @@ __device__ __forceinline__ void prime_sum(const Arith1& M, uint32_t n, uint32_t&
   }
   num = M.fix(N);
   den = M.fix(D);
-  // den changed sign at every i (A, B) or every even i (C); the first term's own sign
-  const uint32_t flips = KIND != 2 ? n : (n + 1u) / 2u;
-  const uint32_t first = KIND != 2 ? n - 1u : (n - 1u) >> 1;
-  if (n != 0 && ((flips ^ first) & 1u)) num = M.neg(num);
+  if (n != 0 && K::negative(0, n)) num = M.neg(num);
 }
 
 // The same over lo <= i < hi, relative to the term at lo (w num / den with w^-(i - lo)), lo
 // even, each lane with its own range; the lanes walk them in step.
 template <int KIND>
-__device__ __forceinline__ void range_sum(const Arith1& M, uint32_t lo, uint32_t hi, uint32_t& num, uint32_t& den) {
-  constexpr uint32_t kW = sum_weight_bits(KIND);
-  constexpr uint32_t kPairTop = KIND == 0 ? 11583u : KIND == 2 ? 1447u : 0u;  // as in prime_sum
+__device__ __forceinline__ void range_sum(const Arith1& M, uint32_t lo, uint32_t hi, uint32_t c0, uint32_t& num,
+                                          uint32_t& den) {
+  using K = SumKind<KIND>;
   const uint32_t steps = __reduce_max_sync(0xffffffffu, hi - lo);
-  const bool pairs = kPairTop != 0u && __reduce_max_sync(0xffffffffu, 2u * hi) <= kPairTop;
+  const bool pairs = K::kPairTop != 0u && __reduce_max_sync(0xffffffffu, K::kStride * hi) <= K::kPairTop;
+  const uint32_t first = K::kStride == 2u ? 1u : c0;
   uint32_t N = 0, D = 1;
   if (pairs) {
-    const bool odd = (hi & 1u) != 0u;
-    const uint32_t n0 = odd ? M.lazy_redc(1u) : 0u;
-    const uint32_t d0 = odd ? M.lazy_redc_neg(static_cast<uint64_t>(2u * hi - 1u) << kW) : 1u;
+    uint32_t n0, d0;
+    pair_start<KIND>(M, hi, first, n0, d0);
+    const uint32_t start = hi / 2u, d_start = pair_sign<KIND>(M, d0);
     uint32_t k = (steps + 1u) / 2u;
-    uint32_t h = lo / 2u + k;  // h - 1: the pair (2 h - 2, 2 h - 1)
-    uint32_t alpha = 16u * h * (h - 1u) + 3u, diff = 32u * (h - 1u);
-    uint32_t beta = KIND == 0 ? 12u * h - 1u : 132u * h - 35u;
-    uint32_t d = 1;
-    const uint32_t d_start = KIND == 0 ? 2u * M.m - d0 : d0, start = hi / 2u;
+    uint32_t h = lo / 2u + k;  // the pair (2 h - 2, 2 h - 1)
+    uint32_t c = K::kStride * (2u * h - 1u) + first, d = 1;
     for (; k > 0u; --k, --h) {
       if (h == start) {
         N = n0;
         d = d_start;
       }
-      N = M.lazy_redc(static_cast<uint64_t>(N) * alpha + static_cast<uint64_t>(d) * beta);
-      const uint64_t t = static_cast<uint64_t>(d) * (alpha << (2u * kW));
-      d = KIND == 0 ? M.lazy_redc(t) : M.lazy_redc_neg(t);
-      alpha -= diff;
-      diff -= 32u;
-      beta -= KIND == 0 ? 12u : 132u;
+      sum_pair<KIND>(M, c, N, d);
+      c -= 2u * K::kStride;
     }
-    D = KIND == 0 ? 2u * M.m - d : d;
+    D = pair_sign<KIND>(M, d);
     if (start == lo / 2u) {  // one term, or none
       N = n0;
       D = d0;
@@ -491,15 +536,7 @@ __device__ __forceinline__ void range_sum(const Arith1& M, uint32_t lo, uint32_t
         D = 1;
       }
       --i;
-      const uint32_t c = 2u * i + 1u;
-      N = M.lazy_redc(static_cast<uint64_t>(N) * c + D);
-      const uint64_t t = static_cast<uint64_t>(D) * (c << kW);
-      if (KIND != 2) {
-        D = M.lazy_redc_neg(t);
-      } else {
-        const uint32_t r = M.lazy_redc(t);
-        D = (i & 1u) ? r : 2u * M.m - r;
-      }
+      sum_step<KIND>(M, i, K::kStride * i + first, N, D);
     }
   }
   if (hi <= lo) {
@@ -508,9 +545,7 @@ __device__ __forceinline__ void range_sum(const Arith1& M, uint32_t lo, uint32_t
   }
   num = M.fix(N);
   den = M.fix(D);
-  const uint32_t flips = KIND != 2 ? hi - lo : (hi + 1u) / 2u - (lo + 1u) / 2u;
-  const uint32_t first = KIND != 2 ? hi - 1u : (hi - 1u) >> 1;
-  if (hi > lo && ((flips ^ first) & 1u)) num = M.neg(num);
+  if (hi > lo && K::negative(lo, hi)) num = M.neg(num);
 }
 
 // The sum over 0 <= i < n shared by GROUP neighbouring lanes with the same prime: each takes
@@ -518,13 +553,12 @@ __device__ __forceinline__ void range_sum(const Arith1& M, uint32_t lo, uint32_t
 //   w num / den = w (num den' w^s + num' den) / (den den' w^s).
 // The group's first lane has the result.
 template <int KIND, int GROUP>
-__device__ __forceinline__ void group_sum(const Arith1& M, uint32_t n, uint32_t& num, uint32_t& den) {
-  constexpr uint32_t kW = sum_weight_bits(KIND);
+__device__ __forceinline__ void group_sum(const Arith1& M, uint32_t n, uint32_t c0, uint32_t& num, uint32_t& den) {
   const uint32_t share = ((n + GROUP - 1) / GROUP + 1u) & ~1u;
   uint32_t lo = (threadIdx.x & (GROUP - 1)) * share, hi = min(n, lo + share);
   if (lo >= n) lo = hi = 0;
-  range_sum<KIND>(M, lo, hi, num, den);
-  uint32_t z = M.one(), e = kW * share;  // w^s
+  range_sum<KIND>(M, lo, hi, c0, num, den);
+  uint32_t z = M.one(), e = SumKind<KIND>::kW * share;  // w^s
   const int bits = 32 - __clz(static_cast<int>(__reduce_max_sync(0xffffffffu, e)));
   for (int b = bits - 1; b >= 0; --b) z = M.mul(z, (e >> b) & 1u ? z + z : z);
 #pragma unroll
@@ -537,37 +571,45 @@ __device__ __forceinline__ void group_sum(const Arith1& M, uint32_t n, uint32_t&
   }
 }
 
+// The largest c = s p at most `last` with c = c0 mod stride, 0 if there is none (p odd)
+template <int KIND>
+__device__ __forceinline__ uint64_t last_multiple(uint64_t last, uint64_t p, uint32_t c0) {
+  constexpr uint32_t mask = SumKind<KIND>::kStride - 1u;
+  const uint64_t s = last / p, s0 = (c0 * p) & mask;  // p^-1 = p mod 4
+  return s < s0 ? 0 : (s - ((s - s0) & mask)) * p;
+}
+
 // The same over lo <= i < hi, relative to the term at lo (w num / den with w^-(i - lo)), the
 // terms with c a multiple of p left out; the lanes walk their ranges in step.  WORD: modulo
 // p, with w a word; else modulo a power of p, with h (a residue in Montgomery form) for w.
 template <int KIND, bool WORD>
-__device__ __forceinline__ void prime_share(const Arith1& M, uint32_t lo, uint32_t hi, uint32_t p, uint32_t h,
-                                            uint32_t& num, uint32_t& den) {
-  constexpr uint32_t kW = sum_weight_bits(KIND);
+__device__ __forceinline__ void prime_share(const Arith1& M, uint32_t lo, uint32_t hi, uint32_t c0, uint32_t p,
+                                            uint32_t h, uint32_t& num, uint32_t& den) {
+  using K = SumKind<KIND>;
   const uint32_t steps = __reduce_max_sync(0xffffffffu, hi > lo ? hi - lo : 0u);
+  const uint32_t first = K::kStride == 2u ? 1u : c0;
   uint32_t i = lo + steps, N = 0, D = 1;
-  uint32_t skip = hi > lo ? (2u * hi - 1u) / p : 0u;  // the last multiple of p: c = skip p, skip odd
-  skip = skip == 0u ? 0u : ((skip - 1u) | 1u) * p;
+  uint32_t skip = hi > lo ? static_cast<uint32_t>(last_multiple<KIND>(K::kStride * (hi - 1u) + first, p, first)) : 0u;
   for (uint32_t k = steps; k > 0; --k) {
     if (i == hi) {
       N = 0;
       D = 1;
     }
     --i;
-    uint32_t c = 2u * i + 1u, add = D;
+    uint32_t c = K::kStride * i + first, add = D;
     if (c == skip) {
       c = 1u;
       add = 0u;
-      skip = skip > p ? skip - 2u * p : 0u;
+      skip = skip > K::kStride * p ? skip - K::kStride * p : 0u;
     }
     N = M.lazy_redc(static_cast<uint64_t>(N) * c + add);
-    const uint64_t t = WORD ? static_cast<uint64_t>(D) * (c << kW)
+    const uint64_t t = WORD ? static_cast<uint64_t>(D) * (c << K::kW)
                             : static_cast<uint64_t>(M.lazy_redc(static_cast<uint64_t>(D) * c)) * h;
-    if (KIND != 2) {
-      D = M.lazy_redc_neg(t);
-    } else {
+    if (K::kInTwos) {
       const uint32_t r = M.lazy_redc(t);
       D = (i & 1u) ? r : 2u * M.m - r;
+    } else {
+      D = K::kAlternates ? M.lazy_redc_neg(t) : M.lazy_redc(t);
     }
   }
   if (hi <= lo) {
@@ -576,40 +618,35 @@ __device__ __forceinline__ void prime_share(const Arith1& M, uint32_t lo, uint32
   }
   num = M.fix(N);
   den = M.fix(D);
-  const uint32_t flips = KIND != 2 ? hi - lo : (hi + 1u) / 2u - (lo + 1u) / 2u;
-  const uint32_t first = KIND != 2 ? hi - 1u : (hi - 1u) >> 1;
-  if (hi > lo && ((flips ^ first) & 1u)) num = M.neg(num);
+  if (hi > lo && K::negative(lo, hi)) num = M.neg(num);
 }
 
 // The same modulo q < 2^46, one term at a time: WORD: q = p and h = w; else q = p^a and
-// h = 2^(bits q) mod q in Montgomery form.  The sign of term i changes with bit `flip` of i.
-template <bool WORD, bool SKIP>
-__device__ __forceinline__ void power_sum(const Arith2& M, uint64_t i0, uint64_t i1, uint32_t flip, uint64_t p,
+// h = 2^(kW q) mod q in Montgomery form.
+template <int KIND, bool WORD, bool SKIP>
+__device__ __forceinline__ void power_sum(const Arith2& M, uint64_t i0, uint64_t i1, uint32_t c0, uint64_t p,
                                           uint64_t h, uint64_t& num, uint64_t& den) {
+  using K = SumKind<KIND>;
   num = 0;
   den = 1;
   if (i0 >= i1) return;
-  uint64_t skip = 0;  // the largest odd multiple of p not above the last c
-  if (SKIP) {
-    skip = (2 * i1 - 1) / p;
-    skip = skip == 0 ? 0 : ((skip - 1) | 1u) * p;
-  }
-  uint32_t c = static_cast<uint32_t>(2 * i1 - 1);
-  const uint32_t c0 = static_cast<uint32_t>(2 * i0 + 1);
-  const uint32_t bit = 2 * flip;  // bit `flip` of i is bit 2 flip of c
-  for (;;) {
+  const uint32_t first = K::kStride == 2u ? 1u : c0;
+  uint64_t skip = SKIP ? last_multiple<KIND>(K::kStride * (i1 - 1) + first, p, first) : 0;
+  uint32_t i = static_cast<uint32_t>(i1);
+  do {
+    --i;
+    const uint32_t c = K::kStride * i + first;
     uint32_t k = c;
     if (SKIP && c == static_cast<uint32_t>(skip)) {
-      skip = skip > p ? skip - 2 * p : 0;
+      skip = skip > K::kStride * p ? skip - K::kStride * p : 0;
       k = 1u;
       num = M.mul_word(num, 1u, 0);
     } else {
-      num = M.mul_word(num, c, (c & bit) ? M.neg(den) : den);
+      const bool minus = K::kAlternates ? (i & 1u) : K::kInTwos ? (i & 2u) : false;
+      num = M.mul_word(num, c, minus ? M.neg(den) : den);
     }
     den = WORD ? M.mul_word(den, k * static_cast<uint32_t>(h), 0) : M.mul(M.mul_word(den, k, 0), h);
-    if (c == c0) break;
-    c -= 2;
-  }
+  } while (i > i0);
 }
 
 template <class A, int LMAX>
@@ -623,13 +660,23 @@ __device__ __forceinline__ void fold_one(const A& M, typename A::T x, uint32_t (
   }
 }
 
-// GROUP lanes per prime: num / den of the three sums, one ladder for the inverse of their
-// denominators and the power of 2.
-//   H = 16 (num_A / den_A - 4 num_B / den_B - num_C / den_C)
+// Terms with c = stride i + c0 up to `top`
+template <int KIND, typename T>
+__device__ __forceinline__ T summands(T top, uint32_t c0) {
+  if (SumKind<KIND>::kStride == 2u) return (top + 1u) / 2u;
+  return top >= c0 ? (top - c0) / 4u + 1u : 0u;
+}
+
+// GROUP lanes per prime: num / den of the formula's three sums, one ladder for the inverse
+// of their denominators and the power of 2.
+//   Eq. 2: H = 16 (num_A / den_A - 4 num_B / den_B - num_C / den_C), times chi(p)
+//   Eq. 1: H = 8 (2 num_D / den_D - num_E / den_E - num_F / den_F) for p = 1 mod 4,
+//          H = -8 (num_D / den_D + 4 num_E / den_E + num_F / den_F) for p = 3 mod 4
 // One lane per prime walks up to 8000 terms in a row where the sums are long; eight lanes
 // bring n = 1e9's longest chain from 600 us (with the SM full) to a quarter.
-template <class A, int GROUP, int LMAX>
+template <class A, int FORMULA, int GROUP, int LMAX>
 __global__ void __launch_bounds__(kHeadThreads) prime_sum_kernel(const __grid_constant__ PrimeArgs G) {
+  constexpr int K0 = FORMULA == 0 ? 0 : 3;
   const uint32_t count = min(*G.count, G.cap);
   uint32_t acc[LMAX];
 #pragma unroll
@@ -640,31 +687,40 @@ __global__ void __launch_bounds__(kHeadThreads) prime_sum_kernel(const __grid_co
     const uint32_t i = at + lane / GROUP;  // a lane past the end repeats the last prime and adds nothing
     const uint64_t p = G.base + G.list[min(i, count - 1)];
     const A M(p);
-    const uint32_t iA = (small_quotient(G.A, p) + 1) / 2, iB = (small_quotient(G.B, p) + 1) / 2,
-                   iC = (small_quotient(G.C, p) + 1) / 2;
-    T nA, dA, nB, dB, nC, dC;
+    const uint32_t r = lo32(p) & 3u;
+    const uint32_t i0 = summands<K0>(small_quotient(G.A, p), r), i1 = summands<K0 + 1>(small_quotient(G.B, p), 4u - r),
+                   i2 = summands<K0 + 2>(small_quotient(G.C, p), 1u);
+    T n0, d0, n1, d1, n2, d2;
     if constexpr (GROUP > 1) {
-      group_sum<0, GROUP>(M, iA, nA, dA);
-      group_sum<1, GROUP>(M, iB, nB, dB);
-      group_sum<2, GROUP>(M, iC, nC, dC);
+      group_sum<K0, GROUP>(M, i0, r, n0, d0);
+      group_sum<K0 + 1, GROUP>(M, i1, 4u - r, n1, d1);
+      group_sum<K0 + 2, GROUP>(M, i2, 1u, n2, d2);
     } else if constexpr (sizeof(T) == 4) {
-      prime_sum<0>(M, iA, nA, dA);
-      prime_sum<1>(M, iB, nB, dB);
-      prime_sum<2>(M, iC, nC, dC);
+      prime_sum<K0>(M, i0, r, n0, d0);
+      prime_sum<K0 + 1>(M, i1, 4u - r, n1, d1);
+      prime_sum<K0 + 2>(M, i2, 1u, n2, d2);
     } else {
-      power_sum<true, false>(M, 0, iA, 1, p, 4, nA, dA);
-      power_sum<true, false>(M, 0, iB, 1, p, 1024, nB, dB);
-      power_sum<true, false>(M, 0, iC, 2, p, 32, nC, dC);
+      power_sum<K0, true, false>(M, 0, i0, r, p, 1u << SumKind<K0>::kW, n0, d0);
+      power_sum<K0 + 1, true, false>(M, 0, i1, 4u - r, p, 1u << SumKind<K0 + 1>::kW, n1, d1);
+      power_sum<K0 + 2, true, false>(M, 0, i2, 1u, p, 1u << SumKind<K0 + 2>::kW, n2, d2);
     }
-    const T bc = M.mul(dB, dC);
-    const T b4 = M.add(nB, nB);
-    T num = M.mul(nA, bc);
-    num = M.add(num, M.neg(M.mul(M.mul(M.add(b4, b4), dA), dC)));
-    num = M.add(num, M.neg(M.mul(M.mul(nC, dA), dB)));
-    const uint64_t e = G.e + 4 - small_quotient(G.e + 4, p - 1) * (p - 1);
-    const T inv = inverse_times_power<A>(M, M.mul(dA, bc), p - 1, e);
+    const T d12 = M.mul(d1, d2);
+    T t0 = M.mul(n0, d12), t1 = M.mul(M.mul(n1, d0), d2);
+    const T t2 = M.mul(M.mul(n2, d0), d1);
+    if (FORMULA == 0 || r == 3u) {  // 4 times the second
+      t1 = M.add(t1, t1);
+      t1 = M.add(t1, t1);
+    } else {
+      t0 = M.add(t0, t0);
+    }
+    const T rest = M.add(t1, t2);
+    // Eq. 2: chi(p) (t0 - rest); Eq. 1: t0 - rest or -(t0 + rest)
+    T num = FORMULA == 0 || r == 1u ? M.add(t0, M.neg(rest)) : M.add(t0, rest);
+    if (r == 3u) num = M.neg(num);
+    const uint64_t e0 = G.e + (FORMULA == 0 ? 4 : 3);
+    const uint64_t e = e0 - small_quotient(e0, p - 1) * (p - 1);
+    const T inv = inverse_times_power<A>(M, M.mul(d0, d12), p - 1, e);
     T x = M.plain(M.mul(num, inv));
-    if (p & 2u) x = M.neg(x);
     if (i >= count || (lane & (GROUP - 1)) != 0u) x = 0;
     fold_one<A, LMAX>(M, x, acc);
   }
@@ -689,44 +745,53 @@ __device__ typename A::T geometric(const A& M, typename A::T r, uint64_t n) {
 
 // What one lane adds of sum KIND to the part of q = p^a: its share of the summands
 // [lo, hi), `times` over, as a fraction added to num / den (all in Montgomery form).
+// Summand i carries s(i) 2^(start - ratio q i) / c.
 template <class A, int KIND, bool PRIME>
 __device__ __forceinline__ void add_share(const A& M, uint64_t p, uint64_t q, uint64_t phi, int64_t e, uint64_t lo,
                                           uint64_t hi, uint64_t period, uint64_t times, uint32_t lane,
                                           typename A::T& num, typename A::T& den) {
   using T = typename A::T;
+  using K = SumKind<KIND>;
   const uint64_t share = (hi - lo + 31) / 32;
   const uint64_t i0 = lo + min(hi - lo, lane * share), i1 = min(hi, i0 + share);
   if (times == 0 || hi <= lo) return;  // the same for every lane
-  constexpr int64_t kRatio = sum_weight_bits(KIND);  // summand i carries 2^(-ratio q i)
+  constexpr int64_t kRatio = K::kW;
   const int64_t sq = static_cast<int64_t>(q);
+  const uint32_t r4 = lo32(q) & 3u, c0 = KIND == 3 ? r4 : KIND == 4 ? 4u - r4 : 1u;
   T n_s, d_s;
   const T h = PRIME ? 0 : power_of_two<A>(M, exponent_mod(kRatio * sq, phi));
   if constexpr (sizeof(T) == 4)
-    prime_share<KIND, PRIME>(M, static_cast<uint32_t>(i0), static_cast<uint32_t>(i1), lo32(p), h, n_s, d_s);
+    prime_share<KIND, PRIME>(M, static_cast<uint32_t>(i0), static_cast<uint32_t>(i1), c0, lo32(p), h, n_s, d_s);
   else
-    power_sum<false, true>(M, i0, i1, KIND == 2 ? 2u : 1u, p, h, n_s, d_s);
-  // the first summand's power of 2, with the h that multiplies the fraction
-  const int64_t start = KIND == 0 ? e + 3 - sq : KIND == 1 ? e + 1 - 5 * sq : e - 1 - 5 * (sq - 1) / 2;
+    power_sum<KIND, false, true>(M, i0, i1, c0, p, h, n_s, d_s);
+  int64_t start = 0;
+  bool minus = true;
+  if (KIND == 0) start = e + 3 - sq, minus = (q & 2u) != 0;
+  if (KIND == 1) start = e + 1 - 5 * sq, minus = (q & 2u) == 0;
+  if (KIND == 2) start = e - 1 - 5 * (sq - 1) / 2, minus = (q & 4u) == 0;
+  if (KIND == 3) start = e + 2 - (sq * c0 - 1) / 2, minus = ((q * c0) & 7u) != 1u;
+  if (KIND == 4) start = e + 2 - sq * c0;
+  if (KIND == 5) start = e + 1 - 2 * sq;
+  // with the h that multiplies the fraction
   T k = power_of_two<A>(M, exponent_mod(start + kRatio * sq * (1 - static_cast<int64_t>(i0)), phi));
   if (times > 1) {
     T r = power_of_two<A>(M, exponent_mod(-kRatio * sq * static_cast<int64_t>(period), phi));
-    if (KIND != 2) r = M.neg(r);  // the period is odd for A and B
+    if (K::kAlternates) r = M.neg(r);  // the period is odd
     k = M.mul(k, geometric<A>(M, r, times));
   }
-  const bool minus = KIND == 0 ? (q & 2u) != 0 : KIND == 1 ? (q & 2u) == 0 : (q & 4u) == 0;
   k = M.mul(k, n_s);
   num = M.add(M.mul(num, d_s), M.mul(minus ? M.neg(k) : k, den));
   den = M.mul(den, d_s);
 }
 
 // Prime power of work item `unit`, 0 if there is none: for PRIME the primes in turn; else
-// p^2 of every prime, then p^3 and p^4 of the first 2560 (p up to 2^14.5 > A^(1/3)), then
+// p^2 of every prime, then p^3 and p^4 of the first 3200 (p up to 29,000 > A^(1/3)), then
 // p^5 ... p^28 of the first 128 (3^28 > A).
 template <bool PRIME>
 __device__ __forceinline__ uint64_t prime_power_of(const PrimeArgs& G, uint32_t unit, uint32_t count, uint64_t* p) {
   uint32_t i = unit, a = 2;
   if (!PRIME && unit >= count) {
-    const uint32_t first = min(count, 2560u), second = min(count, 128u);
+    const uint32_t first = min(count, 3200u), second = min(count, 128u);
     i -= count;
     if (i < 2 * first) {
       a = 3 + i / first;
@@ -749,16 +814,16 @@ __device__ __forceinline__ uint64_t prime_power_of(const PrimeArgs& G, uint32_t 
 
 // One warp per prime power q = p^a: PRIME: a = 1; else a >= 2 and q below (Arith1) or from
 // (Arith2) 2^31 on.  The summands of each sum repeat with a constant
-// ratio after `period` odd c (c^-1 mod q after q of them, the signs after 1 or 4 times
-// that), so at most `period` of them are added up, times a geometric sum: the lanes
+// ratio after `period` of them (c^-1 mod q after q, the signs after 1 or 4 times that), so at most `period` of them are added up, times a geometric sum: the lanes
 // share them evenly, each lane's part being its own fraction over q.
-template <class A, bool PRIME, int LMAX>
+template <class A, int FORMULA, bool PRIME, int LMAX>
 __global__ void __launch_bounds__(kHeadThreads) prime_power_kernel(const __grid_constant__ PrimeArgs G) {
   const uint32_t lane = threadIdx.x & 31u;
   const uint32_t warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   const uint32_t nwarps = (gridDim.x * blockDim.x) >> 5;
   const uint32_t count = min(*G.count, G.cap);
-  const uint32_t units = PRIME ? count : count + 2 * min(count, 2560u) + 24 * min(count, 128u);
+  constexpr int K0 = FORMULA == 0 ? 0 : 3;
+  const uint32_t units = PRIME ? count : count + 2 * min(count, 3200u) + 24 * min(count, 128u);
   using T = typename A::T;
   uint32_t acc[LMAX];
 #pragma unroll
@@ -774,8 +839,11 @@ __global__ void __launch_bounds__(kHeadThreads) prime_power_kernel(const __grid_
     uint64_t whole[3], rest[3], period[3];
 #pragma unroll
     for (int s = 0; s < 3; ++s) {
-      const uint64_t n = (limit[s] / q + 1) / 2;  // odd c up to limit / q
-      period[s] = s == 2 ? 4 * q : q;
+      const uint64_t top = limit[s] / q;
+      const uint32_t r4 = lo32(q) & 3u;
+      const uint64_t n = FORMULA == 0 || s == 2 ? summands<0>(top, 1u)
+                                                : s == 0 ? summands<3>(top, r4) : summands<4>(top, 4u - r4);
+      period[s] = FORMULA == 0 && s == 2 ? 4 * q : q;
       whole[s] = n / period[s];
       rest[s] = n % period[s];
     }
@@ -784,9 +852,9 @@ __global__ void __launch_bounds__(kHeadThreads) prime_power_kernel(const __grid_
       // pass 0: the first `rest` summands, whole + 1 times; pass 1: the others, whole times
       T num = 0, den = M.one();
       const bool f = pass == 0;
-      add_share<A, 0, PRIME>(M, p, q, phi, e, f ? 0 : rest[0], f ? rest[0] : period[0], period[0], whole[0] + f, lane, num, den);
-      add_share<A, 1, PRIME>(M, p, q, phi, e, f ? 0 : rest[1], f ? rest[1] : period[1], period[1], whole[1] + f, lane, num, den);
-      add_share<A, 2, PRIME>(M, p, q, phi, e, f ? 0 : rest[2], f ? rest[2] : period[2], period[2], whole[2] + f, lane, num, den);
+      add_share<A, K0 + 0, PRIME>(M, p, q, phi, e, f ? 0 : rest[0], f ? rest[0] : period[0], period[0], whole[0] + f, lane, num, den);
+      add_share<A, K0 + 1, PRIME>(M, p, q, phi, e, f ? 0 : rest[1], f ? rest[1] : period[1], period[1], whole[1] + f, lane, num, den);
+      add_share<A, K0 + 2, PRIME>(M, p, q, phi, e, f ? 0 : rest[2], f ? rest[2] : period[2], period[2], whole[2] + f, lane, num, den);
       const T x = M.plain(M.mul(num, inverse_times_power<A>(M, den, phi, 0)));  // every lane: warp-wide
       fold_one<A, LMAX>(M, x, acc);
     }

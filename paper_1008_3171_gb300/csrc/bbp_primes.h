@@ -1,14 +1,16 @@
-// The prime form of a whole query's head sum (Bellard's formula, Eq. 2), host side:
-// limits, classes and launch arguments.  Pure C++, no CUDA calls.
+// The prime form of a whole query's head sum, host side: limits, classes and launch
+// arguments.  Pure C++, no CUDA calls.
 //
 // Every head term is 2^e / m mod 1 with m odd.  Splitting 1/m into partial fractions
 // over the prime powers q = p^a that divide m exactly,
 //
 //   1/m = sum_q ((m/q)^-1 mod q) / q   (mod 1),
 //
-// and collecting by q turns the sum over about 0.7 n terms into a sum over the prime
-// powers up to n, about n / ln n of them: one modular exponentiation 2^d mod p per
-// prime serves every term whose modulus p divides.  In terms of odd m,
+// and collecting by q turns the sum over all terms into a sum over the prime powers up to
+// the largest modulus: one modular exponentiation 2^d mod p per prime serves every term
+// whose modulus p divides.
+//
+// Bellard's formula (Eq. 2), in terms of odd m:
 //
 //   series 10k+1, 10k+3, 10k+5, 10k+7, 10k+9 together
 //       =  8 sum_m chi(m) 2^(d-m) / m  -  2 sum_m chi(m) 2^(d-5m) / m      (A and B)
@@ -23,8 +25,18 @@
 //   chi(p) 2^d H / p,   H = 4 sum_(c <= A/p) chi(c) 4^-i / c - 1/16 sum_(c <= B/p) chi(c) 1024^-i / c
 //                           - 1/2 sum_(c <= C/p) psi(c) 32^-i / c    (mod p),  c = 2i + 1 odd,
 //
-// where A, B, C are the largest m of the three sums.  H is one rational number for all
-// primes with the same three limits.
+// where A, B, C are the largest m of the three sums.  The BBP formula (Eq. 1):
+//
+//   series 8k+1, 8k+5:  sum over m = 1 mod 4 of (2/m) 2^(d+2-(m-1)/2) / m   (up to A)
+//   series 4k+3:      - sum over m = 3 mod 4 of 2^(d+2-m) / m               (up to B)
+//   series 2k+1:      - sum over odd m of 2^(d+1-2m) / m                    (up to C)
+//
+// and with (2/p) 2^((p-1)/2) = 1 mod p, p's part is 2^d H / p with
+//
+//   H = 4 sum_(c = p mod 4) (2/c) 2^-((c-1)/2) / c - 4 sum_(c = -p mod 4) 2^-c / c - 2 sum_c 4^-c / c.
+//
+// H is one rational number for all primes with the same three limits (and, for Eq. 1, the
+// same residue mod 4).
 #pragma once
 
 #include <cstdint>
@@ -33,33 +45,34 @@
 namespace bbp {
 
 // Largest moduli of the three sums: every term of a modulus up to these is a head
-// term.  The (at most one) head term above `A` and all tail terms are left to the
+// term.  Eq. 2's (at most one) head term above `A` and all tail terms are left to the
 // term-by-term kernels.
 struct PrimeLimits {
+  int formula = 0;
   uint64_t A = 0, B = 0, C = 0;
 };
-PrimeLimits prime_limits(uint64_t d);
-// First k of series j (formula 0) that the prime form does not cover.
-uint64_t prime_first_k(const PrimeLimits& lim, uint32_t j);
+PrimeLimits prime_limits(int formula, uint64_t d);
+// First k of series j that the prime form does not cover.
+uint64_t prime_first_k(const PrimeLimits& lim, uint32_t j, uint64_t d);
 
 // Primes up to here take the half-reduced ladder: with x <= p + 2^35, x^2 / 2^32 + p stays
 // below 2^48.
 constexpr uint64_t kPrimeHalfMax = 1'020'000'000'000;
 
-// Primes with the same H = num / (den 2^kPrimeShift): those above `above`, up to the
+// Primes with the same +-H = num / (den 2^kPrimeShift), by p mod 4: those above `above`, up to the
 // previous class's `above`.
 constexpr int kPrimeShift = 24;   // every denominator of H up to kPrimeMaxC divides den 2^24
 constexpr uint32_t kPrimeMaxC = 21;  // classes reach down to A / (kPrimeMaxC + 2)
-constexpr int kMaxPrimeClasses = 20;
+constexpr int kMaxPrimeClasses = 24;
 struct PrimeClass {
   uint64_t above;
-  uint64_t num;      // H den 2^24 < 2^54
+  uint64_t num[2];   // |H| den 2^24 < 2^54 for p = 1 and 3 mod 4
   uint64_t den_inv;  // den^-1 mod 2^64
   uint32_t den;      // lcm of the odd numbers up to A / p: 1, 3, 15, ... < 2^24
   uint32_t neg_inv;  // -den^-1 mod 2^32
   uint32_t r2, r3;   // 2^64 mod den, 2^96 mod den
   uint32_t lambda;   // exponent of the group of units mod den, minus 1
-  uint32_t pad;
+  uint32_t negative; // bit 0, 1: the part of p = 1, 3 mod 4 is negative
 };
 // Classes in descending order of `above`; the last one's `above` is A / (kPrimeMaxC + 2).
 std::vector<PrimeClass> prime_classes(const PrimeLimits& lim);

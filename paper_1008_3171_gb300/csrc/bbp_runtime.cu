@@ -399,10 +399,10 @@ bbp_status enqueue_bits(bbp_plan p, int f, uint64_t n, uint32_t P, uint32_t W, u
   float prime_ms = 0;
   p->stats = bbp_stats{};
   if (form != kTerms && !d_limbs && prime_form_serves(f, n, P, W, bound) && prime_workspace(&p->primes, n, kPrimeListMax, s)) {
-    const PrimeLimits lim = prime_limits(n - 1);
+    const PrimeLimits lim = prime_limits(f, n - 1);
     std::vector<TermRange> rest;  // tails, and a head term past the limits
     for (uint32_t j = 0; j < F.count; ++j) {
-      const bbp_status rs = plan_query(p, f, n, W, static_cast<int>(j), prime_first_k(lim, j), UINT64_MAX, rest, nullptr);
+      const bbp_status rs = plan_query(p, f, n, W, static_cast<int>(j), prime_first_k(lim, j, n - 1), UINT64_MAX, rest, nullptr);
       if (rs != BBP_OK) return rs;
     }
     if (p->profile) BBP_CUDA(cudaEventRecord(p->ev2, s));
@@ -410,7 +410,7 @@ bbp_status enqueue_bits(bbp_plan p, int f, uint64_t n, uint32_t P, uint32_t W, u
     const bbp_status ls = launch_ranges(p, f, n, W, rest, p->d_slots, s);
     if (ls != BBP_OK) return ls;
     PrimeRun run;
-    bbp_status ps = run.plan(p->primes, p->sm_count, n, W, p->d_slots);
+    bbp_status ps = run.plan(p->primes, p->sm_count, f, n, W, p->d_slots);
     if (ps == BBP_OK) ps = run.begin(s);
     if (ps == BBP_OK) ps = run.run(0, run.lists(), s);
     if (ps == BBP_OK) ps = run.finish(P, bound, d_out, d_valid, redo, s);
@@ -434,7 +434,7 @@ bbp_status enqueue_bits(bbp_plan p, int f, uint64_t n, uint32_t P, uint32_t W, u
       p->stats.terms += r.count;
       if (!r.tail) p->stats.head_terms += r.count;
     }
-    p->stats.imad_model = prime_form_imad(prime_limits(n - 1), L);
+    p->stats.imad_model = prime_form_imad(prime_limits(f, n - 1), L);
     p->stats.head_launches = prime_launches;
     p->stats.kernel_launches = prime_launches;
     p->stats.head_ms = prime_ms;
@@ -448,7 +448,7 @@ bbp_status enqueue_bits(bbp_plan p, int f, uint64_t n, uint32_t P, uint32_t W, u
   p->stats.kernel_launches += 2 + prime_launches;
   p->stats.head_launches += prime_launches;
   p->stats.head_ms += prime_ms;
-  if (gate) p->stats.imad_model = prime_form_imad(prime_limits(n - 1), L);
+  if (gate) p->stats.imad_model = prime_form_imad(prime_limits(f, n - 1), L);
   return BBP_OK;
 }
 

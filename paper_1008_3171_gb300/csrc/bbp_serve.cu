@@ -229,10 +229,10 @@ bbp_status plan_query_work(bbp_plan p, uint64_t n, uint32_t P, Query* q, bool by
   if (tiles > kMaxQueueTiles) return BBP_ERANGE;  // carry-save limbs could pass 2^64
   q->prime = by_primes && prime_form_serves(BBP_BELLARD, n, P, W, q->bound);
   if (q->prime) {
-    const PrimeLimits lim = prime_limits(n - 1);
+    const PrimeLimits lim = prime_limits(BBP_BELLARD, n - 1);
     ranges.clear();
     for (uint32_t j = 0; j < F.count; ++j)
-      if (plan_series(F, j, n, W, static_cast<uint32_t>(lmax), prime_first_k(lim, j), UINT64_MAX, ranges,
+      if (plan_series(F, j, n, W, static_cast<uint32_t>(lmax), prime_first_k(lim, j, n - 1), UINT64_MAX, ranges,
                       p->wide_min_bits) != 0)
         return BBP_EINVAL;
   }
@@ -454,7 +454,7 @@ void take_primes(ServeEngine* E, std::vector<Query*>& batch, uint64_t budget, st
       if (free_lane < 0 || (is_long && held >= kServeLanes - 1)) continue;
       q->run.reset(new (std::nothrow) PrimeRun());
       const uint64_t slot = static_cast<uint64_t>(q->slot);
-      if (!q->run || q->run->plan(E->lane[free_lane], E->plan->sm_count, q->n, q->W,
+      if (!q->run || q->run->plan(E->lane[free_lane], E->plan->sm_count, BBP_BELLARD, q->n, q->W,
                                   E->d_accum + slot * kMaxLimbs) != BBP_OK) {
         q->run.reset();
         if (plan_query_work(E->plan, q->n, q->P, q, false) != BBP_OK) q->prime = false;  // by its terms instead

@@ -159,17 +159,19 @@ __device__ __forceinline__ uint32_t prime_bits(uint64_t first, uint32_t w, uint6
 }
 
 // Appends the segment's primes, less `origin`, to the list in ascending order; one atomic
-// per segment.  The bits of a word replace its entries for the second pass.
+// per segment: those in the bits `keep` of every 32 entries.  The bits of a word replace its
+// entries for the second pass.
 template <int STEP>
 __device__ void emit_segment(uint64_t first, uint32_t entries, uint64_t above, uint64_t upto, uint8_t* seg,
-                             const uint32_t* tiny, uint64_t origin, uint32_t* list, uint32_t* count, uint32_t cap) {
+                             const uint32_t* tiny, uint32_t keep, uint64_t origin, uint32_t* list, uint32_t* count,
+                             uint32_t cap) {
   __shared__ uint32_t start[kSieveThreads / 32 + 1];
   const uint32_t lane = threadIdx.x & 31u, wid = threadIdx.x >> 5, nwarps = blockDim.x >> 5, words = entries / 32;
   const uint32_t share = (words + nwarps - 1) / nwarps;
   const uint32_t w0 = wid * share, w1 = min(words, w0 + share);
   uint32_t mine = 0;
   for (uint32_t w = w0 + lane; w < w1; w += 32) {
-    const uint32_t v = prime_bits<STEP>(first, w, above, upto, seg, tiny);
+    const uint32_t v = prime_bits<STEP>(first, w, above, upto, seg, tiny) & keep;
     reinterpret_cast<uint32_t*>(seg)[8 * w] = v;
     mine += __popc(v);
   }
@@ -229,7 +231,9 @@ __global__ void __launch_bounds__(kSieveThreads, 4) sieve_kernel(const SieveArgs
   const uint64_t first = a.base + 30ull * skipped + cls;
   if (first > a.upto) return;
   sieve_segment<30>(first, skipped, cls, a.entries, a.upto, a.primes, *a.nprimes, seg, tiny);
-  emit_segment<30>(first, a.entries, a.above, a.upto, seg, tiny, a.base, a.list, a.count, a.cap);
+  // 30 i + first mod 4 alternates
+  const uint32_t keep = a.one_mod_4 == 0u ? ~0u : (first & 3u) == 1u ? 0x55555555u : 0xaaaaaaaau;
+  emit_segment<30>(first, a.entries, a.above, a.upto, seg, tiny, keep, a.base, a.list, a.count, a.cap);
 }
 
 // The base primes, by one CTA: primes below 17 are known, those up to 256 come from a
@@ -253,7 +257,7 @@ __global__ void __launch_bounds__(kSieveThreads) base_primes_kernel(uint32_t upt
     const uint64_t last = min(static_cast<uint64_t>(reach), base + 2 * static_cast<uint64_t>(entries) - 1);
     const uint32_t n = *reinterpret_cast<volatile uint32_t*>(count);
     sieve_segment<2>(base + 1, 0, 0, entries, last, sieve + kSieveTinyPrimes, n - kSieveTinyPrimes, seg, tiny);
-    emit_segment<2>(base + 1, entries, known, last, seg, tiny, 0, primes, count, ~0u);
+    emit_segment<2>(base + 1, entries, known, last, seg, tiny, ~0u, 0, primes, count, ~0u);
     const uint32_t m = *reinterpret_cast<volatile uint32_t*>(count);
     for (uint32_t i = n + tid; i < m; i += blockDim.x) {
       const uint32_t p = primes[i];

@@ -28,6 +28,7 @@ struct SievePrime {
 struct SieveArgs {
   uint64_t base, above, upto;
   uint32_t segments, entries;
+  uint32_t one_mod_4;  // 1: only the primes 1 mod 4
   SievePrime* primes;
   const uint32_t* nprimes;
   uint32_t* list;

@@ -27,14 +27,14 @@ def plans(bbp):
         p.close()
 
 
-def by_terms(bbp, plan, n, P):
+def by_terms(bbp, plan, n, P, formula=0):
     L = plan.working_bits(P) // 32
     slots = torch.zeros(L, dtype=torch.int64, device="cuda")
     out = torch.zeros((P + 7) // 8, dtype=torch.uint8, device="cuda")
     valid = torch.zeros(1, dtype=torch.int32, device="cuda")
     torch.cuda.synchronize()
-    bbp.bbp_accumulate_async(plan.handle, 0, n, P, 0, 1, slots.data_ptr())
-    bbp.bbp_finalize_async(plan.handle, 0, n, P, slots.data_ptr(), out.data_ptr(), valid.data_ptr())
+    bbp.bbp_accumulate_async(plan.handle, formula, n, P, 0, 1, slots.data_ptr())
+    bbp.bbp_finalize_async(plan.handle, formula, n, P, slots.data_ptr(), out.data_ptr(), valid.data_ptr())
     torch.cuda.synchronize()
     return int.from_bytes(bytes(out.cpu().numpy()), "big") >> (8 * len(out) - P), int(valid[0])
 
@@ -56,6 +56,14 @@ def by_async(bbp, plan, n, P):
                                  (2**31 - 1, 64), (2**31 + 2, 256), (23 * 2**29 + 7, 128), (23 * 2**31 + 11, 256)])
 def test_equals_the_terms(bbp, plans, n, P):
     assert plans[64].bits(n, P) == by_terms(bbp, plans[64], n, P)
+
+
+# the BBP formula: residues of n - 1 mod 4, moduli up to 2 n past 2^29 and 2^31, sums in two words
+@pytest.mark.parametrize("n,P", [(16 * 10**6, 64), (16 * 10**6 + 1, 256), (16 * 10**6 + 2, 1000), (16 * 10**6 + 3, 32),
+                                 (2**28 - 1, 100), (2**28 + 2, 448), (2**30 - 2, 64), (2**30 + 1, 704),
+                                 (23 * 2**30 + 5, 128)])
+def test_bbp_formula_equals_the_terms(bbp, plans, n, P):
+    assert plans[64].bits(n, P, 1) == by_terms(bbp, plans[64], n, P, 1)
 
 
 def test_check_sends_uncertain_positions_to_the_terms(bbp, plans):
@@ -100,6 +108,8 @@ def test_batch_of_both_kinds(bbp, plans):
     for _ in range(2):
         vals, valid, _ = bbp.bbp_bits_batch(plan.handle, 0, ns, Ps)
         assert list(zip(vals, valid)) == want
+    vals, valid, _ = bbp.bbp_bits_batch(plan.handle, 1, ns, Ps)
+    assert list(zip(vals, valid)) == [by_terms(bbp, plan, n, P, 1) for n, P in zip(ns, Ps)]
 
 
 def test_async_on_a_stream_and_under_capture(bbp, plans):
