@@ -18,18 +18,18 @@
 namespace bbp {
 namespace {
 
-template <int PATH, int S>
+template <int PATH, int S, Ladder LADDER = kLadderPlain>
 cudaError_t launch_head_t(const HeadArgs& a, int blocks, int threads, cudaStream_t s) {
   const uint64_t tile = 32ull * S * a.run;
   const uint64_t ntiles = (a.count + tile - 1) / tile;
-  head_kernel<BBP_LMAX, PATH, S><<<blocks, threads, 0, s>>>(a, ntiles);
+  head_kernel<BBP_LMAX, PATH, S, LADDER><<<blocks, threads, 0, s>>>(a, ntiles);
   return cudaGetLastError();
 }
 
-template <int PATH, int S>
+template <int PATH, int S, Ladder LADDER = kLadderPlain>
 int head_occupancy_t(int threads) {
   int n = 0;
-  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, head_kernel<BBP_LMAX, PATH, S>, threads, 0) != cudaSuccess)
+  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, head_kernel<BBP_LMAX, PATH, S, LADDER>, threads, 0) != cudaSuccess)
     return 1;
   return n > 0 ? n : 1;
 }
@@ -109,6 +109,8 @@ cudaError_t BBP_CAT(launch_head_l, BBP_LMAX)(const HeadArgs& a, int path, int st
     case 1: return two ? launch_head_t<1, 2>(a, blocks, threads, s) : launch_head_t<1, 1>(a, blocks, threads, s);
     case 2: return two ? launch_head_t<2, 2>(a, blocks, threads, s) : launch_head_t<2, 1>(a, blocks, threads, s);
     case 3: return two ? launch_head_t<3, 2>(a, blocks, threads, s) : launch_head_t<3, 1>(a, blocks, threads, s);
+    case kPathHalf: return two ? launch_head_t<1, 2, kLadderHalf>(a, blocks, threads, s) : launch_head_t<1, 1, kLadderHalf>(a, blocks, threads, s);
+    case kPath47: return two ? launch_head_t<1, 2, kLadder47>(a, blocks, threads, s) : launch_head_t<1, 1, kLadder47>(a, blocks, threads, s);
     default: return cudaErrorInvalidValue;
   }
 }
@@ -120,6 +122,8 @@ int BBP_CAT(head_occupancy_l, BBP_LMAX)(int path, int streams, int threads) {
     case 1: return two ? head_occupancy_t<1, 2>(threads) : head_occupancy_t<1, 1>(threads);
     case 2: return two ? head_occupancy_t<2, 2>(threads) : head_occupancy_t<2, 1>(threads);
     case 3: return two ? head_occupancy_t<3, 2>(threads) : head_occupancy_t<3, 1>(threads);
+    case kPathHalf: return two ? head_occupancy_t<1, 2, kLadderHalf>(threads) : head_occupancy_t<1, 1, kLadderHalf>(threads);
+    case kPath47: return two ? head_occupancy_t<1, 2, kLadder47>(threads) : head_occupancy_t<1, 1, kLadder47>(threads);
     default: return 1;
   }
 }

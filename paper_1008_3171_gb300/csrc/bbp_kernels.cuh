@@ -82,6 +82,10 @@ constexpr int kNumLmaxClasses = static_cast<int>(sizeof(kLmaxClasses) / sizeof(k
 // square (bitlen <= 46); 2 two words, four-word square (bitlen <= 60); 3 one word,
 // fully reduced residues (bitlen 30 or 31).
 constexpr int kNumPaths = 4;
+// launch_head takes two more, for parts of paths 1 and 2 (bbp_tile.cuh, Ladder): moduli of 32
+// bits up to kHalfMaxModulus, and moduli of 47 bits.
+constexpr int kPathHalf = 4, kPath47 = 5;
+constexpr uint64_t kHalfMaxModulus = 1'020'000'000'000;
 constexpr int kQueueVariants = kNumLmaxClasses * kNumPaths;  // limb class x modulus path
 
 // ---------------------------------------------------------------- batches
@@ -134,7 +138,8 @@ struct PrimeArgs {
 
 // Launch helpers (defined in bbp_kernels.cu).  They return cudaGetLastError().
 // path: 0 = one-word moduli, bitlen <= 29; 1 = two-word moduli, bitlen <= 46;
-//       2 = two-word moduli, bitlen <= 60; 3 = one-word moduli of 30 or 31 bits.
+//       2 = two-word moduli, bitlen <= 60; 3 = one-word moduli of 30 or 31 bits;
+//       kPathHalf, kPath47.
 // threads: CTA size, a multiple of 32 in [32, kHeadThreads] (else cudaErrorInvalidValue).
 cudaError_t launch_head(const HeadArgs& a, int path, int streams, int lmax, int blocks, cudaStream_t s,
                         int threads = kHeadThreads);

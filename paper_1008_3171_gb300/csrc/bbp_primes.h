@@ -57,7 +57,7 @@ uint64_t prime_first_k(const PrimeLimits& lim, uint32_t j, uint64_t d);
 
 // Primes up to here take the half-reduced ladder: with x <= p + 2^35, x^2 / 2^32 + p stays
 // below 2^48.
-constexpr uint64_t kPrimeHalfMax = 1'020'000'000'000;
+constexpr uint64_t kPrimeHalfMax = 1'020'000'000'000;  // as kHalfMaxModulus
 
 // Primes with the same +-H = num / (den 2^kPrimeShift), by p mod 4: those above `above`, up to the
 // previous class's `above`.

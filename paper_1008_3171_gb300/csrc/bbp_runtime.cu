@@ -313,34 +313,60 @@ bbp_status launch_ranges(bbp_plan p, int f, uint64_t n, uint32_t W, const std::v
       }
       continue;
     }
-    HeadArgs a = head_args(F, r, n, W);
-    a.slots = slots;
-    a.gate = gate;
-    const int streams = head_streams(p, r.path);
-    const int warps_per_block = p->cta / 32;
-    const int occ = head_occupancy(r.path, streams, lmax, p->cta);
-    const uint64_t resident_warps = static_cast<uint64_t>(occ) * p->sm_count * warps_per_block;
-    // a short range takes fewer consecutive terms per stream, so that its tiles
-    // spread over the GPU's resident warps instead of a few warps running long runs
-    auto tiles_for = [&](uint32_t rn) { return (r.count + 32ull * streams * rn - 1) / (32ull * streams * rn); };
-    const uint32_t run = run_for(static_cast<uint32_t>(p->run), resident_warps, tiles_for);
-    a.run = run;
-    const uint64_t ntiles = tiles_for(run);
-    const uint64_t want = (ntiles + warps_per_block - 1) / warps_per_block;
-    const int blocks = static_cast<int>(std::max<uint64_t>(1, std::min<uint64_t>(want, uint64_t(occ) * p->sm_count)));
-    if (p->profile) BBP_CUDA(cudaEventRecord(p->ev0, st));
-    BBP_CUDA(launch_head(a, r.path, streams, lmax, blocks, st, p->cta));
-    if (p->profile) {
-      BBP_CUDA(cudaEventRecord(p->ev1, st));
-      BBP_CUDA(cudaEventSynchronize(p->ev1));
-      float ms = 0;
-      BBP_CUDA(cudaEventElapsedTime(&ms, p->ev0, p->ev1));
-      total_ms += ms;
+    // parts of paths 1 and 2 that have a ladder of their own
+    TermRange parts[2] = {r, r};
+    int paths[2] = {r.path, r.path};
+    parts[1].count = 0;
+    if ((r.path == 1 && p->wide_min_bits == kWideMinBits) || r.path == 2) {
+      const SeriesDef& s = F.s[r.j];
+      const uint64_t top = r.path == 1 ? kHalfMaxModulus : (1ull << (kSmallMaxBits + 1)) - 1;
+      const uint64_t first_above = top < s.b ? 0 : (top - s.b) / s.a + 1;  // first k past `top`
+      const uint64_t below = first_above > r.k_begin ? std::min(r.count, first_above - r.k_begin) : 0;
+      if (below > 0) {
+        parts[0].count = below;
+        parts[1].k_begin = r.k_begin + below;
+        parts[1].count = r.count - below;
+        paths[0] = r.path == 1 ? kPathHalf : kPath47;
+        uint8_t window;
+        window_params(1, bitlen(static_cast<uint64_t>(s.a) * (r.k_begin + below - 1) + s.b), &window, &parts[0].first,
+                      &parts[0].first_max);
+        parts[0].window = 4;
+      }
     }
-    p->stats.kernel_launches++;
-    p->stats.head_launches++;
-    p->stats.terms += r.count;
-    p->stats.head_terms += r.count;
+    for (int i = 0; i < 2; ++i) {
+      const TermRange& part = parts[i];
+      const int path = paths[i];
+      if (part.count == 0) continue;
+      HeadArgs a = head_args(F, part, n, W);
+      a.slots = slots;
+      a.gate = gate;
+      const int streams = head_streams(p, path);
+      const int warps_per_block = p->cta / 32;
+      const int occ = head_occupancy(path, streams, lmax, p->cta);
+      const uint64_t resident_warps = static_cast<uint64_t>(occ) * p->sm_count * warps_per_block;
+      // a short range takes fewer consecutive terms per stream, so that its tiles
+      // spread over the GPU's resident warps instead of a few warps running long runs
+      auto tiles_for = [&](uint32_t rn) { return (part.count + 32ull * streams * rn - 1) / (32ull * streams * rn); };
+      const uint32_t run = run_for(static_cast<uint32_t>(p->run), resident_warps, tiles_for);
+      a.run = run;
+      const uint64_t ntiles = tiles_for(run);
+      const uint64_t want = (ntiles + warps_per_block - 1) / warps_per_block;
+      const int blocks = static_cast<int>(std::max<uint64_t>(1, std::min<uint64_t>(want, uint64_t(occ) * p->sm_count)));
+      if (p->profile) BBP_CUDA(cudaEventRecord(p->ev0, st));
+      BBP_CUDA(launch_head(a, path, streams, lmax, blocks, st, p->cta));
+      if (p->profile) {
+        BBP_CUDA(cudaEventRecord(p->ev1, st));
+        BBP_CUDA(cudaEventSynchronize(p->ev1));
+        float ms = 0;
+        BBP_CUDA(cudaEventElapsedTime(&ms, p->ev0, p->ev1));
+        total_ms += ms;
+      }
+      p->stats.kernel_launches++;
+      p->stats.head_launches++;
+      p->stats.terms += part.count;
+      p->stats.head_terms += part.count;
+    
+    }
     p->stats.imad_model += r.imad;
   }
   if (tails.n > 0) {

@@ -7,6 +7,7 @@
 #include <vector>
 
 #include "bbp.h"
+#include "bbp_kernels.cuh"
 #include "bbp_planner.h"
 
 struct bbp_plan_s {
@@ -45,7 +46,7 @@ namespace bbp {
 // Term pairs per thread of the head and queue kernels on a modulus path: the tune
 // table's value, else two on path 1 (the three-word squaring has the registers for
 // a second independent pair at three CTAs per SM) and one elsewhere.
-inline int head_streams(const bbp_plan_s* p, int path) { return p->streams > 0 ? p->streams : (path == 1 ? 2 : 1); }
+inline int head_streams(const bbp_plan_s* p, int path) { return p->streams > 0 ? p->streams : (path == 1 || path >= kPathHalf ? 2 : 1); }
 // Terms of one warp tile on that path.
 inline uint64_t tile_terms(const bbp_plan_s* p, int path) {
   return 32ull * static_cast<uint64_t>(head_streams(p, path)) * static_cast<uint64_t>(p->run);

@@ -67,6 +67,13 @@ __device__ __forceinline__ void square_all_general(uint32_t (&x0)[NT], uint32_t 
   for (int t = 0; t < NT; ++t) sqr_shift_redc64(x0[t], x1[t], sh[t], Mod64{m0[t], m1[t], mp[t]}, do_shift);
 }
 
+template <int NT>
+__device__ __forceinline__ void reduce_all(uint32_t (&x0)[NT], uint32_t (&x1)[NT], const uint32_t (&m0)[NT],
+                                           const uint32_t (&m1)[NT], const uint32_t (&mp)[NT]) {
+#pragma unroll
+  for (int t = 0; t < NT; ++t) reduce_once64(x0[t], x1[t], Mod64{m0[t], m1[t], mp[t]});
+}
+
 // Quotient digits of every term, least significant first, folded straight into
 // the LMAX-limb sum with a signed carry (odd terms subtracted when NEG_ODD).  A
 // term of a lane past the range has x = 0, whose digits are all 0.
@@ -111,9 +118,29 @@ __device__ __forceinline__ void square_group(int len, uint32_t (&x0)[NT], uint32
   square_all<PATH, NT>(x0, x1, m0, m1, mp, sh, true);
 }
 
+// Ladders of path 1 for parts of its and path 2's moduli (two words, three-word square).
+enum Ladder {
+  kLadderPlain,
+  // Moduli up to kHalfMaxModulus: every second squaring takes one reduction step
+  // (sqr_half64_p1).  All factors are powers of two, so a value is followed by its exponent
+  // f: a squaring with two steps and a window shift s takes f to 2 f - 64 + s, one with a
+  // step to 2 f - 32, the two together to 4 f - 128 + s.  After c plain squarings from
+  // R 2^w0 (f = 64 + w0) and k pairs, f = 4^k f1 - 128 (4^k - 1) / 3 + S with
+  // f1 = 64 + (w0 and c bits), so f1 and S are the top and the low 2 k bits of
+  // U = E + 128 (4^k - 1) / 3.  k is the largest with f1 >= 64.
+  // (n = 1e12, 40-bit moduli: 36 squarings with 72 steps -> 35 with 53; a slice of 2e8
+  // terms 8.13 -> 7.35 ms.)
+  kLadderHalf,
+  // Moduli of 47 bits: a squaring without shift leaves x < m + 2^31, one with a shift of 15
+  // x < m + 2^46.3 < 2^47.7, and that x's square still fits three words, its first reduction
+  // two.  Only the unreduced first window may leave more, so it is reduced fully.
+  // (n = 1e14, a slice of 2e8 terms: 10.8 ms on path 2, 9.0 here.)
+  kLadder47
+};
+
 // One warp tile: terms [ti * tile, (ti + 1) * tile) of the run list of A, added
 // into this lane's sum.  Every lane of the warp must call it (warp-wide reductions).
-template <int LMAX, int PATH, int S>
+template <int LMAX, int PATH, int S, Ladder LADDER = kLadderPlain>
 __device__ __forceinline__ void process_tile(const HeadArgs& A, const uint64_t ti, const uint32_t lane,
                                              uint32_t (&acc)[LMAX]) {
   constexpr int NT = 2 * S;
@@ -163,6 +190,46 @@ __device__ __forceinline__ void process_tile(const HeadArgs& A, const uint64_t t
         nbl = max(nbl, bitlen64(v[t]));
       }
     }
+    if constexpr (LADDER == kLadderHalf) {
+      // the warp's largest and smallest exponents: first lane's first term, last lane's last
+      const uint64_t e_max = __shfl_sync(0xffffffffu, v[0], 0) + RB;
+      const uint64_t e_min = __shfl_sync(0xffffffffu, v[NT - 1], 31) + RB;
+      const int k = (bitlen64((3 * e_min - 128) >> 6) - 1) / 2;  // 64 4^k <= 3 E - 128
+      const uint64_t low = (1ull << (2 * k)) - 1ull, off = (0x5555555555555555ull & low) << 7;
+      int c = 1;
+      while ((((e_max + off) >> (2 * k)) - 64) >> c > A.first_max) ++c;
+      uint64_t rem[NT];
+      uint32_t sh[NT];
+#pragma unroll
+      for (int t = 0; t < NT; ++t) {
+        const uint64_t u = v[t] + RB + off;
+        const uint32_t f1 = static_cast<uint32_t>(u >> (2 * k)) - 64u;
+        const uint64_t x = make64(x0[t], x1[t]) << (f1 >> c);
+        x0[t] = lo32(x);
+        x1[t] = hi32(x);
+        rem[t] = (static_cast<uint64_t>(f1 & ((1u << c) - 1u)) << (2 * k)) | (u & low);
+      }
+      // the c bits of f1, the first on the general routine
+      int p = 2 * k + c - 1;
+#pragma unroll
+      for (int t = 0; t < NT; ++t) sh[t] = static_cast<uint32_t>(rem[t] >> p) & 1u;
+      square_all_general<NT>(x0, x1, m0, m1, mp, sh, true);
+      while (p > 2 * k) {
+        --p;
+#pragma unroll
+        for (int t = 0; t < NT; ++t) sh[t] = static_cast<uint32_t>(rem[t] >> p) & 1u;
+        square_all<PATH, NT>(x0, x1, m0, m1, mp, sh, true);
+      }
+      reduce_all<NT>(x0, x1, m0, m1, mp);
+      while (p > 0) {
+        p -= 2;
+#pragma unroll
+        for (int t = 0; t < NT; ++t) sh[t] = static_cast<uint32_t>(rem[t] >> p) & 3u;
+#pragma unroll
+        for (int t = 0; t < NT; ++t) sqr_half64_p1(x0[t], x1[t], Mod64{m0[t], m1[t], mp[t]});
+        square_all<PATH, NT>(x0, x1, m0, m1, mp, sh, true);
+      }
+    } else {
     const int nb = static_cast<int>(__reduce_max_sync(0xffffffffu, static_cast<uint32_t>(nbl)));
     int h = nb > 0 ? min(static_cast<int>(A.first), nb - 1) : 0;
     if (A.first_max >= (1u << h) && h + 1 <= nb - 1) {
@@ -206,8 +273,10 @@ __device__ __forceinline__ void process_tile(const HeadArgs& A, const uint64_t t
       for (int t = 0; t < NT; ++t) sh[t] = static_cast<uint32_t>(rem[t] >> p) & ((1u << len) - 1u);
       if (len == 1) {
         square_all_general<NT>(x0, x1, m0, m1, mp, sh, true);
+        if constexpr (LADDER == kLadder47) reduce_all<NT>(x0, x1, m0, m1, mp);
       } else {
         square_all_general<NT>(x0, x1, m0, m1, mp, zero, false);
+        if constexpr (LADDER == kLadder47) reduce_all<NT>(x0, x1, m0, m1, mp);
         square_group<PATH, NT>(len - 1, x0, x1, m0, m1, mp, sh);
       }
     }
@@ -231,6 +300,7 @@ __device__ __forceinline__ void process_tile(const HeadArgs& A, const uint64_t t
 #pragma unroll
       for (int t = 0; t < NT; ++t) sh[t] = static_cast<uint32_t>(rem[t] >> p) & ((1u << len) - 1u);
       square_group<PATH, NT>(len, x0, x1, m0, m1, mp, sh);
+    }
     }
     // s = 2^E mod m (0 for a lane past the range), then the W-bit quotient digits
     // folded into the signed sum
@@ -292,8 +362,12 @@ __device__ __forceinline__ void flush_cta(uint32_t (&acc)[LMAX], uint32_t L, uns
   }
 }
 
-template <int LMAX, int PATH, int S>
-__global__ void __launch_bounds__(kHeadThreads) head_kernel(const HeadArgs A, const uint64_t ntiles) {
+// The half-reduced ladder with two term pairs a thread is held to 80 registers, three CTAs
+// an SM (7.35 against 7.58 ms on its slice); the others are faster with the 102 the compiler
+// takes, and two (8.58 against 8.89 ms on 43-bit moduli).
+template <int LMAX, int PATH, int S, Ladder LADDER = kLadderPlain>
+__global__ void __launch_bounds__(kHeadThreads, LADDER == kLadderHalf && S == 2 && LMAX <= 16 ? 3 : 0)
+head_kernel(const HeadArgs A, const uint64_t ntiles) {
   if (A.gate && *A.gate == 0u) return;
   const uint32_t lane = threadIdx.x & 31u;
   const uint64_t warp = (static_cast<uint64_t>(blockIdx.x) * blockDim.x + threadIdx.x) >> 5;
@@ -302,7 +376,7 @@ __global__ void __launch_bounds__(kHeadThreads) head_kernel(const HeadArgs A, co
   uint32_t acc[LMAX];
 #pragma unroll
   for (int i = 0; i < LMAX; ++i) acc[i] = 0;
-  for (uint64_t ti = warp; ti < ntiles; ti += nwarps) process_tile<LMAX, PATH, S>(A, ti, lane, acc);
+  for (uint64_t ti = warp; ti < ntiles; ti += nwarps) process_tile<LMAX, PATH, S, LADDER>(A, ti, lane, acc);
 
   if (A.negate) negate_limbs<LMAX>(acc);
   flush_cta<LMAX>(acc, A.L, A.slots);
