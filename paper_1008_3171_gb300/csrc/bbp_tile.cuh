@@ -52,7 +52,7 @@ __device__ __forceinline__ void square_all(uint32_t (&x0)[NT], uint32_t (&x1)[NT
   for (int t = 0; t < NT; ++t) {
     if (PATH == 1) sqr_redc64_p1(x0[t], x1[t], sh[t], Mod64{m0[t], m1[t], mp[t]}, do_shift);
     else if (PATH == 2) sqr_shift_redc64(x0[t], x1[t], sh[t], Mod64{m0[t], m1[t], mp[t]}, do_shift);
-    else x0[t] = sqr_shift_redc32<PATH == 3>(x0[t], sh[t], Mod32{m0[t], mp[t]}, do_shift);
+    else x0[t] = sqr_shift_redc32<PATH == 3>(x0[t], sh[t], m0[t], m1[t], do_shift);  // m1: m^-1 mod 2^32
   }
 }
 
@@ -186,6 +186,7 @@ __device__ __forceinline__ void process_tile(const HeadArgs& A, const uint64_t t
         m0[t] = lo32(st[s].m);
         m1[t] = hi32(st[s].m);
         mp[t] = neg_inverse32(m0[t]);
+        if (!WIDE) m1[t] = 0u - mp[t];  // no high word: the inverse itself
         v[t] = st[s].E - RB;  // E >= W >= RB for head terms
         nbl = max(nbl, bitlen64(v[t]));
       }
