@@ -78,6 +78,7 @@ cudaError_t BBP_CAT(launch_prime_l, BBP_LMAX)(const PrimeArgs& a, PrimeKernel k,
     case kPrimes1: return launch_prime_t(prime_kernel<BBP_LMAX, 1, false>, a, sms, s);
     case kPrimesHalf: return launch_prime_t(prime_kernel<BBP_LMAX, 1, true>, a, sms, s);
     case kPrimes3: return launch_prime_t(prime_kernel<BBP_LMAX, 3, false>, a, sms, s);
+    case kSums32: return launch_prime_t(f ? prime_sum_kernel<Arith1, 1, 32, BBP_LMAX> : prime_sum_kernel<Arith1, 0, 32, BBP_LMAX>, a, sms, s);
     case kSums8: return launch_prime_t(f ? prime_sum_kernel<Arith1, 1, 8, BBP_LMAX> : prime_sum_kernel<Arith1, 0, 8, BBP_LMAX>, a, sms, s);
     case kSums1: return launch_prime_t(f ? prime_sum_kernel<Arith1, 1, 1, BBP_LMAX> : prime_sum_kernel<Arith1, 0, 1, BBP_LMAX>, a, sms, s);
     case kSums2: return launch_prime_t(f ? prime_sum_kernel<Arith2, 1, 1, BBP_LMAX> : prime_sum_kernel<Arith2, 0, 1, BBP_LMAX>, a, sms, s);

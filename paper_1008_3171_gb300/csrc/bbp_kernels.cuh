@@ -167,9 +167,9 @@ int head_lmax_for(int L, int bump = 0);
 int head_occupancy(int path, int streams, int lmax, int threads = kHeadThreads);
 // A prime kernel over the primes of `a`, on every SM.  kPrimes0, 1, 3: prime_kernel on
 // that modulus path (primes above A / 23), kPrimesHalf on path 1 up to kPrimeHalfMax; kSums1, kSums2: prime_sum_kernel in one or two
-// words, kSums8 in one word with eight lanes a prime; kPrimeWarps: prime_power_kernel, a = 1 (p < 2^31); kPowers1, kPowers2: a >= 2 (p < 2^23), p^a
+// words, kSums8 and kSums32 in one word with 8 and 32 lanes a prime; kPrimeWarps: prime_power_kernel, a = 1 (p < 2^31); kPowers1, kPowers2: a >= 2 (p < 2^23), p^a
 // below 2^31 or from there on.
-enum PrimeKernel { kPrimes0, kPrimes1, kPrimesHalf, kPrimes3, kSums8, kSums1, kSums2, kPrimeWarps, kPowers1, kPowers2 };
+enum PrimeKernel { kPrimes0, kPrimes1, kPrimesHalf, kPrimes3, kSums32, kSums8, kSums1, kSums2, kPrimeWarps, kPowers1, kPowers2 };
 cudaError_t launch_prime(const PrimeArgs& a, PrimeKernel k, int formula, int lmax, int sms, cudaStream_t s);
 // blocks: CTAs for the head ranges, besides q.tail_blocks; both together at least 1.
 cudaError_t launch_query(const QuerySet& q, int streams, int lmax, int blocks, int threads, cudaStream_t s);

@@ -23,12 +23,10 @@ namespace bbp {
 
 namespace {
 
-constexpr uint32_t kMaxBase = (1u << 23) - 1;       // base primes up to here: 564,162 odd ones
-constexpr uint32_t kBaseCap = 565000;
+constexpr uint32_t kBaseCap = 565000;               // odd primes below 2^23: 564,162
 constexpr uint32_t kMaxLists = 1u << 17;            // 7.6e4 lists of 6 M primes at the largest position
 constexpr uint32_t kSieveEntries = 64u << 10;       // of a sieve segment: three CTAs an SM
-constexpr uint64_t kLongSum = 32000;                // primes below A / this take a warp each,
-constexpr uint64_t kGroupSum = 1000;                // those below A / this eight lanes
+constexpr uint64_t kLongSum = 8000, kGroupSum = 1000;  // primes below A / these take 32, 8 lanes
 
 uint64_t isqrt(uint64_t v) {
   uint64_t r = static_cast<uint64_t>(std::sqrt(static_cast<double>(v)));
@@ -155,14 +153,17 @@ bbp_status PrimeRun::plan(PrimeState* state, int sm_count, int formula, uint64_t
   std::copy(classes.begin(), classes.end(), a.classes);
   e_ = n - 1 + W;
   const uint64_t root = isqrt(lim.A);
-  base_to_ = static_cast<uint32_t>(std::min<uint64_t>(kMaxBase, std::max(root, lim.A / kLongSum)));
+  base_to_ = static_cast<uint32_t>(root);  // below 2^23
   const uint64_t bottom = classes.back().above;
   // lists: primes in (base_to, A], cut where their kernel changes
   struct Span { uint64_t lo, hi; PrimeKernel k; };
   std::vector<Span> spans;
   {
-    const uint64_t grouped = std::min<uint64_t>(lim.A / kGroupSum, (1ull << 31) - 1);
-    const uint64_t cuts[] = {grouped, bottom, (1ull << 29) - 1, (1ull << 31) - 1, kPrimeHalfMax,
+    const uint64_t one_word = (1ull << 31) - 1;
+    // a list of its own pays from about n = 6e8 on
+    const uint64_t shared32 = lim.A / kLongSum > 3 * root ? std::min(lim.A / kLongSum, one_word) : 0;
+    const uint64_t shared8 = std::min(lim.A / kGroupSum, one_word);
+    const uint64_t cuts[] = {shared32, shared8, bottom, (1ull << 29) - 1, (1ull << 31) - 1, kPrimeHalfMax,
                              formula == 1 ? lim.B : lim.A, lim.A};
     std::vector<uint64_t> c(std::begin(cuts), std::end(cuts));
     std::sort(c.begin(), c.end());
@@ -171,7 +172,7 @@ bbp_status PrimeRun::plan(PrimeState* state, int sm_count, int formula, uint64_t
       hi = std::min(hi, lim.A);
       if (hi <= lo) continue;
       PrimeKernel k;
-      if (hi <= bottom) k = hi <= grouped ? kSums8 : hi < (1ull << 31) ? kSums1 : kSums2;
+      if (hi <= bottom) k = hi <= shared32 ? kSums32 : hi <= shared8 ? kSums8 : hi <= one_word ? kSums1 : kSums2;
       else k = hi < (1ull << 29) ? kPrimes0 : hi < (1ull << 31) ? kPrimes3 : hi <= kPrimeHalfMax ? kPrimesHalf : kPrimes1;
       spans.push_back(Span{lo, hi, k});
       lo = hi;
@@ -258,7 +259,7 @@ bbp_status PrimeRun::run(size_t first, size_t last, cudaStream_t st) {
     a.base = l.base;
     a.count = lengths + i;
     a.taken = lengths + lists_.size() + i;
-    const bool sums = l.kernel == kSums1 || l.kernel == kSums2 || l.kernel == kSums8;
+    const bool sums = l.kernel == kSums1 || l.kernel == kSums2 || l.kernel == kSums8 || l.kernel == kSums32;
     a.e = sums ? e_ : e_ - kPrimeShift + 64;  // the product with H leaves a factor 2^-64
     chk(launch_prime(a, l.kernel, formula_, lmax_, sms_, st));
     chk(cudaEventRecord(S->used[slot], st));

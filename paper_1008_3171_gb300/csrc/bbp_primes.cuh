@@ -3,8 +3,8 @@
 //
 //   prime_kernel       primes above A / 23: H is one of a few rational constants, so a
 //                      prime costs one modular power of 2, a product and W bits of quotient
-//   prime_sum_kernel   primes below: H summed mod p, one prime per thread or eight threads
-//   prime_power_kernel primes and prime powers with long sums: one warp each
+//   prime_sum_kernel   primes below, down to sqrt(A): H summed mod p, 1, 8 or 32 threads each
+//   prime_power_kernel primes up to sqrt(A) and prime powers: one warp each
 //
 // Every part is a residue x = 2^W r mod q of a fraction r / q; its W bits are the
 // exact-division digits of -x / q, as for a term (bbp_device.cuh).  Each is rounded
@@ -255,7 +255,9 @@ __global__ void __launch_bounds__(kHeadThreads) prime_kernel(const __grid_consta
 struct Arith1 {
   using T = uint32_t;
   uint32_t m, mp, minv;  // mp = -m^-1, minv = m^-1 mod 2^32
-  __device__ explicit Arith1(uint64_t q) : m(lo32(q)), mp(neg_inverse32(lo32(q))), minv(0u - mp) {}
+  uint32_t r1;           // 2^32 mod m: 1 in Montgomery form
+  __device__ explicit Arith1(uint64_t q)
+      : m(lo32(q)), mp(neg_inverse32(lo32(q))), minv(0u - mp), r1(static_cast<uint32_t>(r_mod_m_bitserial<32>(q).r)) {}
   __device__ __forceinline__ T lazy_redc(uint64_t t) const {  // t 2^-32, t < m 2^32 (or below 2 m for hi(t) < m)
     return hi32(t) + m - __umulhi(lo32(t) * minv, m);
   }
@@ -267,7 +269,7 @@ struct Arith1 {
   __device__ __forceinline__ T mul(T a, T b) const { return redc(static_cast<uint64_t>(a) * b); }
   __device__ __forceinline__ T add(T a, T b) const { return fix(a + b); }
   __device__ __forceinline__ T neg(T a) const { return a != 0u ? m - a : 0u; }
-  __device__ __forceinline__ T one() const { return static_cast<T>(r_mod_m_bitserial<32>(m).r); }
+  __device__ __forceinline__ T one() const { return r1; }
   __device__ __forceinline__ T plain(T a) const { return redc(a); }  // out of Montgomery form
   __device__ __forceinline__ uint32_t digit(T& x) const {            // next exact-division digit
     const uint32_t q = x * mp;
@@ -281,7 +283,8 @@ struct Arith2 {
   using T = uint64_t;
   static constexpr int kBits = 64;
   uint64_t m, mp;
-  __device__ explicit Arith2(uint64_t q) : m(q) {
+  uint64_t r1;  // 2^64 mod m
+  __device__ explicit Arith2(uint64_t q) : m(q), r1(r_mod_m_bitserial<64>(q).r) {
     const uint64_t x = 0u - neg_inverse32(lo32(q));
     mp = 0ull - x * (2ull - q * x);
   }
@@ -300,7 +303,7 @@ struct Arith2 {
   }
   __device__ __forceinline__ T add(T a, T b) const { return fix(a + b); }
   __device__ __forceinline__ T neg(T a) const { return a != 0 ? m - a : 0; }
-  __device__ __forceinline__ T one() const { return r_mod_m_bitserial<64>(m).r; }
+  __device__ __forceinline__ T one() const { return r1; }
   __device__ __forceinline__ T plain(T a) const { return mul(a, 1); }
   __device__ __forceinline__ uint32_t digit(T& x) const {
     uint32_t x0 = lo32(x), x1 = hi32(x);
@@ -672,8 +675,9 @@ __device__ __forceinline__ T summands(T top, uint32_t c0) {
 //   Eq. 2: H = 16 (num_A / den_A - 4 num_B / den_B - num_C / den_C), times chi(p)
 //   Eq. 1: H = 8 (2 num_D / den_D - num_E / den_E - num_F / den_F) for p = 1 mod 4,
 //          H = -8 (num_D / den_D + 4 num_E / den_E + num_F / den_F) for p = 3 mod 4
-// One lane per prime walks up to 8000 terms in a row where the sums are long; eight lanes
-// bring n = 1e9's longest chain from 600 us (with the SM full) to a quarter.
+// One lane per prime would walk up to sqrt(A) / 2 terms in a row where the sums are long
+// (n = 1e9: 600 us with the SM full, for 180 us of work): 32 lanes share a prime below
+// A / 8000, eight one below A / 1000.
 template <class A, int FORMULA, int GROUP, int LMAX>
 __global__ void __launch_bounds__(kHeadThreads) prime_sum_kernel(const __grid_constant__ PrimeArgs G) {
   constexpr int K0 = FORMULA == 0 ? 0 : 3;
@@ -744,19 +748,19 @@ __device__ typename A::T geometric(const A& M, typename A::T r, uint64_t n) {
 }
 
 // What one lane adds of sum KIND to the part of q = p^a: its share of the summands
-// [lo, hi), `times` over, as a fraction added to num / den (all in Montgomery form).
-// Summand i carries s(i) 2^(start - ratio q i) / c.
+// [lo, hi), times `factor`, as a fraction added to num / den (all in Montgomery form).
+// Summand i carries s(i) 2^(start - ratio q i) / c; e is taken mod phi.
 template <class A, int KIND, bool PRIME>
 __device__ __forceinline__ void add_share(const A& M, uint64_t p, uint64_t q, uint64_t phi, int64_t e, uint64_t lo,
-                                          uint64_t hi, uint64_t period, uint64_t times, uint32_t lane,
-                                          typename A::T& num, typename A::T& den) {
+                                          uint64_t hi, typename A::T factor, uint32_t lane, typename A::T& num,
+                                          typename A::T& den) {
   using T = typename A::T;
   using K = SumKind<KIND>;
   const uint64_t share = (hi - lo + 31) / 32;
   const uint64_t i0 = lo + min(hi - lo, lane * share), i1 = min(hi, i0 + share);
-  if (times == 0 || hi <= lo) return;  // the same for every lane
+  if (hi <= lo) return;  // the same for every lane
   constexpr int64_t kRatio = K::kW;
-  const int64_t sq = static_cast<int64_t>(q);
+  const int64_t sq = static_cast<int64_t>(PRIME ? 1 : q);  // 2^p = 2 mod p
   const uint32_t r4 = lo32(q) & 3u, c0 = KIND == 3 ? r4 : KIND == 4 ? 4u - r4 : 1u;
   T n_s, d_s;
   const T h = PRIME ? 0 : power_of_two<A>(M, exponent_mod(kRatio * sq, phi));
@@ -768,18 +772,13 @@ __device__ __forceinline__ void add_share(const A& M, uint64_t p, uint64_t q, ui
   bool minus = true;
   if (KIND == 0) start = e + 3 - sq, minus = (q & 2u) != 0;
   if (KIND == 1) start = e + 1 - 5 * sq, minus = (q & 2u) == 0;
-  if (KIND == 2) start = e - 1 - 5 * (sq - 1) / 2, minus = (q & 4u) == 0;
-  if (KIND == 3) start = e + 2 - (sq * c0 - 1) / 2, minus = ((q * c0) & 7u) != 1u;
+  if (KIND == 2) start = e - 1 - 5 * (static_cast<int64_t>(q) - 1) / 2, minus = (q & 4u) == 0;
+  if (KIND == 3) start = e + 2 - (static_cast<int64_t>(q) * c0 - 1) / 2, minus = ((q * c0) & 7u) != 1u;
   if (KIND == 4) start = e + 2 - sq * c0;
   if (KIND == 5) start = e + 1 - 2 * sq;
   // with the h that multiplies the fraction
   T k = power_of_two<A>(M, exponent_mod(start + kRatio * sq * (1 - static_cast<int64_t>(i0)), phi));
-  if (times > 1) {
-    T r = power_of_two<A>(M, exponent_mod(-kRatio * sq * static_cast<int64_t>(period), phi));
-    if (K::kAlternates) r = M.neg(r);  // the period is odd
-    k = M.mul(k, geometric<A>(M, r, times));
-  }
-  k = M.mul(k, n_s);
+  k = M.mul(M.mul(k, factor), n_s);
   num = M.add(M.mul(num, d_s), M.mul(minus ? M.neg(k) : k, den));
   den = M.mul(den, d_s);
 }
@@ -833,28 +832,35 @@ __global__ void __launch_bounds__(kHeadThreads) prime_power_kernel(const __grid_
     const uint64_t q = prime_power_of<PRIME>(G, unit, count, &p);
     if (q == 0 || (!PRIME && (q < (1ull << 31)) != (sizeof(T) == 4))) continue;
     const A M(q);
-    const uint64_t phi = q / p * (p - 1);
-    const int64_t e = static_cast<int64_t>(G.e);
-    const uint64_t limit[3] = {G.A, G.B, G.C};
-    uint64_t whole[3], rest[3], period[3];
-#pragma unroll
-    for (int s = 0; s < 3; ++s) {
-      const uint64_t top = limit[s] / q;
-      const uint32_t r4 = lo32(q) & 3u;
-      const uint64_t n = FORMULA == 0 || s == 2 ? summands<0>(top, 1u)
-                                                : s == 0 ? summands<3>(top, r4) : summands<4>(top, 4u - r4);
-      period[s] = FORMULA == 0 && s == 2 ? 4 * q : q;
-      whole[s] = n / period[s];
-      rest[s] = n % period[s];
+    const uint64_t phi = PRIME ? p - 1 : q / p * (p - 1);
+    const int64_t e = static_cast<int64_t>(G.e % phi);
+    // lane s < 3 works out sum s's repetitions: n summands, `whole` periods of them and `rest`
+    const uint32_t s = min(lane, 2u), r4 = lo32(q) & 3u;
+    const uint64_t top = (s == 0 ? G.A : s == 1 ? G.B : G.C) / q;
+    const uint64_t n = FORMULA == 0 || s == 2 ? summands<0>(top, 1u) : s == 0 ? summands<3>(top, r4) : summands<4>(top, 4u - r4);
+    const uint64_t period_s = FORMULA == 0 && s == 2 ? 4 * q : q;
+    const uint64_t whole_s = n / period_s, rest_s = n - whole_s * period_s;
+    T once = M.one(), more = 0;  // the first `rest` summands count whole + 1 times, the others whole times
+    const bool repeats = __any_sync(0xffffffffu, whole_s != 0);
+    if (repeats) {
+      const uint32_t ratio = s == 0 ? SumKind<K0>::kW : s == 1 ? SumKind<K0 + 1>::kW : SumKind<K0 + 2>::kW;
+      const bool alternates = s == 0 ? SumKind<K0>::kAlternates : s == 1 && SumKind<K0 + 1>::kAlternates;
+      // (where nothing repeats, q^2 may pass 64 bits: then `whole` is 0 and r is not used)
+      const uint64_t turn = (PRIME ? 1 : q % phi) * (period_s % phi) % phi * ratio;
+      T r = power_of_two<A>(M, exponent_mod(-static_cast<int64_t>(turn), phi));
+      if (alternates) r = M.neg(r);  // the period is odd
+      more = geometric<A>(M, r, whole_s);
+      once = M.add(M.mul(more, r), M.one());
     }
-    const bool repeats = (whole[0] | whole[1] | whole[2]) != 0;
+    auto of = [&](auto v, int k) { return __shfl_sync(0xffffffffu, v, k); };
     for (int pass = 0; pass < (repeats ? 2 : 1); ++pass) {
-      // pass 0: the first `rest` summands, whole + 1 times; pass 1: the others, whole times
       T num = 0, den = M.one();
       const bool f = pass == 0;
-      add_share<A, K0 + 0, PRIME>(M, p, q, phi, e, f ? 0 : rest[0], f ? rest[0] : period[0], period[0], whole[0] + f, lane, num, den);
-      add_share<A, K0 + 1, PRIME>(M, p, q, phi, e, f ? 0 : rest[1], f ? rest[1] : period[1], period[1], whole[1] + f, lane, num, den);
-      add_share<A, K0 + 2, PRIME>(M, p, q, phi, e, f ? 0 : rest[2], f ? rest[2] : period[2], period[2], whole[2] + f, lane, num, den);
+      const T factor = f ? once : more;
+      const uint64_t lo = f ? 0 : rest_s, hi = f ? rest_s : whole_s ? period_s : rest_s;
+      add_share<A, K0, PRIME>(M, p, q, phi, e, of(lo, 0), of(hi, 0), of(factor, 0), lane, num, den);
+      add_share<A, K0 + 1, PRIME>(M, p, q, phi, e, of(lo, 1), of(hi, 1), of(factor, 1), lane, num, den);
+      add_share<A, K0 + 2, PRIME>(M, p, q, phi, e, of(lo, 2), of(hi, 2), of(factor, 2), lane, num, den);
       const T x = M.plain(M.mul(num, inverse_times_power<A>(M, den, phi, 0)));  // every lane: warp-wide
       fold_one<A, LMAX>(M, x, acc);
     }
