@@ -2,8 +2,10 @@
 """Benchmark: BBP digit extraction of pi, n = 1e12, P = 256 (+64 guard bits), one GB300.
 
 One step is one whole query: every series of Bellard's formula (Eq. 2), head and
-tail terms, the exact reduction and the finalize (certified bits + output bytes),
-through the library's public API with host output buffers.  The device time of a
+tail terms, the exact reduction and the certified bits, through the library's public
+API with host output buffers.  The library sums the head terms by primes (partial
+fractions of their moduli): value counts the terms of the sum, and the roofline the
+multiplies of the prime form.  The device time of a
 step comes from CUDA events on the plan's stream; the end-to-end time is the
 wall clock around the same API call (it includes the device->host read of the
 result).  Between timed steps the L2 is flushed by writing a 256 MiB buffer.
@@ -437,23 +439,10 @@ def run_gpu(args):
                    "parallelism": f"k-range shards x{world}" if world > 1 else "single GPU"},
         "e2e": {"value": e2e_value, "unit": "terms/s", "h2d_bytes_per_step": 0,
                 "d2h_bytes_per_step": nbytes + 4,
-                "note": "bbp_bits with host output; the query (n, P) travels as kernel arguments"},
+                "note": "bbp_bits with host output; the query (n, P) travels as kernel arguments, the kernels "
+                        "write the result to pinned host memory"},
         "gpu_launches": launches,
-        "roofline": {"bound": "alu", "achieved": achieved_model, "peak": peak, "unit": "T IMAD/s",
-                     "frac": (achieved_model / peak) if achieved_model else None,
-                     "traffic": ncu.get("dram_bytes_per_launch"),
-                     "model": "per term: 16 ceil(log2 e) + 4L + 50 IMAD per two-limb term, 5 ceil(log2 e) + 3L + 25 "
-                              "per one-limb term, summed over the query's exponents",
-                     "achieved_half_products": achieved,
-                     "frac_half_products": (achieved / peak) if achieved else None,
-                     "half_products_model": "32-bit product halves the method needs: 13 per two-limb squaring "
-                                            "(14 when x1^2 needs its high word), 4 per one-limb squaring, 4 (2) per "
-                                            "quotient digit, 6 for m^-1 mod 2^32",
-                     "ncu_imad_pipe_frac": ncu.get("fma_pipe_frac_of_imad_rate"),
-                     "kernel": "head_kernel", "head_launches": head_launches,
-                     "peak_basis": f"{sms} SMs x {IMAD_LANES_PER_CLK_PER_SM} IMAD lanes/clk (mul.lo issue rate, "
-                                   f"measured) x {max_mhz:.0f} MHz; achieved = modelled multiplies of the "
-                                   "head terms / summed CUDA-event time of the head launches"},
+        "roofline": roofline(sms, peak, max_mhz, achieved, achieved_model, ncu, head_launches, world),
         "cpu_baseline": cpu,
         "clocks": clocks,
         "verified": verified,
@@ -461,6 +450,35 @@ def run_gpu(args):
     })
     if world > 1:
         dist.destroy_process_group()
+
+
+def roofline(sms, peak, max_mhz, achieved, achieved_terms, ncu, launches, world) -> dict:
+    """The bench line's roofline object.  One GPU: the query is summed by primes, whose modelled
+    32-bit product halves are the achieved work; the multiplies that the terms would take one by
+    one, over the same time, are given beside it and are no rate of executed work.  Several
+    GPUs: each sums its shard term by term."""
+    basis = (f"{sms} SMs x {IMAD_LANES_PER_CLK_PER_SM} IMAD lanes/clk (mul.lo issue rate, measured) x "
+             f"{max_mhz:.0f} MHz; achieved = modelled multiplies / summed CUDA-event time of the head launches")
+    out = {"bound": "alu", "peak": peak, "unit": "T IMAD/s", "traffic": ncu.get("dram_bytes_per_launch"),
+           "head_launches": launches, "peak_basis": basis}
+    if world == 1:
+        out.update({
+            "achieved": achieved, "frac": (achieved / peak) if achieved else None,
+            "kernel": "prime_kernel, prime_sum_kernel, prime_power_kernel, sieve_kernel",
+            "model": "32-bit product halves of the prime form: per prime above A / 23 13 per two-limb or 4 per "
+                     "one-limb squaring of its ladder, 4 or 2 per quotient digit, 22 or 16 for the inverse and the "
+                     "product with H; per prime below two ladders and 12 per summand; primes counted as the "
+                     "integral of 1 / ln x; the sieve is not counted",
+            "term_by_term_equivalent": (achieved_terms / peak) if achieved_terms else None})
+    else:
+        out.update({
+            "achieved": achieved_terms, "frac": (achieved_terms / peak) if achieved_terms else None,
+            "kernel": "head_kernel",
+            "model": "per term: 16 ceil(log2 e) + 4L + 50 IMAD per two-limb term, 5 ceil(log2 e) + 3L + 25 per "
+                     "one-limb term, summed over the query's exponents",
+            "achieved_half_products": achieved, "frac_half_products": (achieved / peak) if achieved else None,
+            "ncu_imad_pipe_frac": ncu.get("fma_pipe_frac_of_imad_rate")})
+    return out
 
 
 # ---------------------------------------------------------------- batched workload

@@ -480,12 +480,24 @@ __device__ __forceinline__ void prime_sum(const Arith1& M, uint32_t n, uint32_t 
     const uint32_t start = n >> 1, d_start = pair_sign<KIND>(M, d0);
     uint32_t d = pair_sign<KIND>(M, D);
     const bool late = n <= i;  // starts within the pairs
-    for (uint32_t h = i / 2; h > 0; --h) {
+    // down to where every lane has started, then without looking
+    const uint32_t all = min(i / 2u, __reduce_min_sync(0xffffffffu, start));
+    uint32_t h = i / 2;
+    for (; h > all; --h) {
       if (late && h == start) {
         N = n0;
         d = d_start;
       }
       sum_pair<KIND>(M, K::kStride * (2u * h - 1u) + first, N, d);
+    }
+    if (late && h == start) {
+      N = n0;
+      d = d_start;
+    }
+    uint32_t c = K::kStride * (2u * h - 1u) + first;
+    for (; h > 0; --h) {
+      sum_pair<KIND>(M, c, N, d);
+      c -= 2u * K::kStride;
     }
     D = pair_sign<KIND>(M, d);
     if (late && start == 0u) {  // n = 1 (or none): no pair
@@ -502,7 +514,8 @@ __device__ __forceinline__ void prime_sum(const Arith1& M, uint32_t n, uint32_t 
 }
 
 // The same over lo <= i < hi, relative to the term at lo (w num / den with w^-(i - lo)), lo
-// even, each lane with its own range; the lanes walk them in step.
+// even, each lane with its own range; the lanes walk them in step, and none looks for its
+// start once all have started.
 template <int KIND>
 __device__ __forceinline__ void range_sum(const Arith1& M, uint32_t lo, uint32_t hi, uint32_t c0, uint32_t& num,
                                           uint32_t& den) {
@@ -514,32 +527,49 @@ __device__ __forceinline__ void range_sum(const Arith1& M, uint32_t lo, uint32_t
   if (pairs) {
     uint32_t n0, d0;
     pair_start<KIND>(M, hi, first, n0, d0);
-    const uint32_t start = hi / 2u, d_start = pair_sign<KIND>(M, d0);
+    const uint32_t d_start = pair_sign<KIND>(M, d0);
     uint32_t k = (steps + 1u) / 2u;
-    uint32_t h = lo / 2u + k;  // the pair (2 h - 2, 2 h - 1)
-    uint32_t c = K::kStride * (2u * h - 1u) + first, d = 1;
-    for (; k > 0u; --k, --h) {
-      if (h == start) {
+    uint32_t c = K::kStride * (2u * (lo / 2u + k) - 1u) + first, d = 1;
+    const uint32_t mine = (hi - lo) / 2u, all = __reduce_min_sync(0xffffffffu, hi > lo ? mine : k);
+    auto begin = [&] {
+      if (k == mine) {
         N = n0;
         d = d_start;
       }
+    };
+    for (; k > all; --k) {
+      begin();
+      sum_pair<KIND>(M, c, N, d);
+      c -= 2u * K::kStride;
+    }
+    begin();
+    for (; k > 0u; --k) {
       sum_pair<KIND>(M, c, N, d);
       c -= 2u * K::kStride;
     }
     D = pair_sign<KIND>(M, d);
-    if (start == lo / 2u) {  // one term, or none
+    if (mine == 0u) {  // one term, or none
       N = n0;
       D = d0;
     }
   } else {
-    uint32_t i = lo + steps;
-    for (uint32_t k = steps; k > 0u; --k) {
-      if (i == hi) {
+    uint32_t k = steps, c = K::kStride * (lo + steps) + first;
+    const uint32_t mine = hi - lo, all = __reduce_min_sync(0xffffffffu, hi > lo ? mine : k);
+    auto begin = [&] {
+      if (k == mine) {
         N = 0;
         D = 1;
       }
-      --i;
-      sum_step<KIND>(M, i, K::kStride * i + first, N, D);
+    };
+    for (; k > all; --k) {
+      begin();
+      c -= K::kStride;
+      sum_step<KIND>(M, lo + k - 1u, c, N, D);
+    }
+    begin();
+    for (; k > 0u; --k) {
+      c -= K::kStride;
+      sum_step<KIND>(M, lo + k - 1u, c, N, D);
     }
   }
   if (hi <= lo) {
@@ -552,25 +582,28 @@ __device__ __forceinline__ void range_sum(const Arith1& M, uint32_t lo, uint32_t
 }
 
 // The sum over 0 <= i < n shared by GROUP neighbouring lanes with the same prime: each takes
-// an even number s of terms, and the fractions are put together two by two,
+// about as many terms, an even number but for the last, and the fractions are put together
+// two by two, w^s with the s terms of the lower one:
 //   w num / den = w (num den' w^s + num' den) / (den den' w^s).
 // The group's first lane has the result.
 template <int KIND, int GROUP>
 __device__ __forceinline__ void group_sum(const Arith1& M, uint32_t n, uint32_t c0, uint32_t& num, uint32_t& den) {
-  const uint32_t share = ((n + GROUP - 1) / GROUP + 1u) & ~1u;
-  uint32_t lo = (threadIdx.x & (GROUP - 1)) * share, hi = min(n, lo + share);
-  if (lo >= n) lo = hi = 0;
+  const uint32_t g = threadIdx.x & (GROUP - 1), share = n / GROUP & ~1u;
+  const uint32_t extra = (n & ~1u) - share * GROUP;  // even: two more for the first lanes
+  const uint32_t lo = share * g + min(2u * g, extra);
+  const uint32_t hi = g == GROUP - 1 ? n : lo + share + (2u * g < extra ? 2u : 0u);
   range_sum<KIND>(M, lo, hi, c0, num, den);
-  uint32_t z = M.one(), e = SumKind<KIND>::kW * share;  // w^s
+  uint32_t z = M.one(), e = SumKind<KIND>::kW * (hi - lo);  // w^s
   const int bits = 32 - __clz(static_cast<int>(__reduce_max_sync(0xffffffffu, e)));
   for (int b = bits - 1; b >= 0; --b) z = M.mul(z, (e >> b) & 1u ? z + z : z);
 #pragma unroll
   for (int d = 1; d < GROUP; d <<= 1) {
     const uint32_t num2 = __shfl_down_sync(0xffffffffu, num, d, GROUP);
     const uint32_t den2 = __shfl_down_sync(0xffffffffu, den, d, GROUP);
+    const uint32_t z2 = __shfl_down_sync(0xffffffffu, z, d, GROUP);
     num = M.add(M.mul(M.mul(num, z), den2), M.mul(den, num2));
     den = M.mul(M.mul(den, z), den2);
-    z = M.mul(z, z);
+    z = M.mul(z, z2);
   }
 }
 
@@ -591,15 +624,19 @@ __device__ __forceinline__ void prime_share(const Arith1& M, uint32_t lo, uint32
   using K = SumKind<KIND>;
   const uint32_t steps = __reduce_max_sync(0xffffffffu, hi > lo ? hi - lo : 0u);
   const uint32_t first = K::kStride == 2u ? 1u : c0;
-  uint32_t i = lo + steps, N = 0, D = 1;
+  uint32_t k = steps, N = 0, D = 1;
+  uint32_t last = K::kStride * (lo + steps) + first;  // one stride above c
   uint32_t skip = hi > lo ? static_cast<uint32_t>(last_multiple<KIND>(K::kStride * (hi - 1u) + first, p, first)) : 0u;
-  for (uint32_t k = steps; k > 0; --k) {
-    if (i == hi) {
+  const uint32_t mine = hi > lo ? hi - lo : 0u, all = __reduce_min_sync(0xffffffffu, mine ? mine : k);
+  auto begin = [&] {
+    if (k == mine) {
       N = 0;
       D = 1;
     }
-    --i;
-    uint32_t c = K::kStride * i + first, add = D;
+  };
+  auto step = [&] {
+    last -= K::kStride;
+    uint32_t c = last, add = D;
     if (c == skip) {
       c = 1u;
       add = 0u;
@@ -610,11 +647,17 @@ __device__ __forceinline__ void prime_share(const Arith1& M, uint32_t lo, uint32
                             : static_cast<uint64_t>(M.lazy_redc(static_cast<uint64_t>(D) * c)) * h;
     if (K::kInTwos) {
       const uint32_t r = M.lazy_redc(t);
-      D = (i & 1u) ? r : 2u * M.m - r;
+      D = ((lo + k - 1u) & 1u) ? r : 2u * M.m - r;
     } else {
       D = K::kAlternates ? M.lazy_redc_neg(t) : M.lazy_redc(t);
     }
+  };
+  for (; k > all; --k) {
+    begin();
+    step();
   }
+  begin();
+  for (; k > 0u; --k) step();
   if (hi <= lo) {
     N = 0;
     D = 1;
