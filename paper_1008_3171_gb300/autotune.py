@@ -13,9 +13,9 @@ Sweeps the launch parameters the C ABI reads from a tune table
 * grab          -- warp tiles handed out per queue operation in batched passes.
 
 run x streams, then cta, then limb_bump are timed on a slice of the n = 1e12
-query (series 0, 1e9 terms of the 64-bit path); wide_min_bits on the whole
-n = 3e9, P = 128 query (moduli up to 2^31.5, so every crossover moves terms);
-grab on a seeded calibration batch.
+query (series 0, 1e9 terms of the 64-bit path); wide_min_bits on the seven
+series of the n = 3e9, P = 128 query, term by term (moduli up to 2^31.5, so every
+crossover moves terms); grab on a seeded calibration batch.
 Every setting computes bit-identical results (the sum is exact; the sweep checks
 it), so only time is compared.
 
@@ -126,9 +126,12 @@ def tune(out_path: str, slice_terms: int = 1_000_000_000, batch: int = 512) -> d
     setting["cta"] = _sweep(bbp, "cta", CTAS, setting, slice_work, measured)
     setting["limb_bump"] = _sweep(bbp, "limb_bump", LIMB_BUMPS, setting, slice_work, measured)
 
-    def n3e9_work(p):
-        v = p.bits(3 * 10**9, 128)
-        return v, p.stats()["terms"]
+    def n3e9_work(p):  # whole queries are summed by primes: the series one by one are not
+        terms, sums = 0, []
+        for j in range(7):
+            sums.append(p.partial_sum(0, j, 0, None, 3 * 10**9, 128))
+            terms += p.stats()["terms"]
+        return sums, terms
 
     setting["wide_min_bits"] = _sweep(bbp, "wide_min_bits", WIDE_MIN_BITS, setting, n3e9_work, measured, reps=5)
     ns, Ps = workloads.batched_queries(count=batch, seed=3, lo=4.0, hi=8.5)
