@@ -57,16 +57,22 @@ cudaError_t launch_query_t(const QuerySet& q, int blocks, int threads, cudaStrea
 }
 
 template <typename K>
-cudaError_t launch_prime_t(K kernel, const PrimeArgs& a, int sms, cudaStream_t s) {
+cudaError_t launch_prime_t(K kernel, const PrimeArgs& a, int sms, cudaStream_t s, int most = 32) {
   // the sieve's CTAs need the SM's shared memory while these run
   cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributePreferredSharedMemoryCarveout,
                                        cudaSharedmemCarveoutMaxShared);
   int n = 0;
   if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, kernel, kHeadThreads, 0);
   if (e != cudaSuccess) return e;
-  kernel<<<std::max(1, n) * sms, kHeadThreads, 0, s>>>(a);
+  kernel<<<std::max(1, std::min(n, most)) * sms, kHeadThreads, 0, s>>>(a);
   return cudaGetLastError();
 }
+
+// prime_kernel's CTAs per SM: two of the four that fit, so that the next list's sieve has
+// registers all along.  With four the sieve, of higher priority, takes most of the SM until it
+// is done, and the rest runs alone: n = 4e10 86.4 ms, with three 84.9, two 83.5 (although the
+// lists alone, nothing beside them, take 57.9 ms with two and 55.0 with four).
+constexpr int kPrimeCtas = 2;
 
 }  // namespace
 
@@ -74,10 +80,10 @@ cudaError_t BBP_CAT(launch_prime_l, BBP_LMAX)(const PrimeArgs& a, PrimeKernel k,
                                               cudaStream_t s) {
   const bool f = formula != 0;
   switch (k) {
-    case kPrimes0: return launch_prime_t(prime_kernel<BBP_LMAX, 0, false>, a, sms, s);
-    case kPrimes1: return launch_prime_t(prime_kernel<BBP_LMAX, 1, false>, a, sms, s);
-    case kPrimesHalf: return launch_prime_t(prime_kernel<BBP_LMAX, 1, true>, a, sms, s);
-    case kPrimes3: return launch_prime_t(prime_kernel<BBP_LMAX, 3, false>, a, sms, s);
+    case kPrimes0: return launch_prime_t(prime_kernel<BBP_LMAX, 0, false>, a, sms, s, kPrimeCtas);
+    case kPrimes1: return launch_prime_t(prime_kernel<BBP_LMAX, 1, false>, a, sms, s, kPrimeCtas);
+    case kPrimesHalf: return launch_prime_t(prime_kernel<BBP_LMAX, 1, true>, a, sms, s, kPrimeCtas);
+    case kPrimes3: return launch_prime_t(prime_kernel<BBP_LMAX, 3, false>, a, sms, s, kPrimeCtas);
     case kSums32: return launch_prime_t(f ? prime_sum_kernel<Arith1, 1, 32, BBP_LMAX> : prime_sum_kernel<Arith1, 0, 32, BBP_LMAX>, a, sms, s);
     case kSums8: return launch_prime_t(f ? prime_sum_kernel<Arith1, 1, 8, BBP_LMAX> : prime_sum_kernel<Arith1, 0, 8, BBP_LMAX>, a, sms, s);
     case kSums1: return launch_prime_t(f ? prime_sum_kernel<Arith1, 1, 1, BBP_LMAX> : prime_sum_kernel<Arith1, 0, 1, BBP_LMAX>, a, sms, s);
