@@ -71,7 +71,8 @@ cudaError_t launch_prime_t(K kernel, const PrimeArgs& a, int sms, cudaStream_t s
 // prime_kernel's CTAs per SM: two of the four that fit, so that the next list's sieve has
 // registers all along.  With four the sieve, of higher priority, takes most of the SM until it
 // is done, and the rest runs alone: n = 4e10 86.4 ms, with three 84.9, two 83.5 (although the
-// lists alone, nothing beside them, take 57.9 ms with two and 55.0 with four).
+// lists alone, nothing beside them, take 57.9 ms with two and 55.0 with four; all with four
+// primes a thread, kPrimeNT).
 constexpr int kPrimeCtas = 2;
 
 }  // namespace
