@@ -217,9 +217,11 @@ __device__ __forceinline__ uint32_t take_primes(uint32_t* taken, uint32_t n, uin
 
 // Primes per thread: independent chains that keep the multiply pipe fed at two CTAs an SM
 // (n = 4e10, two words: 83.5 ms with four, 82.4 with five, 84.8 with six; one word: 1.745 ms
-// at n = 1e9 with four, 1.751 with five).
-template <int PATH>
-constexpr int kPrimeNT = PathTraits<PATH>::kWide ? 5 : 4;
+// at n = 1e9 with four, 1.751 with five).  With 16 or 24 accumulator limbs the fifth takes the
+// registers that the sieve runs in (n = 1e10, P = 400 and 600: 21.2 and 22.7 ms with four, 21.4
+// and 24.1 with five); with 40 there are none for it either way (P = 1000: 27.4, 26.7 ms).
+template <int LMAX, int PATH>
+constexpr int kPrimeNT = PathTraits<PATH>::kWide && (LMAX <= 10 || LMAX == 40) ? 5 : 4;
 
 template <int LMAX, int PATH, bool HALF>
 __global__ void __launch_bounds__(kHeadThreads) prime_kernel(const __grid_constant__ PrimeArgs A) {
@@ -227,7 +229,7 @@ __global__ void __launch_bounds__(kHeadThreads) prime_kernel(const __grid_consta
   for (uint32_t i = threadIdx.x; i < A.nclasses * (sizeof(PrimeClass) / 4); i += blockDim.x)
     reinterpret_cast<uint32_t*>(classes)[i] = reinterpret_cast<const uint32_t*>(A.classes)[i];
   __syncthreads();
-  constexpr int NT = kPrimeNT<PATH>;
+  constexpr int NT = kPrimeNT<LMAX, PATH>;
   const uint32_t lane = threadIdx.x & 31u;
   const uint32_t count = min(*A.count, A.cap);
   uint32_t acc[LMAX];
