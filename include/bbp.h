@@ -142,7 +142,11 @@ bbp_status bbp_bits_formula(bbp_plan p, bbp_formula f, uint64_t n, uint32_t P, u
 /* Device-pointer form: d_out (ceil(P/8) bytes), d_valid (one uint32, may be NULL)
  * and d_limbs (W/32 uint32 of the raw sum, may be NULL) are caller-owned device
  * memory; returns once queued on `stream` (NULL: the plan's stream).  With d_limbs the
- * terms are summed one by one (the raw sum holds every term's rounding). */
+ * terms are summed one by one (the raw sum holds every term's rounding).
+ * Under stream capture the call allocates nothing: a plan without the buffers that the sum
+ * over primes needs at this n (a query of the same n or a larger one makes them) has the
+ * terms captured.  The graph may be replayed until the plan is destroyed, whatever the
+ * plan does in between; as with every use of a plan, one replay or call at a time. */
 bbp_status bbp_bits_async(bbp_plan p, bbp_formula f, uint64_t n, uint32_t P, uint8_t* d_out,
                           uint32_t* d_valid, uint32_t* d_limbs, void* stream);
 

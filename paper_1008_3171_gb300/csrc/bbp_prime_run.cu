@@ -42,6 +42,14 @@ uint64_t isqrt(uint64_t v) {
 struct PrimeState {
   uint32_t* list[2] = {};
   uint32_t list_cap = 0;
+  // A capture has recorded the lists: a graph may be replayed while the plan lives, so lists
+  // that are replaced by longer ones are kept until it goes.  Those are at least twice as long
+  // then, from 1.1e6 to 2.5e7 primes: no more than kKeptLists are ever kept, together less than
+  // twice the longest.
+  static constexpr int kKeptLists = 12;
+  bool captured = false;
+  int nkept = 0;
+  uint32_t* kept[kKeptLists] = {};
   uint32_t* primes = nullptr;  // base primes
   bbp::SievePrime* sieve_primes = nullptr;
   // [0] base primes, [1] those from 17 on; then the length of each list, then the primes of
@@ -89,6 +97,7 @@ void release_prime_state(PrimeState** state) {
   if (s->sieve) cudaStreamDestroy(s->sieve);
   if (s->sums) cudaStreamDestroy(s->sums);
   for (uint32_t* l : s->list) cudaFree(l);
+  for (uint32_t* l : s->kept) cudaFree(l);
   cudaFree(s->primes);
   cudaFree(s->sieve_primes);
   cudaFree(s->counts);
@@ -99,13 +108,18 @@ void release_prime_state(PrimeState** state) {
 bool prime_workspace(PrimeState** state, uint64_t n, uint32_t max_list, cudaStream_t st) {
   // primes of one list: all of them up to the limit
   const double x = static_cast<double>(n);
-  const uint32_t want = static_cast<uint32_t>(std::min<double>(max_list, 1.2 * x / std::log(x) + 4096.0));
-  if (*state && (*state)->list_cap >= want) return true;
+  uint32_t want = static_cast<uint32_t>(std::min<double>(max_list, 1.2 * x / std::log(x) + 4096.0));
   cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-  if (cudaStreamIsCapturing(st, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone) {
+  if (cudaStreamIsCapturing(st, &cap) != cudaSuccess) {
     cudaGetLastError();
     return false;
   }
+  const bool capturing = cap != cudaStreamCaptureStatusNone;
+  if (*state && (*state)->list_cap >= want) {
+    (*state)->captured |= capturing;
+    return true;
+  }
+  if (capturing) return false;
   if (!*state) {
     *state = new (std::nothrow) PrimeState();
     if (!*state) return false;
@@ -116,6 +130,15 @@ bool prime_workspace(PrimeState** state, uint64_t n, uint32_t max_list, cudaStre
     }
   }
   PrimeState* s = *state;
+  if (s->captured) {
+    if (s->nkept + 2 > PrimeState::kKeptLists) return false;
+    want = std::max(want, std::min(max_list, 2 * s->list_cap));
+    for (uint32_t*& l : s->list) {
+      s->kept[s->nkept++] = l;
+      l = nullptr;
+    }
+    s->captured = false;
+  }
   s->list_cap = 0;
   for (uint32_t*& l : s->list) {
     cudaFree(l);  // waits for the work that reads it

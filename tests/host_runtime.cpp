@@ -1,0 +1,338 @@
+// The library's host runtime (plans, queries by primes, batches, serving) on a CUDA runtime
+// that only keeps books: which allocations live, which operation of a stream comes after
+// which, what a capture has recorded.  Kernels do nothing.  Run with the name of a case;
+// exits 0 if it holds (test_host_runtime.py).
+#include <cuda_runtime.h>
+
+#include <cstdio>
+#include <cstdlib>
+#include <cstring>
+#include <map>
+#include <mutex>
+#include <set>
+#include <string>
+#include <thread>
+#include <vector>
+
+#include "bbp.h"
+#include "bbp_kernels.cuh"
+#include "bbp_sieve.cuh"
+
+namespace {
+
+std::recursive_mutex mu;  // the serving engine has a thread of its own
+
+struct Op {
+  std::string what;
+  std::vector<size_t> after;
+  std::vector<const void*> reads;
+  bool captured = false, complete = false;
+};
+struct Stream {
+  long last = -1, last_real = -1;
+  bool capturing = false;
+};
+struct Event {
+  long op = -1;
+};
+std::vector<Op> ops;
+std::set<Stream*> streams;
+std::map<const void*, size_t> live;
+int sms = 152;
+uint32_t verdict = 0;                      // what the prime form's check says
+std::map<std::string, int> calls, fail_at;  // fails from that call on (negative: that call alone)
+
+#define REQUIRE(x)                                              \
+  do {                                                          \
+    if (!(x)) {                                                 \
+      std::printf("line %d: %s does not hold\n", __LINE__, #x); \
+      std::exit(1);                                             \
+    }                                                           \
+  } while (0)
+
+bool fails(const std::string& name) {
+  std::lock_guard<std::recursive_mutex> l(mu);
+  const int k = ++calls[name];
+  const auto f = fail_at.find(name);
+  return f != fail_at.end() && (f->second < 0 ? k == -f->second : k >= f->second);
+}
+
+Stream* of(cudaStream_t s) { return reinterpret_cast<Stream*>(s); }
+
+cudaError_t add(cudaStream_t st, const std::string& what, std::vector<const void*> reads = {}, long also_after = -1) {
+  std::lock_guard<std::recursive_mutex> l(mu);
+  Stream* s = of(st);
+  REQUIRE(streams.count(s));
+  for (const void* p : reads) REQUIRE(!p || live.count(p));
+  Op op;
+  op.what = what;
+  op.reads = reads;
+  if (s->last >= 0) op.after.push_back(static_cast<size_t>(s->last));
+  if (also_after >= 0) op.after.push_back(static_cast<size_t>(also_after));
+  op.captured = s->capturing;
+  ops.push_back(op);
+  s->last = static_cast<long>(ops.size()) - 1;
+  if (!s->capturing) s->last_real = s->last;
+  return cudaSuccess;
+}
+
+std::vector<bool> before(long op) {  // the operations that have ended when `op` has
+  std::vector<bool> in(ops.size(), false);
+  std::vector<size_t> todo;
+  if (op >= 0) todo.push_back(static_cast<size_t>(op));
+  while (!todo.empty()) {
+    const size_t i = todo.back();
+    todo.pop_back();
+    if (in[i]) continue;
+    in[i] = true;
+    for (size_t a : ops[i].after) todo.push_back(a);
+  }
+  return in;
+}
+
+cudaError_t wait_for(long op) {
+  std::lock_guard<std::recursive_mutex> l(mu);
+  const std::vector<bool> in = before(op);
+  for (size_t i = 0; i < ops.size(); ++i)
+    if (in[i]) ops[i].complete = true;
+  return cudaSuccess;
+}
+
+// What torch.cuda.graph does around a call
+void begin_capture(cudaStream_t s) {
+  of(s)->capturing = true;
+  of(s)->last = -1;
+}
+void end_capture() {
+  for (Stream* s : streams) {
+    s->capturing = false;
+    s->last = s->last_real;
+  }
+}
+
+size_t in_flight() {
+  size_t n = 0;
+  for (const Op& o : ops) n += !o.complete && !o.captured;
+  return n;
+}
+
+}  // namespace
+
+extern "C" {
+
+cudaError_t cudaGetDeviceCount(int* n) { *n = 1; return cudaSuccess; }
+cudaError_t cudaSetDevice(int) { return cudaSuccess; }
+cudaError_t cudaGetLastError() { return cudaSuccess; }
+cudaError_t cudaGetDeviceProperties(cudaDeviceProp* p, int) {
+  std::memset(p, 0, sizeof(*p));
+  p->multiProcessorCount = sms;
+  return cudaSuccess;
+}
+cudaError_t cudaDeviceGetStreamPriorityRange(int* a, int* b) { *a = 0; *b = -5; return cudaSuccess; }
+
+cudaError_t cudaMalloc(void** p, size_t n) {
+  if (fails("cudaMalloc")) return cudaErrorMemoryAllocation;
+  std::lock_guard<std::recursive_mutex> l(mu);
+  *p = std::calloc(1, n ? n : 1);
+  live[*p] = n;
+  return cudaSuccess;
+}
+cudaError_t cudaFree(void* p) {
+  std::lock_guard<std::recursive_mutex> l(mu);
+  if (!p) return cudaSuccess;
+  REQUIRE(live.erase(p) == 1);
+  for (Op& o : ops) o.complete |= !o.captured;  // waits for the device
+  return cudaSuccess;  // the memory stays, so that no address comes back
+}
+cudaError_t cudaMallocHost(void** p, size_t n) { *p = std::calloc(1, n ? n : 1); return cudaSuccess; }
+cudaError_t cudaHostAlloc(void** p, size_t n, unsigned int) { return cudaMallocHost(p, n); }
+cudaError_t cudaFreeHost(void* p) { std::free(p); return cudaSuccess; }
+
+cudaError_t cudaStreamCreateWithPriority(cudaStream_t* s, unsigned int, int) {
+  std::lock_guard<std::recursive_mutex> l(mu);
+  Stream* n = new Stream();
+  streams.insert(n);
+  *s = reinterpret_cast<cudaStream_t>(n);
+  return cudaSuccess;
+}
+cudaError_t cudaStreamCreateWithFlags(cudaStream_t* s, unsigned int) { return cudaStreamCreateWithPriority(s, 0, 0); }
+cudaError_t cudaStreamDestroy(cudaStream_t s) {
+  std::lock_guard<std::recursive_mutex> l(mu);
+  REQUIRE(streams.erase(of(s)) == 1);
+  return cudaSuccess;
+}
+cudaError_t cudaStreamSynchronize(cudaStream_t s) { return wait_for(of(s)->last_real); }
+cudaError_t cudaStreamIsCapturing(cudaStream_t s, cudaStreamCaptureStatus* c) {
+  *c = of(s)->capturing ? cudaStreamCaptureStatusActive : cudaStreamCaptureStatusNone;
+  return cudaSuccess;
+}
+cudaError_t cudaStreamWaitEvent(cudaStream_t st, cudaEvent_t e, unsigned int) {
+  std::lock_guard<std::recursive_mutex> l(mu);
+  const long op = reinterpret_cast<Event*>(e)->op;
+  if (op < 0) return cudaSuccess;
+  Stream* s = of(st);
+  const bool captured = ops[static_cast<size_t>(op)].captured;
+  if (captured && !s->capturing) {  // the stream joins the capture that is going on
+    bool any = false;
+    for (Stream* o : streams) any |= o->capturing;
+    if (!any) return cudaErrorCapturedEvent;
+    s->capturing = true;
+    s->last = -1;
+  }
+  if (s->capturing && !captured) return cudaErrorStreamCaptureIsolation;
+  return add(st, "wait", {}, op);
+}
+
+cudaError_t cudaEventCreateWithFlags(cudaEvent_t* e, unsigned int) {
+  *e = reinterpret_cast<cudaEvent_t>(new Event());
+  return cudaSuccess;
+}
+cudaError_t cudaEventCreate(cudaEvent_t* e) { return cudaEventCreateWithFlags(e, 0); }
+cudaError_t cudaEventDestroy(cudaEvent_t e) { delete reinterpret_cast<Event*>(e); return cudaSuccess; }
+cudaError_t cudaEventRecord(cudaEvent_t e, cudaStream_t s) {
+  std::lock_guard<std::recursive_mutex> l(mu);
+  if (of(s)->last < 0) add(s, "nothing");
+  reinterpret_cast<Event*>(e)->op = of(s)->last;
+  return cudaSuccess;
+}
+cudaError_t cudaEventSynchronize(cudaEvent_t e) { return wait_for(reinterpret_cast<Event*>(e)->op); }
+cudaError_t cudaEventElapsedTime(float* ms, cudaEvent_t, cudaEvent_t) { *ms = 1.0f; return cudaSuccess; }
+
+cudaError_t cudaMemsetAsync(void* p, int v, size_t n, cudaStream_t s) {
+  if (n && !of(s)->capturing) std::memset(p, v, n);
+  return add(s, "memset");
+}
+cudaError_t cudaMemcpyAsync(void* d, const void* src, size_t n, cudaMemcpyKind, cudaStream_t s) {
+  if (n && !of(s)->capturing) std::memcpy(d, src, n);
+  return add(s, "memcpy");
+}
+
+cudaError_t cudaStreamBeginCapture(cudaStream_t s, cudaStreamCaptureMode) {
+  begin_capture(s);
+  return cudaSuccess;
+}
+cudaError_t cudaStreamEndCapture(cudaStream_t s, cudaGraph_t* g) {
+  of(s)->capturing = false;
+  of(s)->last = of(s)->last_real;
+  *g = reinterpret_cast<cudaGraph_t>(1);
+  return cudaSuccess;
+}
+cudaError_t cudaGraphInstantiate(cudaGraphExec_t* e, cudaGraph_t, unsigned long long) {
+  *e = reinterpret_cast<cudaGraphExec_t>(1);
+  return cudaSuccess;
+}
+cudaError_t cudaGraphExecUpdate(cudaGraphExec_t, cudaGraph_t, cudaGraphExecUpdateResultInfo*) { return cudaSuccess; }
+cudaError_t cudaGraphLaunch(cudaGraphExec_t, cudaStream_t s) { return add(s, "graph"); }
+cudaError_t cudaGraphDestroy(cudaGraph_t) { return cudaSuccess; }
+cudaError_t cudaGraphExecDestroy(cudaGraphExec_t) { return cudaSuccess; }
+
+}  // extern "C"
+
+namespace bbp {
+
+int head_lmax_for(int L, int bump) {
+  if (fails("head_lmax_for")) return 0;
+  for (int i = 0; i < kNumLmaxClasses; ++i)
+    if (kLmaxClasses[i] >= L) return kLmaxClasses[std::min(i + bump, kNumLmaxClasses - 1)];
+  return 0;
+}
+int head_occupancy(int, int, int, int) { return 2; }
+int query_occupancy(int, int, int) { return 2; }
+int queue_occupancy(int, int, int) { return 2; }
+cudaError_t launch_head(const HeadArgs& a, int, int, int, int, cudaStream_t s, int) { return add(s, "head", {a.slots}); }
+cudaError_t launch_tail_set(const TailSet&, cudaStream_t s) { return add(s, "tails"); }
+cudaError_t launch_query(const QuerySet& q, int, int, int, int, cudaStream_t s) { return add(s, "query", {q.slots}); }
+cudaError_t launch_zero_slots(unsigned long long* p, int, cudaStream_t s, const uint32_t*) { return add(s, "zero", {p}); }
+cudaError_t launch_fold_limbs(const unsigned long long* p, int, uint32_t*, cudaStream_t s) { return add(s, "fold", {p}); }
+cudaError_t launch_finalize_bits(const unsigned long long* p, int, uint32_t, uint64_t, uint8_t*, uint32_t*, uint32_t*,
+                                 cudaStream_t s, const uint32_t*) {
+  return add(s, "finalize", {p});
+}
+cudaError_t launch_queue(const BatchDev& b, uint32_t, uint32_t, unsigned long long*, int, int, int, int, cudaStream_t s) {
+  return add(s, "queue", {b.accum});
+}
+cudaError_t launch_queue_tail(const BatchDev& b, uint32_t, uint32_t, unsigned long long*, int, cudaStream_t s) {
+  return add(s, "queue tails", {b.accum});
+}
+cudaError_t launch_timestamp(unsigned long long*, cudaStream_t s) { return add(s, "time"); }
+cudaError_t launch_imad_probe(int, int, int, int, unsigned long long*, uint32_t*, uint32_t*, cudaStream_t s) {
+  return add(s, "probe");
+}
+cudaError_t launch_base_primes(uint32_t, uint32_t* p, SievePrime* sp, uint32_t* c, uint32_t*, cudaStream_t s) {
+  return add(s, "base", {p, sp, c});
+}
+cudaError_t launch_sieve(const SieveArgs& a, int, cudaStream_t s) { return add(s, "sieve", {a.list}); }
+cudaError_t launch_prime(const PrimeArgs& a, PrimeKernel, int, int, int, cudaStream_t s) {
+  if (fails("launch_prime")) return cudaErrorLaunchOutOfResources;
+  return add(s, "primes", {a.list});
+}
+cudaError_t launch_prime_check(const unsigned long long* slots, int, uint32_t, uint64_t, const uint32_t*, uint32_t, uint32_t,
+                               uint8_t*, uint32_t*, uint32_t* redo, cudaStream_t s) {
+  *redo = verdict;
+  (void)slots;
+  return add(s, "check");
+}
+
+}  // namespace bbp
+
+namespace {
+
+struct Caller {
+  bbp_plan plan = nullptr;
+  cudaStream_t a = nullptr, b = nullptr;
+  void* out = nullptr;
+  Caller() {
+    REQUIRE(bbp_plan_create(&plan, nullptr) == BBP_OK);
+    cudaStreamCreateWithFlags(&a, 0);
+    cudaStreamCreateWithFlags(&b, 0);
+    cudaMalloc(&out, 256);
+  }
+  bbp_status async(uint64_t n, cudaStream_t s) {
+    return bbp_bits_async(plan, BBP_BELLARD, n, 128, static_cast<uint8_t*>(out), nullptr, nullptr, s);
+  }
+  bbp_status bits(uint64_t n, bbp_formula f = BBP_BELLARD) {
+    uint8_t bytes[160];
+    return bbp_bits_formula(plan, f, n, 128, bytes, nullptr);
+  }
+};
+
+// A captured query by primes, then larger ones that need longer lists, captured again and
+// again: what the captures use is there until the plan goes, and goes with it.  What is held
+// stays bounded.
+void captured_lists_stay() {
+  const size_t outside = 1;  // Caller::out
+  Caller c;
+  REQUIRE(c.bits(17'000'000) == BBP_OK);
+  uint64_t largest = 0;
+  for (uint64_t n = 17'000'000; n < 2'000'000'000; n += n / 9) {
+    begin_capture(c.a);
+    REQUIRE(c.async(n, c.a) == BBP_OK);
+    end_capture();
+    REQUIRE(c.bits(n + n / 9) == BBP_OK);
+    for (const Op& o : ops)
+      if (o.captured)
+        for (const void* p : o.reads) REQUIRE(!p || live.count(p));
+    size_t held = 0;
+    for (const auto& m : live) held += m.second;
+    largest = std::max<uint64_t>(largest, held);
+  }
+  size_t captured = 0;
+  for (const Op& o : ops) captured += o.captured && o.what == "sieve";
+  REQUIRE(captured > 0);
+  REQUIRE(largest < 512ull << 20);  // two lists of 96 MB, and as much again of shorter ones
+  REQUIRE(bbp_plan_destroy(c.plan) == BBP_OK);
+  REQUIRE(live.size() == outside);
+}
+
+const std::map<std::string, void (*)()> kCases = {
+    {"captured_lists_stay", captured_lists_stay},
+};
+
+}  // namespace
+
+int main(int argc, char** argv) {
+  const auto c = kCases.find(argc > 1 ? argv[1] : "");
+  REQUIRE(c != kCases.end());
+  c->second();
+  return 0;
+}

@@ -1,0 +1,43 @@
+"""Calls by primes beside other uses of a plan and of the device, each against the
+term-by-term kernels or the printed rows, tolerance 0."""
+
+import pytest
+
+from test_gpu_primes import bbp, by_terms, plans  # noqa: F401  (fixtures)
+
+pytestmark = pytest.mark.gpu
+
+torch = pytest.importorskip("torch")
+
+
+def value(out, P):
+    return int.from_bytes(bytes(out.cpu().numpy()), "big") >> (8 * len(out) - P)
+
+
+def test_graph_replayed_after_a_longer_query(bbp, plans):  # noqa: F811
+    """Captured at 1e8, then a query of 6e8 whose lists do not fit the captured ones, replayed."""
+    n, P = 10**8 + 79, 128
+    plan = bbp.Plan(device=0, guard_bits=64)
+    plan.bits(n, P)
+    out = torch.zeros(P // 8, dtype=torch.uint8, device="cuda")
+    valid = torch.zeros(1, dtype=torch.int32, device="cuda")
+    stream = torch.cuda.Stream()
+    torch.cuda.synchronize()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph, stream=stream):
+        bbp.bbp_bits_async(plan.handle, 0, n, P, out.data_ptr(), valid.data_ptr(), 0, stream.cuda_stream)
+    want = by_terms(bbp, plans[64], n, P)
+    longer = by_terms(bbp, plans[64], 6 * 10**8 + 1, P)
+    free = torch.cuda.mem_get_info()[0]
+    assert plan.bits(6 * 10**8 + 1, P) == longer
+    # the longer lists came on top of the captured ones: two of 24 M primes
+    assert free - torch.cuda.mem_get_info()[0] >= 2 * 4 * (24 << 20)
+    out.zero_()
+    valid.zero_()
+    torch.cuda.synchronize()
+    graph.replay()
+    torch.cuda.synchronize()
+    assert (value(out, P), int(valid[0])) == want
+    assert plan.bits(6 * 10**8 + 1, P) == longer
+    del graph
+    plan.close()
