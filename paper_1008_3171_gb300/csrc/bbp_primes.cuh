@@ -319,13 +319,11 @@ struct Arith2 {
   }
 };
 
-// a / p for quotients below 2^21 (a < 2^44): single precision is off by at most one
+// a / p for the limits of the sums and primes from sqrt(A) on
+template <int FORMULA>
 __device__ __forceinline__ uint32_t small_quotient(uint64_t a, uint64_t p) {
-  uint32_t q = static_cast<uint32_t>(__fdividef(static_cast<float>(a), static_cast<float>(p)));
-  int64_t rem = static_cast<int64_t>(a) - static_cast<int64_t>(q * p);
-  if (rem < 0) --q;
-  if (rem >= static_cast<int64_t>(p)) ++q;
-  return q;
+  const float q = __fdividef(static_cast<float>(a), static_cast<float>(p));
+  return corrected_quotient<FORMULA>(static_cast<uint32_t>(q), a, p);
 }
 
 // den^-1 2^e (Montgomery form) for a unit `den` mod m whose group of units has
@@ -741,8 +739,8 @@ __global__ void __launch_bounds__(kHeadThreads) prime_sum_kernel(const __grid_co
     const uint64_t p = G.base + G.list[min(i, count - 1)];
     const A M(p);
     const uint32_t r = lo32(p) & 3u;
-    const uint32_t i0 = summands<K0>(small_quotient(G.A, p), r), i1 = summands<K0 + 1>(small_quotient(G.B, p), 4u - r),
-                   i2 = summands<K0 + 2>(small_quotient(G.C, p), 1u);
+    const uint32_t i0 = summands<K0>(small_quotient<FORMULA>(G.A, p), r), i1 = summands<K0 + 1>(small_quotient<FORMULA>(G.B, p), 4u - r),
+                   i2 = summands<K0 + 2>(small_quotient<FORMULA>(G.C, p), 1u);
     T n0, d0, n1, d1, n2, d2;
     if constexpr (GROUP > 1) {
       group_sum<K0, GROUP>(M, i0, r, n0, d0);
@@ -771,7 +769,7 @@ __global__ void __launch_bounds__(kHeadThreads) prime_sum_kernel(const __grid_co
     T num = FORMULA == 0 || r == 1u ? M.add(t0, M.neg(rest)) : M.add(t0, rest);
     if (r == 3u) num = M.neg(num);
     const uint64_t e0 = G.e + (FORMULA == 0 ? 4 : 3);
-    const uint64_t e = e0 - small_quotient(e0, p - 1) * (p - 1);
+    const uint64_t e = e0 - small_quotient<FORMULA>(e0, p - 1) * (p - 1);
     const T inv = inverse_times_power<A>(M, M.mul(d0, d12), p - 1, e);
     T x = M.plain(M.mul(num, inv));
     if (i >= count || (lane & (GROUP - 1)) != 0u) x = 0;

@@ -42,7 +42,31 @@
 #include <cstdint>
 #include <vector>
 
+#ifdef __CUDACC__
+#define BBP_HOST_DEVICE __host__ __device__
+#else
+#define BBP_HOST_DEVICE
+#endif
+
 namespace bbp {
+
+// floor(a / p) from q, the single-precision quotient cut to a whole number.  That is off by two
+// ulps and the rounding of a and p (2^-24 each, nothing for p < 2^24).  Quotients of the sums are
+// at most sqrt(A): up to 2^21.7 for Eq. 2, whose ulps are 1/4, so that one correction is enough;
+// up to 2^22.2 for Eq. 1, where an ulp is 1/2, and past 2^22 (n > 8.8e12) it may take two.
+// (Two for both: 0.7 % of a whole query at n = 1e9 and 4e10.)
+template <int FORMULA>
+BBP_HOST_DEVICE inline uint32_t corrected_quotient(uint32_t q, uint64_t a, uint64_t p) {
+  const int64_t m = static_cast<int64_t>(p);
+  int64_t rem = static_cast<int64_t>(a) - static_cast<int64_t>(q * p);
+  if (FORMULA == 1 && q >= 1u << 21) {
+    if (rem < 0) --q, rem += m;
+    if (rem >= m) ++q, rem -= m;
+  }
+  if (rem < 0) --q;
+  if (rem >= m) ++q;
+  return q;
+}
 
 // Largest moduli of the three sums: every term of a modulus up to these is a head
 // term.  Eq. 2's (at most one) head term above `A` and all tail terms are left to the
@@ -92,6 +116,9 @@ double prime_form_imad(const PrimeLimits& lim, int limbs);
 // P = 128, term by term and by primes: n = 2e7 334 and 217 us, 3e7 474 and 241, 1e8 1560 and 354.
 // About 200 us of the latter are launches and chains.
 constexpr uint64_t kPrimeMinN = 16'000'000;
-constexpr uint64_t kPrimeMaxN = 10'900'000'000'000;  // 1024 sqrt(0.4 n) < 2^31: word products of the sums
+// The largest product of w = 2^10 and a c in the sums mod p (Eq. 2's second sum, c <= sqrt(0.4 n))
+// stays below 2^31; Eq. 1's (w = 2^4, c <= sqrt(4 n)) are smaller.  Its A = 2 n is below 2^44.4, where
+// small_quotient and the 46-bit arithmetic reach.
+constexpr uint64_t kPrimeMaxN = 10'900'000'000'000;
 
 }  // namespace bbp

@@ -4,11 +4,14 @@
 // exits 0 if it holds (test_host_runtime.py).
 #include <cuda_runtime.h>
 
+#include <algorithm>
+#include <cmath>
 #include <cstdio>
 #include <cstdlib>
 #include <cstring>
 #include <map>
 #include <mutex>
+#include <random>
 #include <set>
 #include <string>
 #include <thread>
@@ -16,6 +19,7 @@
 
 #include "bbp.h"
 #include "bbp_kernels.cuh"
+#include "bbp_primes.h"
 #include "bbp_sieve.cuh"
 
 namespace {
@@ -275,6 +279,8 @@ cudaError_t launch_prime_check(const unsigned long long* slots, int, uint32_t, u
 
 }  // namespace bbp
 
+using namespace bbp;
+
 namespace {
 
 struct Caller {
@@ -324,7 +330,31 @@ void captured_lists_stay() {
   REQUIRE(live.size() == outside);
 }
 
+// Quotients of the sums' limits by primes from their square root on, from every single-precision
+// estimate that the division's two ulps allow, up to the largest position of both formulas.
+void sum_quotients() {
+  std::mt19937_64 rng(7);
+  for (int i = 0; i < 400000; ++i) {
+    const int formula = i & 1;
+    const uint64_t n = i < 1000 ? kPrimeMaxN - i : kPrimeMinN + rng() % (kPrimeMaxN - kPrimeMinN + 1);
+    const PrimeLimits lim = prime_limits(formula, n - 1);
+    const uint64_t root = static_cast<uint64_t>(std::sqrt(static_cast<double>(lim.A)));
+    const uint64_t p = root + rng() % (i & 2 ? 100 : i & 4 ? root : 22 * root);
+    uint64_t a[4] = {lim.A, lim.B, lim.C, n + 1280};
+    a[3] -= rng() % p;
+    a[0] = i & 8 ? a[0] / p * p - (i >> 4 & 1) : a[0];  // at a multiple, and one below
+    for (uint64_t v : a) {
+      const float near = static_cast<float>(v) / static_cast<float>(p);
+      float q = std::nextafter(std::nextafter(near, 0.0f), 0.0f);
+      for (int ulp = -2; ulp <= 2; ++ulp, q = std::nextafter(q, 1e30f))
+        REQUIRE((formula ? corrected_quotient<1>(static_cast<uint32_t>(q), v, p)
+                         : corrected_quotient<0>(static_cast<uint32_t>(q), v, p)) == v / p);
+    }
+  }
+}
+
 const std::map<std::string, void (*)()> kCases = {
+    {"sum_quotients", sum_quotients},
     {"captured_lists_stay", captured_lists_stay},
 };
 
