@@ -162,7 +162,7 @@ struct BatchPlan {
   uint32_t tail_begin[kMaxWaves + 1] = {};               // tail jobs of a wave
   uint64_t terms = 0, head_terms = 0;
   double imad = 0;
-  struct Prime { uint32_t q, W; uint64_t n, bound; };
+  struct Prime { uint32_t q, W; uint64_t n, bound; bool planned; };
   std::vector<Prime> primes;  // queries by the prime form, smallest first
 };
 
@@ -207,7 +207,7 @@ static bbp_status plan_batch(bbp_plan p, int f, uint32_t count, const uint64_t* 
     if (prime) {  // the queue takes what the prime form leaves
       const PrimeLimits lim = prime_limits(f, n[q] - 1);
       bp->imad += prime_form_imad(lim, static_cast<int>(L));
-      bp->primes.push_back(BatchPlan::Prime{q, W, n[q], bound});
+      bp->primes.push_back(BatchPlan::Prime{q, W, n[q], bound, true});
       ranges.clear();
       for (uint32_t j = 0; j < F.count; ++j)
         if (plan_series(F, j, n[q], W, static_cast<uint32_t>(lmax), prime_first_k(lim, j, n[q] - 1), UINT64_MAX, ranges,
@@ -485,12 +485,13 @@ static bbp_status run_batch(bbp_plan p, bbp_formula f, uint32_t count, const uin
     const int used = static_cast<int>(std::min<size_t>(kPrimeLanes, bp.primes.size()));
     for (int i = 0; i < used; ++i) BBP_TRY(cudaStreamWaitEvent(b->lane_stream[i], b->ready, 0));
     for (size_t i = 0; i < bp.primes.size(); ++i) {
-      const BatchPlan::Prime& r = bp.primes[i];
+      BatchPlan::Prime& r = bp.primes[i];
       const int k = static_cast<int>(i % kPrimeLanes);
       const cudaStream_t to = b->lane_stream[k];
       PrimeRun run;
-      bbp_status ls = run.plan(b->lane[k], p->sm_count, f, r.n, r.W, b->d_accum + static_cast<uint64_t>(r.q) * kMaxLimbs);
-      if (ls == BBP_OK) ls = run.begin(to);
+      r.planned = run.plan(b->lane[k], p->sm_count, f, r.n, r.W, b->d_accum + static_cast<uint64_t>(r.q) * kMaxLimbs) == BBP_OK;
+      if (!r.planned) continue;  // by its terms, in the second pass
+      bbp_status ls = run.begin(to);
       if (ls == BBP_OK) ls = run.run(0, run.lists(), to);
       if (ls == BBP_OK)
         ls = run.finish(P[r.q], r.bound, b->d_out + static_cast<size_t>(r.q) * kOutStride, b->d_valid + r.q,
@@ -522,6 +523,11 @@ static bbp_status run_batch(bbp_plan p, bbp_formula f, uint32_t count, const uin
     BBP_TRY(cudaEventElapsedTime(&ms, p->ev0, p->ev1));
     p->stats.head_ms = ms;
   }
+  for (const BatchPlan::Prime& r : bp.primes)
+    if (!r.planned) {  // nothing was written for it
+      b->h_redo[r.q] = 1;
+      b->h_done[1 + r.q] = b->h_done[0];
+    }
   double last_ms = 0;
   for (uint32_t q = 0; q < count; ++q) {
     std::memcpy(out + static_cast<size_t>(q) * out_stride, b->h_out + static_cast<size_t>(q) * kOutStride,

@@ -23,7 +23,9 @@ namespace bbp {
 namespace {
 
 constexpr uint32_t kBaseCap = 565000;               // odd primes below 2^23: 564,162
-constexpr uint32_t kMaxLists = 1u << 17;            // 7.6e4 lists of 6 M primes at the largest position
+// At the largest position lists of 6 M primes number 7.3e4 for Eq. 2 and 1.46e5 for Eq. 1, whose
+// moduli reach 2 n (152 SMs; 1.9e5 at most from 120 to 160).
+constexpr uint32_t kMaxLists = 1u << 18;
 constexpr uint32_t kSieveEntries = 64u << 10;       // of a sieve segment: three CTAs an SM
 constexpr uint64_t kLongSum = 8000, kGroupSum = 1000;  // primes below A / these take 32, 8 lanes
 

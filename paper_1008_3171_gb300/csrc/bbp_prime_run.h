@@ -27,7 +27,8 @@ void release_prime_state(PrimeState** state);
 class PrimeRun {
  public:
   // The query at position n, W working bits, into `slots` (to which the terms that the
-  // prime form does not cover are added by the caller).
+  // prime form does not cover are added by the caller).  Host work alone; not BBP_OK: the caller
+  // sums the terms.
   bbp_status plan(PrimeState* state, int sm_count, int formula, uint64_t n, uint32_t W, unsigned long long* slots);
   size_t lists() const { return lists_.size(); }
   double share(size_t i) const;  // list i's part of the numbers up to n

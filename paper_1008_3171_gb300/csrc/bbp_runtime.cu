@@ -437,20 +437,22 @@ bbp_status enqueue_bits(bbp_plan p, int f, uint64_t n, uint32_t P, uint32_t W, u
     const bbp_status ls = launch_ranges(p, f, n, W, rest, p->d_slots, s);
     if (ls != BBP_OK) return ls;
     PrimeRun run;
-    bbp_status ps = run.plan(p->primes, p->sm_count, f, n, W, p->d_slots);
-    if (ps == BBP_OK) ps = run.begin(s);
-    if (ps == BBP_OK) ps = run.run(0, run.lists(), s);
-    if (ps == BBP_OK) ps = run.finish(P, bound, d_out, d_valid, redo, s);
-    prime_launches = run.launches();
-    if (ps != BBP_OK) return ps;
-    if (p->profile) {
-      BBP_CUDA(cudaEventRecord(p->ev1, s));
-      BBP_CUDA(cudaEventSynchronize(p->ev1));
-      BBP_CUDA(cudaEventElapsedTime(&prime_ms, p->ev2, p->ev1));
+    if (run.plan(p->primes, p->sm_count, f, n, W, p->d_slots) == BBP_OK) {  // else all by terms
+      bbp_status ps = run.begin(s);
+      if (ps == BBP_OK) ps = run.run(0, run.lists(), s);
+      if (ps == BBP_OK) ps = run.finish(P, bound, d_out, d_valid, redo, s);
+      prime_launches = run.launches();
+      if (ps != BBP_OK) return ps;
+      if (p->profile) {
+        BBP_CUDA(cudaEventRecord(p->ev1, s));
+        BBP_CUDA(cudaEventSynchronize(p->ev1));
+        BBP_CUDA(cudaEventElapsedTime(&prime_ms, p->ev2, p->ev1));
+      }
+      prime_launches += p->stats.kernel_launches + 1;
+      gate = redo;
     }
-    prime_launches += p->stats.kernel_launches + 1;
-    gate = redo;
-  } else {
+  }
+  if (!gate) {
     bool done = false;
     const bbp_status os = launch_one(p, f, n, W, P, ranges, bound, d_out, d_valid, d_limbs, s, &done);
     if (os != BBP_OK || done) return os;

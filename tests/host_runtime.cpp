@@ -353,7 +353,50 @@ void sum_quotients() {
   }
 }
 
+// The largest positions of both formulas, in lists of each length, on several numbers of SMs.
+void largest_positions() {
+  for (int n_sms : {120, 132, 148, 152, 160}) {
+    sms = n_sms;
+    Caller c;
+    for (bbp_formula f : {BBP_BELLARD, BBP_BBP}) {
+      const uint64_t n[2] = {kPrimeMaxN, kPrimeMaxN + 1};
+      const uint32_t P[2] = {64, 64};
+      uint8_t out[16];
+      calls["launch_prime"] = 0;
+      REQUIRE(bbp_bits_batch(c.plan, f, 1, n, P, out, 8, nullptr, nullptr) == BBP_OK);
+      REQUIRE(calls["launch_prime"] > 10000);  // by primes
+      if (n_sms == 152) REQUIRE(c.bits(kPrimeMaxN, f) == BBP_OK);
+      ops.clear();
+      for (Stream* s : streams) s->last = s->last_real = -1;
+    }
+    bbp_plan_destroy(c.plan);
+  }
+}
+
+// A query whose lists cannot be planned is summed by its terms: alone, and in a batch.
+void no_plan_no_primes() {
+  Caller c;
+  REQUIRE(c.bits(100'000'000) == BBP_OK);
+  const int primes = calls["launch_prime"];
+  calls["head_lmax_for"] = 0;
+  fail_at["head_lmax_for"] = -10;  // the lists': after the query's, seven series' leftovers and their launch
+  REQUIRE(c.bits(100'000'000) == BBP_OK);
+  REQUIRE(calls["head_lmax_for"] > 10 && calls["launch_prime"] == primes);
+  const uint64_t n[3] = {50'000'000, 1'000'000, 100'000'000};
+  const uint32_t P[3] = {64, 64, 64};
+  uint8_t out[24];
+  double ms[3];
+  calls["head_lmax_for"] = 0;
+  fail_at["head_lmax_for"] = -4;  // three queries, then the first one's lists
+  REQUIRE(bbp_bits_batch(c.plan, BBP_BELLARD, 3, n, P, out, 8, nullptr, ms) == BBP_OK);
+  size_t graphs = 0;
+  for (const Op& o : ops) graphs += o.what == "graph";
+  REQUIRE(graphs == 2);  // the second pass
+}
+
 const std::map<std::string, void (*)()> kCases = {
+    {"largest_positions", largest_positions},
+    {"no_plan_no_primes", no_plan_no_primes},
     {"sum_quotients", sum_quotients},
     {"captured_lists_stay", captured_lists_stay},
 };
