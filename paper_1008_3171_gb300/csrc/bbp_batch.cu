@@ -113,6 +113,16 @@ struct BatchState {
 
 namespace bbp {
 
+// Waits for everything a batch has queued: after a call that failed half way, no kernel may
+// still add to the accumulators nor a copy read the staging that the next call fills.
+static void wait_batch(BatchState* b) {
+  if (b->stream) cudaStreamSynchronize(b->stream);
+  for (int i = 0; i < kPrimeLanes; ++i) {
+    if (b->lane_stream[i]) cudaStreamSynchronize(b->lane_stream[i]);
+    wait_prime_state(b->lane[i]);
+  }
+}
+
 void release_batch_state(bbp_plan p) {
   BatchState* b = p->batch;
   if (!b) return;
@@ -589,13 +599,17 @@ extern "C" bbp_status bbp_bits_batch(bbp_plan p, bbp_formula f, uint32_t count, 
     std::vector<uint32_t> valid(count);
     std::vector<double> ms(count);
     const bbp_status st = run_batch(p, f, count, n, P, out, out_stride, valid.data(), ms.data(), true);
-    if (st != BBP_OK) return st;
+    if (st != BBP_OK) {
+      wait_batch(p->batch);
+      return st;
+    }
     if (valid_bits) std::copy(valid.begin(), valid.end(), valid_bits);
     if (latency_ms) std::copy(ms.begin(), ms.end(), latency_ms);
     if (p->strict)
       for (uint32_t q = 0; q < count; ++q)
         if (valid[q] < P[q]) return BBP_EINVALID_BITS;
   } catch (const std::bad_alloc&) {
+    wait_batch(p->batch);
     return BBP_ENOMEM;
   }
   return BBP_OK;

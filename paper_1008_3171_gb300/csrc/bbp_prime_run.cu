@@ -85,11 +85,16 @@ bool make_state(PrimeState* s) {
 }
 }  // namespace
 
-void release_prime_state(PrimeState** state) {
-  PrimeState* s = *state;
+void wait_prime_state(PrimeState* s) {
   if (!s) return;
   if (s->sieve) cudaStreamSynchronize(s->sieve);
   if (s->sums) cudaStreamSynchronize(s->sums);
+}
+
+void release_prime_state(PrimeState** state) {
+  PrimeState* s = *state;
+  if (!s) return;
+  wait_prime_state(s);
   for (cudaEvent_t e : s->ready)
     if (e) cudaEventDestroy(e);
   for (cudaEvent_t e : s->used)

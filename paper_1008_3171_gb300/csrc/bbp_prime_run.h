@@ -22,6 +22,8 @@ constexpr uint32_t kPrimeListMax = 24u << 20;      // single queries: two lists 
 constexpr uint32_t kPrimeLaneListMax = 6u << 20;   // each of several workspaces: two of 24 MB
 bool prime_workspace(PrimeState** state, uint64_t n, uint32_t max_list, cudaStream_t st);
 void release_prime_state(PrimeState** state);
+// Waits for what runs on the workspace's own streams, beside the caller's (NULL: nothing).
+void wait_prime_state(PrimeState* state);
 
 // One query on one workspace and one stream: begin, every list in order, finish.
 class PrimeRun {

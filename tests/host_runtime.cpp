@@ -394,7 +394,23 @@ void no_plan_no_primes() {
   REQUIRE(graphs == 2);  // the second pass
 }
 
+// A batch that fails among its prime forms has waited for all it queued when it returns.
+void failed_batch_leaves_nothing() {
+  Caller c;
+  const uint64_t n[4] = {50'000'000, 1'000'000, 1'000'000'000, 100'000'000};
+  const uint32_t P[4] = {64, 64, 64, 64};
+  uint8_t out[32];
+  for (int at = 1; at < 30; ++at) {
+    calls["launch_prime"] = 0;
+    fail_at["launch_prime"] = -at;
+    REQUIRE(bbp_bits_batch(c.plan, BBP_BELLARD, 4, n, P, out, 8, nullptr, nullptr) == BBP_ECUDA);
+    REQUIRE(calls["launch_prime"] >= at);
+    REQUIRE(in_flight() == 0);
+  }
+}
+
 const std::map<std::string, void (*)()> kCases = {
+    {"failed_batch_leaves_nothing", failed_batch_leaves_nothing},
     {"largest_positions", largest_positions},
     {"no_plan_no_primes", no_plan_no_primes},
     {"sum_quotients", sum_quotients},
