@@ -123,6 +123,7 @@ struct Query {
   int lane = -1;                  // workspace kept between iterations
   size_t next_list = 0;
   uint64_t terms_done = 0;
+  bbp_status broken = BBP_OK;     // could not be planned again: fails with this at the iteration's end
   bool final_in_flight = false;
   std::vector<uint8_t> out;
   uint32_t valid = 0;
@@ -426,6 +427,16 @@ bool make_lanes(ServeEngine* E) {
   return true;
 }
 
+// Back to the terms for a query that has not begun; if they cannot be planned it leaves with
+// this iteration, without a result.
+void plan_by_terms(ServeEngine* E, Query* q) {
+  q->run.reset();
+  q->broken = plan_query_work(E->plan, q->n, q->P, q, false);
+  if (q->broken == BBP_OK) return;
+  q->prime = false;
+  q->work.clear();
+}
+
 // What an iteration does for one query by primes: its lists [first, last) on a workspace.
 struct PrimePart {
   Query* q;
@@ -456,8 +467,7 @@ void take_primes(ServeEngine* E, std::vector<Query*>& batch, uint64_t budget, st
       const uint64_t slot = static_cast<uint64_t>(q->slot);
       if (!q->run || q->run->plan(E->lane[free_lane], E->plan->sm_count, BBP_BELLARD, q->n, q->W,
                                   E->d_accum + slot * kMaxLimbs) != BBP_OK) {
-        q->run.reset();
-        if (plan_query_work(E->plan, q->n, q->P, q, false) != BBP_OK) q->prime = false;  // by its terms instead
+        plan_by_terms(E, q);
         continue;
       }
       q->next_list = 0;
@@ -507,7 +517,7 @@ bool enqueue_iteration(ServeEngine* E, HostStage& H, std::vector<Query*>& batch,
   for (Query* q : batch) primes |= q->prime;
   if (primes && !make_lanes(E))
     for (Query* q : batch)
-      if (q->prime && plan_query_work(p, q->n, q->P, q, false) != BBP_OK) return false;
+      if (q->prime) plan_by_terms(E, q);
   size_t by_terms = 0;
   for (Query* q : batch) by_terms += q->prime ? 0 : 1;
   // half of an iteration for either kind while there are both
@@ -664,14 +674,16 @@ bool finish_iteration(ServeEngine* E, HostStage& H) {
       q->next = 0;
       q->tile_off = 0;
       q->final_in_flight = false;
-      const bbp_status ps = plan_query_work(E->plan, q->n, q->P, q, false);
-      if (ps == BBP_OK) {
+      plan_by_terms(E, q);
+      if (q->broken == BBP_OK) {
         E->rezero.push_back(q->slot);
         E->active.push_back(q);
         continue;
       }
+    }
+    if (q->broken != BBP_OK) {
       q->state = kFailed;
-      q->error = ps;
+      q->error = q->broken;
       E->free_slots.push_back(q->slot);
       q->slot = -1;
       continue;

@@ -409,7 +409,30 @@ void failed_batch_leaves_nothing() {
   }
 }
 
+bbp_status served(bbp_plan plan, bbp_ticket t) {
+  uint8_t out[160];
+  bbp_status st;
+  while ((st = bbp_poll(plan, t, out, nullptr)) == BBP_PENDING) std::this_thread::yield();
+  return st;
+}
+
+// A submitted query whose lists and then whose terms cannot be planned fails: no result is made
+// of the few terms that the primes leave.
+void unplanned_query_fails() {
+  Caller c;
+  bbp_ticket t = 0;
+  calls["head_lmax_for"] = 0;
+  fail_at["head_lmax_for"] = 2;  // after the submission's own
+  REQUIRE(bbp_submit(c.plan, 100'000'000, 64, &t) == BBP_OK);
+  REQUIRE(served(c.plan, t) == BBP_EINVAL);
+  fail_at.clear();
+  REQUIRE(bbp_submit(c.plan, 100'000'000, 64, &t) == BBP_OK);
+  REQUIRE(served(c.plan, t) == BBP_OK);
+  REQUIRE(bbp_plan_destroy(c.plan) == BBP_OK);
+}
+
 const std::map<std::string, void (*)()> kCases = {
+    {"unplanned_query_fails", unplanned_query_fails},
     {"failed_batch_leaves_nothing", failed_batch_leaves_nothing},
     {"largest_positions", largest_positions},
     {"no_plan_no_primes", no_plan_no_primes},
