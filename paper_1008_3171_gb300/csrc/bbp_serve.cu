@@ -703,8 +703,14 @@ bool finish_iteration(ServeEngine* E, HostStage& H) {
 
 // An iteration could not be enqueued or did not complete: every admitted query
 // fails (bbp_poll returns BBP_ECUDA) and gives its slot back, so that later
-// submissions are admitted again (a fresh slot is zeroed on admission).
+// submissions are admitted again (a fresh slot is zeroed on admission).  What the iteration
+// has queued ends first: none of it may add to a slot that has a new query.
 void fail_all(ServeEngine* E) {
+  cudaStreamSynchronize(E->stream);
+  for (int i = 0; i < kServeLanes; ++i) {
+    if (E->lane_stream[i]) cudaStreamSynchronize(E->lane_stream[i]);
+    wait_prime_state(E->lane[i]);
+  }
   std::lock_guard<std::mutex> lock(E->mu);
   auto fail = [&](Query* q) {
     q->state = kFailed;

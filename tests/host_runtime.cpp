@@ -431,7 +431,27 @@ void unplanned_query_fails() {
   REQUIRE(bbp_plan_destroy(c.plan) == BBP_OK);
 }
 
+// An iteration that fails among its prime forms has ended when its queries are given back.
+void failed_iteration_leaves_nothing() {
+  for (int at : {1, 2, 3, 5, 9}) {
+    Caller c;
+    bbp_ticket t = 0;
+    calls["launch_prime"] = 0;
+    fail_at["launch_prime"] = -at;
+    REQUIRE(bbp_submit(c.plan, 1'000'000'000, 64, &t) == BBP_OK);
+    REQUIRE(served(c.plan, t) == BBP_ECUDA);
+    {
+      std::lock_guard<std::recursive_mutex> l(mu);
+      REQUIRE(in_flight() == 0);
+    }
+    REQUIRE(bbp_submit(c.plan, 100'000'000, 64, &t) == BBP_OK);
+    REQUIRE(served(c.plan, t) == BBP_OK);
+    REQUIRE(bbp_plan_destroy(c.plan) == BBP_OK);
+  }
+}
+
 const std::map<std::string, void (*)()> kCases = {
+    {"failed_iteration_leaves_nothing", failed_iteration_leaves_nothing},
     {"unplanned_query_fails", unplanned_query_fails},
     {"failed_batch_leaves_nothing", failed_batch_leaves_nothing},
     {"largest_positions", largest_positions},
