@@ -112,6 +112,19 @@ void release_prime_state(PrimeState** state) {
   *state = nullptr;
 }
 
+// Lets this thread allocate while some other stream is being captured, which a capture in the
+// default mode forbids and would not survive: queries that allocate nothing but at a plan's
+// first use are called beside captures.
+class AllocateBesideCaptures {
+ public:
+  AllocateBesideCaptures() { cudaThreadExchangeStreamCaptureMode(&mode_); }
+  ~AllocateBesideCaptures() { cudaThreadExchangeStreamCaptureMode(&mode_); }
+  AllocateBesideCaptures(const AllocateBesideCaptures&) = delete;
+
+ private:
+  cudaStreamCaptureMode mode_ = cudaStreamCaptureModeRelaxed;
+};
+
 bool prime_workspace(PrimeState** state, uint64_t n, uint32_t max_list, cudaStream_t st) {
   // primes of one list: all of them up to the limit
   const double x = static_cast<double>(n);
@@ -127,6 +140,7 @@ bool prime_workspace(PrimeState** state, uint64_t n, uint32_t max_list, cudaStre
     return true;
   }
   if (capturing) return false;
+  const AllocateBesideCaptures guard;
   if (!*state) {
     *state = new (std::nothrow) PrimeState();
     if (!*state) return false;

@@ -43,6 +43,9 @@ std::vector<Op> ops;
 std::set<Stream*> streams;
 std::map<const void*, size_t> live;
 int sms = 152;
+thread_local cudaStreamCaptureMode mode = cudaStreamCaptureModeGlobal;
+bool other_capture = false;                // a stream of some other code is captured in the default mode,
+bool other_broken = false;                 // and a call of ours has ended that
 uint32_t verdict = 0;                      // what the prime form's check says
 std::map<std::string, int> calls, fail_at;  // fails from that call on (negative: that call alone)
 
@@ -53,6 +56,13 @@ std::map<std::string, int> calls, fail_at;  // fails from that call on (negative
       std::exit(1);                                             \
     }                                                           \
   } while (0)
+
+// A call that a capture in the default mode forbids
+bool forbidden() {
+  if (!other_capture || mode == cudaStreamCaptureModeRelaxed) return false;
+  other_broken = true;
+  return true;
+}
 
 bool fails(const std::string& name) {
   std::lock_guard<std::recursive_mutex> l(mu);
@@ -135,13 +145,16 @@ cudaError_t cudaGetDeviceProperties(cudaDeviceProp* p, int) {
 cudaError_t cudaDeviceGetStreamPriorityRange(int* a, int* b) { *a = 0; *b = -5; return cudaSuccess; }
 
 cudaError_t cudaMalloc(void** p, size_t n) {
+  if (forbidden()) return cudaErrorStreamCaptureUnsupported;
   if (fails("cudaMalloc")) return cudaErrorMemoryAllocation;
   std::lock_guard<std::recursive_mutex> l(mu);
   *p = std::calloc(1, n ? n : 1);
   live[*p] = n;
   return cudaSuccess;
 }
+cudaError_t cudaThreadExchangeStreamCaptureMode(cudaStreamCaptureMode* m) { std::swap(*m, mode); return cudaSuccess; }
 cudaError_t cudaFree(void* p) {
+  if (forbidden()) return cudaErrorStreamCaptureUnsupported;
   std::lock_guard<std::recursive_mutex> l(mu);
   if (!p) return cudaSuccess;
   REQUIRE(live.erase(p) == 1);
@@ -450,7 +463,21 @@ void failed_iteration_leaves_nothing() {
   }
 }
 
+// Stream queries beside a capture of some other stream, at a plan's first use and where its
+// lists have to grow: the capture goes on, and the query runs by primes.
+void beside_a_capture() {
+  Caller c;
+  other_capture = true;
+  for (uint64_t n : {100'000'000, 1'000'000'000}) {
+    const int primes = calls["launch_prime"];
+    REQUIRE(c.async(n, c.a) == BBP_OK);
+    REQUIRE(!other_broken && calls["launch_prime"] > primes);
+    REQUIRE(mode == cudaStreamCaptureModeGlobal);
+  }
+}
+
 const std::map<std::string, void (*)()> kCases = {
+    {"beside_a_capture", beside_a_capture},
     {"failed_iteration_leaves_nothing", failed_iteration_leaves_nothing},
     {"unplanned_query_fails", unplanned_query_fails},
     {"failed_batch_leaves_nothing", failed_batch_leaves_nothing},

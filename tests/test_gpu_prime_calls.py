@@ -41,3 +41,27 @@ def test_graph_replayed_after_a_longer_query(bbp, plans):  # noqa: F811
     assert plan.bits(6 * 10**8 + 1, P) == longer
     del graph
     plan.close()
+
+
+def test_beside_a_capture_of_another_stream(bbp, plans):  # noqa: F811
+    """A plan's first query by primes, and one whose lists grow, on one stream while another is
+    captured in the default mode: both are right."""
+    plan = bbp.Plan(device=0, guard_bits=64)
+    queries = [(10**8 + 81, 128), (4 * 10**8 + 3, 64)]
+    outs = [torch.zeros(P // 8, dtype=torch.uint8, device="cuda") for _, P in queries]
+    valid = torch.zeros(2, dtype=torch.int32, device="cuda")
+    x = torch.zeros(1024, device="cuda")
+    side, stream = torch.cuda.Stream(), torch.cuda.Stream()
+    torch.cuda.synchronize()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph, stream=stream, capture_error_mode="global"):
+        x.add_(1)
+        for i, (n, P) in enumerate(queries):
+            bbp.bbp_bits_async(plan.handle, 0, n, P, outs[i].data_ptr(), valid.data_ptr() + 4 * i, 0, side.cuda_stream)
+    graph.replay()
+    torch.cuda.synchronize()
+    assert float(x.sum()) == 1024
+    for i, (n, P) in enumerate(queries):
+        assert (value(outs[i], P), int(valid[i])) == by_terms(bbp, plans[64], n, P)
+    del graph
+    plan.close()
