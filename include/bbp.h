@@ -20,7 +20,9 @@
  *   - Output bit strings are MSB-first bytes: out[0] bit 7 is bit n; the unused low
  *     bits of the last byte are 0.
  *   - Every function returns a bbp_status; no C++ exception crosses the ABI.
- *   - A plan is not thread-safe: one host thread at a time per plan.
+ *   - A plan is not thread-safe: one host thread at a time per plan.  Its queries and partial
+ *     sums share one set of accumulators: the caller orders those queued on several streams
+ *     (bbp_accumulate_async and bbp_finalize_async use the caller's alone).
  *   - Buffers named h_* or without prefix are host memory owned by the caller;
  *     d_* are device memory on the plan's device owned by the caller.
  *   - Moduli must stay below 2^60: n up to about 1.1e18 (BBP_ERANGE beyond).

@@ -59,6 +59,9 @@ struct PrimeState {
   uint32_t* counts = nullptr;
   cudaStream_t sieve = nullptr, sums = nullptr;  // beside the caller's stream
   cudaEvent_t ready[2] = {}, used[2] = {}, base = nullptr, done = nullptr;
+  cudaEvent_t idle = nullptr;   // the last run that was not captured, on
+  cudaStream_t last = nullptr;  // this stream
+  bool ran = false;
 };
 
 namespace bbp {
@@ -81,6 +84,7 @@ bool make_state(PrimeState* s) {
   for (cudaEvent_t& e : s->used) event(&e);
   event(&s->base);
   event(&s->done);
+  event(&s->idle);
   return ok;
 }
 }  // namespace
@@ -101,6 +105,7 @@ void release_prime_state(PrimeState** state) {
     if (e) cudaEventDestroy(e);
   if (s->base) cudaEventDestroy(s->base);
   if (s->done) cudaEventDestroy(s->done);
+  if (s->idle) cudaEventDestroy(s->idle);
   if (s->sieve) cudaStreamDestroy(s->sieve);
   if (s->sums) cudaStreamDestroy(s->sums);
   for (uint32_t* l : s->list) cudaFree(l);
@@ -253,6 +258,11 @@ bbp_status PrimeRun::begin(cudaStream_t st) {
   PrimeState* const S = state_;
   cudaError_t err = cudaSuccess;
   auto chk = [&](cudaError_t r) { if (err == cudaSuccess) err = r; };
+  // a run on another stream may still read the lists that this one writes
+  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+  chk(cudaStreamIsCapturing(st, &cap));
+  captured_ = cap != cudaStreamCaptureStatusNone;
+  if (S->ran && S->last != st && !captured_) chk(cudaStreamWaitEvent(st, S->idle, 0));
   chk(cudaMemsetAsync(S->counts, 0, sizeof(uint32_t) * (kCountHead + 2 * lists_.size()), st));
   chk(launch_base_primes(base_to_, S->primes, S->sieve_primes, S->counts, S->counts + 1, st));
   chk(cudaEventRecord(S->base, st));
@@ -318,6 +328,11 @@ bbp_status PrimeRun::finish(uint32_t P, uint64_t bound, uint8_t* d_out, uint32_t
     err = launch_prime_check(args_.slots, static_cast<int>(args_.L), P, bound, state_->counts + kCountHead,
                              static_cast<uint32_t>(lists_.size()), state_->list_cap, d_out, d_valid, d_redo, st);
   ++launches_;
+  if (!captured_) {
+    if (err == cudaSuccess) err = cudaEventRecord(state_->idle, st);
+    state_->last = st;
+    state_->ran = err == cudaSuccess;
+  }
   return err == cudaSuccess ? BBP_OK : BBP_ECUDA;
 }
 

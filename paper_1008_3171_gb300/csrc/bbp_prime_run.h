@@ -25,7 +25,9 @@ void release_prime_state(PrimeState** state);
 // Waits for what runs on the workspace's own streams, beside the caller's (NULL: nothing).
 void wait_prime_state(PrimeState* state);
 
-// One query on one workspace and one stream: begin, every list in order, finish.
+// One query on one workspace and one stream: begin, every list in order, finish.  Runs on a
+// workspace follow one another, on whatever streams; captured ones are ordered by who replays
+// them.
 class PrimeRun {
  public:
   // The query at position n, W working bits, into `slots` (to which the terms that the
@@ -52,6 +54,7 @@ class PrimeRun {
   };
   PrimeState* state_ = nullptr;
   int sms_ = 0, lmax_ = 0, formula_ = 0;
+  bool captured_ = false;
   uint32_t base_to_ = 0;
   uint64_t e_ = 0, launches_ = 0;
   PrimeArgs args_{};

@@ -476,7 +476,26 @@ void beside_a_capture() {
   }
 }
 
+// Queries on one stream after another, with captured ones between them: none sieves before
+// those before it have used the workspace.
+void runs_follow_one_another() {
+  Caller c;
+  auto uses = [](const Op& o) { return o.what == "base" || o.what == "sieve" || o.what == "primes" || o.what == "check"; };
+  for (cudaStream_t s : {c.a, c.b, c.b, c.a, c.b}) {
+    const size_t first = ops.size();
+    REQUIRE(c.async(1'000'000'000, s) == BBP_OK);
+    size_t sieve = first;
+    while (ops[sieve].what != "sieve") ++sieve;
+    const std::vector<bool> ended = before(static_cast<long>(sieve));
+    for (size_t i = 0; i < first; ++i) REQUIRE(ended[i] || ops[i].captured || !uses(ops[i]));
+    begin_capture(c.a);
+    REQUIRE(c.async(1'000'000'000, c.a) == BBP_OK);
+    end_capture();
+  }
+}
+
 const std::map<std::string, void (*)()> kCases = {
+    {"runs_follow_one_another", runs_follow_one_another},
     {"beside_a_capture", beside_a_capture},
     {"failed_iteration_leaves_nothing", failed_iteration_leaves_nothing},
     {"unplanned_query_fails", unplanned_query_fails},
