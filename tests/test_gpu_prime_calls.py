@@ -65,3 +65,13 @@ def test_beside_a_capture_of_another_stream(bbp, plans):  # noqa: F811
         assert (value(outs[i], P), int(valid[i])) == by_terms(bbp, plans[64], n, P)
     del graph
     plan.close()
+
+
+def test_primes_past_the_half_reduced_ladder(bbp, plans, pins):  # noqa: F811
+    """Primes past 1.02e12 take the plain two-word ladder: the printed row at 1e13 + 1 by Eq. 2
+    (half a minute), and Eq. 1, whose moduli reach 2 n, against Eq. 2 at 6e11."""
+    row = pins["table2_m13"]
+    want = int(row["hex"], 16) >> (len(row["hex"]) * 4 - 256)
+    assert plans[64].bits(10**13 + 1, 256) == (want, 256)
+    n = 6 * 10**11 + 7
+    assert plans[64].bits(n, 128, 1) == plans[64].bits(n, 128)
