@@ -294,6 +294,13 @@ bbp_status launch_one(bbp_plan p, int f, uint64_t n, uint32_t W, uint32_t P, con
   return BBP_OK;
 }
 
+// A range that crosses the line between two ladders is split where that pays: a second launch
+// costs some 13 us (600,000 terms across 2^47: 70 us in one, 72 to 85 in two; across 1.02e12 58, 61
+// to 73), and the cheaper ladder saves 9 to 17 % of its part.  From 2^21 terms on two are as fast
+// or faster (3e6 terms across 2^47: 199 to 236 us, 255 before the ladders), with few terms below
+// the line one (1000 of 4e6: 292, 306 in two).
+constexpr uint64_t kSplitTerms = 1u << 21, kSplitBelow = 1u << 17;
+
 // Launches every range of `ranges` (all of one query, same W) into `slots`.
 bbp_status launch_ranges(bbp_plan p, int f, uint64_t n, uint32_t W, const std::vector<TermRange>& ranges,
                          unsigned long long* slots, cudaStream_t st, const uint32_t* gate) {
@@ -323,7 +330,7 @@ bbp_status launch_ranges(bbp_plan p, int f, uint64_t n, uint32_t W, const std::v
       const uint64_t top = r.path == 1 ? kHalfMaxModulus : (1ull << (kSmallMaxBits + 1)) - 1;
       const uint64_t first_above = top < s.b ? 0 : (top - s.b) / s.a + 1;  // first k past `top`
       const uint64_t below = first_above > r.k_begin ? std::min(r.count, first_above - r.k_begin) : 0;
-      if (below > 0) {
+      if (below == r.count || (below >= kSplitBelow && r.count >= kSplitTerms)) {
         parts[0].count = below;
         parts[1].k_begin = r.k_begin + below;
         parts[1].count = r.count - below;

@@ -5,6 +5,7 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
+#include <array>
 #include <cmath>
 #include <cstdio>
 #include <cstdlib>
@@ -494,7 +495,26 @@ void runs_follow_one_another() {
   }
 }
 
+// A range across the line between two ladders is one launch while it is short, two when it is
+// long enough on both sides.
+void short_ranges_stay_whole() {
+  Caller c;
+  uint32_t limbs[10];
+  for (uint64_t line : {kHalfMaxModulus, uint64_t{1} << 47}) {
+    const uint64_t k = (line - 1) / 10 + 1;  // first k of series 10 k + 1 past it
+    for (auto [below, above, launches] : {std::array<uint64_t, 3>{700, 700, 1}, {1000, 599'000, 1}, {1'000'000, 1'000'000, 1},
+                                          {1000, 5'000'000, 1}, {1'500'000, 1'500'000, 2}, {5'000'000, 0, 1}, {0, 5'000'000, 1}}) {
+      const size_t first = ops.size();
+      REQUIRE(bbp_partial_sum(c.plan, BBP_BELLARD, 0, k - below, k + above, 100 * line, 256, limbs) == BBP_OK);
+      uint64_t heads = 0;
+      for (size_t i = first; i < ops.size(); ++i) heads += ops[i].what == "head";
+      REQUIRE(heads == launches);
+    }
+  }
+}
+
 const std::map<std::string, void (*)()> kCases = {
+    {"short_ranges_stay_whole", short_ranges_stay_whole},
     {"runs_follow_one_another", runs_follow_one_another},
     {"beside_a_capture", beside_a_capture},
     {"failed_iteration_leaves_nothing", failed_iteration_leaves_nothing},
