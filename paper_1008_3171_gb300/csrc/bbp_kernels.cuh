@@ -86,6 +86,16 @@ constexpr int kNumPaths = 4;
 // bits up to kHalfMaxModulus, and moduli of 47 bits.
 constexpr int kPathHalf = 4, kPath47 = 5;
 constexpr uint64_t kHalfMaxModulus = 1'020'000'000'000;
+// And two kernels of 10 limbs for long ranges of paths 1 and kPath47: the gated ones, for which
+// the compiler takes 102 and 104 registers, two CTAs an SM, in the place of 80 and three (1e8
+// terms: 4.80 against 4.86 and 5.22 against 5.33 ms; 450,000 terms: 57 against 51 us, 600,000: 57
+// against 68).
+constexpr int kPathRoomy = 6, kPathRoomy47 = 7;
+constexpr uint64_t kRoomyTerms = 1u << 19;
+inline int roomy_path(int path, int streams, int lmax, uint64_t count) {
+  if (lmax != 10 || streams != 2 || count < kRoomyTerms) return path;
+  return path == 1 ? kPathRoomy : path == kPath47 ? kPathRoomy47 : path;
+}
 constexpr int kQueueVariants = kNumLmaxClasses * kNumPaths;  // limb class x modulus path
 
 // ---------------------------------------------------------------- batches
@@ -139,7 +149,7 @@ struct PrimeArgs {
 // Launch helpers (defined in bbp_kernels.cu).  They return cudaGetLastError().
 // path: 0 = one-word moduli, bitlen <= 29; 1 = two-word moduli, bitlen <= 46;
 //       2 = two-word moduli, bitlen <= 60; 3 = one-word moduli of 30 or 31 bits;
-//       kPathHalf, kPath47.
+//       kPathHalf, kPath47, kPathRoomy, kPathRoomy47.
 // threads: CTA size, a multiple of 32 in [32, kHeadThreads] (else cudaErrorInvalidValue).
 cudaError_t launch_head(const HeadArgs& a, int path, int streams, int lmax, int blocks, cudaStream_t s,
                         int threads = kHeadThreads);

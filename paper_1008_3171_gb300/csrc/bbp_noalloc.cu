@@ -116,6 +116,7 @@ extern "C" bbp_status bbp_partial_sum_noalloc(bbp_formula f, uint32_t denominato
       const int streams = path == 1 || path >= kPathHalf ? 2 : 1;
       window_params(path >= kPathHalf ? 1 : path, lbits, &window, &first, &first_max);
       if (path >= kPathHalf) window = 4;
+      path = roomy_path(path, streams, lmax, ke - kb);
       HeadArgs a{};
       a.d = d;
       a.k_begin = kb;

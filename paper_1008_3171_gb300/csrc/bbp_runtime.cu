@@ -343,12 +343,12 @@ bbp_status launch_ranges(bbp_plan p, int f, uint64_t n, uint32_t W, const std::v
     }
     for (int i = 0; i < 2; ++i) {
       const TermRange& part = parts[i];
-      const int path = paths[i];
       if (part.count == 0) continue;
       HeadArgs a = head_args(F, part, n, W);
       a.slots = slots;
       a.gate = gate;
-      const int streams = head_streams(p, path);
+      const int streams = head_streams(p, paths[i]);
+      const int path = roomy_path(paths[i], streams, lmax, part.count);
       const int warps_per_block = p->cta / 32;
       const int occ = head_occupancy(path, streams, lmax, p->cta);
       const uint64_t resident_warps = static_cast<uint64_t>(occ) * p->sm_count * warps_per_block;

@@ -364,12 +364,14 @@ __device__ __forceinline__ void flush_cta(uint32_t (&acc)[LMAX], uint32_t L, uns
 }
 
 // The half-reduced ladder with two term pairs a thread is held to 80 registers, three CTAs
-// an SM (7.35 against 7.58 ms on its slice); the others are faster with the 102 the compiler
-// takes, and two (8.58 against 8.89 ms on 43-bit moduli).
-template <int LMAX, int PATH, int S, Ladder LADDER = kLadderPlain>
+// an SM (7.35 against 7.58 ms on its slice).  GATED: nothing is done when *A.gate is 0.  The
+// test is a template's because its early return costs the ladders up to 2 % by what the
+// compiler then makes of them (P = 128, 41-bit moduli, 1e8 terms: 4.71 ms without, 4.79 with),
+// or saves as much; launch_head (bbp_inst.cuh) takes the faster one.
+template <int LMAX, int PATH, int S, Ladder LADDER = kLadderPlain, bool GATED = false>
 __global__ void __launch_bounds__(kHeadThreads, LADDER == kLadderHalf && S == 2 && LMAX <= 16 ? 3 : 0)
 head_kernel(const HeadArgs A, const uint64_t ntiles) {
-  if (A.gate && *A.gate == 0u) return;
+  if (GATED && A.gate && *A.gate == 0u) return;
   const uint32_t lane = threadIdx.x & 31u;
   const uint64_t warp = (static_cast<uint64_t>(blockIdx.x) * blockDim.x + threadIdx.x) >> 5;
   const uint64_t nwarps = (static_cast<uint64_t>(gridDim.x) * blockDim.x) >> 5;

@@ -33,3 +33,18 @@ def test_ranges_at_a_line(plan, line, n, formula, j):
         P = (64, 256, 100)[i % 3]
         assert plan.partial_sum(formula, j, k - below, k + above, n, P) == \
             oracle.c_partial_sum(formula, j, k - below, k + above, n, P, 64), (below, above, P)
+
+
+@pytest.mark.parametrize("streams", [0, 1])
+@pytest.mark.parametrize("P", [256, 170, 64])
+def test_kernels_of_ten_limbs_by_length(P, streams, tmp_path):
+    """Moduli of 42 and 47 bits, at the length from which ranges of 10 limbs take other kernels."""
+    import paper_1008_3171_gb300 as bbp
+
+    table = tmp_path / "tune.json"
+    table.write_text('{"streams": %d}' % streams if streams else "{}")
+    with bbp.Plan(device=0, guard_bits=64, tune_table=str(table)) as p:
+        for m, n in ((3 * 10**12, 10**14 + 1), (10**14, 10**15)):
+            for count in (2**19 - 1, 2**19):
+                k = m // 10 + count
+                assert p.partial_sum(0, 0, k, k + count, n, P) == oracle.c_partial_sum(0, 0, k, k + count, n, P, 64)
