@@ -86,6 +86,10 @@ constexpr int kNumPaths = 4;
 // bits up to kHalfMaxModulus, and moduli of 47 bits.
 constexpr int kPathHalf = 4, kPath47 = 5;
 constexpr uint64_t kHalfMaxModulus = 1'020'000'000'000;
+// Ranges of 47-bit moduli take kPath47 from here on, where path 2 has a CTA for each of 152 SMs.
+// kPath47's threads have four terms each, path 2's two: a shorter range lasts longer there (60,000
+// terms, P = 256: 33.8 us, on path 2 30.7; 100,000: 34.1 and 35.5).
+constexpr uint64_t k47Terms = 76u << 10;
 // And two kernels of 10 limbs for long ranges of paths 1 and kPath47: the gated ones, for which
 // the compiler takes 102 and 104 registers, two CTAs an SM, in the place of 80 and three (1e8
 // terms: 4.80 against 4.86 and 5.22 against 5.33 ms; 450,000 terms: 57 against 51 us, 600,000: 57

@@ -111,7 +111,7 @@ extern "C" bbp_status bbp_partial_sum_noalloc(bbp_formula f, uint32_t denominato
       int path = path_for_bits(lbits);
       uint8_t window, first, first_max;
       const bool half = path == 1 && static_cast<uint64_t>(s.a) * (ke - 1) + s.b <= kHalfMaxModulus;
-      if (path == 2 && lbits == kSmallMaxBits + 1) path = kPath47;
+      if (path == 2 && lbits == kSmallMaxBits + 1 && ke - kb >= k47Terms) path = kPath47;
       if (half) path = kPathHalf;
       const int streams = path == 1 || path >= kPathHalf ? 2 : 1;
       window_params(path >= kPathHalf ? 1 : path, lbits, &window, &first, &first_max);

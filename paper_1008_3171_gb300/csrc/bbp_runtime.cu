@@ -330,7 +330,8 @@ bbp_status launch_ranges(bbp_plan p, int f, uint64_t n, uint32_t W, const std::v
       const uint64_t top = r.path == 1 ? kHalfMaxModulus : (1ull << (kSmallMaxBits + 1)) - 1;
       const uint64_t first_above = top < s.b ? 0 : (top - s.b) / s.a + 1;  // first k past `top`
       const uint64_t below = first_above > r.k_begin ? std::min(r.count, first_above - r.k_begin) : 0;
-      if (below == r.count || (below >= kSplitBelow && r.count >= kSplitTerms)) {
+      const bool whole = below == r.count && (r.path == 1 || r.count >= k47Terms);
+      if (whole || (below >= kSplitBelow && r.count >= kSplitTerms)) {
         parts[0].count = below;
         parts[1].k_begin = r.k_begin + below;
         parts[1].count = r.count - below;

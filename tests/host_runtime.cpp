@@ -257,7 +257,11 @@ int head_lmax_for(int L, int bump) {
 int head_occupancy(int, int, int, int) { return 2; }
 int query_occupancy(int, int, int) { return 2; }
 int queue_occupancy(int, int, int) { return 2; }
-cudaError_t launch_head(const HeadArgs& a, int, int, int, int, cudaStream_t s, int) { return add(s, "head", {a.slots}); }
+std::vector<int> head_paths;
+cudaError_t launch_head(const HeadArgs& a, int path, int, int, int, cudaStream_t s, int) {
+  head_paths.push_back(path);
+  return add(s, "head", {a.slots});
+}
 cudaError_t launch_tail_set(const TailSet&, cudaStream_t s) { return add(s, "tails"); }
 cudaError_t launch_query(const QuerySet& q, int, int, int, int, cudaStream_t s) { return add(s, "query", {q.slots}); }
 cudaError_t launch_zero_slots(unsigned long long* p, int, cudaStream_t s, const uint32_t*) { return add(s, "zero", {p}); }
@@ -513,7 +517,20 @@ void short_ranges_stay_whole() {
   }
 }
 
+// Ranges of 47-bit moduli that leave SMs idle stay on the four-word path.
+void short_47_bit_ranges() {
+  Caller c;
+  uint32_t limbs[6];
+  for (auto [count, path] : {std::array<int, 2>{1000, 2}, {77'000, 2}, {78'000, kPath47}, {2'000'000, kPath47}}) {
+    head_paths.clear();
+    const uint64_t k = (uint64_t{1} << 46) / 10 + 10;
+    REQUIRE(bbp_partial_sum(c.plan, BBP_BELLARD, 0, k, k + static_cast<uint64_t>(count), 1'000'000'000'000'000, 128, limbs) == BBP_OK);
+    REQUIRE(head_paths == std::vector<int>{path});
+  }
+}
+
 const std::map<std::string, void (*)()> kCases = {
+    {"short_47_bit_ranges", short_47_bit_ranges},
     {"short_ranges_stay_whole", short_ranges_stay_whole},
     {"runs_follow_one_another", runs_follow_one_another},
     {"beside_a_capture", beside_a_capture},

@@ -27,7 +27,7 @@ def plan():
 def test_ranges_at_a_line(plan, line, n, formula, j):
     s = o1.FORMULAS[formula].series[j]
     k = (line - s.b) // s.a + 1            # first k past the line
-    for i, (below, above) in enumerate([(700, 0), (0, 700), (1, 1), (701, 4000), (4000, 701),
+    for i, (below, above) in enumerate([(700, 0), (0, 700), (1, 1), (701, 4000), (4000, 701), (76 * 1024 - 1, 0), (76 * 1024, 0),
                                         (BELOW, TERMS - BELOW - 1), (BELOW - 1, TERMS - BELOW + 1),
                                         (BELOW, TERMS - BELOW), (TERMS - 1, 1), (TERMS, 0), (0, TERMS)]):
         P = (64, 256, 100)[i % 3]
