@@ -225,6 +225,11 @@ uint32_t run_for(uint32_t run, uint64_t resident_warps, F count_tiles) {
 
 }  // namespace
 
+// Of 40 limbs no more head terms go into one launch: its kernel is 5 to 18 % slower a term than the
+// ranges' own, which pays for eight launches up to n = 2e7 (P = 1000: 562 us in one, 579 in nine; 4e7:
+// 1124 and 1057; 5e8: 14.6 and 12.3 ms).  Of fewer limbs one launch is the faster one throughout.
+constexpr uint64_t kOneLaunchTerms40 = 20'000'000;
+
 // Queues a whole query as one launch if all its head ranges are on modulus path 0 (n up
 // to 2^29); *done says whether it did.
 bbp_status launch_one(bbp_plan p, int f, uint64_t n, uint32_t W, uint32_t P, const std::vector<TermRange>& ranges,
@@ -234,10 +239,13 @@ bbp_status launch_one(bbp_plan p, int f, uint64_t n, uint32_t W, uint32_t P, con
   const int lmax = pick_lmax(W, p->limb_bump);
   if (lmax == 0) return BBP_EINVAL;
   uint32_t heads = 0, tails = 0;
+  uint64_t head_terms = 0;
   for (const TermRange& r : ranges) {
     if (!r.tail && r.path != 0) return BBP_OK;
     ++(r.tail ? tails : heads);
+    head_terms += r.tail ? 0 : r.count;
   }
+  if (lmax == 40 && head_terms > kOneLaunchTerms40) return BBP_OK;
   if (heads > static_cast<uint32_t>(kMaxQueryRanges) || tails > static_cast<uint32_t>(kMaxTailSet)) return BBP_OK;
   QuerySet q{};
   q.slots = p->d_query;

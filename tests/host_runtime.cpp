@@ -529,7 +529,24 @@ void short_47_bit_ranges() {
   }
 }
 
+// Whole queries term by term (the raw sum wanted): one launch, but for many terms of 40 limbs.
+void one_launch_by_size() {
+  Caller c;
+  void* limbs;
+  cudaMalloc(&limbs, 256);
+  for (auto [n, P, one] : {std::array<uint64_t, 3>{20'000'000, 1000, 1}, {40'000'000, 1000, 0}, {500'000'000, 1000, 0},
+                           {500'000'000, 700, 1}, {500'000'000, 256, 1}}) {
+    const size_t first = ops.size();
+    REQUIRE(bbp_bits_async(c.plan, BBP_BELLARD, n, static_cast<uint32_t>(P), static_cast<uint8_t*>(c.out), nullptr,
+                           static_cast<uint32_t*>(limbs), c.a) == BBP_OK);
+    size_t queries = 0, heads = 0;
+    for (size_t i = first; i < ops.size(); ++i) queries += ops[i].what == "query", heads += ops[i].what == "head";
+    REQUIRE(queries == one && (heads == 0) == (one == 1));
+  }
+}
+
 const std::map<std::string, void (*)()> kCases = {
+    {"one_launch_by_size", one_launch_by_size},
     {"short_47_bit_ranges", short_47_bit_ranges},
     {"short_ranges_stay_whole", short_ranges_stay_whole},
     {"runs_follow_one_another", runs_follow_one_another},
