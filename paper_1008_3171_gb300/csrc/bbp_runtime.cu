@@ -230,6 +230,18 @@ uint32_t run_for(uint32_t run, uint64_t resident_warps, F count_tiles) {
 // 1124 and 1057; 5e8: 14.6 and 12.3 ms).  Of fewer limbs one launch is the faster one throughout.
 constexpr uint64_t kOneLaunchTerms40 = 20'000'000;
 
+// The same on path 2 up to 10 limbs, whose threads have two terms, four CTAs an SM, and start a
+// run in a third of a term's time: the longest run that fills the resident warps, unless the
+// shorter ones' rounds, the last one whole, are less work (P = 256: 1e6 terms 97 us by this, 103 by
+// shorter runs; 3e6 terms 268 and 233).  Of more limbs the shorter ones are the faster throughout.
+template <typename F>
+uint32_t run_for_path2(uint32_t run, uint64_t resident_warps, F count_tiles) {
+  const uint32_t fine = run_for(run, resident_warps, count_tiles);
+  while (run % 4 == 0 && count_tiles(run) < resident_warps) run /= 2;
+  auto work = [&](uint32_t r) { return (count_tiles(r) + resident_warps - 1) / resident_warps * (3 * r + 1); };
+  return 49 * work(run) <= 50 * work(fine) ? run : fine;
+}
+
 // Queues a whole query as one launch if all its head ranges are on modulus path 0 (n up
 // to 2^29); *done says whether it did.
 bbp_status launch_one(bbp_plan p, int f, uint64_t n, uint32_t W, uint32_t P, const std::vector<TermRange>& ranges,
@@ -364,7 +376,8 @@ bbp_status launch_ranges(bbp_plan p, int f, uint64_t n, uint32_t W, const std::v
       // a short range takes fewer consecutive terms per stream, so that its tiles
       // spread over the GPU's resident warps instead of a few warps running long runs
       auto tiles_for = [&](uint32_t rn) { return (part.count + 32ull * streams * rn - 1) / (32ull * streams * rn); };
-      const uint32_t run = run_for(static_cast<uint32_t>(p->run), resident_warps, tiles_for);
+      const uint32_t run = path == 2 && lmax <= 10 ? run_for_path2(static_cast<uint32_t>(p->run), resident_warps, tiles_for)
+                                                   : run_for(static_cast<uint32_t>(p->run), resident_warps, tiles_for);
       a.run = run;
       const uint64_t ntiles = tiles_for(run);
       const uint64_t want = (ntiles + warps_per_block - 1) / warps_per_block;
