@@ -270,7 +270,9 @@ cudaError_t launch_finalize_bits(const unsigned long long* p, int, uint32_t, uin
                                  cudaStream_t s, const uint32_t*) {
   return add(s, "finalize", {p});
 }
-cudaError_t launch_queue(const BatchDev& b, uint32_t, uint32_t, unsigned long long*, int, int, int, int, cudaStream_t s) {
+std::vector<std::array<int, 2>> queues;  // tiles a hand-out, CTAs
+cudaError_t launch_queue(const BatchDev& b, uint32_t, uint32_t, unsigned long long*, int, int, int, int blocks, cudaStream_t s) {
+  queues.push_back({static_cast<int>(b.grab), blocks});
   return add(s, "queue", {b.accum});
 }
 cudaError_t launch_queue_tail(const BatchDev& b, uint32_t, uint32_t, unsigned long long*, int, cudaStream_t s) {
@@ -545,7 +547,25 @@ void one_launch_by_size() {
   }
 }
 
+// A small batch is spread over the SMs, a large one takes what fits, four tiles at a time.
+void small_groups_spread() {
+  Caller c;
+  std::vector<uint64_t> n(150, 1'000'000);
+  std::vector<uint32_t> P(150, 64);
+  std::vector<uint8_t> out(8 * 150);
+  for (auto [count, grab, least, most] : {std::array<int, 4>{1, 1, sms, 2 * sms}, {150, 4, 2 * sms, 2 * sms}}) {
+    queues.clear();
+    REQUIRE(bbp_bits_batch(c.plan, BBP_BBP, static_cast<uint32_t>(count), n.data(), P.data(), out.data(), 8, nullptr, nullptr) == BBP_OK);
+    REQUIRE(queues.size() == 1 && queues[0][0] == grab && queues[0][1] >= least && queues[0][1] <= most);
+  }
+  n[0] = 60;  // a handful of terms: a CTA for each tile
+  queues.clear();
+  REQUIRE(bbp_bits_batch(c.plan, BBP_BBP, 1, n.data(), P.data(), out.data(), 8, nullptr, nullptr) == BBP_OK);
+  REQUIRE(queues.size() == 1 && queues[0][0] == 1 && queues[0][1] >= 1 && queues[0][1] < 32);
+}
+
 const std::map<std::string, void (*)()> kCases = {
+    {"small_groups_spread", small_groups_spread},
     {"one_launch_by_size", one_launch_by_size},
     {"short_47_bit_ranges", short_47_bit_ranges},
     {"short_ranges_stay_whole", short_ranges_stay_whole},

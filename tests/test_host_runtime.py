@@ -44,7 +44,7 @@ def program(tmp_path_factory):
                                   "failed_batch_leaves_nothing", "unplanned_query_fails",
                                   "failed_iteration_leaves_nothing", "beside_a_capture",
                                   "runs_follow_one_another", "short_ranges_stay_whole",
-                                  "short_47_bit_ranges", "one_launch_by_size"])
+                                  "short_47_bit_ranges", "one_launch_by_size", "small_groups_spread"])
 def test_case(program, case):
     r = subprocess.run([program, case], capture_output=True, text=True, timeout=120)
     assert r.returncode == 0, r.stdout + r.stderr
