@@ -80,9 +80,9 @@ typedef struct bbp_plan_opts {
 
 /* Counters of the most recent compute call on a plan. */
 typedef struct bbp_stats {
-  uint64_t terms;           /* terms evaluated (head + tail) */
-  uint64_t head_terms;      /* head terms (modular exponentiations) */
-  uint64_t head_launches;   /* head-kernel launches */
+  uint64_t terms;           /* terms of the sum (head + tail), evaluated one by one or summed by primes */
+  uint64_t head_terms;      /* head terms (term by term: modular exponentiations) */
+  uint64_t head_launches;   /* launches of head kernels, or of the sum by primes */
   uint64_t kernel_launches; /* all kernel launches */
   double imad_model;        /* 32-bit integer multiplies the evaluation needs (model), term by term or, for
                                a whole query summed by primes, by that form */
@@ -132,7 +132,12 @@ bbp_status bbp_partial_sum_async(bbp_plan p, bbp_formula f, uint32_t denominator
  * bits to spare are summed over the primes up to n instead of over the terms (partial
  * fractions of the moduli); the sum is checked on the device, and where it is too close
  * to a carry to have the term-by-term sum's bits for certain, the terms are summed.  The
- * bits and the certified count are the term-by-term ones in every case.  out: caller-owned ceil(P/8) host bytes, MSB first.
+ * bits and the certified count are the term-by-term ones in every case.
+ * The first such query of a plan makes its buffers, a larger one longer lists: two of up to
+ * 96 MiB and 12 MiB beside them, until the plan is destroyed (a captured query's lists are
+ * kept too).  Batches and the serving engine make four workspaces of up to 61 MiB each of
+ * their own.  Where they cannot be had the terms are summed.
+ * out: caller-owned ceil(P/8) host bytes, MSB first.
  * valid_bits (may be NULL): how many leading bits the guard-bit error bound certifies
  * (|S - exact| < N + J + 1 units for N evaluated terms and J series).  Blocks. */
 bbp_status bbp_bits(bbp_plan p, uint64_t n, uint32_t P, uint8_t* out, uint32_t* valid_bits);
@@ -144,7 +149,10 @@ bbp_status bbp_bits_formula(bbp_plan p, bbp_formula f, uint64_t n, uint32_t P, u
 /* Device-pointer form: d_out (ceil(P/8) bytes), d_valid (one uint32, may be NULL)
  * and d_limbs (W/32 uint32 of the raw sum, may be NULL) are caller-owned device
  * memory; returns once queued on `stream` (NULL: the plan's stream).  With d_limbs the
- * terms are summed one by one (the raw sum holds every term's rounding).
+ * terms are summed one by one (the raw sum holds every term's rounding).  Summed over
+ * primes, a query is three launches for every 20 million primes (some 5,700 at n = 1e12), which
+ * may hold the host for most of its run, and the term kernels behind them, which return at
+ * once; making or enlarging the buffers (see bbp_bits) waits for the device.
  * Under stream capture the call allocates nothing: a plan without the buffers that the sum
  * over primes needs at this n (a query of the same n or a larger one makes them) has the
  * terms captured.  The graph may be replayed until the plan is destroyed, whatever the

@@ -1,7 +1,7 @@
 // Runs the prime form of a query's head sum (bbp_primes.h) on a plan: base primes, the
 // prime powers with long sums, then the primes up to n in lists of bounded length, each
-// sieved and summed.  One list buffer and one stream: a list's kernels end before the
-// next is sieved.
+// sieved and summed.  Two list buffers and three streams: the caller's stream sums a list
+// while the next is sieved on a second one, and the prime powers run on a third.
 //
 // Measured on a GB300, whole bbp_bits calls, term by term -> by primes: n = 1e9, P = 128:
 // 15.6 -> 1.75 ms; n = 1e9, P = 64 by Eq. 1: 20.5 -> 2.54 ms; n = 3e8, P = 1000:

@@ -103,7 +103,7 @@ std::vector<PrimeClass> prime_classes(const PrimeLimits& lim);
 
 // Whether the prime form serves this query: position in range, and the error bound
 // small enough against the guard bits that its result is almost always certain to
-// equal the term-by-term one (see prime_check in bbp_primes.cu).
+// equal the term-by-term one (see launch_prime_check in bbp_sieve.cuh).
 bool prime_form_serves(int formula, uint64_t n, uint32_t P, uint32_t W, uint64_t bound);
 
 // 32-bit product halves the prime form multiplies for a query of `limbs` limbs (a model,

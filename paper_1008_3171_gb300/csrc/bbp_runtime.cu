@@ -395,7 +395,6 @@ bbp_status launch_ranges(bbp_plan p, int f, uint64_t n, uint32_t W, const std::v
       p->stats.head_launches++;
       p->stats.terms += part.count;
       p->stats.head_terms += part.count;
-    
     }
     p->stats.imad_model += r.imad;
   }
@@ -424,10 +423,6 @@ bbp_status plan_query(bbp_plan p, int f, uint64_t n, uint32_t W, int j_only, uin
 }
 
 }  // namespace bbp
-
-extern "C" {
-
-}  // extern "C"
 
 namespace {
 
