@@ -5,8 +5,8 @@
 //
 // Measured on a GB300, whole bbp_bits calls, term by term -> by primes: n = 1e9, P = 128:
 // 15.6 -> 1.75 ms; n = 1e9, P = 64 by Eq. 1: 20.5 -> 2.54 ms; n = 3e8, P = 1000:
-// 7.88 -> 0.91 ms; n = 4e10, P = 256: 1005 -> 82.4 ms.  At 4e10 the kernels one after
-// another: 58 ms primes above A / 23, 14.2 those below, 4.0 prime powers, 13.9 sieve.
+// 7.88 -> 0.91 ms; n = 4e10, P = 256: 1005 -> 82.3 ms.  At 4e10 the kernels one after
+// another: 56.1 ms primes above A / 23, 14.3 those below, 4.0 prime powers, 13.9 sieve.
 #include <cuda_runtime.h>
 
 #include <algorithm>
