@@ -230,7 +230,7 @@ uint32_t run_for(uint32_t run, uint64_t resident_warps, F count_tiles) {
 // 1124 and 1057; 5e8: 14.6 and 12.3 ms).  Of fewer limbs one launch is the faster one throughout.
 constexpr uint64_t kOneLaunchTerms40 = 20'000'000;
 
-// The same on path 2 up to 10 limbs, whose threads have two terms, four CTAs an SM, and start a
+// run_for on path 2 up to 10 limbs, whose threads have two terms, four CTAs an SM, and start a
 // run in a third of a term's time: the longest run that fills the resident warps, unless the
 // shorter ones' waves, the last one whole, are less work (P = 256: 1e6 terms 97 us by this, 103 by
 // shorter runs; 3e6 terms 268 and 233).  Of more limbs the shorter ones are the faster throughout.
